@@ -12,13 +12,12 @@
 //                 the item's last block O / l -> bf16 -> global memory
 //     warps 4-7   the same for slot 1
 //     warp 8      TMA producer of the K / V ring (all lanes in lock step, one elected lane issues)
-//     warp 9      MMA scheduler (likewise): checks ahead of time that K / V, Q and O of each visit are in
-//                 place and queues the visit for the issuer; owns the TMEM allocation
+//     warp 9      owns the TMEM allocation
 //     warp 10     TMA producer of the Q tiles (likewise)
-//     warp 11     MMA issuer (likewise): waits for P of the queued visit and issues its MMAs; P V starts on
+//     warp 11     MMA issuer (likewise): waits for K / V, Q, O and P of each visit and issues its MMAs; P V starts on
 //                 the leading key columns while the softmax still works on the last 32
 // TMEM columns: S/P of slot 0, S/P of slot 1, O of slot 0, O of slot 1 (128 columns each).
-// The MMA scheduler visits the slots alternately; a visit issues P V of the slot's previous block and
+// The MMA issuer visits the slots alternately; a visit issues P V of the slot's previous block and
 // then Q K^T of its next block (P overwrites S, so the order inside a visit is fixed).  The K / V
 // producer walks the same visit sequence, so one shared ring serves both slots in order.  A slot's
 // items follow each other without a gap: Q K^T of the next item's first block is issued right
@@ -53,7 +52,6 @@ constexpr int kQBufsMax = 3;                             // Q tiles: one per slo
 constexpr int kSlotBytes = 32 * 1024;
 constexpr int kQBytes = 32 * 1024;
 constexpr int kTmemCols = 512;
-constexpr int kCmdSlots = 4;
 constexpr int kSpareQMaxList = 256;                      // longest list (blocks) served with the spare Q tile
 constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X; S/P at 128 X
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
@@ -62,11 +60,7 @@ constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after:
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4 };
 enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarCmdFull, kBarCmdEmpty, kBarPEarly };
-// One visit of the MMA issuer as a command word.
-enum Cmd : uint32_t { kCmdPv = 1u, kCmdQk = 2u, kCmdPvFirst = 4u, kCmdPvLast = 8u, kCmdQkLast = 16u, kCmdSlot1 = 32u,
-                      kCmdPPar = 64u,  // phase parity of p_ready the P V of this visit waits for
-                      kCmdExit = 0x80000000u };
+                   kBarDrain, kBarPEarly };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -82,10 +76,7 @@ struct Smem {
   static constexpr int o_full = p_early + 16;
   static constexpr int o_free = o_full + 16;
   static constexpr int drain = o_free + 16;
-  static constexpr int cmd_full = drain + 8;               // scheduler -> issuer command ring
-  static constexpr int cmd_empty = cmd_full + 8 * kCmdSlots;
-  static constexpr int cmd_word = cmd_empty + 8 * kCmdSlots;
-  static constexpr int tmem_ptr = cmd_word + 4 * kCmdSlots;
+  static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
   static constexpr int total = abort_flag + 4;
 };
@@ -136,28 +127,6 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
   return done;
 }
 
-// Up to four independent probes issued back to back (so their shared-memory round trips overlap);
-// a disabled probe (en == 0) counts as complete.  Returns 1 when every enabled barrier phase is done.
-__device__ __forceinline__ uint32_t mbar_try4(uint32_t b0, uint32_t p0, uint32_t e0, uint32_t b1, uint32_t p1, uint32_t e1,
-                                              uint32_t b2, uint32_t p2, uint32_t e2, uint32_t b3, uint32_t p3, uint32_t e3) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred q0, q1, q2, q3, r0, r1, r2, r3;\n\t"
-      "setp.ne.b32 q0, %3, 0;\n\tsetp.ne.b32 q1, %6, 0;\n\tsetp.ne.b32 q2, %9, 0;\n\tsetp.ne.b32 q3, %12, 0;\n\t"
-      "setp.eq.b32 r0, 0, 0;\n\tsetp.eq.b32 r1, 0, 0;\n\tsetp.eq.b32 r2, 0, 0;\n\tsetp.eq.b32 r3, 0, 0;\n\t"
-      "@q0 mbarrier.try_wait.parity.shared::cta.b64 r0, [%1], %2;\n\t"
-      "@q1 mbarrier.try_wait.parity.shared::cta.b64 r1, [%4], %5;\n\t"
-      "@q2 mbarrier.try_wait.parity.shared::cta.b64 r2, [%7], %8;\n\t"
-      "@q3 mbarrier.try_wait.parity.shared::cta.b64 r3, [%10], %11;\n\t"
-      "and.pred r0, r0, r1;\n\tand.pred r2, r2, r3;\n\tand.pred r0, r0, r2;\n\t"
-      "selp.u32 %0, 1, 0, r0;\n\t}"
-      : "=r"(done)
-      : "r"(b0), "r"(p0), "r"((uint32_t)e0), "r"(b1), "r"(p1), "r"((uint32_t)e1), "r"(b2), "r"(p2), "r"((uint32_t)e2),
-        "r"(b3), "r"(p3), "r"((uint32_t)e3)
-      : "memory");
-  return done;
-}
-
 struct Ctx {
   volatile int* abort_flag;  // shared memory
   int32_t* status;           // global memory status words
@@ -190,7 +159,38 @@ __device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, co
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const Ctx& c, int bar_id,
                                           uint64_t limit_ns = kWaitLimitNs) {
   if (mbar_try(bar, parity)) return true;
+  if (mbar_try(bar, parity)) return true;  // a second probe before the timer is read
   return mbar_wait_slow(bar, parity, c, bar_id, limit_ns);
+}
+
+// The issuer's form of the bounded wait: nothing but the probe and one branch when the phase is complete.  A wait that
+// gives up raises the CTA's abort flag and leaves `id` in `failed`, which the caller looks at when it is cheap to; what
+// it issues in between works on undefined data inside the CTA's own shared and tensor memory.
+__device__ __forceinline__ void mbar_wait_sticky(uint32_t bar, uint32_t parity, uint32_t abort_addr, int id, int& failed) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 f;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE_%=;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE_%=;\n\t"
+      "mov.u64 t0, %%globaltimer;\n\t"
+      "LOOP_%=:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE_%=;\n\t"
+      "ld.volatile.shared::cta.u32 f, [%3];\n\t"
+      "setp.ne.u32 p, f, 0;\n\t"
+      "@p bra FAIL_%=;\n\t"
+      "mov.u64 t1, %%globaltimer;\n\t"
+      "sub.u64 t1, t1, t0;\n\t"
+      "setp.le.u64 p, t1, %5;\n\t"
+      "@p bra LOOP_%=;\n\t"
+      "FAIL_%=:\n\t"
+      "mov.u32 %0, %4;\n\t"
+      "st.volatile.shared::cta.u32 [%3], 1;\n\t"
+      "DONE_%=:\n\t}"
+      : "+r"(failed)
+      : "r"(bar), "r"(parity), "r"(abort_addr), "r"(id), "l"(kWaitLimitNs)
+      : "memory");
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
@@ -355,6 +355,41 @@ struct ItemCursor {
   }
 };
 
+// The list lengths of one slot's items, in the ItemCursor's order, for the MMA issuer: the loads that lead to the length
+// of the next item are started an item ahead (the work entry two items ahead), so that next() waits for none of them.
+struct LengthCursor {
+  int idx, step;       // the item whose length `raw` is
+  int raw, h2, R2;     // length of item idx as loaded; work entry of item idx + step
+  int n;
+  __device__ __forceinline__ int length(const AttnArgs& a, int h, int R) const {
+    return a.sel_idx ? a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R] : a.rows.row_r[R] + 1;
+  }
+  __device__ __forceinline__ void entry(const AttnArgs& a, int i) {
+    const int j = min(i, a.n_items - 1);
+    h2 = a.work[2 * j];
+    R2 = a.work[2 * j + 1];
+  }
+  __device__ __forceinline__ void init(const AttnArgs& a, int slot) {
+    step = 2 * (int)gridDim.x;
+    idx = (int)blockIdx.x + slot * (int)gridDim.x;
+    entry(a, idx);
+    raw = length(a, h2, R2);
+    entry(a, idx + step);
+  }
+  // Moves to the next item with a non-empty list; false when the slot has no more items.
+  __device__ __forceinline__ bool next(const AttnArgs& a) {
+    do {
+      if (idx >= a.n_items) { n = 0; return false; }
+      n = uni(raw);
+      if (a.sel_idx) n = min(max(n, 0), a.k_max);
+      idx += step;
+      raw = length(a, h2, R2);
+      entry(a, idx + step);
+    } while (n == 0);
+    return true;
+  }
+};
+
 template <int BLK, bool kSpareQ>
 __global__ void __launch_bounds__(kThreads, 1)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -388,7 +423,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
     }
     mbar_init(bar(Smem::drain, 0), 1);
-    for (int i = 0; i < kCmdSlots; ++i) { mbar_init(bar(Smem::cmd_full, i), 1); mbar_init(bar(Smem::cmd_empty, i), 1); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -571,7 +605,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       ++ord;
     }
   } else {
-    // The three issuing roles run with all 32 lanes in lock step on warp-uniform values (loads are
+    // The issuing roles run with all 32 lanes in lock step on warp-uniform values (loads are
     // broadcast through lane 0), so that descriptors, coordinates and barrier addresses live in
     // uniform registers; only the TMA / MMA / commit instructions themselves are issued by one
     // elected lane.
@@ -632,7 +666,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       enter(s0); enter(s1);
       bool ok = true;
       // With the spare Q tile slot 1 starts half an item behind slot 0, so that the two slots' item boundaries (and
-      // their claims on the spare) do not fall together.  The scheduler skips the same visits.
+      // their claims on the spare) do not fall together.  The MMA issuer skips the same visits.
       const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;
       for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
         ok = visit(s0);
@@ -650,10 +684,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // ============================== Q producer ==============================
       Ctx ctx{abort_flag, a.status, kRoleQProducer};
       if constexpr (kSpareQ) {
-        // The two slots advance one block per scheduler iteration, so the iteration at which a slot's item ends is the
+        // The two slots advance one block per round of the MMA issuer, so the round at which a slot's item ends is the
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
         // next tile, loaded into the spare buffer long before it is wanted; the buffer the slot leaves becomes the
-        // spare once the last Q K^T of its item has read it.  The scheduler rotates the buffers by the same rule.
+        // spare once the last Q K^T of its item has read it.  The MMA issuer rotates the buffers by the same rule.
         ItemCursor c0, c1;
         c0.init(0); c1.init(1);
         bool has0 = c0.next(a), has1 = c1.next(a);
@@ -675,9 +709,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           q_odd ^= 1u << b;
           return true;
         };
-        uint32_t end0 = 0, end1 = 0;  // scheduler iteration at which the slot's latest loaded item ends
+        uint32_t end0 = 0, end1 = 0;  // round of the MMA issuer at which the slot's latest loaded item ends
         int buf0 = 0, buf1 = 1, spare = 2;
-        const uint32_t delay1 = has0 ? (uint32_t)c0.n / 2u : 0u;  // slot 1 starts this many iterations late
+        const uint32_t delay1 = has0 ? (uint32_t)c0.n / 2u : 0u;  // slot 1 starts this many rounds late
         if (has0) { ok = load_into(c0, buf0); end0 = (uint32_t)c0.n; has0 = c0.next(a); }
         if (ok && has1) { ok = load_into(c1, buf1); end1 = delay1 + (uint32_t)c1.n; has1 = c1.next(a); }
         while (ok && (has0 || has1)) {
@@ -740,72 +774,88 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           while (ord1 > 0 && !mbar_try(bar(Smem::q_full, 1), (ord1 - 1) & 1) && globaltimer() - t1 < 4000000ull) {}
         }
       }
-    } else if (warp == 9) {
-      // ============================== MMA scheduler ==============================
-      // Decides what the tensor core does next and checks ahead of time that it can be done (K / V
-      // and Q landed, O drained); the MMAs themselves are issued by warp 11 from a small command
-      // ring.  The scheduler runs ahead of the issuer, so that a visit's command is already waiting
-      // when the slot's softmax warps publish P: the issuer alone waits for P, and the path from
-      // "P stored" to "P V issued" is one barrier wake-up instead of a chain of book-keeping.
+    } else if (warp == 11) {
+      // ============================== MMA issuer ==============================
+      // Visits the slots in turn.  A visit issues O_X (+)= P V of the slot's previous block, then S_X = Q K^T of its
+      // next block (which overwrites the P just consumed), with the commits that publish them.
+      // This warp is what the tensor core waits for: a visit's 16 MMAs run 1024 cycles, only a few of them can be
+      // queued, and every instruction here competes with two softmax warps for issue.  So the waits cost a probe and
+      // a branch when there is nothing to wait for, a wait that gave up is looked at once per round, the MMA loops are
+      // unrolled and the list lengths are fetched an item ahead (LengthCursor).  Dense 16K tokens: 1234 TFLOP/s; rolled
+      // loops 1200; waits that return a flag and vote 1053; a second warp that checks ahead and queues commands 1197.
       Ctx ctx{abort_flag, a.status, kRoleMma};
-      volatile uint32_t* cmd_word = (volatile uint32_t*)(smem_gen + Smem::cmd_word);
-      uint32_t ci = 0, cpar = 0;  // next command slot and its phase
+      const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
+      enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {
-        ItemCursor cur;
-        bool has, pend, pend_first, pend_last;
-        int e;
-        uint32_t p_par, q_par, o_par;  // phase parities of p_ready, q_full, o_full / o_free
+        LengthCursor cur;
+        int left;                      // blocks of the current item whose Q K^T is still to come (0: no item left)
+        uint32_t st;                   // kPend: a P V is due, of its item's first (kFirst) / last (kLast) block;
+                                       // kNewItem: the next Q K^T is the first of its item
+        uint32_t p_par, q_par, o_par;  // phase parities of p_early / p_ready, q_full, o_full / o_free
         int qbuf;                      // Q buffer of the slot's current item
       };
       uint32_t ring = 0, ring_par = 0;  // next K / V ring slot to consume and its phase
       int q_spare = 2;      // kSpareQ: the buffer that receives the next item's tile, and per buffer (bit b) whether an
       uint32_t q_odd = 3u;  // odd number of items was assigned to it so far - the Q producer's rule, step for step
-      // One visit.  Every barrier the visit depends on is probed up front in one go (independent
-      // shared-memory operations in flight together); only a failed probe falls back to the bounded waits.
-      auto visit = [&](MmaSlot& s, const int X) -> bool {
-        const bool do_pv = s.pend, do_qk = s.has;
-        const uint32_t slot_v = ring, par_v = ring_par;
-        uint32_t slot_k = ring, par_k = ring_par;
-        if (do_pv && ++slot_k == kKvSlots) { slot_k = 0; par_k ^= 1; }
-        const bool need_o = do_pv && s.pend_first, need_q = do_qk && s.e == 0;
-        const bool last = do_qk && s.e == s.cur.n - 1;
-        const uint32_t all_done =
-            mbar_try4(bar(Smem::kv_full, slot_v), par_v, do_pv, bar(Smem::o_free, X), s.o_par ^ 1, need_o,
-                      bar(Smem::kv_full, slot_k), par_k, do_qk, bar(Smem::q_full, s.qbuf), s.q_par, need_q);
-        if (!__all_sync(0xffffffffu, all_done != 0)) {
-          bool ok = true;
-          if (do_pv) ok = mbar_wait(bar(Smem::kv_full, slot_v), par_v, ctx, kBarKvFull);
-          if (ok && need_o) ok = mbar_wait(bar(Smem::o_free, X), s.o_par ^ 1, ctx, kBarOFree);
-          if (ok && do_qk) ok = mbar_wait(bar(Smem::kv_full, slot_k), par_k, ctx, kBarKvFull);
-          if (ok && need_q) ok = mbar_wait(bar(Smem::q_full, s.qbuf), s.q_par, ctx, kBarQFull);
-          if (!__all_sync(0xffffffffu, ok)) return false;
-        }
-        // everything the visit needs is in place: hand it to the issuing warp
-        if (!__all_sync(0xffffffffu, mbar_wait(bar(Smem::cmd_empty, ci), cpar ^ 1, ctx, kBarCmdEmpty))) return false;
-        if (lane == 0) {
-          cmd_word[ci] = (do_pv ? kCmdPv : 0u) | (do_qk ? kCmdQk : 0u) | (s.pend_first ? kCmdPvFirst : 0u) |
-                         (s.pend_last ? kCmdPvLast : 0u) | (last ? kCmdQkLast : 0u) | (X ? kCmdSlot1 : 0u) |
-                         (s.p_par ? kCmdPPar : 0u) | (slot_v << 8) | (slot_k << 12) | ((uint32_t)s.qbuf << 16);
-          mbar_arrive(bar(Smem::cmd_full, ci));  // release: the word and everything observed above
-        }
-        __syncwarp();
-        if (++ci == kCmdSlots) { ci = 0; cpar ^= 1; }
-        if (do_pv) {
-          s.p_par ^= 1;
-          if (s.pend_last) s.o_par ^= 1;
-          s.pend = false;
-        }
-        ring = slot_k; ring_par = par_k;
-        if (do_qk) {
+      constexpr int kEarlySteps = (BLK / 32 - 1) * 2;  // 16-key steps of P V covered by p_early
+      const uint32_t abort_addr = smem_base + Smem::abort_flag;
+      int failed = 0;
+      auto visit = [&](MmaSlot& s, const int X) {
+        const uint32_t s_tmem = tmem_base + X * 128;
+        const uint32_t o_tmem = tmem_base + kOCol + X * 128;
+        const uint32_t st = s.st;
+        if (st & kPend) {
+          const uint32_t v_addr = smem_base + kKvOff + ring * kSlotBytes;
+          mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
+          if (st & kFirst) mbar_wait_sticky(bar(Smem::o_free, X), s.o_par ^ 1, abort_addr, kBarOFree, failed);
+          // P V starts on the leading key columns while the softmax still works on the last 32
+          mbar_wait_sticky(bar(Smem::p_early, X), s.p_par, abort_addr, kBarPEarly, failed);
+          tc_fence_after();
+          if (leader) {
+            const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
+#pragma unroll
+            for (int k = 0; k < kEarlySteps; ++k)
+              mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, (k == 0 && (st & kFirst)) ? 0u : 1u);
+          }
+          __syncwarp();
+          mbar_wait_sticky(bar(Smem::p_ready, X), s.p_par, abort_addr, kBarPReady, failed);
+          tc_fence_after();
+          if (leader) {
+            const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
+#pragma unroll
+            for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
+            tc_commit(bar(Smem::kv_empty, ring));
+            if (st & kLast) tc_commit(bar(Smem::o_full, X));
+          }
+          __syncwarp();
           if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
-          s.pend = true;
-          s.pend_first = s.e == 0;
-          s.pend_last = last;
+          s.p_par ^= 1;
+          if (st & kLast) s.o_par ^= 1;
+          s.st = st & kNewItem;
+        }
+        if (s.left > 0) {
+          mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
+          if (st & kNewItem) mbar_wait_sticky(bar(Smem::q_full, s.qbuf), s.q_par, abort_addr, kBarQFull, failed);
+          tc_fence_after();
+          const bool last = --s.left == 0;
+          if (leader) {
+            const uint64_t da = smem_desc(smem_base + Smem::q + s.qbuf * kQBytes, 16, 1024);
+            const uint64_t db = smem_desc(smem_base + kKvOff + ring * kSlotBytes, 16, 1024);
+#pragma unroll
+            for (int k = 0; k < kHeadDim / 16; ++k)  // 16 columns = 32 bytes on; the second four steps: the other 64-column half
+              mma_ss(s_tmem, da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4), db + (((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4),
+                     kIdescS, k > 0 ? 1u : 0u);
+            tc_commit(bar(Smem::kv_empty, ring));
+            tc_commit(bar(Smem::s_full, X));
+            if (last) tc_commit(bar(Smem::q_empty, s.qbuf));
+          }
+          __syncwarp();
+          if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
+          s.st = kPend | ((st & kNewItem) ? kFirst : 0u) | (last ? kLast | kNewItem : 0u);
           if (last) {
-            s.has = s.cur.next(a);
-            s.e = 0;
+            s.left = s.cur.next(a) ? s.cur.n : 0;
             if constexpr (kSpareQ) {
-              if (s.has) {  // the next item's tile is (or will be) in the spare buffer; this item's buffer becomes the spare
+              if (s.left > 0) {  // the next item's tile is (or will be) in the spare buffer; this item's buffer becomes the spare
                 const int old = s.qbuf;
                 s.qbuf = q_spare;
                 q_spare = old;
@@ -815,109 +865,24 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             } else {
               s.q_par ^= 1;
             }
-          } else {
-            ++s.e;
           }
         }
-        return true;
       };
       MmaSlot s0, s1;
-      s0.cur.init(0); s1.cur.init(1);
-      s0.has = s0.cur.next(a); s1.has = s1.cur.next(a);
-      s0.pend = s1.pend = s0.pend_first = s1.pend_first = s0.pend_last = s1.pend_last = false;
-      s0.e = s1.e = 0;
+      s0.cur.init(a, 0); s1.cur.init(a, 1);
+      s0.left = s0.cur.next(a) ? s0.cur.n : 0;
+      s1.left = s1.cur.next(a) ? s1.cur.n : 0;
+      s0.st = s1.st = kNewItem;
       s0.p_par = s1.p_par = s0.q_par = s1.q_par = s0.o_par = s1.o_par = 0;
       s0.qbuf = 0; s1.qbuf = 1;
-      bool ok = true;
-      const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;  // as in the K / V producer
-      for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
-        ok = visit(s0, 0);
-        if (ok && (!kSpareQ || it >= delay1)) ok = visit(s1, 1);
+      const uint32_t delay1 = kSpareQ ? (uint32_t)s0.left / 2u : 0u;  // as in the K / V producer
+      for (uint32_t it = 0; s0.left > 0 || s1.left > 0 || ((s0.st | s1.st) & kPend); ++it) {
+        visit(s0, 0);
+        if (!kSpareQ || it >= delay1) visit(s1, 1);
+        if (__any_sync(0xffffffffu, failed != 0)) break;
       }
-      // tell the issuing warp that nothing follows (also when aborting: its own waits are bounded too)
-      if (__all_sync(0xffffffffu, mbar_wait(bar(Smem::cmd_empty, ci), cpar ^ 1, ctx, kBarCmdEmpty)) && lane == 0) {
-        cmd_word[ci] = kCmdExit;
-        mbar_arrive(bar(Smem::cmd_full, ci));
-      }
-    } else if (warp == 11) {
-      // ============================== MMA issuer ==============================
-      // Executes the scheduler's commands in order: O_X (+)= P V of a block, then S_X = Q K^T of the
-      // slot's next block (which overwrites the P just consumed), with the commits that publish them.
-      Ctx ctx{abort_flag, a.status, kRoleMma};
-      volatile uint32_t* cmd_word = (volatile uint32_t*)(smem_gen + Smem::cmd_word);
-      uint32_t ci = 0, cpar = 0;
-      bool ok = true;
-      const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
-      for (;;) {
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::cmd_full, ci), cpar, ctx, kBarCmdFull));
-        if (!ok) break;
-        const uint32_t cmd = (uint32_t)uni((int)cmd_word[ci]);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(Smem::cmd_empty, ci));
-        if (++ci == kCmdSlots) { ci = 0; cpar ^= 1; }
-        if (cmd & kCmdExit) break;
-        const uint32_t X = (cmd & kCmdSlot1) ? 1u : 0u;
-        const uint32_t slot_v = (cmd >> 8) & 15u, slot_k = (cmd >> 12) & 15u;
-        const uint32_t s_tmem = tmem_base + X * 128;
-        const uint32_t o_tmem = tmem_base + kOCol + X * 128;
-        constexpr int kEarlySteps = (BLK / 32 - 1) * 2;  // 16-key steps of P V covered by p_early
-        const uint32_t v_addr = smem_base + kKvOff + slot_v * kSlotBytes;
-        const uint32_t p_par = (cmd & kCmdPPar) ? 1u : 0u;
-        if (cmd & kCmdPv) {
-          // The one condition the scheduler leaves open: the slot's softmax warps have stored P.
-          // P V starts on the leading key columns while the softmax still works on the last 32.
-          ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::p_early, X), p_par, ctx, kBarPEarly));
-          if (!ok) break;
-          tc_fence_after();
-          if (leader) {
-            const uint32_t first = (cmd & kCmdPvFirst) ? 1u : 0u;
-            uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
-            uint32_t acc = first ^ 1u;
-#pragma unroll 1
-            for (int k = 0; k < kEarlySteps; ++k) {  // rolled: the issuing loop stays within a few instruction-cache lines
-              mma_ts(o_tmem, s_tmem + k * 8, db, kIdescPV, acc);
-              db += 2048 >> 4;
-              acc = 1u;
-            }
-          }
-          __syncwarp();
-          ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::p_ready, X), p_par, ctx, kBarPReady));
-          if (!ok) break;
-        }
-        tc_fence_after();
-        if (leader) {
-          if (cmd & kCmdPv) {
-            uint64_t db = smem_desc(v_addr + kEarlySteps * 2048, kHalfBytes, 1024);
-#pragma unroll 1
-            for (int k = kEarlySteps; k < BLK / 16; ++k) {
-              mma_ts(o_tmem, s_tmem + k * 8, db, kIdescPV, 1u);
-              db += 2048 >> 4;
-            }
-            tc_commit(bar(Smem::kv_empty, slot_v));
-            if (cmd & kCmdPvLast) tc_commit(bar(Smem::o_full, X));
-          }
-          if (cmd & kCmdQk) {
-            const uint32_t qb = (cmd >> 16) & 3u;
-            const uint32_t q_addr = smem_base + Smem::q + qb * kQBytes;
-            const uint32_t k_addr = smem_base + kKvOff + slot_k * kSlotBytes;
-            uint64_t da = smem_desc(q_addr, 16, 1024);
-            uint64_t db = smem_desc(k_addr, 16, 1024);
-            uint32_t acc = 0u;
-#pragma unroll 1
-            for (int k = 0; k < kHeadDim / 16; ++k) {
-              mma_ss(s_tmem, da, db, kIdescS, acc);
-              acc = 1u;
-              // 16 columns = 32 bytes on; after four steps the next 64-column half of the tile
-              da += (k == 3) ? (uint64_t)((kTileM * 128 - 96) >> 4) : (uint64_t)(32 >> 4);
-              db += (k == 3) ? (uint64_t)((kHalfBytes - 96) >> 4) : (uint64_t)(32 >> 4);
-            }
-            tc_commit(bar(Smem::kv_empty, slot_k));
-            tc_commit(bar(Smem::s_full, X));
-            if (cmd & kCmdQkLast) tc_commit(bar(Smem::q_empty, qb));
-          }
-        }
-        __syncwarp();
-      }
+      const bool ok = !__any_sync(0xffffffffu, failed != 0);
+      if (failed != 0) raise_abort(ctx, failed);
       if (!ok && lane == 0) {
         // aborting: let the tensor-core work already issued finish (bounded) before TMEM is freed
         tc_commit(bar(Smem::drain, 0));
