@@ -100,7 +100,10 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   const int last_ntok = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1];
   const int nfull = last_ntok == BLK ? nb : nb - 1;
   // nothing to do when the tile holds no full row or no full column
-  if (r0 + ti * kTile >= nfull || tj * kTile >= nfull) return;
+  if (r0 + ti * kTile >= nfull || tj * kTile >= nfull) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // before it counts as done: see the partial-row kernel
+    return;
+  }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
@@ -114,8 +117,9 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   }
   // Launched as a programmatic dependent of the pooling kernel (which writes MV), everything above overlaps
   // its tail.  (Without that launch attribute both are no-ops.)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The partial-row kernel may start behind the wait: it needs MV as well, and nothing of this kernel's.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x < kTile) {
     const int c = threadIdx.x;
     bias[c] = (tj * kTile + c < nb) ? a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + tj * kTile + c] : 0.f;
@@ -212,63 +216,115 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
 }
 
 // The metric row of a sequence's partial last block (when it belongs to the query chunk): for every j <= r the
-// mean over the anti-diagonal pairs whose two tokens exist.  One CTA per (sequence, query head); a warp takes
-// 32 consecutive columns at a time, the lanes share each dot product (4 elements of d per lane).
+// mean over the anti-diagonal pairs whose two tokens exist.  One CTA per (32 columns, sequence, kv head).  A half-warp
+// reads 256-byte rows with 16-byte loads and multiplies the key rows of four columns with the matching query rows of
+// four heads of the group, 8 loads for 16 products (with a column at a time the L1 traffic of the query rows bounds the
+// kernel, with one row in flight the latency: a 60-token block against 255 full blocks at 32 / 8 heads took 0.76 ms);
+// two warps share four columns, each taking every other pair of rows.
+constexpr int kPartThreads = 512;
+constexpr int kPartMaxGroup = 32;
 template <int BLK>
-__global__ void __launch_bounds__(256) antidiag_partial_kernel(const AntiArgs a) {
-  const int seq = blockIdx.x, h = blockIdx.y, kvh = h / a.g;
+__global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const AntiArgs a) {
+  __shared__ float part[2][kPartMaxGroup][32];
+  const int g = a.g, Hkv = a.Hq / g;
+  const int seq = blockIdx.y / Hkv, kvh = blockIdx.y - seq * Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int half = lane >> 4, chunk = lane & 15;
   const int nb = a.rows.seq_nblk[seq], r0 = a.rows.seq_r0[seq];
   const int r = nb - 1;
   const int ntok = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + r];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (ntok == BLK || r < r0) return;
+  const int j0 = (int)blockIdx.x * 32;
+  if (ntok == BLK || r < r0 || j0 > r) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int R = a.rows.seq_row_off[seq] + (r - r0);
-  const __nv_bfloat16* qblk = a.Q + (int64_t)a.rows.row_tok0[R] * a.q_st + (int64_t)h * a.q_sh;
-  const __nv_bfloat16* kseq = a.K + (int64_t)a.rows.seq_tok0[seq] * a.kv_st + (int64_t)kvh * a.kv_sh;
-  const int stride = (nb + 31) & ~31;
-  uint32_t* planes = (uint32_t*)a.M + (int64_t)h * a.mt_tot + a.rows.seq_mt_off[seq] + (int64_t)(r - r0) * stride;
-  float* mrow = a.M + (int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)(r - r0) * nb;
-  const float score_scale = a.scale * (float)BLK;
-  for (int j0 = warp * 32; j0 <= r; j0 += 8 * 32) {
-    float mine = 0.f;  // lane c keeps the value of column j0 + c
-    for (int c = 0; c < 32; ++c) {
-      const int j = j0 + c;
-      if (j > r) break;  // warp-uniform
-      const int ktok = j == r ? ntok : BLK;
-      float acc = 0.f;
-      int pairs = 0;
-      for (int s = 0; s < BLK; ++s) {
-        const int tq = BLK - 1 - s;
-        if (tq >= ntok || s >= ktok) continue;  // warp-uniform
-        const uint2 qv = *(const uint2*)(qblk + (int64_t)tq * a.q_st + lane * 4);
-        const uint2 kv = *(const uint2*)(kseq + (int64_t)(j * BLK + s) * a.kv_st + lane * 4);
-        acc = fmaf(__uint_as_float(qv.x << 16), __uint_as_float(kv.x << 16), acc);
-        acc = fmaf(__uint_as_float(qv.x & 0xffff0000u), __uint_as_float(kv.x & 0xffff0000u), acc);
-        acc = fmaf(__uint_as_float(qv.y << 16), __uint_as_float(kv.y << 16), acc);
-        acc = fmaf(__uint_as_float(qv.y & 0xffff0000u), __uint_as_float(kv.y & 0xffff0000u), acc);
-        ++pairs;
+  const int s_lo = BLK - ntok;  // steps s whose query token B-1-s exists
+  const int c0 = (warp & 7) * 4, which = warp >> 3;
+  if (j0 + c0 <= r) {
+    const __nv_bfloat16* kseq = a.K + (int64_t)a.rows.seq_tok0[seq] * a.kv_st + (int64_t)kvh * a.kv_sh + chunk * 8;
+    const __nv_bfloat16* kcol[4];
+    int s_hi[4];  // steps whose key token s exists as well
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = j0 + c0 + c;
+      s_hi[c] = j < r ? BLK : (j == r ? ntok : 0);
+      kcol[c] = kseq + (int64_t)min(j, r) * BLK * a.kv_st;
+    }
+    const __nv_bfloat16* qblk = a.Q + (int64_t)a.rows.row_tok0[R] * a.q_st + (int64_t)(kvh * g) * a.q_sh + chunk * 8;
+    for (int h0 = 0; h0 < g; h0 += 4) {
+      float acc[4][4];
+      const __nv_bfloat16* qh[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        qh[q] = qblk + (int64_t)min(h0 + q, g - 1) * a.q_sh;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[q][c] = 0.f;
+      }
+#pragma unroll 2
+      for (int s = s_lo + 2 * which + half; s < BLK; s += 4) {
+        uint4 kv[4], qv[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) kv[c] = s < s_hi[c] ? *(const uint4*)(kcol[c] + (int64_t)s * a.kv_st) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) qv[q] = *(const uint4*)(qh[q] + (int64_t)(BLK - 1 - s) * a.q_st);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float kl[4], kh[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t w = i == 0 ? kv[c].x : i == 1 ? kv[c].y : i == 2 ? kv[c].z : kv[c].w;
+            kl[c] = __uint_as_float(w << 16);
+            kh[c] = __uint_as_float(w & 0xffff0000u);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t w = i == 0 ? qv[q].x : i == 1 ? qv[q].y : i == 2 ? qv[q].z : qv[q].w;
+            const float ql = __uint_as_float(w << 16), qu = __uint_as_float(w & 0xffff0000u);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[q][c] = fmaf(qu, kh[c], fmaf(ql, kl[c], acc[q][c]));
+          }
+        }
       }
 #pragma unroll
-      for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-      const float val = score_scale * (pairs > 0 ? acc / (float)pairs : 0.f) +
-                        a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + j];
-      if (lane == c) mine = val;
+      for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) acc[q][c] += __shfl_xor_sync(0xffffffffu, acc[q][c], d);
+          if (lane == 0 && h0 + q < g) part[which][h0 + q][c0 + c] = acc[q][c];
+        }
+      }
     }
+  }
+  __syncthreads();
+  // (MV is complete since before this kernel started: the contraction kernel lets it start only behind its own wait.)
+  const int stride = (nb + 31) & ~31;
+  const int j = j0 + lane;
+  const bool valid = j <= r;
+  const int pairs = max((j < r ? BLK : ntok) - s_lo, 0);
+  const float scale = pairs > 0 ? a.scale * (float)BLK / (float)pairs : 0.f;
+  const float bias = valid ? a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + j] : 0.f;
+  for (int hh = warp; hh < g; hh += kPartThreads / 32) {
+    const int h = kvh * g + hh;
+    const float val = valid ? fmaf(scale, part[0][hh][lane] + part[1][hh][lane], bias) : 0.f;
     if (a.as_keys) {
       // the 32 columns' keys as 32 bit planes: lane k stores plane k
-      const uint32_t key = j0 + lane <= r ? metric_key(mine) : 0u;
+      uint32_t* planes = (uint32_t*)a.M + (int64_t)h * a.mt_tot + a.rows.seq_mt_off[seq] + (int64_t)(r - r0) * stride;
+      const uint32_t key = valid ? metric_key(val) : 0u;
       uint32_t word = 0u;
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         const uint32_t bal = __ballot_sync(0xffffffffu, (key >> k) & 1u);
         if (lane == k) word = bal;
       }
-      planes[j0 + lane] = word;
-    } else if (j0 + lane <= r) {
-      mrow[j0 + lane] = mine;
+      planes[j] = word;
+    } else if (valid) {
+      a.M[(int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)(r - r0) * nb + j] = val;
     }
   }
+  // This kernel is not complete before the contraction is: what follows on the stream reads both kernels' rows.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace
@@ -333,12 +389,14 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   if (e != cudaSuccess) return e;
   ++*launched;
   if (!any_partial) return e;
-  // the metric rows of partial last blocks (stream-ordered behind the contraction; it waits for the pooling
-  // kernel's MV through the contraction kernel)
+  // the metric rows of partial last blocks, beside the contraction (the rows are not those the contraction writes, and
+  // MV is complete once every CTA of the contraction is past its wait or gone)
   cudaLaunchConfig_t cfg2 = {};
-  cfg2.gridDim = dim3((unsigned)batch, (unsigned)a.Hq);
-  cfg2.blockDim = dim3(256);
+  cfg2.gridDim = dim3((unsigned)((p.max_nblk + 31) / 32), (unsigned)(batch * p.cfg.num_kv_heads));
+  cfg2.blockDim = dim3(kPartThreads);
   cfg2.stream = s;
+  cfg2.attrs = attr;
+  cfg2.numAttrs = 1;
   e = B == 128 ? cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<128>, a) : cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<64>, a);
   if (e == cudaSuccess) ++*launched;
   return e;

@@ -117,3 +117,24 @@ def test_32k_layer_in_antidiagonal_mode():
     check_attention(from_dev_bf16(out), O_ref, mask, label=f"{w.name} anti-diagonal mode ({len(rows)} lists)")
     assert torch.isfinite(out.float()).all()
     plan.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (128, (128 * 33 + 1,), 1, 1),           # one token in the last block, 34 columns: a second column group
+    (128, (128 * 31 + 127, 60), 10, 2),     # all but one token; a sequence without any full block; five heads per group
+    (64, (64 * 64 + 33,), 16, 1),           # 65 columns, four rounds of heads
+])
+def test_antidiagonal_metric_row_of_a_partial_last_block(block, seqlens, hq, hkv):
+    w = wl.small("ad_partial", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=200, seed=77)
+    data = wl.make_qkv(w)
+    M_ref, _ = so.score_antidiag(data["q"], data["k"], data["v"], data["cu_seqlens"], oracle_params(w))
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w, score_mode=1)
+    M = torch.full((hq, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_score(plan, q, k, v, M)
+    assert binding.stem_check_status(plan)[0] == 0
+    M_g = M.cpu().numpy()
+    defined = ~np.isnan(M_ref)
+    assert np.array_equal(np.isnan(M_g), ~defined)
+    assert np.all(np.abs(M_g[defined] - M_ref[defined]) <= METRIC_ABS + METRIC_REL * np.abs(M_ref[defined]))
+    plan.close()
