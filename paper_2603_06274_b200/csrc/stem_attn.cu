@@ -53,6 +53,7 @@ constexpr int kSlotBytes = 32 * 1024;
 constexpr int kQBytes = 32 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSpareQMaxList = 256;                      // longest list (blocks) served with the spare Q tile
+constexpr int kMaskedFactor = 1;                         // token lists: the masked form up to this times 128 / g x k_max tokens
 constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X; S/P at 128 X
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
 constexpr float kRescaleThreshold = 8.0f;                // log2 units
@@ -60,7 +61,7 @@ constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after:
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4 };
 enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarPEarly };
+                   kBarDrain, kBarPEarly, kBarMask };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -75,7 +76,8 @@ struct Smem {
   static constexpr int p_early = p_ready + 16;            // all of P but its last 32 key columns stored
   static constexpr int o_full = p_early + 16;
   static constexpr int o_free = o_full + 16;
-  static constexpr int drain = o_free + 16;
+  static constexpr int mask_bar = o_free + 16;            // kTok: the softmax warps of a slot among themselves
+  static constexpr int drain = mask_bar + 16;
   static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
   static constexpr int total = abort_flag + 4;
@@ -127,18 +129,21 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
   return done;
 }
 
+__device__ int32_t g_masked_status[4];  // status words of the token-list form, which is given no workspace
+
 struct Ctx {
   volatile int* abort_flag;  // shared memory
-  int32_t* status;           // global memory status words
+  int32_t* status;           // global memory status words (null: g_masked_status)
   int role;
 };
 
 __device__ __forceinline__ void raise_abort(const Ctx& c, int bar_id) {
   *c.abort_flag = 1;
-  if (atomicCAS(c.status, 0, 1) == 0) {
-    c.status[1] = (int32_t)blockIdx.x;
-    c.status[2] = c.role;
-    c.status[3] = bar_id;
+  int32_t* st = c.status ? c.status : g_masked_status;
+  if (atomicCAS(st, 0, c.status ? 1 : 4) == 0) {
+    st[1] = (int32_t)blockIdx.x;
+    st[2] = c.role;
+    st[3] = bar_id;
   }
 }
 
@@ -327,12 +332,32 @@ struct AttnArgs {
   RowTables rows;
   int n_items, Hq, g, R_tot, k_max, T;
   int list_div;             // query heads per index list: 1, or g when the lists are per kv head
+  // token lists (kTok): sel_idx / sel_cnt are [n_kvh, T, k_max] / [n_kvh, T] lists of single tokens
+  int n_kvh;                // kv heads
+  int tok_tile;             // query tokens of an item: as many as give at most 128 rows (tokens x query heads of a group)
+  int win_blocks;           // key blocks whose masks fit a slot's share of shared memory at a time
+  int vec_lists;            // the lists may be read 16 bytes at a time
   float scale_log2;
 };
+
+// kTok: the tensors themselves, for the rows that exact_token_row computes.
+struct TokRows {
+  const __nv_bfloat16 *Q, *K, *V;
+  int64_t q_st, q_sh, kv_st, kv_sh;
+};
+
+// kTok: item i is (kv head, tile of query tokens), the longest prefixes first; n = key blocks up to its last token.
+__device__ __forceinline__ void tok_item(const AttnArgs& a, int i, int& kvh, int& tile, int& n) {
+  const int q = i / a.n_kvh;
+  kvh = i - q * a.n_kvh;
+  tile = (a.T - 1) / a.tok_tile - q;
+  n = (min((tile + 1) * a.tok_tile, a.T) - 1) / kTileM + 1;
+}
 
 // Walks the items of one slot of this CTA: item i of the work order belongs to CTA i % gridDim.x,
 // slot (i / gridDim.x) % 2.  Items with an empty list are skipped (the slot's softmax warps zero
 // their output rows).  Used by whole warps in lock step (values are broadcast from lane 0).
+template <bool kTok>
 struct ItemCursor {
   int idx, step;
   int h, R, r, n;
@@ -343,6 +368,14 @@ struct ItemCursor {
   }
   // Moves to the next item with a non-empty list; false when the slot has no more items.
   __device__ __forceinline__ bool next(const AttnArgs& a) {
+    if constexpr (kTok) {
+      idx += step;
+      n = 0;
+      if (idx >= a.n_items) return false;
+      tok_item(a, idx, h, R, n);
+      r = n - 1;
+      return true;
+    }
     for (idx += step; idx < a.n_items; idx += step) {
       h = uni(a.work[2 * idx]);
       R = uni(a.work[2 * idx + 1]);
@@ -357,6 +390,7 @@ struct ItemCursor {
 
 // The list lengths of one slot's items, in the ItemCursor's order, for the MMA issuer: the loads that lead to the length
 // of the next item are started an item ahead (the work entry two items ahead), so that next() waits for none of them.
+template <bool kTok>
 struct LengthCursor {
   int idx, step;       // the item whose length `raw` is
   int raw, h2, R2;     // length of item idx as loaded; work entry of item idx + step
@@ -372,6 +406,7 @@ struct LengthCursor {
   __device__ __forceinline__ void init(const AttnArgs& a, int slot) {
     step = 2 * (int)gridDim.x;
     idx = (int)blockIdx.x + slot * (int)gridDim.x;
+    if constexpr (kTok) return;
     entry(a, idx);
     raw = length(a, h2, R2);
     entry(a, idx + step);
@@ -380,6 +415,12 @@ struct LengthCursor {
   __device__ __forceinline__ bool next(const AttnArgs& a) {
     do {
       if (idx >= a.n_items) { n = 0; return false; }
+      if constexpr (kTok) {
+        int kvh, tile;
+        tok_item(a, idx, kvh, tile, n);
+        idx += step;
+        return true;
+      }
       n = uni(raw);
       if (a.sel_idx) n = min(max(n, 0), a.k_max);
       idx += step;
@@ -390,10 +431,57 @@ struct LengthCursor {
   }
 };
 
-template <int BLK, bool kSpareQ>
+// One output row of the token-list form straight from its definition, for the rows the masked form cannot do: a list
+// with the same token twice (a mask holds it once), or a row that met a non-finite value (0 times a V row that the list
+// does not name).  One thread, fp32; four passes over the output columns keep it small.
+__device__ __noinline__ void exact_token_row(float scale_log2, const __nv_bfloat16* K, const __nv_bfloat16* V, const __nv_bfloat16* q,
+                                             int64_t kv_st, const int32_t* list, int n, int t, __nv_bfloat16* o, float* lse) {
+  auto score = [&](int i) -> float {
+    const __nv_bfloat16* k = K + (int64_t)min(max(list[i], 0), t) * kv_st;
+    float acc = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < kHeadDim; c += 8) {
+      const uint4 kv = *(const uint4*)(k + c), qv = *(const uint4*)(q + c);
+      const uint32_t kw[4] = {kv.x, kv.y, kv.z, kv.w}, qw[4] = {qv.x, qv.y, qv.z, qv.w};
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        acc = fmaf(__uint_as_float(qw[w] << 16), __uint_as_float(kw[w] << 16), acc);
+        acc = fmaf(__uint_as_float(qw[w] & 0xffff0000u), __uint_as_float(kw[w] & 0xffff0000u), acc);
+      }
+    }
+    return acc * scale_log2;
+  };
+  float m = -INFINITY, l = 0.f;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) m = fmaxf(m, score(i));
+#pragma unroll 1
+  for (int c0 = 0; c0 < kHeadDim; c0 += 32) {
+    float acc[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+    l = 0.f;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const float p = fast_exp2(score(i) - m);
+      l += p;
+      const __nv_bfloat16* v = V + (int64_t)min(max(list[i], 0), t) * kv_st + c0;
+#pragma unroll
+      for (int c = 0; c < 32; c += 2) {
+        const uint32_t w = *(const uint32_t*)(v + c);
+        acc[c] = fmaf(p, __uint_as_float(w << 16), acc[c]);
+        acc[c + 1] = fmaf(p, __uint_as_float(w & 0xffff0000u), acc[c + 1]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 32; c += 2) *(uint32_t*)(o + c0 + c) = pack_bf16(acc[c] / l, acc[c + 1] / l);
+  }
+  if (lse) *lse = (m + log2f(l)) * 0.6931471805599453f;
+}
+
+template <int BLK, bool kSpareQ, bool kTok>
 __global__ void __launch_bounds__(kThreads, 1)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const AttnArgs a) {
+                   const __grid_constant__ CUtensorMap map_v, const AttnArgs a, const TokRows tok) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = ((uint32_t)__cvta_generic_to_shared(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem_gen = smem_raw + (smem_base - (uint32_t)__cvta_generic_to_shared(smem_raw));
@@ -405,7 +493,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // kSpareQ: three Q tiles (the next item's tile is loaded into a spare while the current items run) and a ring of
   // four K / V slots, for lists of tens of blocks, where an item boundary that waits for Q costs two blocks' time;
   // otherwise two Q tiles and a ring of five, for long lists (and the dense mode), where the deeper ring pays.
-  constexpr int kKvSlots = kSpareQ ? 4 : 5;
+  // kTok: two Q tiles, a ring of four, and one tile's room for the token masks of the two slots.
+  static_assert(!kTok || (BLK == 128 && !kSpareQ), "the token-list form has two Q tiles and key blocks of 128");
+  constexpr int kKvSlots = (kSpareQ || kTok) ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
 
@@ -422,6 +512,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::o_full, i), 1);
       mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
     }
+    for (int i = 0; i < 2; ++i) mbar_init(bar(Smem::mask_bar, i), 4);
     mbar_init(bar(Smem::drain, 0), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -442,7 +533,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   constexpr uint32_t kHalfBytes = BLK * 128;    // one 64-column half of it
   constexpr uint32_t kIdescS = make_idesc(BLK, 0);
   constexpr uint32_t kIdescPV = make_idesc(kHeadDim, 1);
-  const bool dense = a.sel_idx == nullptr;
+  const bool dense = kTok || a.sel_idx == nullptr;
 
   if (warp < 8) {
     // ============================== softmax of slot X ==============================
@@ -456,12 +547,83 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     uint32_t blk = 0;   // blocks of this slot so far (phase of s_full / p_ready)
     uint32_t ord = 0;   // non-empty items of this slot so far (phase of o_full / o_free)
     bool ok = true;
+    // kTok: row m is query head m % g of the tile's token m / g.  Which keys a token's list names is kept as a bit mask
+    // in shared memory, win_blocks key blocks at a time, built by the slot's own 128 threads: the g threads of a token
+    // share its list in chunks of four entries.
+    const int tokl = kTok ? m / a.g : 0, sub = kTok ? m - tokl * a.g : 0;
+    const uint32_t mask_stride = kTok ? a.win_blocks * 16 + 16 : 0;  // bytes per token (padded: tokens on other banks)
+    const uint32_t mask_s = smem_base + kKvOff + kKvSlots * kSlotBytes + X * (kSlotBytes / 2);
+    uint32_t mask_par = 0;
+    auto mask_sync = [&]() -> bool {  // the slot's softmax warps among themselves (bounded, unlike bar.sync)
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(Smem::mask_bar, X));
+      const bool done = mbar_wait(bar(Smem::mask_bar, X), mask_par, ctx, kBarMask);
+      mask_par ^= 1;
+      return __all_sync(0xffffffffu, done);
+    };
+    int chunk0 = 0;           // this thread's first chunk with an entry behind the window
+    bool ascending = true;    // this thread's chunks are in ascending order (else every window reads them all)
+    auto build_masks = [&](const int32_t* list, const int nl, const int t, const int lo) -> bool {
+      const uint32_t span = (uint32_t)a.win_blocks * kTileM;
+      if (!mask_sync()) return false;  // everyone has read the previous window
+      for (uint32_t o = (uint32_t)m * 16; o < (uint32_t)a.tok_tile * mask_stride; o += 128 * 16)
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(mask_s + o), "r"(0) : "memory");
+      if (!mask_sync()) return false;
+      const uint32_t row_s = mask_s + (uint32_t)tokl * mask_stride;
+      const bool first = lo == 0;
+      if (first) { chunk0 = sub; ascending = true; }
+      const int behind = lo + (int)span;
+      int prev = -1, found = -1;
+      uint32_t word = 0xffffffffu, bits = 0u;
+      int c = ascending ? chunk0 : sub;
+      for (; 4 * c < nl; c += 4 * a.g) {
+        int e[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // four chunks in flight
+          const int i0 = 4 * (c + u * a.g);
+          if (a.vec_lists) {
+            int4 v = make_int4(0, 0, 0, 0);
+            if (i0 < nl) v = *(const int4*)(list + i0);
+            e[u][0] = v.x; e[u][1] = v.y; e[u][2] = v.z; e[u][3] = v.w;
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) e[u][q] = i0 + q < nl ? list[i0 + q] : 0;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i0 = 4 * (c + u * a.g);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (i0 + q < nl) {
+              const int x = min(max(e[u][q], 0), t);
+              if (first) ascending = ascending && x >= prev;
+              prev = x;
+              if (x >= behind && found < 0) found = c + u * a.g;
+              const uint32_t off = (uint32_t)(x - lo);
+              if (off < span) {
+                if ((off >> 5) != word) {
+                  if (bits) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(row_s + word * 4), "r"(bits) : "memory");
+                  word = off >> 5;
+                  bits = 0u;
+                }
+                bits |= 1u << (off & 31u);
+              }
+            }
+          }
+        }
+        if (!first && ascending && prev >= behind) break;
+      }
+      if (bits) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(row_s + word * 4), "r"(bits) : "memory");
+      chunk0 = found >= 0 ? found : c;
+      return mask_sync();
+    };
     // The list length of an item and whether its list ends on the diagonal block sit at the end of a
     // chain of dependent global loads (work order -> row table -> length -> last entry).  The chain
     // of the next item is walked while the current item's blocks are processed, and its result kept
     // in one register (length, bit 31 = diagonal); the item's other fields are then cache hits.
     auto list_info = [&](const int item) -> uint32_t {
-      if (item >= a.n_items) return 0u;
+      if (kTok || item >= a.n_items) return 0u;
       const int h = a.work[2 * item], R = a.work[2 * item + 1];
       const int r = a.rows.row_r[R];
       if (dense) return (uint32_t)(r + 1) | 0x80000000u;
@@ -474,11 +636,32 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     for (int item = (int)blockIdx.x + X * (int)gridDim.x; item < a.n_items && ok; item += 2 * (int)gridDim.x) {
       const uint32_t info = next_info;
       next_info = list_info(item + 2 * (int)gridDim.x);
-      const int h = a.work[2 * item], R = a.work[2 * item + 1];
-      const int q_tok0 = a.rows.row_tok0[R];
-      const int ntok = a.rows.row_ntok[R];
-      const int n = (int)(info & 0x7fffffffu);
+      int h, R, q_tok0, ntok, n;
+      if constexpr (kTok) {
+        int kvh, tile;
+        tok_item(a, item, kvh, tile, n);
+        h = kvh * a.g + sub;
+        R = kvh;
+        q_tok0 = tile * a.tok_tile + tokl - m;  // so that q_tok0 + m is the row's token
+        ntok = (tokl < a.tok_tile && tile * a.tok_tile + tokl < a.T) ? kTileM : 0;
+      } else {
+        h = a.work[2 * item];
+        R = a.work[2 * item + 1];
+        q_tok0 = a.rows.row_tok0[R];
+        ntok = a.rows.row_ntok[R];
+        n = (int)(info & 0x7fffffffu);
+      }
       const bool row_valid = m < ntok;
+      // kTok: the row's token list, and how many distinct tokens of it the masks have shown
+      const int t_row = q_tok0 + m;
+      const int32_t* list = nullptr;
+      int list_n = 0, seen = 0;
+      if constexpr (kTok) {
+        if (row_valid) {
+          list = a.sel_idx + ((int64_t)R * a.T + t_row) * a.k_max;
+          list_n = min(max(a.sel_cnt[(int64_t)R * a.T + t_row], 0), min(a.k_max, t_row + 1));
+        }
+      }
       if (n == 0) {
         if (row_valid) {
           __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
@@ -490,7 +673,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
       const bool has_diag = (info >> 31) != 0u;
       float m_run = -INFINITY, l_run = 0.f;
+      int in_win = kTok ? a.win_blocks : 0;  // key blocks of the current mask window so far
       for (int e = 0; e < n; ++e, ++blk) {
+        if constexpr (kTok) {
+          if (in_win == a.win_blocks) {
+            ok = build_masks(list, list_n, t_row, e * kTileM);
+            if (!ok) break;
+            in_win = 0;
+          }
+        }
         // S of block e is complete; so is every earlier tensor-core operation of this slot,
         // P V of block e-1 included (the commit behind Q K^T covers all earlier operations)
         ok = mbar_wait(bar(Smem::s_full, X), blk & 1, ctx, kBarSFull);
@@ -501,7 +692,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
         for (int c = 0; c < BLK / 32; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
         tmem_ld_wait();
-        if (e == n - 1 && has_diag) {
+        if constexpr (kTok) {
+          uint32_t w[4];
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                       : "r"(mask_s + (uint32_t)min(tokl, a.tok_tile - 1) * mask_stride + (uint32_t)in_win * 16) : "memory");
+          ++in_win;
+          seen += __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
+#pragma unroll
+          for (int c = 0; c < BLK; ++c) s[c] = (w[c >> 5] & (1u << (c & 31))) ? s[c] : -INFINITY;
+        } else if (e == n - 1 && has_diag) {
 #pragma unroll
           for (int c = 0; c < BLK; ++c) s[c] = (c <= m) ? s[c] : -INFINITY;
         }
@@ -515,7 +715,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         const float mx_c = fmaxf(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], max3(mx[5], mx[6], mx[7]))) * a.scale_log2;
         if (e == 0) {
-          m_run = mx_c;
+          m_run = kTok ? fmaxf(mx_c, -1e30f) : mx_c;  // finite: a block may hold no token of the row's list
         } else {
           const bool grow = mx_c > m_run + kRescaleThreshold;
           if (__any_sync(0xffffffffu, grow)) {
@@ -571,7 +771,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const float inv_l = 1.f / l_run;
+      const float inv_l = (kTok && list_n == 0) ? 0.f : 1.f / l_run;
+      float finite = 0.f;  // kTok: turns NaN with the first value that is not finite
       const bool o_al32 = ((uintptr_t)a.O & 31u) == 0u;  // rows are multiples of 256 bytes apart
       __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
 #pragma unroll
@@ -589,6 +790,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           uint32_t w[16];
 #pragma unroll
           for (int q = 0; q < 16; ++q) w[q] = pack_bf16(o[2 * q] * inv_l, o[2 * q + 1] * inv_l);
+          if constexpr (kTok) {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) finite = fmaf(o[q], 0.f, finite);
+          }
           if (o_al32) {
             // whole 32-byte sectors per store: a thread writes its own 256-byte row, so the stores of
             // a warp are 32 separate sectors either way, and this halves their number
@@ -601,7 +806,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           }
         }
       }
-      if (a.lse && row_valid) a.lse[(int64_t)h * a.T + q_tok0 + m] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+      if (a.lse && row_valid)
+        a.lse[(int64_t)h * a.T + q_tok0 + m] = (kTok && list_n == 0) ? -INFINITY : (m_run + log2f(l_run)) * 0.6931471805599453f;
+      if constexpr (kTok) {
+        if (row_valid && list_n > 0 && (seen != list_n || !(finite == 0.f && l_run < INFINITY)))
+          exact_token_row(a.scale_log2, tok.K + R * tok.kv_sh, tok.V + R * tok.kv_sh, tok.Q + (int64_t)t_row * tok.q_st + h * tok.q_sh, tok.kv_st, list,
+                          list_n, t_row, o_row, a.lse ? a.lse + (int64_t)h * a.T + t_row : nullptr);
+        else if (row_valid && list_n == 0)
+#pragma unroll
+          for (int c = 0; c < 16; ++c) *(uint4*)(o_row + c * 8) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+      }
       ++ord;
     }
   } else {
@@ -614,7 +829,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // ============================== K / V producer ==============================
       Ctx ctx{abort_flag, a.status, kRoleProducer};
       struct KvSlot {
-        ItemCursor cur;
+        ItemCursor<kTok> cur;
         bool has, pend;
         int e, j_next, pend_tok, pend_kvh, seq_tok0;
         const int32_t* list;
@@ -623,7 +838,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         s.has = s.cur.next(a);
         s.e = 0;
         if (s.has) {
-          s.seq_tok0 = uni(a.rows.seq_tok0[uni(a.rows.row_seq[s.cur.R])]);
+          s.seq_tok0 = kTok ? 0 : uni(a.rows.seq_tok0[uni(a.rows.row_seq[s.cur.R])]);
           s.list = dense ? nullptr : a.sel_idx + ((int64_t)(s.cur.h / a.list_div) * a.R_tot + s.cur.R) * a.k_max;
           s.j_next = dense ? 0 : uni(s.list[0]);
         }
@@ -651,7 +866,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         if (s.has) {
           const int j = min(max(s.j_next, 0), s.cur.r);
-          const int kvh = s.cur.h / a.g;
+          const int kvh = kTok ? s.cur.h : s.cur.h / a.g;
           const int tok = s.seq_tok0 + j * BLK;
           if (!load(&map_k, kvh, tok)) return false;
           s.pend = true; s.pend_tok = tok; s.pend_kvh = kvh;
@@ -688,12 +903,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
         // next tile, loaded into the spare buffer long before it is wanted; the buffer the slot leaves becomes the
         // spare once the last Q K^T of its item has read it.  The MMA issuer rotates the buffers by the same rule.
-        ItemCursor c0, c1;
+        ItemCursor<kTok> c0, c1;
         c0.init(0); c1.init(1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t q_used = 0u, q_odd = 0u;  // per buffer (bit b): a tile was loaded; an odd number of tiles was loaded
         bool ok = true;
-        auto load_into = [&](const ItemCursor& cur, const int b) -> bool {
+        auto load_into = [&](const ItemCursor<kTok>& cur, const int b) -> bool {
           if (((q_used >> b) & 1u) &&
               !__all_sync(0xffffffffu, mbar_wait(bar(Smem::q_empty, b), ((q_odd >> b) & 1u) ^ 1u, ctx, kBarQEmpty)))
             return false;
@@ -734,19 +949,20 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             while (((q_used >> b) & 1u) && !mbar_try(bar(Smem::q_full, b), ((q_odd >> b) & 1u) ^ 1u) && globaltimer() - t1 < 4000000ull) {}
         }
       } else {
-        ItemCursor c0, c1;
+        ItemCursor<kTok> c0, c1;
         c0.init(0); c1.init(1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t ord0 = 0, ord1 = 0;
         // Loads the slot's next Q tile as soon as the last Q K^T of its previous item has read the buffer.
-        auto try_load = [&](ItemCursor& cur, bool& has, uint32_t& ord, const int X) -> bool {
+        auto try_load = [&](ItemCursor<kTok>& cur, bool& has, uint32_t& ord, const int X) -> bool {
           if (!has || !uni((int)mbar_test(bar(Smem::q_empty, X), (ord & 1) ^ 1))) return false;
-          const int q_tok0 = uni(a.rows.row_tok0[cur.R]);
+          const int q_tok0 = kTok ? cur.R * a.tok_tile : uni(a.rows.row_tok0[cur.R]);
+          const int q_head = kTok ? cur.h * a.g : cur.h;
           const uint32_t dst = smem_base + Smem::q + X * kQBytes;
           if (elect_one()) {
-            mbar_expect_tx(bar(Smem::q_full, X), kQBytes);
-            tma_load_3d(dst, &map_q, bar(Smem::q_full, X), 0, cur.h, q_tok0);
-            tma_load_3d(dst + kTileM * 128, &map_q, bar(Smem::q_full, X), 64, cur.h, q_tok0);
+            mbar_expect_tx(bar(Smem::q_full, X), kTok ? a.tok_tile * a.g * 256 : kQBytes);
+            tma_load_3d(dst, &map_q, bar(Smem::q_full, X), 0, q_head, q_tok0);
+            tma_load_3d(dst + kTileM * 128, &map_q, bar(Smem::q_full, X), 64, q_head, q_tok0);
           }
           __syncwarp();
           ++ord;
@@ -787,7 +1003,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {
-        LengthCursor cur;
+        LengthCursor<kTok> cur;
         int left;                      // blocks of the current item whose Q K^T is still to come (0: no item left)
         uint32_t st;                   // kPend: a P V is due, of its item's first (kFirst) / last (kLast) block;
                                        // kNewItem: the next Q K^T is the first of its item
@@ -907,9 +1123,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // ------------------------------------------------------------------------------------------------
 // [T, H, 128] bf16 with element strides (tok, head): TMA dims (innermost first) = (128, H, T);
 // one box = 64 columns x 1 head x `rows` tokens = rows x 128 bytes, 128-byte swizzled.
-bool make_map(CUtensorMap* map, const void* base, int64_t T, int H, int64_t stride_tok, int64_t stride_head, int rows) {
+bool make_map(CUtensorMap* map, const void* base, int64_t T, int H, int64_t stride_tok, int64_t stride_head, int rows, int heads = 1) {
   return ptx::make_bf16_map_3d(map, base, {(uint64_t)kHeadDim, (uint64_t)H, (uint64_t)T},
-                               {(uint64_t)stride_head * 2, (uint64_t)stride_tok * 2}, {64u, 1u, (uint32_t)rows});
+                               {(uint64_t)stride_head * 2, (uint64_t)stride_tok * 2}, {64u, (uint32_t)heads, (uint32_t)rows});
 }
 
 }  // namespace
@@ -942,10 +1158,10 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   static bool attr_set[64] = {};
   const int dev_slot = p.device & 63;
   if (!attr_set[dev_slot]) {
-    e = cudaFuncSetAttribute(sparse_attn_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[dev_slot] = true;
   }
@@ -954,13 +1170,57 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // and longer lists: the deeper K / V ring.
   const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList;
   if (B == 128) {
-    if (spare_q) sparse_attn_kernel<128, true><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a);
-    else sparse_attn_kernel<128, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a);
+    if (spare_q) sparse_attn_kernel<128, true, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
+    else sparse_attn_kernel<128, false, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
   } else {
-    if (spare_q) sparse_attn_kernel<64, true><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a);
-    else sparse_attn_kernel<64, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a);
+    if (spare_q) sparse_attn_kernel<64, true, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
+    else sparse_attn_kernel<64, false, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
   }
   return cudaGetLastError();
+}
+
+// Attention over token lists with every causal key block computed and the keys outside a token's list masked out.
+// It costs key blocks x 128 keys for T = 128 / g query tokens at once, the gather kernel its list for every token: both
+// take about 2000 cycles per 128 keys, so the masked form wins until a causal prefix (n_tokens / 2 on average) is T
+// times as long as a list.
+cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
+                                int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
+                                void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s) {
+  *taken = false;
+  const int g = Hq / Hkv, tile = kTileM / g;
+  if ((int64_t)N > (int64_t)kMaskedFactor * tile * k_max) return cudaSuccess;
+  CUtensorMap mq, mk, mv;
+  if (!make_map(&mq, Q, N, Hq, q_st, q_sh, tile, g) || !make_map(&mk, K, N, Hkv, kv_st, kv_sh, kTileM) ||
+      !make_map(&mv, V, N, Hkv, kv_st, kv_sh, kTileM))
+    return cudaSuccess;  // strides that a tensor map cannot hold: the gather kernel takes them
+  *taken = true;
+  AttnArgs a{};
+  a.sel_idx = sel_idx; a.sel_cnt = sel_cnt;
+  a.O = (__nv_bfloat16*)O; a.lse = lse; a.status = nullptr;
+  a.n_items = ((N + tile - 1) / tile) * Hkv;
+  a.Hq = Hq; a.g = g; a.k_max = k_max; a.T = N; a.list_div = g; a.n_kvh = Hkv; a.tok_tile = tile;
+  a.win_blocks = kSlotBytes / 2 / 16 / tile - 1;
+  a.vec_lists = k_max % 4 == 0 && ((uintptr_t)sel_idx & 15u) == 0u;
+  a.scale_log2 = softmax_scale * 1.4426950408889634f;
+  const TokRows tok{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, q_st, q_sh, kv_st, kv_sh};
+  static bool attr_set[64] = {};
+  if (!attr_set[device & 63]) {
+    const cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    attr_set[device & 63] = true;
+  }
+  sparse_attn_kernel<128, false, true><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
+  return cudaGetLastError();
+}
+
+// Reads (and clears) the status words of the masked form after the caller synchronised the stream.
+cudaError_t masked_status_words(int32_t* out4) {
+  cudaError_t e = cudaMemcpyFromSymbol(out4, g_masked_status, sizeof(g_masked_status));
+  if (e == cudaSuccess && out4[0] != 0) {
+    const int32_t zero[4] = {0, 0, 0, 0};
+    e = cudaMemcpyToSymbol(g_masked_status, zero, sizeof(zero));
+  }
+  return e;
 }
 
 }  // namespace stem

@@ -138,6 +138,12 @@ cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_ma
 cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st,
                                    int64_t kv_sh, int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx,
                                    const int32_t* sel_cnt, float softmax_scale, void* O, float* lse, cudaStream_t s);
+// The same attention with every causal key block computed and masked by the lists (stem_attn.cu); *taken = false (and nothing
+// enqueued) where the gather form is the better one.
+cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
+                                int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
+                                void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s);
+cudaError_t masked_status_words(int32_t* out4);
 // The status words {4, CTA, role, barrier} of the gather-attention kernel on the current device, read to the host
 // and cleared when set (the caller has synchronised).
 cudaError_t token_status_words(int32_t* out4);

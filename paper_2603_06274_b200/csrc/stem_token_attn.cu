@@ -498,6 +498,9 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
+  bool taken = false;
+  e = launch_token_masked(Q, K, V, q_st, q_sh, kv_st, kv_sh, N, Hq, Hkv, k_max, sel_idx, sel_cnt, softmax_scale, O, lse, dev, sms, &taken, s);
+  if (e != cudaSuccess || taken) return e;
   if (!attr_set[dev & 63]) {
     e = cudaFuncSetAttribute(token_attn_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(token_attn_tc_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
@@ -531,8 +534,9 @@ cudaError_t token_status_words(int32_t* out4) {
   if (out4[0] != 0) {
     const int32_t zero[4] = {0, 0, 0, 0};
     e = cudaMemcpyToSymbol(g_token_status, zero, sizeof(zero));
+    return e;
   }
-  return e;
+  return masked_status_words(out4);
 }
 
 }  // namespace stem

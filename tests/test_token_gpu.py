@@ -165,3 +165,91 @@ def test_token_level_argument_errors():
     with pytest.raises(binding.StemError) as e:
         binding.stem_token_attention(q, kv, kv, idx, cnt, torch.empty_like(q))     # 17 query heads per kv head
     assert e.value.status == binding.STEM_ERR_UNSUPPORTED
+
+
+def _lists(r, n, hkv, k_max, order="ascending", repeat=False):
+    """Lists of 0 .. min(t + 1, k_max) tokens; with ``repeat`` some lists name a token twice."""
+    idx = np.full((hkv, n, k_max), -1, np.int32)
+    cnt = np.zeros((hkv, n), np.int32)
+    for h in range(hkv):
+        for t in range(n):
+            top = min(t + 1, k_max)
+            m = int(r.choice([0, 1, top, int(r.integers(0, top + 1))], p=[0.05, 0.05, 0.3, 0.6]))
+            pick = r.choice(t + 1, size=m, replace=False)
+            if repeat and m > 1 and r.random() < 0.3:
+                pick[0] = pick[1]
+            idx[h, t, :m] = np.sort(pick) if order == "ascending" else pick
+            cnt[h, t] = m
+    return idx, cnt
+
+
+def _plain_attention(q, k, v, idx, cnt, rows):
+    """fp64 attention of the listed rows (h, t): softmax over the list's entries, a repeated entry counted as often as it appears."""
+    hq, hkv = q.shape[1], k.shape[1]
+    out, lse = {}, {}
+    for h, t in rows:
+        kvh = h // (hq // hkv)
+        ids = np.clip(idx[kvh, t, :cnt[kvh, t]], 0, t)
+        s = k[ids, kvh].astype(np.float64) @ q[t, h].astype(np.float64) / np.sqrt(128.0)
+        p = np.exp(s - s.max())
+        out[h, t] = (p / p.sum()) @ v[ids, kvh].astype(np.float64)
+        lse[h, t] = s.max() + np.log(p.sum())
+    return out, lse
+
+
+# The masked form (every causal key block, the keys outside a list masked out) is taken when n <= 128 / g x k_max, the
+# gather form beyond.  Window edges of the masks: 128-token tiles of one head hold masks of 7 key blocks at a time.
+@pytest.mark.parametrize("n,hq,hkv,k_max,order,repeat,what", [
+    (1930, 2, 2, 64, "ascending", False, "masked, three mask windows, one head per group"),
+    (1930, 2, 2, 61, "any", False, "masked, lists in any order, entries read one at a time"),
+    (897, 7, 1, 300, "ascending", True, "masked, 18-token tiles, lists that name a token twice"),
+    (129, 16, 1, 128, "any", True, "masked, 8-token tiles, one token past a key block"),
+    (1100, 16, 1, 128, "ascending", False, "gather: the prefix is too long for the masks to pay"),
+    (700, 5, 1, 27, "any", True, "gather, lists in any order and with repeats"),
+])
+def test_token_attention_forms(n, hq, hkv, k_max, order, repeat, what):
+    r = np.random.default_rng(n + k_max)
+    w = wl.small("token_forms", seqlens=(n,), hq=hq, hkv=hkv, block=64, permille=100, sink=True, seed=n)
+    data = wl.make_qkv(w)
+    idx, cnt = _lists(r, n, hkv, k_max, order, repeat)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    out = torch.full((n, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((hq, n), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_token_attention(q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out, lse)
+    st, detail = binding.stem_token_check_status()
+    assert st == 0, detail
+    g = hq // hkv
+    rows = [(h, t) for h in range(hq) for t in sorted({0, 1, 127, 128, n // 2, n - 1, *r.integers(0, n, 150).tolist()}) if t < n and cnt[h // g, t] > 0]
+    O_ref, lse_ref = _plain_attention(from_dev_bf16(q), from_dev_bf16(k), from_dev_bf16(v), idx, cnt, rows)
+    got, got_lse = from_dev_bf16(out), lse.cpu().numpy()
+    ref = np.stack([O_ref[x] for x in rows])
+    check_attention(np.stack([got[t, h] for h, t in rows]), ref, np.ones(ref.shape, bool), label=what)
+    assert max(abs(got_lse[h, t] - lse_ref[h, t]) for h, t in rows) < 1e-3
+    empty = np.repeat(cnt == 0, g, axis=0)
+    assert (got.transpose(1, 0, 2)[empty] == 0).all() and np.isneginf(got_lse[empty]).all()
+    assert np.isfinite(got).all()
+
+
+def test_token_attention_ignores_rows_no_list_names():
+    # a value row that is not finite reaches only the queries whose lists name it, and so does a key row
+    n, hq, hkv, k_max = 400, 4, 2, 100
+    w = wl.small("token_nan", seqlens=(n,), hq=hq, hkv=hkv, block=64, permille=100, sink=False, seed=5)
+    data = wl.make_qkv(w)
+    r = np.random.default_rng(5)
+    idx, cnt = _lists(r, n, hkv, k_max)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    outs = []
+    for bad in (False, True):
+        if bad:
+            v[37] = float("inf")
+            k[38] = float("nan")
+        out = torch.empty((n, hq, 128), dtype=torch.bfloat16, device="cuda")
+        binding.stem_token_attention(q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out)
+        st, detail = binding.stem_token_check_status()
+        assert st == 0, detail
+        outs.append(from_dev_bf16(out))
+    named = np.array([[np.isin([37, 38], idx[h, t, :cnt[h, t]]).any() for t in range(n)] for h in range(hkv)])
+    clean = np.repeat(~named, hq // hkv, axis=0).T
+    assert clean.any() and not clean.all()
+    check_attention(outs[1][clean], outs[0][clean], np.ones(outs[0][clean].shape, bool), label="rows whose lists name no bad row")
+    assert not np.isfinite(outs[1][~clean]).all(axis=1).any()
