@@ -281,7 +281,8 @@ int stem_token_select(const float* scores, int32_t n_tokens, int32_t list_heads,
  * (STEM_ERR_UNSUPPORTED otherwise).  Strides in elements, multiples of 8; Q, K, V, O 16-byte aligned.
  * softmax_scale 0 means 1/sqrt(128).  O bf16 [n_tokens, num_q_heads, 128] (contiguous); lse fp32
  * [num_q_heads, n_tokens] or NULL.  Probabilities are rounded to bf16 before they meet V (as in stem_sparse_prefill).
- * The call only enqueues; a bounded device-side wait that gave up is reported by stem_token_check_status. */
+ * The call only enqueues; O serves as scratch memory until its kernels are done.  A bounded device-side wait that gave up
+ * is reported by stem_token_check_status. */
 int stem_token_attention(const void* Q, const void* K, const void* V, int32_t n_tokens, int32_t num_q_heads,
                          int32_t num_kv_heads, int64_t q_stride_tok, int64_t q_stride_head, int64_t kv_stride_tok,
                          int64_t kv_stride_head, const int32_t* sel_idx, const int32_t* sel_cnt, int32_t k_max,

@@ -61,7 +61,7 @@ constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after:
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4 };
 enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarPEarly, kBarMask };
+                   kBarDrain, kBarPEarly };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -76,8 +76,7 @@ struct Smem {
   static constexpr int p_early = p_ready + 16;            // all of P but its last 32 key columns stored
   static constexpr int o_full = p_early + 16;
   static constexpr int o_free = o_full + 16;
-  static constexpr int mask_bar = o_free + 16;            // kTok: the softmax warps of a slot among themselves
-  static constexpr int drain = mask_bar + 16;
+  static constexpr int drain = o_free + 16;
   static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
   static constexpr int total = abort_flag + 4;
@@ -332,11 +331,12 @@ struct AttnArgs {
   RowTables rows;
   int n_items, Hq, g, R_tot, k_max, T;
   int list_div;             // query heads per index list: 1, or g when the lists are per kv head
-  // token lists (kTok): sel_idx / sel_cnt are [n_kvh, T, k_max] / [n_kvh, T] lists of single tokens
-  int n_kvh;                // kv heads
+  // token lists (kTok): sel_idx / sel_cnt are [n_kvh, T, k_max] / [n_kvh, T] lists of single tokens; the launch computes
+  // the query tokens tok_a .. tok_b - 1
+  int n_kvh, tok_a, tok_b;
   int tok_tile;             // query tokens of an item: as many as give at most 128 rows (tokens x query heads of a group)
-  int win_blocks;           // key blocks whose masks fit a slot's share of shared memory at a time
-  int vec_lists;            // the lists may be read 16 bytes at a time
+  const unsigned char* masks;            // token t, kv head h: bit mask of its list at masks + (t - tok_a) mask_st + h mask_sh
+  int64_t mask_st, mask_sh;
   float scale_log2;
 };
 
@@ -350,8 +350,8 @@ struct TokRows {
 __device__ __forceinline__ void tok_item(const AttnArgs& a, int i, int& kvh, int& tile, int& n) {
   const int q = i / a.n_kvh;
   kvh = i - q * a.n_kvh;
-  tile = (a.T - 1) / a.tok_tile - q;
-  n = (min((tile + 1) * a.tok_tile, a.T) - 1) / kTileM + 1;
+  tile = (a.tok_b - a.tok_a - 1) / a.tok_tile - q;
+  n = (min(a.tok_a + (tile + 1) * a.tok_tile, a.tok_b) - 1) / kTileM + 1;
 }
 
 // Walks the items of one slot of this CTA: item i of the work order belongs to CTA i % gridDim.x,
@@ -493,9 +493,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // kSpareQ: three Q tiles (the next item's tile is loaded into a spare while the current items run) and a ring of
   // four K / V slots, for lists of tens of blocks, where an item boundary that waits for Q costs two blocks' time;
   // otherwise two Q tiles and a ring of five, for long lists (and the dense mode), where the deeper ring pays.
-  // kTok: two Q tiles, a ring of four, and one tile's room for the token masks of the two slots.
   static_assert(!kTok || (BLK == 128 && !kSpareQ), "the token-list form has two Q tiles and key blocks of 128");
-  constexpr int kKvSlots = (kSpareQ || kTok) ? 4 : 5;
+  constexpr int kKvSlots = kSpareQ ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
 
@@ -512,7 +511,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::o_full, i), 1);
       mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
     }
-    for (int i = 0; i < 2; ++i) mbar_init(bar(Smem::mask_bar, i), 4);
     mbar_init(bar(Smem::drain, 0), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -547,77 +545,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     uint32_t blk = 0;   // blocks of this slot so far (phase of s_full / p_ready)
     uint32_t ord = 0;   // non-empty items of this slot so far (phase of o_full / o_free)
     bool ok = true;
-    // kTok: row m is query head m % g of the tile's token m / g.  Which keys a token's list names is kept as a bit mask
-    // in shared memory, win_blocks key blocks at a time, built by the slot's own 128 threads: the g threads of a token
-    // share its list in chunks of four entries.
+    // kTok: row m is query head m % g of the tile's token m / g
     const int tokl = kTok ? m / a.g : 0, sub = kTok ? m - tokl * a.g : 0;
-    const uint32_t mask_stride = kTok ? a.win_blocks * 16 + 16 : 0;  // bytes per token (padded: tokens on other banks)
-    const uint32_t mask_s = smem_base + kKvOff + kKvSlots * kSlotBytes + X * (kSlotBytes / 2);
-    uint32_t mask_par = 0;
-    auto mask_sync = [&]() -> bool {  // the slot's softmax warps among themselves (bounded, unlike bar.sync)
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(Smem::mask_bar, X));
-      const bool done = mbar_wait(bar(Smem::mask_bar, X), mask_par, ctx, kBarMask);
-      mask_par ^= 1;
-      return __all_sync(0xffffffffu, done);
-    };
-    int chunk0 = 0;           // this thread's first chunk with an entry behind the window
-    bool ascending = true;    // this thread's chunks are in ascending order (else every window reads them all)
-    auto build_masks = [&](const int32_t* list, const int nl, const int t, const int lo) -> bool {
-      const uint32_t span = (uint32_t)a.win_blocks * kTileM;
-      if (!mask_sync()) return false;  // everyone has read the previous window
-      for (uint32_t o = (uint32_t)m * 16; o < (uint32_t)a.tok_tile * mask_stride; o += 128 * 16)
-        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(mask_s + o), "r"(0) : "memory");
-      if (!mask_sync()) return false;
-      const uint32_t row_s = mask_s + (uint32_t)tokl * mask_stride;
-      const bool first = lo == 0;
-      if (first) { chunk0 = sub; ascending = true; }
-      const int behind = lo + (int)span;
-      int prev = -1, found = -1;
-      uint32_t word = 0xffffffffu, bits = 0u;
-      int c = ascending ? chunk0 : sub;
-      for (; 4 * c < nl; c += 4 * a.g) {
-        int e[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {  // four chunks in flight
-          const int i0 = 4 * (c + u * a.g);
-          if (a.vec_lists) {
-            int4 v = make_int4(0, 0, 0, 0);
-            if (i0 < nl) v = *(const int4*)(list + i0);
-            e[u][0] = v.x; e[u][1] = v.y; e[u][2] = v.z; e[u][3] = v.w;
-          } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) e[u][q] = i0 + q < nl ? list[i0 + q] : 0;
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i0 = 4 * (c + u * a.g);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (i0 + q < nl) {
-              const int x = min(max(e[u][q], 0), t);
-              if (first) ascending = ascending && x >= prev;
-              prev = x;
-              if (x >= behind && found < 0) found = c + u * a.g;
-              const uint32_t off = (uint32_t)(x - lo);
-              if (off < span) {
-                if ((off >> 5) != word) {
-                  if (bits) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(row_s + word * 4), "r"(bits) : "memory");
-                  word = off >> 5;
-                  bits = 0u;
-                }
-                bits |= 1u << (off & 31u);
-              }
-            }
-          }
-        }
-        if (!first && ascending && prev >= behind) break;
-      }
-      if (bits) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(row_s + word * 4), "r"(bits) : "memory");
-      chunk0 = found >= 0 ? found : c;
-      return mask_sync();
-    };
     // The list length of an item and whether its list ends on the diagonal block sit at the end of a
     // chain of dependent global loads (work order -> row table -> length -> last entry).  The chain
     // of the next item is walked while the current item's blocks are processed, and its result kept
@@ -642,8 +571,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         tok_item(a, item, kvh, tile, n);
         h = kvh * a.g + sub;
         R = kvh;
-        q_tok0 = tile * a.tok_tile + tokl - m;  // so that q_tok0 + m is the row's token
-        ntok = (tokl < a.tok_tile && tile * a.tok_tile + tokl < a.T) ? kTileM : 0;
+        q_tok0 = a.tok_a + tile * a.tok_tile + tokl - m;  // so that q_tok0 + m is the row's token
+        ntok = (tokl < a.tok_tile && q_tok0 + m < a.tok_b) ? kTileM : 0;
       } else {
         h = a.work[2 * item];
         R = a.work[2 * item + 1];
@@ -652,14 +581,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         n = (int)(info & 0x7fffffffu);
       }
       const bool row_valid = m < ntok;
-      // kTok: the row's token list, and how many distinct tokens of it the masks have shown
+      // kTok: the row's mask words of the next key block, its list's length, and how many tokens of it the masks have shown
       const int t_row = q_tok0 + m;
-      const int32_t* list = nullptr;
+      const uint4* mask = nullptr;
+      uint4 mask_next = make_uint4(0, 0, 0, 0);
       int list_n = 0, seen = 0;
       if constexpr (kTok) {
         if (row_valid) {
-          list = a.sel_idx + ((int64_t)R * a.T + t_row) * a.k_max;
           list_n = min(max(a.sel_cnt[(int64_t)R * a.T + t_row], 0), min(a.k_max, t_row + 1));
+          mask = (const uint4*)(a.masks + (t_row - a.tok_a) * a.mask_st + R * a.mask_sh);
+          mask_next = mask[0];
         }
       }
       if (n == 0) {
@@ -673,15 +604,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
       const bool has_diag = (info >> 31) != 0u;
       float m_run = -INFINITY, l_run = 0.f;
-      int in_win = kTok ? a.win_blocks : 0;  // key blocks of the current mask window so far
       for (int e = 0; e < n; ++e, ++blk) {
-        if constexpr (kTok) {
-          if (in_win == a.win_blocks) {
-            ok = build_masks(list, list_n, t_row, e * kTileM);
-            if (!ok) break;
-            in_win = 0;
-          }
-        }
         // S of block e is complete; so is every earlier tensor-core operation of this slot,
         // P V of block e-1 included (the commit behind Q K^T covers all earlier operations)
         ok = mbar_wait(bar(Smem::s_full, X), blk & 1, ctx, kBarSFull);
@@ -693,11 +616,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int c = 0; c < BLK / 32; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
         tmem_ld_wait();
         if constexpr (kTok) {
-          uint32_t w[4];
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                       : "r"(mask_s + (uint32_t)min(tokl, a.tok_tile - 1) * mask_stride + (uint32_t)in_win * 16) : "memory");
-          ++in_win;
+          const uint32_t w[4] = {mask_next.x, mask_next.y, mask_next.z, mask_next.w};
+          if (row_valid && e + 1 < n) mask_next = mask[e + 1];  // used in the next turn
           seen += __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
 #pragma unroll
           for (int c = 0; c < BLK; ++c) s[c] = (w[c >> 5] & (1u << (c & 31))) ? s[c] : -INFINITY;
@@ -810,7 +730,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         a.lse[(int64_t)h * a.T + q_tok0 + m] = (kTok && list_n == 0) ? -INFINITY : (m_run + log2f(l_run)) * 0.6931471805599453f;
       if constexpr (kTok) {
         if (row_valid && list_n > 0 && (seen != list_n || !(finite == 0.f && l_run < INFINITY)))
-          exact_token_row(a.scale_log2, tok.K + R * tok.kv_sh, tok.V + R * tok.kv_sh, tok.Q + (int64_t)t_row * tok.q_st + h * tok.q_sh, tok.kv_st, list,
+          exact_token_row(a.scale_log2, tok.K + R * tok.kv_sh, tok.V + R * tok.kv_sh, tok.Q + (int64_t)t_row * tok.q_st + h * tok.q_sh, tok.kv_st, a.sel_idx + ((int64_t)R * a.T + t_row) * a.k_max,
                           list_n, t_row, o_row, a.lse ? a.lse + (int64_t)h * a.T + t_row : nullptr);
         else if (row_valid && list_n == 0)
 #pragma unroll
@@ -956,7 +876,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // Loads the slot's next Q tile as soon as the last Q K^T of its previous item has read the buffer.
         auto try_load = [&](ItemCursor<kTok>& cur, bool& has, uint32_t& ord, const int X) -> bool {
           if (!has || !uni((int)mbar_test(bar(Smem::q_empty, X), (ord & 1) ^ 1))) return false;
-          const int q_tok0 = kTok ? cur.R * a.tok_tile : uni(a.rows.row_tok0[cur.R]);
+          const int q_tok0 = kTok ? a.tok_a + cur.R * a.tok_tile : uni(a.rows.row_tok0[cur.R]);
           const int q_head = kTok ? cur.h * a.g : cur.h;
           const uint32_t dst = smem_base + Smem::q + X * kQBytes;
           if (elect_one()) {
@@ -1182,7 +1102,11 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
 // Attention over token lists with every causal key block computed and the keys outside a token's list masked out.
 // It costs key blocks x 128 keys for T = 128 / g query tokens at once, the gather kernel its list for every token: both
 // take about 2000 cycles per 128 keys, so the masked form wins until a causal prefix (n_tokens / 2 on average) is T
-// times as long as a list.
+// times as long as a list.  8K tokens, 32 / 8 heads, top 2048: 0.72 ms against 6.4 (start: 7.3), of which 0.52 attention.
+// The masks, one bit per key of the prefix, are built by a kernel of their own (token_mask_kernel) into the rows of O that
+// are not yet final: of the query tokens themselves, whose masks are read before their rows are written, if a prefix has no
+// more bits than a row of the group (2048 g); else the tokens are computed from the last ones on, as many at a time as find
+// room for their masks in the rows of the tokens before them.
 cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
                                 int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
                                 void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s) {
@@ -1197,10 +1121,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
   AttnArgs a{};
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt;
   a.O = (__nv_bfloat16*)O; a.lse = lse; a.status = nullptr;
-  a.n_items = ((N + tile - 1) / tile) * Hkv;
   a.Hq = Hq; a.g = g; a.k_max = k_max; a.T = N; a.list_div = g; a.n_kvh = Hkv; a.tok_tile = tile;
-  a.win_blocks = kSlotBytes / 2 / 16 / tile - 1;
-  a.vec_lists = k_max % 4 == 0 && ((uintptr_t)sel_idx & 15u) == 0u;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
   const TokRows tok{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, q_st, q_sh, kv_st, kv_sh};
   static bool attr_set[64] = {};
@@ -1209,8 +1130,29 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
     if (e != cudaSuccess) return e;
     attr_set[device & 63] = true;
   }
-  sparse_attn_kernel<128, false, true><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
-  return cudaGetLastError();
+  const int64_t row_bytes = (int64_t)g * kHeadDim * 2;  // of O, per token and kv head
+  for (int b = N; b > 0; b = a.tok_a) {
+    const int64_t mask_bytes = (int64_t)((b + kTileM - 1) / kTileM) * (kTileM / 8);
+    a.masks = (const unsigned char*)O;
+    if (mask_bytes <= row_bytes) {
+      a.tok_a = 0;
+      a.mask_st = Hkv * row_bytes;
+      a.mask_sh = row_bytes;
+    } else {
+      // (b - tok_a) masks fit tok_a rows
+      a.tok_a = (int)(((int64_t)b * mask_bytes + mask_bytes + row_bytes - 1) / (mask_bytes + row_bytes));
+      a.mask_st = Hkv * mask_bytes;
+      a.mask_sh = mask_bytes;
+    }
+    a.tok_b = b;
+    a.n_items = ((b - a.tok_a + tile - 1) / tile) * Hkv;
+    cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, tile, O, a.mask_st, a.mask_sh, s);
+    if (e != cudaSuccess) return e;
+    sparse_attn_kernel<128, false, true><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Reads (and clears) the status words of the masked form after the caller synchronised the stream.

@@ -144,6 +144,11 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
                                 int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
                                 void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s);
 cudaError_t masked_status_words(int32_t* out4);
+// Bit masks of the token lists of query tokens t0 .. t1 - 1: bit x of the mask of (token t, kv head h), at
+// masks + (t - t0) st + h sh bytes, says whether the list names token x <= t; whole 128-key blocks up to that
+// of the last token of t's tile of `tile` tokens.
+cudaError_t launch_token_masks(const int32_t* sel_idx, const int32_t* sel_cnt, int N, int Hkv, int k_max, int t0, int t1, int tile, void* masks,
+                               int64_t st, int64_t sh, cudaStream_t s);
 // The status words {4, CTA, role, barrier} of the gather-attention kernel on the current device, read to the host
 // and cleared when set (the caller has synchronised).
 cudaError_t token_status_words(int32_t* out4);

@@ -179,7 +179,76 @@ __global__ void __launch_bounds__(kSelThreads) token_select_kernel(const float* 
   if (threadIdx.x == 0) sel_cnt[(int64_t)lh * N + t] = total;
 }
 
+// ------------------------------------------------------------------------------------------------
+// Token lists as bit masks, for the attention that computes every causal key block (stem_attn.cu).  One warp per (query
+// token, kv head): a byte per key in shared memory is set for every listed token (plain stores: atomic ORs of bits take
+// 14 cycles of the SM per warp instruction and would bound the kernel), then 32 bytes at a time are packed into a word.
+// Keys are taken a window of kMaskWindow at a time; a list is read once per window.
+// ------------------------------------------------------------------------------------------------
+constexpr int kMaskThreads = 256;
+constexpr int kMaskWindow = 4096;
+
+__global__ void __launch_bounds__(kMaskThreads) token_mask_kernel(const int32_t* __restrict__ sel_idx, const int32_t* __restrict__ sel_cnt,
+                                                                  int N, int Hkv, int k_max, int t0, int t1, int tile,
+                                                                  unsigned char* masks, int64_t st, int64_t sh, int vec) {
+  __shared__ __align__(16) unsigned char flags_all[kMaskThreads / 32][kMaskWindow];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t item = (int64_t)blockIdx.x * (kMaskThreads / 32) + warp;
+  if (item >= (int64_t)(t1 - t0) * Hkv) return;
+  const int h = (int)(item % Hkv), t = t1 - 1 - (int)(item / Hkv);  // long prefixes first
+  unsigned char* flags = flags_all[warp];
+  const int64_t row = (int64_t)h * N + t;
+  const int32_t* list = sel_idx + row * k_max;
+  const int n = min(max(sel_cnt[row], 0), min(k_max, t + 1));
+  const int n_vec = vec ? n / 4 : 0;
+  unsigned char* dst = masks + (int64_t)(t - t0) * st + (int64_t)h * sh;
+  // a row goes up to the last key block that its tile of queries reads
+  const int keys = (min(t0 + ((t - t0) / tile + 1) * tile, t1) + 127) / 128 * 128;
+  for (int lo = 0; lo < keys; lo += kMaskWindow) {
+    const int span = min(kMaskWindow, keys - lo);  // a multiple of 128
+    const uint32_t in = (uint32_t)max(min(span, t + 1 - lo), 0);
+    for (int o = lane * 16; o < span; o += 512) *(uint4*)(flags + o) = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    if (in > 0) {
+#pragma unroll 4
+      for (int i = lane; i < n_vec; i += 32) {
+        const int4 v = *(const int4*)(list + 4 * i);
+        if ((uint32_t)(v.x - lo) < in) flags[v.x - lo] = 1;
+        if ((uint32_t)(v.y - lo) < in) flags[v.y - lo] = 1;
+        if ((uint32_t)(v.z - lo) < in) flags[v.z - lo] = 1;
+        if ((uint32_t)(v.w - lo) < in) flags[v.w - lo] = 1;
+      }
+      for (int i = 4 * n_vec + lane; i < n; i += 32) {
+        const int x = list[i];
+        if ((uint32_t)(x - lo) < in) flags[x - lo] = 1;
+      }
+    }
+    __syncwarp();
+    for (int o = lane * 32; o < span; o += 1024) {
+      uint32_t word = 0u;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint4 f = *(const uint4*)(flags + o + 16 * q);
+        // four bytes of 0 / 1 -> four bits: the product's top byte collects them
+        word |= ((f.x * 0x10204080u) >> 28) << (16 * q) | ((f.y * 0x10204080u) >> 28) << (16 * q + 4) |
+                ((f.z * 0x10204080u) >> 28) << (16 * q + 8) | ((f.w * 0x10204080u) >> 28) << (16 * q + 12);
+      }
+      *(uint32_t*)(dst + (lo + o) / 8) = word;
+    }
+    __syncwarp();
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_token_masks(const int32_t* sel_idx, const int32_t* sel_cnt, int N, int Hkv, int k_max, int t0, int t1, int tile, void* masks,
+                               int64_t st, int64_t sh, cudaStream_t s) {
+  const int64_t items = (int64_t)(t1 - t0) * Hkv;
+  const unsigned grid = (unsigned)((items + kMaskThreads / 32 - 1) / (kMaskThreads / 32));
+  const int vec = k_max % 4 == 0 && ((uintptr_t)sel_idx & 15u) == 0u;
+  token_mask_kernel<<<grid, kMaskThreads, 0, s>>>(sel_idx, sel_cnt, N, Hkv, k_max, t0, t1, tile, (unsigned char*)masks, st, sh, vec);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_max, const int32_t* k_tok, int stem, int local,
                                 int32_t* sel_idx, int32_t* sel_cnt, cudaStream_t s) {

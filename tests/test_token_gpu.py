@@ -198,10 +198,11 @@ def _plain_attention(q, k, v, idx, cnt, rows):
 
 
 # The masked form (every causal key block, the keys outside a list masked out) is taken when n <= 128 / g x k_max, the
-# gather form beyond.  Window edges of the masks: 128-token tiles of one head hold masks of 7 key blocks at a time.
+# gather form beyond.  Masks live in the token's own rows of O up to 2048 g keys, beyond in rows of earlier tokens.
 @pytest.mark.parametrize("n,hq,hkv,k_max,order,repeat,what", [
-    (1930, 2, 2, 64, "ascending", False, "masked, three mask windows, one head per group"),
-    (1930, 2, 2, 61, "any", False, "masked, lists in any order, entries read one at a time"),
+    (2048, 2, 2, 64, "ascending", False, "masked, masks that just fit the tokens' own rows"),
+    (2049, 1, 1, 64, "ascending", False, "masked, two launches: masks in rows of earlier tokens"),
+    (4300, 2, 2, 61, "any", True, "masked, four launches, two windows of flags, entries read one at a time"),
     (897, 7, 1, 300, "ascending", True, "masked, 18-token tiles, lists that name a token twice"),
     (129, 16, 1, 128, "any", True, "masked, 8-token tiles, one token past a key block"),
     (1100, 16, 1, 128, "ascending", False, "gather: the prefix is too long for the masks to pay"),
