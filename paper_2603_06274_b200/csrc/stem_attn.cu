@@ -53,7 +53,6 @@ constexpr int kSlotBytes = 32 * 1024;
 constexpr int kQBytes = 32 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSpareQMaxList = 256;                      // longest list (blocks) served with the spare Q tile
-constexpr int kMaskedFactor = 1;                         // token lists: the masked form up to this times 128 / g x k_max tokens
 constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X; S/P at 128 X
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
 constexpr float kRescaleThreshold = 8.0f;                // log2 units
@@ -581,16 +580,14 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         n = (int)(info & 0x7fffffffu);
       }
       const bool row_valid = m < ntok;
-      // kTok: the row's mask words of the next key block, its list's length, and how many tokens of it the masks have shown
+      // kTok: the row's mask, its list's length, and how many tokens of it the mask has shown
       const int t_row = q_tok0 + m;
       const uint4* mask = nullptr;
-      uint4 mask_next = make_uint4(0, 0, 0, 0);
       int list_n = 0, seen = 0;
       if constexpr (kTok) {
         if (row_valid) {
           list_n = min(max(a.sel_cnt[(int64_t)R * a.T + t_row], 0), min(a.k_max, t_row + 1));
           mask = (const uint4*)(a.masks + (t_row - a.tok_a) * a.mask_st + R * a.mask_sh);
-          mask_next = mask[0];
         }
       }
       if (n == 0) {
@@ -605,6 +602,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       const bool has_diag = (info >> 31) != 0u;
       float m_run = -INFINITY, l_run = 0.f;
       for (int e = 0; e < n; ++e, ++blk) {
+        uint4 mask_w = make_uint4(0, 0, 0, 0);  // kTok: the block's mask words, here while S is still awaited
+        if constexpr (kTok) {
+          if (row_valid) mask_w = mask[e];
+          seen += __popc(mask_w.x) + __popc(mask_w.y) + __popc(mask_w.z) + __popc(mask_w.w);
+        }
         // S of block e is complete; so is every earlier tensor-core operation of this slot,
         // P V of block e-1 included (the commit behind Q K^T covers all earlier operations)
         ok = mbar_wait(bar(Smem::s_full, X), blk & 1, ctx, kBarSFull);
@@ -616,9 +618,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int c = 0; c < BLK / 32; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
         tmem_ld_wait();
         if constexpr (kTok) {
-          const uint32_t w[4] = {mask_next.x, mask_next.y, mask_next.z, mask_next.w};
-          if (row_valid && e + 1 < n) mask_next = mask[e + 1];  // used in the next turn
-          seen += __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
+          const uint32_t w[4] = {mask_w.x, mask_w.y, mask_w.z, mask_w.w};
 #pragma unroll
           for (int c = 0; c < BLK; ++c) s[c] = (w[c >> 5] & (1u << (c & 31))) ? s[c] : -INFINITY;
         } else if (e == n - 1 && has_diag) {
@@ -1099,10 +1099,41 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   return cudaGetLastError();
 }
 
-// Attention over token lists with every causal key block computed and the keys outside a token's list masked out.
-// It costs key blocks x 128 keys for T = 128 / g query tokens at once, the gather kernel its list for every token: both
-// take about 2000 cycles per 128 keys, so the masked form wins until a causal prefix (n_tokens / 2 on average) is T
-// times as long as a list.  8K tokens, 32 / 8 heads, top 2048: 0.72 ms against 6.4 (start: 7.3), of which 0.52 attention.
+// The masks of the query tokens below b need mask_bytes each: from which token on they are computed in one launch.
+// All of them (0) if a mask fits the token's own rows of O; else as many as find room in the rows of the tokens before.
+static int first_token_of_launch(int b, int64_t mask_bytes, int64_t row_bytes) {
+  return mask_bytes <= row_bytes ? 0 : (int)(((int64_t)b * mask_bytes + mask_bytes + row_bytes - 1) / (mask_bytes + row_bytes));
+}
+static int64_t mask_bytes_of(int b) { return (int64_t)((b + kTileM - 1) / kTileM) * (kTileM / 8); }
+
+// Whether computing every causal key block is cheaper than gathering the lists, by estimates in microseconds that were
+// fitted to both (148 SMs, within 25 % from 0.02 to 7 ms):
+//   gather   a list entry tile of 128 costs 1.05, an item (token, kv head) 0.7 + 0.14 g on top, spread over the SMs
+//   masked   a launch 12, then a block of 128 keys x 128 rows 2.1 on a CTA whose two slots are busy, 1.7 on one whose
+//            first alone is, along the items of the CTA that gets the longest ones; reading the lists 5 TB/s
+// Measured gather / masked in us: 8192 tokens, 32/8 heads, top 2048: 6440 / 609; 12000, 32/2, 1024: 1877 / 1025;
+// 12000, 8/2, 256: 448 / 425; 12000, 8/2, 128: 337 / 422; 12000, 32/2, 256: 881 / 1004; 12000, 2/2, 128: 306 / 715 (ten
+// launches); 512, 4/1, 128: 15.5 / 21.8.
+static bool masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count) {
+  const double sms = sm_count, k = std::min(k_max, N);
+  const double gather = 8.0 + (double)N * Hkv / sms * (0.7 + 0.14 * g + 1.05 * std::max(1.0, k / kTileM * (1.0 - 0.5 * k / N)));
+  double masked = 0.0;
+  const int tile = kTileM / g;
+  for (int b = N; b > 0 && masked < gather;) {
+    const int a = first_token_of_launch(b, mask_bytes_of(b), (int64_t)g * kHeadDim * 2);
+    const int tiles = (b - a + tile - 1) / tile;
+    const int64_t items = (int64_t)tiles * Hkv;
+    int64_t path = 0;
+    for (int64_t i = 0; i < items; i += 2 * sm_count)
+      path += (std::min(a + (tiles - (int)(i / Hkv)) * tile, b) + kTileM - 1) / kTileM;
+    masked += 12.0 + path * (items > sm_count ? 2.1 : 1.7) + (double)(b - a) * Hkv * k * 4e-6 / 5.0;
+    b = a;
+  }
+  return masked < gather;
+}
+
+// Attention over token lists with every causal key block computed and the keys outside a token's list masked out, for
+// 128 / g query tokens (128 rows) at once.
 // The masks, one bit per key of the prefix, are built by a kernel of their own (token_mask_kernel) into the rows of O that
 // are not yet final: of the query tokens themselves, whose masks are read before their rows are written, if a prefix has no
 // more bits than a row of the group (2048 g); else the tokens are computed from the last ones on, as many at a time as find
@@ -1112,7 +1143,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
                                 void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s) {
   *taken = false;
   const int g = Hq / Hkv, tile = kTileM / g;
-  if ((int64_t)N > (int64_t)kMaskedFactor * tile * k_max) return cudaSuccess;
+  if (!masked_is_cheaper(N, Hkv, g, k_max, sm_count)) return cudaSuccess;
   CUtensorMap mq, mk, mv;
   if (!make_map(&mq, Q, N, Hq, q_st, q_sh, tile, g) || !make_map(&mk, K, N, Hkv, kv_st, kv_sh, kTileM) ||
       !make_map(&mv, V, N, Hkv, kv_st, kv_sh, kTileM))
@@ -1132,18 +1163,12 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
   }
   const int64_t row_bytes = (int64_t)g * kHeadDim * 2;  // of O, per token and kv head
   for (int b = N; b > 0; b = a.tok_a) {
-    const int64_t mask_bytes = (int64_t)((b + kTileM - 1) / kTileM) * (kTileM / 8);
+    const int64_t mask_bytes = mask_bytes_of(b);
+    const bool own_rows = mask_bytes <= row_bytes;
     a.masks = (const unsigned char*)O;
-    if (mask_bytes <= row_bytes) {
-      a.tok_a = 0;
-      a.mask_st = Hkv * row_bytes;
-      a.mask_sh = row_bytes;
-    } else {
-      // (b - tok_a) masks fit tok_a rows
-      a.tok_a = (int)(((int64_t)b * mask_bytes + mask_bytes + row_bytes - 1) / (mask_bytes + row_bytes));
-      a.mask_st = Hkv * mask_bytes;
-      a.mask_sh = mask_bytes;
-    }
+    a.tok_a = first_token_of_launch(b, mask_bytes, row_bytes);
+    a.mask_sh = own_rows ? row_bytes : mask_bytes;
+    a.mask_st = Hkv * a.mask_sh;
     a.tok_b = b;
     a.n_items = ((b - a.tok_a + tile - 1) / tile) * Hkv;
     cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, tile, O, a.mask_st, a.mask_sh, s);

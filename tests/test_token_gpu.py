@@ -197,16 +197,17 @@ def _plain_attention(q, k, v, idx, cnt, rows):
     return out, lse
 
 
-# The masked form (every causal key block, the keys outside a list masked out) is taken when n <= 128 / g x k_max, the
-# gather form beyond.  Masks live in the token's own rows of O up to 2048 g keys, beyond in rows of earlier tokens.
+# The masked form (every causal key block, the keys outside a list masked out) is taken where it is estimated to be the
+# faster one, the gather form for lists that are short against the prefix.  Masks live in the token's own rows of O up to
+# 2048 g keys, beyond in rows of earlier tokens.
 @pytest.mark.parametrize("n,hq,hkv,k_max,order,repeat,what", [
-    (2048, 2, 2, 64, "ascending", False, "masked, masks that just fit the tokens' own rows"),
-    (2049, 1, 1, 64, "ascending", False, "masked, two launches: masks in rows of earlier tokens"),
-    (4300, 2, 2, 61, "any", True, "masked, four launches, two windows of flags, entries read one at a time"),
-    (897, 7, 1, 300, "ascending", True, "masked, 18-token tiles, lists that name a token twice"),
-    (129, 16, 1, 128, "any", True, "masked, 8-token tiles, one token past a key block"),
-    (1100, 16, 1, 128, "ascending", False, "gather: the prefix is too long for the masks to pay"),
-    (700, 5, 1, 27, "any", True, "gather, lists in any order and with repeats"),
+    (2048, 4, 4, 512, "ascending", False, "masked, masks that just fit the tokens' own rows"),
+    (2049, 4, 4, 512, "ascending", False, "masked, two launches: masks in rows of earlier tokens"),
+    (4300, 2, 2, 1501, "any", True, "masked, four launches, two windows of flags, entries read one at a time"),
+    (897, 28, 4, 300, "ascending", True, "masked, 18-token tiles, lists that name a token twice"),
+    (129, 64, 4, 128, "any", True, "masked, 8-token tiles, one token past a key block"),
+    (3000, 2, 2, 20, "ascending", False, "gather: lists short against the prefix"),
+    (300, 5, 1, 27, "any", True, "gather, lists in any order and with repeats"),
 ])
 def test_token_attention_forms(n, hq, hkv, k_max, order, repeat, what):
     r = np.random.default_rng(n + k_max)
