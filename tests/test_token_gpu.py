@@ -255,3 +255,44 @@ def test_token_attention_ignores_rows_no_list_names():
     assert clean.any() and not clean.all()
     check_attention(outs[1][clean], outs[0][clean], np.ones(outs[0][clean].shape, bool), label="rows whose lists name no bad row")
     assert not np.isfinite(outs[1][~clean]).all(axis=1).any()
+
+
+@pytest.mark.parametrize("n,heads,k_start,stem,local,ties", [
+    (33, 2, 7, 0, 1, True),          # less than a warp's row
+    (1024, 1, 300, 3, 5, True),      # one warp to a row, its last row full
+    (1025, 2, 1000, 0, 1, False),    # the first row of two warps; N not a multiple of four: scalar loads
+    (2052, 1, 64, 1, 2, True),       # rows of two and of four warps
+    (4097, 1, 2048, 0, 1, False),    # the first row of eight warps
+    (8200, 1, 500, 4, 8, True),      # rows of sixteen warps
+    (16388, 1, 700, 0, 1, True),     # longer than the registers hold: the other kernel for all rows
+])
+def test_token_selection_row_lengths(n, heads, k_start, stem, local, ties):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    sc = torch.randn((heads, n, n), generator=g, device="cuda")
+    if ties:
+        sc = torch.round(sc * 2.0) / 2.0 * torch.where(torch.rand((heads, n, n), generator=g, device="cuda") < 0.5, 1.0, -1.0)
+        sc[0, n - 1, 3:9] = float("nan")
+        sc[0, n // 2, ::5] = float("inf")
+        sc[0, n // 3, 1::4] = float("-inf")
+    k_tok = binding.stem_token_budget(n, k_start, (7, 10), stem, local)
+    k_max = int(k_tok.max())
+    idx = torch.full((heads, n, k_max), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.full((heads, n), -7, dtype=torch.int32, device="cuda")
+    binding.stem_token_select(sc, k_tok.cuda(), idx, cnt, stem, local)
+    torch.cuda.synchronize()
+    rows = sorted({0, 1, stem + local - 1, k_start - 1, k_start, n // 3, n // 2, n - 1, 1023, 1024, 2047, 2048, 4095, 4096, 8191, 8192}
+                  | set(np.random.default_rng(n).integers(0, n, 40).tolist()))
+    for h in range(heads):
+        for t in [t for t in rows if 0 <= t < n]:
+            s = sc[h, t, :t + 1].cpu().numpy().astype(np.float64)
+            s[np.isnan(s)] = -np.inf
+            forced = (np.arange(t + 1) < stem) | (np.arange(t + 1) > t - local)
+            free = np.flatnonzero(~forced)
+            want = max(int(k_tok[t]) - int(forced.sum()), 0)
+            best = free[np.lexsort((free, -s[free]))][:want]
+            ref = np.sort(np.concatenate([np.flatnonzero(forced), best]))
+            got = idx[h, t].cpu().numpy()
+            assert int(cnt[h, t]) == len(ref)
+            assert np.array_equal(got[:len(ref)], ref), (h, t)
+            assert (got[len(ref):] == -1).all()
