@@ -390,19 +390,23 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
 // from it.  (Two ways of overlapping the HBM-bound pooling with the scoring were measured and dropped: phases
 // on two streams lose more to cross-stream event waits than they gain, and one persistent kernel
 // with a shared ticket list leaves too few warps per SM to stream HBM.)
+// first_word: the status words from it on are cleared (those of the metric kernels, 4; with the attention behind, all).
 static int enqueue_score_select(const Plan& p, const void* Q, const void* K, const void* V, void* kcache, uint8_t* w,
-                                int32_t* idx, int32_t* cnt, cudaStream_t s) {
+                                int32_t* idx, int32_t* cnt, int first_word, cudaStream_t s) {
   const KSide ks = k_side(p, w, kcache);
   float* M = (float*)(w + p.ws.metric);  // holds the bit planes of the selection keys, not the floats
-  int rc = cuda_rc(cudaMemsetAsync(w + p.ws.status + 16, 0, 16, s));  // the metric kernel's status words
-  if (rc != STEM_OK) return rc;
-  // (the anti-diagonal mode has no use for the pooled query vectors)
-  rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, false, s));
+  // (the anti-diagonal mode has no use for the pooled query vectors; the pooling kernel clears all status words)
+  int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, false,
+                               (int32_t*)(w + p.ws.status) + first_word, kStatusWords - first_word, s));
   if (rc != STEM_OK) return rc;
   p.last_launches++;
-  rc = enqueue_metric(p, Q, K, w, ks, M, true, true, s);
-  if (rc != STEM_OK) return rc;
-  rc = cuda_rc(launch_select_planes(p, (const uint32_t*)M, p.score_mode != 1, idx, cnt, s));
+  if (small_score_select(p)) {
+    rc = cuda_rc(launch_small_score_select(p, w + p.ws.qsplit, ks.ksplit, ks.mv, idx, cnt, s));
+  } else {
+    rc = enqueue_metric(p, Q, K, w, ks, M, true, true, s);
+    if (rc != STEM_OK) return rc;
+    rc = cuda_rc(launch_select_planes(p, (const uint32_t*)M, p.score_mode != 1, idx, cnt, s));
+  }
   if (rc == STEM_OK) p.last_launches++;
   return rc;
 }
@@ -419,9 +423,8 @@ int stem_score(const stem_plan* plan, const void* Q, const void* K, const void* 
   cudaStream_t s = (cudaStream_t)stream;
   p.last_launches = 0;
   float* mv = (float*)(w + p.ws.mv);
-  rc = cuda_rc(cudaMemsetAsync(w + p.ws.status + 16, 0, 16, s));  // the metric kernel's status words
-  if (rc != STEM_OK) return rc;
-  rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, mv, w + p.ws.qsplit, w + p.ws.ksplit, false, s));
+  rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, mv, w + p.ws.qsplit, w + p.ws.ksplit, false,
+                           (int32_t*)(w + p.ws.status) + 4, 4, s));  // ... and the metric kernel's status words
   if (rc != STEM_OK) return rc;
   p.last_launches++;
   if (M) rc = enqueue_metric(p, Q, K, w, k_side(p, w, nullptr), M, false, true, s);
@@ -467,7 +470,7 @@ int stem_score_select(const stem_plan* plan, const void* Q, const void* K, const
   if (rc != STEM_OK) return rc;
   uint8_t* w = (uint8_t*)ws;
   p.last_launches = 0;
-  return enqueue_score_select(p, Q, K, V, nullptr, w, sel_idx, sel_cnt, (cudaStream_t)stream);
+  return enqueue_score_select(p, Q, K, V, nullptr, w, sel_idx, sel_cnt, 4, (cudaStream_t)stream);
 }
 
 int stem_pool_kv(const stem_plan* plan, const void* K, const void* V, void* kcache, void* stream) {
@@ -477,7 +480,7 @@ int stem_pool_kv(const stem_plan* plan, const void* K, const void* V, void* kcac
   if (p.kcache_blocks == 0) return STEM_ERR_INVALID_ARG;
   const KSide ks = k_side(p, nullptr, kcache);
   p.last_launches = 0;
-  const int rc = cuda_rc(launch_pool(p, nullptr, K, V, ks.mv, nullptr, ks.ksplit, true, (cudaStream_t)stream));
+  const int rc = cuda_rc(launch_pool(p, nullptr, K, V, ks.mv, nullptr, ks.ksplit, true, nullptr, 0, (cudaStream_t)stream));
   if (rc == STEM_OK) p.last_launches++;
   return rc;
 }
@@ -492,7 +495,7 @@ int stem_score_select_cached(const stem_plan* plan, const void* Q, const void* k
   int rc = check_ws(p, ws, ws_bytes);
   if (rc != STEM_OK) return rc;
   p.last_launches = 0;
-  return enqueue_score_select(p, Q, nullptr, nullptr, const_cast<void*>(kcache), (uint8_t*)ws, sel_idx, sel_cnt,
+  return enqueue_score_select(p, Q, nullptr, nullptr, const_cast<void*>(kcache), (uint8_t*)ws, sel_idx, sel_cnt, 4,
                               (cudaStream_t)stream);
 }
 
@@ -506,7 +509,7 @@ int stem_sparse_prefill(const stem_plan* plan, const void* Q, const void* K, con
   if (rc != STEM_OK) return rc;
   p.last_launches = 0;
   rc = cuda_rc(launch_sparse_attention(p, Q, K, V, sel_idx, sel_cnt, p.share_group, O, lse,
-                                       (int32_t*)((uint8_t*)ws + p.ws.status), (cudaStream_t)stream));
+                                       (int32_t*)((uint8_t*)ws + p.ws.status), false, (cudaStream_t)stream));
   if (rc == STEM_OK) p.last_launches++;
   return rc;
 }
@@ -520,13 +523,13 @@ static int enqueue_prefill(const Plan& p, const void* Q, const void* K, const vo
   int rc = STEM_OK;
   if (kcache && update_cache) {
     const KSide ks = k_side(p, w, kcache);
-    rc = cuda_rc(launch_pool(p, nullptr, K, V, ks.mv, nullptr, ks.ksplit, true, s));
+    rc = cuda_rc(launch_pool(p, nullptr, K, V, ks.mv, nullptr, ks.ksplit, true, nullptr, 0, s));
     if (rc != STEM_OK) return rc;
     p.last_launches++;
   }
-  rc = enqueue_score_select(p, Q, kcache ? nullptr : K, kcache ? nullptr : V, kcache, w, idx, cnt, s);
+  rc = enqueue_score_select(p, Q, kcache ? nullptr : K, kcache ? nullptr : V, kcache, w, idx, cnt, 0, s);
   if (rc != STEM_OK) return rc;
-  rc = cuda_rc(launch_sparse_attention(p, Q, K, V, idx, cnt, p.share_group, O, lse, (int32_t*)(w + p.ws.status), s));
+  rc = cuda_rc(launch_sparse_attention(p, Q, K, V, idx, cnt, p.share_group, O, lse, (int32_t*)(w + p.ws.status), true, s));
   if (rc != STEM_OK) return rc;
   p.last_launches++;
   return STEM_OK;

@@ -131,17 +131,17 @@ __device__ int32_t g_masked_status[4];  // status words of the token-list form, 
 
 struct Ctx {
   volatile int* abort_flag;  // shared memory
-  int32_t* status;           // global memory status words (null: g_masked_status)
+  int32_t* status;           // global memory status words
   int role;
+  int code;                  // what the first of them says: 1, or 4 for the token-list form
 };
 
 __device__ __forceinline__ void raise_abort(const Ctx& c, int bar_id) {
   *c.abort_flag = 1;
-  int32_t* st = c.status ? c.status : g_masked_status;
-  if (atomicCAS(st, 0, c.status ? 1 : 4) == 0) {
-    st[1] = (int32_t)blockIdx.x;
-    st[2] = c.role;
-    st[3] = bar_id;
+  if (atomicCAS(c.status, 0, c.code) == 0) {
+    c.status[1] = (int32_t)blockIdx.x;
+    c.status[2] = c.role;
+    c.status[3] = bar_id;
   }
 }
 
@@ -487,6 +487,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
 
   volatile int* abort_flag = (volatile int*)(smem_gen + Smem::abort_flag);
+  int32_t* const status = kTok ? g_masked_status : a.status;
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(smem_gen + Smem::tmem_ptr);
   auto bar = [&](int off, int idx) { return smem_base + off + 8 * idx; };
   // kSpareQ: three Q tiles (the next item's tile is loaded into a spare while the current items run) and a ring of
@@ -521,6 +522,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // Launched as a programmatic dependent of the selection, everything above overlaps its tail; lists, Q, K, V and O are
+  // touched only below.  (Without that launch attribute this is a no-op.)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -536,7 +540,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // ============================== softmax of slot X ==============================
     set_max_regs_inc<kRegsSoftmax>();
     const int X = warp >> 2;
-    Ctx ctx{abort_flag, a.status, kRoleSoftmax};
+    Ctx ctx{abort_flag, status, kRoleSoftmax, kTok ? 4 : 1};
     const int m = (warp & 3) * 32 + lane;  // query row inside the tile == TMEM lane
     const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_addr = lane_addr + X * 128;
@@ -747,7 +751,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     set_max_regs_dec<kRegsOther>();
     if (warp == 8) {
       // ============================== K / V producer ==============================
-      Ctx ctx{abort_flag, a.status, kRoleProducer};
+      Ctx ctx{abort_flag, status, kRoleProducer, kTok ? 4 : 1};
       struct KvSlot {
         ItemCursor<kTok> cur;
         bool has, pend;
@@ -817,7 +821,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
     } else if (warp == 10) {
       // ============================== Q producer ==============================
-      Ctx ctx{abort_flag, a.status, kRoleQProducer};
+      Ctx ctx{abort_flag, status, kRoleQProducer, kTok ? 4 : 1};
       if constexpr (kSpareQ) {
         // The two slots advance one block per round of the MMA issuer, so the round at which a slot's item ends is the
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
@@ -919,7 +923,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // a branch when there is nothing to wait for, a wait that gave up is looked at once per round, the MMA loops are
       // unrolled and the list lengths are fetched an item ahead (LengthCursor).  Dense 16K tokens: 1234 TFLOP/s; rolled
       // loops 1200; waits that return a flag and vote 1053; a second warp that checks ahead and queues commands 1197.
-      Ctx ctx{abort_flag, a.status, kRoleMma};
+      Ctx ctx{abort_flag, status, kRoleMma, kTok ? 4 : 1};
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {
@@ -1052,7 +1056,7 @@ bool make_map(CUtensorMap* map, const void* base, int64_t T, int H, int64_t stri
 
 cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K, const void* V, const int32_t* sel_idx,
                                     const int32_t* sel_cnt, bool list_group, void* O, float* lse, int32_t* status,
-                                    cudaStream_t s) {
+                                    bool dependent, cudaStream_t s) {
   const int B = p.cfg.block;
   CUtensorMap mq, mk, mv;
   // With H == 1 the head stride is irrelevant to addressing but must still be a legal TMA stride.
@@ -1070,9 +1074,10 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   a.list_div = list_group ? a.g : 1;
   a.scale_log2 = p.softmax_scale * 1.4426950408889634f;
 
+  cudaError_t e = cudaSuccess;
   // this kernel's status words only: words 4.. belong to the metric kernel, whose record of a wait that gave up
   // must survive until stem_check_status reads it
-  cudaError_t e = cudaMemsetAsync(status, 0, 4 * sizeof(int32_t), s);
+  if (!dependent) e = cudaMemsetAsync(status, 0, 4 * sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
   // the attribute belongs to the device's context: set it once per device of this process
   static bool attr_set[64] = {};
@@ -1089,14 +1094,21 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Lists of up to a few hundred blocks: the spare Q tile (an item boundary then costs no wait for Q); the dense mode
   // and longer lists: the deeper K / V ring.
   const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList;
-  if (B == 128) {
-    if (spare_q) sparse_attn_kernel<128, true, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
-    else sparse_attn_kernel<128, false, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
-  } else {
-    if (spare_q) sparse_attn_kernel<64, true, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
-    else sparse_attn_kernel<64, false, false><<<grid, kThreads, kSmemBytes, s>>>(mq, mk, mv, a, TokRows{});
-  }
-  return cudaGetLastError();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
+  // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
+  cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
+  auto kernel = B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false> : sparse_attn_kernel<128, false, false>)
+                         : (spare_q ? sparse_attn_kernel<64, true, false> : sparse_attn_kernel<64, false, false>);
+  return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, a, TokRows{});
 }
 
 // The masks of the query tokens below b need mask_bytes each: from which token on they are computed in one launch.

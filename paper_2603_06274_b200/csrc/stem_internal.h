@@ -98,9 +98,9 @@ inline size_t kcache_bytes(const Plan& p) { return kcache_mv_offset(p) + (size_t
 // Alg. 1 step 1.  Q side (Q != null): Qbar of every query row as hi + mid + lo bf16 parts into qsplit
 // [3, H_list, R_tot, d] (the mean over the heads of a kv group as well, with share_group).  K side (K, V != null):
 // Kbar parts into ksplit [3, H_kv, KB_tot, d] and MV into mv [H_kv, KB_tot], for every key block of the plan or,
-// with only_new, for the blocks the chunk adds.
+// with only_new, for the blocks the chunk adds.  The n_clear status words at `clear` are set to zero.
 cudaError_t launch_pool(const Plan& p, const void* Q, const void* K, const void* V, float* mv, void* qsplit, void* ksplit,
-                        bool only_new, cudaStream_t s);
+                        bool only_new, int32_t* clear, int n_clear, cudaStream_t s);
 
 // Metric of every causal block (layout of stem_score's M) from the split pooled vectors, on the tensor cores.
 // as_keys: instead of the floats, store bit planes of the selection's order-preserving keys: row r of sequence b at
@@ -126,10 +126,18 @@ cudaError_t launch_select_rows(const Plan& p, const float* M, bool dependent, in
 cudaError_t launch_select_planes(const Plan& p, const uint32_t* Mt, bool dependent, int32_t* sel_idx, int32_t* sel_cnt,
                                  cudaStream_t s);
 
+// Metric and selection of short sequences in one kernel, straight from the split pooled vectors (Alg. 1 steps 3a-3c):
+// whether a plan is one for it, and its launch (a programmatic dependent of the pooling kernel).
+bool small_score_select(const Plan& p);
+cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
+                                      int32_t* sel_cnt, cudaStream_t s);
+
+// dependent: launched as a programmatic dependent of the selection kernel enqueued just before, its status words cleared by
+// an earlier kernel; otherwise the launch clears them itself.
 // list_group: the lists are per kv head ([H_kv, R_tot, k_max]); every query head of a group walks its group's list.
 cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K, const void* V,
                                     const int32_t* sel_idx, const int32_t* sel_cnt, bool list_group, void* O, float* lse,
-                                    int32_t* status, cudaStream_t s);
+                                    int32_t* status, bool dependent, cudaStream_t s);
 
 // Token-level selection and gather attention (one sequence; lists per kv head).
 int token_attn_max_group();

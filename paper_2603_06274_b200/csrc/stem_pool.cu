@@ -43,6 +43,8 @@ struct PoolArgs {
   RowTables rows;
   float* mv;
   __nv_bfloat16 *qsplit, *ksplit;
+  int32_t* clear;  // status words the kernels behind this one start from zero with (or null)
+  int n_clear;
 };
 
 template <int kBlock, bool kGroupMean>
@@ -53,6 +55,7 @@ __global__ void __launch_bounds__(128) pool_kernel(const PoolArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = lane >> 4, chunk = lane & 15;
+  if (blockIdx.x == 0 && (int)threadIdx.x < a.n_clear) a.clear[threadIdx.x] = 0;  // (a memset of its own costs 2.5 us of a small call)
 
   const __nv_bfloat16* base;
   int64_t st, sh;
@@ -167,8 +170,9 @@ __global__ void __launch_bounds__(128) pool_kernel(const PoolArgs a) {
 }  // namespace
 
 cudaError_t launch_pool(const Plan& p, const void* Q, const void* K, const void* V, float* mv, void* qsplit, void* ksplit,
-                        bool only_new, cudaStream_t s) {
+                        bool only_new, int32_t* clear, int n_clear, cudaStream_t s) {
   PoolArgs a{};
+  a.clear = clear; a.n_clear = n_clear;
   a.Q = (const __nv_bfloat16*)Q; a.K = (const __nv_bfloat16*)K; a.V = (const __nv_bfloat16*)V;
   a.q_st = p.cfg.q_stride_tok; a.q_sh = p.cfg.q_stride_head; a.kv_st = p.cfg.kv_stride_tok; a.kv_sh = p.cfg.kv_stride_head;
   a.H_list = p.H_list; a.heads_per_list = p.cfg.num_q_heads / p.H_list; a.Hkv = p.cfg.num_kv_heads;

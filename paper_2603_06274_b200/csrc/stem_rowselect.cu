@@ -15,6 +15,7 @@
 //   select_planes_kernel  from the bit planes the metric kernel writes for the fused path: one
 //                         128-byte line per lane, nothing to convert or transpose.
 // Both are bound by the integer pipe, so the stages are written for few logic instructions.
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "stem_internal.h"
@@ -25,6 +26,7 @@ namespace stem {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int64_t kSmallRowsMax = 8192;  // (list head, row) pairs of the small kernel
 
 // Monotone map float -> uint32 with -0 == +0 and NaN below everything (as -inf).  Every key is >= 1.
 __device__ __forceinline__ uint32_t metric_key(float f) {
@@ -203,6 +205,7 @@ __device__ __forceinline__ int warp_scan(int v, int lane) {
 template <int SETS>
 __global__ void __launch_bounds__(kThreads, SETS == 1 ? 4 : 2) select_planes_kernel(const SelArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t item = (int64_t)blockIdx.x * (kThreads / 32) + warp;
   if (item >= (int64_t)a.Hq * a.R_tot) return;
   const int h = (int)(item % a.Hq);
@@ -301,7 +304,145 @@ __global__ void __launch_bounds__(kThreads, SETS == 1 ? 4 : 2) select_planes_ker
   if (lane == 0) a.sel_cnt[(int64_t)h * a.R_tot + R] = total;
 }
 
+// ------------------------------------------------------------------------------------------------
+// Metric and selection of short sequences (up to 64 blocks) in one kernel: one CTA per (list head, row).  A half-warp reads
+// a pooled key vector (its three parts, 256 bytes each) and multiplies it with the row's query vector; then one warp has
+// column j in lane j mod 32, a ballot per key bit gives that bit of all columns to every lane, and the radix descent needs
+// no reductions.  The tensor-core metric kernel and the selection behind it are bound by latency at these sizes (tensor
+// memory, tensor maps, a chain of copies and MMAs): 9.6 + 1.3 us at 12 blocks, where this takes 2.
+// ------------------------------------------------------------------------------------------------
+struct SmallArgs {
+  const __nv_bfloat16 *q, *k;  // split pooled vectors [3, H_list, R_tot, d], [3, H_kv, KB_tot, d]
+  const float* mv;
+  int32_t *sel_idx, *sel_cnt;
+  RowTables rows;
+  int H_list, Hkv, R_tot, KB_tot, k_max, stem, local;
+  float scale, beta;
+};
+
+constexpr int kSmallBlocks = 64;
+constexpr int kSmallThreads = 128;
+
+// Eight pooled values of one lane: the sum of the three bf16 parts is the fp32 value exactly.
+__device__ __forceinline__ void load_split8(const __nv_bfloat16* p, int64_t plane, float (&f)[8]) {
+  const uint4 hi = *(const uint4*)p, mid = *(const uint4*)(p + plane), lo = *(const uint4*)(p + 2 * plane);
+  const uint32_t a[4] = {hi.x, hi.y, hi.z, hi.w}, b[4] = {mid.x, mid.y, mid.z, mid.w}, c[4] = {lo.x, lo.y, lo.z, lo.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = __uint_as_float(a[i] << 16) + __uint_as_float(b[i] << 16) + __uint_as_float(c[i] << 16);
+    f[2 * i + 1] = __uint_as_float(a[i] & 0xffff0000u) + __uint_as_float(b[i] & 0xffff0000u) + __uint_as_float(c[i] & 0xffff0000u);
+  }
+}
+
+__global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const SmallArgs a) {
+  __shared__ float dots[kSmallBlocks];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int half = lane >> 4, chunk = lane & 15;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int item = blockIdx.x;
+  const int h = item % a.H_list, R = a.R_tot - 1 - item / a.H_list;  // long rows first
+  const int kvh = h / (a.H_list / a.Hkv);
+  const int seq = a.rows.row_seq[R], r = a.rows.row_r[R];
+  const int kb0 = a.rows.seq_kb_off[seq];
+  const int i = r + 1;
+  const int n_stem = min(a.stem, i);
+  const int c_lo = n_stem, c_hi = max(max(i - a.local, 0), n_stem);  // candidates [c_lo, c_hi)
+  const int n_cand = c_hi - c_lo;
+  const int need = max(min(a.rows.row_keff[R] - (i - n_cand), n_cand), 0);
+  auto range = [](int lo, int hi) -> uint64_t {  // bits lo .. hi - 1
+    return (hi >= 64 ? ~0ull : (1ull << hi) - 1ull) & ~(lo >= 64 ? ~0ull : (1ull << lo) - 1ull);
+  };
+  const uint64_t all = range(0, i), cand = range(c_lo, c_hi);
+  uint64_t sel = all & ~cand;  // the forced blocks
+  const bool ranked = need > 0 && need < n_cand;
+  if (need > 0 && !ranked) sel = all;
+
+  // everything above overlaps the tail of the pooling kernel, whose results are read below
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (ranked) {
+    // warp w: the columns 16 w .. 16 w + 15, eight per half-warp, all of their loads in flight together
+    const int64_t q_plane = (int64_t)a.H_list * a.R_tot * kHeadDim, k_plane = (int64_t)a.Hkv * a.KB_tot * kHeadDim;
+    const int j0 = 16 * warp;
+    if (j0 < c_hi) {
+      const __nv_bfloat16* krow = a.k + ((int64_t)kvh * a.KB_tot + kb0) * kHeadDim + chunk * 8;
+      float q[8], acc[8];
+      load_split8(a.q + ((int64_t)h * a.R_tot + R) * kHeadDim + chunk * 8, q_plane, q);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        float k[8];
+        load_split8(krow + (int64_t)min(j0 + 2 * u + half, r) * kHeadDim, k_plane, k);
+        acc[u] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[u] = fmaf(q[c], k[c], acc[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], d);
+        if (chunk == 0) dots[j0 + 2 * u + half] = acc[u];
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const float* mv = a.mv + (int64_t)kvh * a.KB_tot + kb0;
+      const float d0 = lane < c_hi ? dots[lane] : 0.f, d1 = lane + 32 < c_hi ? dots[lane + 32] : 0.f;
+      const uint32_t key0 = metric_key(fmaf(a.scale, d0, a.beta * mv[min(lane, r)]));
+      const uint32_t key1 = metric_key(fmaf(a.scale, d1, a.beta * mv[min(lane + 32, r)]));
+      uint64_t act = cand, gt = 0ull;
+      int k = need;
+#pragma unroll 1
+      for (int b = 31; b >= 0; --b) {
+        const uint64_t plane = (uint64_t)__ballot_sync(0xffffffffu, (key0 >> b) & 1u) |
+                               ((uint64_t)__ballot_sync(0xffffffffu, (key1 >> b) & 1u) << 32);
+        const uint64_t ones = act & plane;
+        const int cnt = __popcll(ones);
+        const bool inside = cnt >= k;  // the k-th largest key has this bit set
+        gt |= inside ? 0ull : ones;
+        k -= inside ? 0 : cnt;
+        act = inside ? ones : act & ~plane;
+      }
+      // of the equal keys the first k by block id
+      while (k < __popcll(act)) act &= ~(1ull << (63 - __clzll((long long)act)));
+      sel |= gt | act;
+    }
+  }
+  if (warp != 0) return;
+  int32_t* out = a.sel_idx + ((int64_t)h * a.R_tot + R) * a.k_max;
+  const int total = __popcll(sel);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int col = lane + 32 * s;
+    if ((sel >> col) & 1ull) out[__popcll(sel & ((1ull << col) - 1ull))] = col;
+  }
+  for (int q = total + lane; q < a.k_max; q += 32) out[q] = -1;
+  if (lane == 0) a.sel_cnt[(int64_t)h * a.R_tot + R] = total;
+}
+
 }  // namespace
+
+// Sequences of up to 64 blocks, and not so many rows that the tensor cores pay.
+bool small_score_select(const Plan& p) {
+  return p.score_mode == 0 && p.max_nblk <= kSmallBlocks && (int64_t)p.H_list * p.R_tot <= kSmallRowsMax;
+}
+
+cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
+                                      int32_t* sel_cnt, cudaStream_t s) {
+  SmallArgs a{};
+  a.q = (const __nv_bfloat16*)qsplit; a.k = (const __nv_bfloat16*)ksplit; a.mv = mv;
+  a.sel_idx = sel_idx; a.sel_cnt = sel_cnt; a.rows = p.rows;
+  a.H_list = p.H_list; a.Hkv = p.cfg.num_kv_heads; a.R_tot = p.R_tot; a.KB_tot = p.KB_tot; a.k_max = p.k_max;
+  a.stem = p.cfg.stem_blocks; a.local = p.cfg.local_blocks; a.scale = p.score_scale; a.beta = p.cfg.beta;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(p.H_list * p.R_tot));
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, small_score_select_kernel, a);
+}
 
 int row_select_max_blocks() { return 2 * 1024; }
 

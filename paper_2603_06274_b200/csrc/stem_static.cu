@@ -82,7 +82,7 @@ extern "C" int stem_score_static(const stem_plan* plan, const void* Q, const voi
   // (tiles that reach past a sequence's last block read rows of a neighbour or stale rows, and only
   // into entries the epilogue never stores).
   if (cudaMemsetAsync(status, 0, kStatusWords * sizeof(int32_t), s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
-  if (launch_pool(p, Q, K, V, mv, qsplit, ksplit, false, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
+  if (launch_pool(p, Q, K, V, mv, qsplit, ksplit, false, nullptr, 0, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
   p.last_launches++;
   if (launch_metric_gemm(p, qsplit, ksplit, mv, M, false, true, status, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
   p.last_launches++;

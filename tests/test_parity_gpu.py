@@ -241,3 +241,32 @@ def test_argument_errors_enqueue_nothing():
     with pytest.raises(binding.StemError) as e:
         binding.stem_prefill(plan, q.view(-1)[1:-7].view(-1), k, v, out)  # 2-byte offset: misaligned
     assert e.value.status == binding.STEM_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv,share", [
+    (64, (64 * 64,), 4, 2, False),                    # 64 blocks: the longest sequence of the one-kernel scoring
+    (64, (64 * 64 + 1, 700), 4, 2, False),            # one block more: the tensor-core metric
+    (128, (1, 128, 129, 63 * 128 + 5), 2, 1, False),  # sequences of one and two blocks beside one of 64
+    (64, (2000, 900), 8, 2, True),                    # one list per kv head
+    (64, (64 * 64, 64 * 64, 33 * 64), 56, 8, False),  # so many rows that the tensor cores take them
+])
+def test_scoring_of_short_sequences(block, seqlens, hq, hkv, share):
+    w = wl.small("short", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=150, sink=True, seed=sum(seqlens))
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w, share_group=share)
+    info = plan.info
+    idx = torch.full((info.list_heads, info.total_q_blocks, info.k_max), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.full((info.list_heads, info.total_q_blocks), -7, dtype=torch.int32, device="cuda")
+    binding.stem_score_select(plan, q, k, v, idx, cnt)
+    assert binding.stem_check_status(plan)[0] == 0
+    # the lists of the fused path against those selected from the metric that the same library hands out (the tensor cores)
+    M = torch.full((info.list_heads, info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_score(plan, q, k, v, M)
+    M_g = M.cpu().numpy()
+    nblk = so.n_blocks(w.seqlens, w.block)
+    idx_ref, cnt_ref = so.select(np.nan_to_num(M_g, nan=0.0), nblk, plan.budget().numpy(), w.stem_blocks, w.local_blocks)
+    idx_g, cnt_g = idx.cpu().numpy(), cnt.cpu().numpy()
+    ties = compare_selection(idx_g, cnt_g, idx_ref, cnt_ref, M_g, nblk, w)
+    assert len(ties) <= max(2, idx_g.shape[0] * idx_g.shape[1] // 200)
+    plan.close()
