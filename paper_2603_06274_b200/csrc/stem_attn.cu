@@ -60,7 +60,7 @@ constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after:
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4 };
 enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarPEarly };
+                   kBarDrain, kBarPEarly, kBarHalves };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -75,7 +75,8 @@ struct Smem {
   static constexpr int p_early = p_ready + 16;            // all of P but its last 32 key columns stored
   static constexpr int o_full = p_early + 16;
   static constexpr int o_free = o_full + 16;
-  static constexpr int drain = o_free + 16;
+  static constexpr int halves = o_free + 16;              // both slots' parts of a list that was cut in halves
+  static constexpr int drain = halves + 8;
   static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
   static constexpr int total = abort_flag + 4;
@@ -330,6 +331,7 @@ struct AttnArgs {
   RowTables rows;
   int n_items, Hq, g, R_tot, k_max, T;
   int list_div;             // query heads per index list: 1, or g when the lists are per kv head
+  int split;                // every CTA has one item, whose list is cut in halves for its two slots
   // token lists (kTok): sel_idx / sel_cnt are [n_kvh, T, k_max] / [n_kvh, T] lists of single tokens; the launch computes
   // the query tokens tok_a .. tok_b - 1
   int n_kvh, tok_a, tok_b;
@@ -353,15 +355,26 @@ __device__ __forceinline__ void tok_item(const AttnArgs& a, int i, int& kvh, int
   n = (min(a.tok_a + (tile + 1) * a.tok_tile, a.tok_b) - 1) / kTileM + 1;
 }
 
+// A slot's part of a list of n entries that the two slots share.
+__device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
+  const int first = (n + 1) >> 1;
+  off = slot ? first : 0;
+  n = slot ? n - first : first;
+}
+
 // Walks the items of one slot of this CTA: item i of the work order belongs to CTA i % gridDim.x,
 // slot (i / gridDim.x) % 2.  Items with an empty list are skipped (the slot's softmax warps zero
 // their output rows).  Used by whole warps in lock step (values are broadcast from lane 0).
-template <bool kTok>
+// kSplit: with a.split both slots take the same item, slot 0 the first half of its list (rounded up), slot 1 the rest; `off` is
+// the first entry of the slot's part.
+template <bool kTok, bool kSplit>
 struct ItemCursor {
-  int idx, step;
+  int idx, step, slot, off;
   int h, R, r, n;
-  __device__ __forceinline__ void init(int slot) {
-    idx = (int)blockIdx.x + slot * (int)gridDim.x - 2 * (int)gridDim.x;
+  __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
+    slot = slot_;
+    off = 0;
+    idx = (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x) - 2 * (int)gridDim.x;
     step = 2 * (int)gridDim.x;
     n = 0;
   }
@@ -380,6 +393,7 @@ struct ItemCursor {
       R = uni(a.work[2 * idx + 1]);
       r = uni(a.rows.row_r[R]);
       n = a.sel_idx ? min(max(uni(a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R]), 0), a.k_max) : r + 1;
+      if (kSplit && a.split) part_of_list(slot, n, off);
       if (n > 0) return true;
     }
     n = 0;
@@ -389,9 +403,9 @@ struct ItemCursor {
 
 // The list lengths of one slot's items, in the ItemCursor's order, for the MMA issuer: the loads that lead to the length
 // of the next item are started an item ahead (the work entry two items ahead), so that next() waits for none of them.
-template <bool kTok>
+template <bool kTok, bool kSplit>
 struct LengthCursor {
-  int idx, step;       // the item whose length `raw` is
+  int idx, step, slot; // the item whose length `raw` is
   int raw, h2, R2;     // length of item idx as loaded; work entry of item idx + step
   int n;
   __device__ __forceinline__ int length(const AttnArgs& a, int h, int R) const {
@@ -402,9 +416,10 @@ struct LengthCursor {
     h2 = a.work[2 * j];
     R2 = a.work[2 * j + 1];
   }
-  __device__ __forceinline__ void init(const AttnArgs& a, int slot) {
+  __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
+    slot = slot_;
     step = 2 * (int)gridDim.x;
-    idx = (int)blockIdx.x + slot * (int)gridDim.x;
+    idx = (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x);
     if constexpr (kTok) return;
     entry(a, idx);
     raw = length(a, h2, R2);
@@ -422,6 +437,8 @@ struct LengthCursor {
       }
       n = uni(raw);
       if (a.sel_idx) n = min(max(n, 0), a.k_max);
+      int off;
+      if (kSplit && a.split) part_of_list(slot, n, off);
       idx += step;
       raw = length(a, h2, R2);
       entry(a, idx + step);
@@ -494,6 +511,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // four K / V slots, for lists of tens of blocks, where an item boundary that waits for Q costs two blocks' time;
   // otherwise two Q tiles and a ring of five, for long lists (and the dense mode), where the deeper ring pays.
   static_assert(!kTok || (BLK == 128 && !kSpareQ), "the token-list form has two Q tiles and key blocks of 128");
+  constexpr bool kSplit = !kSpareQ && !kTok;  // the layout that may cut lists in halves (a.split)
   constexpr int kKvSlots = kSpareQ ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
@@ -511,6 +529,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::o_full, i), 1);
       mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
     }
+    mbar_init(bar(Smem::halves, 0), 8);
     mbar_init(bar(Smem::drain, 0), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -521,6 +540,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                  "n"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (!kTok && threadIdx.x < 2) {
+    // the plan's tables do not depend on the kernels before this one: fetch what the first items need of them
+    const int item = (int)blockIdx.x + (kSplit && a.split ? 0 : (int)threadIdx.x * (int)gridDim.x);
+    if (item < a.n_items) {
+      const int R = a.work[2 * item + 1];
+      const int seq = a.rows.row_seq[R];
+      asm volatile("" ::"r"(a.work[2 * item]), "r"(a.rows.row_r[R]), "r"(a.rows.row_tok0[R]), "r"(a.rows.row_ntok[R]), "r"(a.rows.seq_tok0[seq]));
+    }
   }
   // Launched as a programmatic dependent of the selection, everything above overlaps its tail; lists, Q, K, V and O are
   // touched only below.  (Without that launch attribute this is a no-op.)
@@ -558,14 +586,25 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       if (kTok || item >= a.n_items) return 0u;
       const int h = a.work[2 * item], R = a.work[2 * item + 1];
       const int r = a.rows.row_r[R];
-      if (dense) return (uint32_t)(r + 1) | 0x80000000u;
-      const int64_t lh = h / a.list_div;
-      const int n = min(max(a.sel_cnt[lh * a.R_tot + R], 0), a.k_max);
-      const bool diag = n > 0 && a.sel_idx[(lh * a.R_tot + R) * a.k_max + n - 1] >= r;
-      return (uint32_t)n | (diag ? 0x80000000u : 0u);
+      int n = r + 1;
+      bool diag = true;
+      if (!dense) {
+        const int64_t lh = h / a.list_div;
+        n = min(max(a.sel_cnt[lh * a.R_tot + R], 0), a.k_max);
+        diag = n > 0 && a.sel_idx[(lh * a.R_tot + R) * a.k_max + n - 1] >= r;
+      }
+      uint32_t halves = 0u;
+      if (kSplit && a.split) {
+        // the last entry is in slot 1's part if that has any; bit 30: both slots have one
+        if (n > 1) { halves = 0x40000000u; diag = diag && X == 1; }
+        int off;
+        part_of_list(X, n, off);
+      }
+      return (uint32_t)n | (diag ? 0x80000000u : 0u) | halves;
     };
-    uint32_t next_info = list_info((int)blockIdx.x + X * (int)gridDim.x);
-    for (int item = (int)blockIdx.x + X * (int)gridDim.x; item < a.n_items && ok; item += 2 * (int)gridDim.x) {
+    const int first_item = (int)blockIdx.x + (kSplit && a.split ? 0 : X * (int)gridDim.x);
+    uint32_t next_info = list_info(first_item);
+    for (int item = first_item; item < a.n_items && ok; item += 2 * (int)gridDim.x) {
       const uint32_t info = next_info;
       next_info = list_info(item + 2 * (int)gridDim.x);
       int h, R, q_tok0, ntok, n;
@@ -581,7 +620,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         R = a.work[2 * item + 1];
         q_tok0 = a.rows.row_tok0[R];
         ntok = a.rows.row_ntok[R];
-        n = (int)(info & 0x7fffffffu);
+        n = (int)(info & 0x3fffffffu);
       }
       const bool row_valid = m < ntok;
       // kTok: the row's mask, its list's length, and how many tokens of it the mask has shown
@@ -595,7 +634,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
       }
       if (n == 0) {
-        if (row_valid) {
+        if (row_valid && !(kSplit && a.split && X == 1)) {  // (an item cut in halves is slot 0's to clear)
           __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
 #pragma unroll
           for (int c = 0; c < 16; ++c) *(uint4*)(o_row + c * 8) = make_uint4(0, 0, 0, 0);
@@ -695,6 +734,60 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
+      if constexpr (kSplit) {
+        if ((info & 0x40000000u) != 0u) {
+          // Two halves of one list: each slot finishes 64 of the 128 columns, for which the other hands over its O, its
+          // reference and its sum through the K / V ring, which nobody uses once both slots' last P V are complete.
+          ok = mbar_wait(bar(Smem::o_full, X ^ 1), 0, ctx, kBarOFull);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const uint32_t mine_s = smem_base + kKvOff + X * kSlotBytes + m * 4, theirs_s = smem_base + kKvOff + (X ^ 1) * kSlotBytes + m * 4;
+          const uint32_t ml_s = smem_base + kKvOff + 2 * kSlotBytes + m * 8;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            float o[32];
+            tmem_ld32(o_addr + (X ^ 1) * 64 + c * 32, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int q = 0; q < 32; ++q) asm volatile("st.shared.f32 [%0], %1;" ::"r"(mine_s + (c * 32 + q) * 512), "f"(o[q]) : "memory");
+          }
+          asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(ml_s + X * 1024), "f"(m_run), "f"(l_run) : "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(Smem::halves, 0));
+          ok = mbar_wait(bar(Smem::halves, 0), 0, ctx, kBarHalves);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          float m_o, l_o;
+          asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(m_o), "=f"(l_o) : "r"(ml_s + (X ^ 1) * 1024) : "memory");
+          const float m_both = fmaxf(m_run, m_o);
+          const float w_mine = fast_exp2(m_run - m_both), w_o = fast_exp2(m_o - m_both);
+          const float l_both = l_run * w_mine + l_o * w_o;
+          const float f_mine = w_mine / l_both, f_o = w_o / l_both;
+          __nv_bfloat16* o_half = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim + X * 64;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            float o[32];
+            tmem_ld32(o_addr + X * 64 + c * 32, o);
+            tmem_ld_wait();
+            uint32_t w[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+              float t0, t1;
+              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(t0) : "r"(theirs_s + (c * 32 + 2 * q) * 512) : "memory");
+              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(t1) : "r"(theirs_s + (c * 32 + 2 * q + 1) * 512) : "memory");
+              w[q] = pack_bf16(fmaf(o[2 * q], f_mine, t0 * f_o), fmaf(o[2 * q + 1], f_mine, t1 * f_o));
+            }
+            if (row_valid) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                *(uint4*)(o_half + c * 32 + q * 8) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            }
+          }
+          if (a.lse && row_valid && X == 0) a.lse[(int64_t)h * a.T + q_tok0 + m] = (m_both + log2f(l_both)) * 0.6931471805599453f;
+          ++ord;
+          continue;
+        }
+      }
       const float inv_l = (kTok && list_n == 0) ? 0.f : 1.f / l_run;
       float finite = 0.f;  // kTok: turns NaN with the first value that is not finite
       const bool o_al32 = ((uintptr_t)a.O & 31u) == 0u;  // rows are multiples of 256 bytes apart
@@ -753,7 +846,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // ============================== K / V producer ==============================
       Ctx ctx{abort_flag, status, kRoleProducer, kTok ? 4 : 1};
       struct KvSlot {
-        ItemCursor<kTok> cur;
+        ItemCursor<kTok, kSplit> cur;
         bool has, pend;
         int e, j_next, pend_tok, pend_kvh, seq_tok0;
         const int32_t* list;
@@ -763,8 +856,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         s.e = 0;
         if (s.has) {
           s.seq_tok0 = kTok ? 0 : uni(a.rows.seq_tok0[uni(a.rows.row_seq[s.cur.R])]);
-          s.list = dense ? nullptr : a.sel_idx + ((int64_t)(s.cur.h / a.list_div) * a.R_tot + s.cur.R) * a.k_max;
-          s.j_next = dense ? 0 : uni(s.list[0]);
+          s.list = dense ? nullptr : a.sel_idx + ((int64_t)(s.cur.h / a.list_div) * a.R_tot + s.cur.R) * a.k_max + s.cur.off;
+          s.j_next = dense ? s.cur.off : uni(s.list[0]);
         }
       };
       uint32_t ring = 0, ring_par = 0;  // next ring slot to fill and its phase
@@ -794,13 +887,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const int tok = s.seq_tok0 + j * BLK;
           if (!load(&map_k, kvh, tok)) return false;
           s.pend = true; s.pend_tok = tok; s.pend_kvh = kvh;
-          if (++s.e < s.cur.n) s.j_next = dense ? s.e : uni(s.list[s.e]);  // consumed on the slot's next visit
+          if (++s.e < s.cur.n) s.j_next = dense ? s.cur.off + s.e : uni(s.list[s.e]);  // consumed on the slot's next visit
           else enter(s);
         }
         return true;
       };
       KvSlot s0, s1;
-      s0.cur.init(0); s1.cur.init(1);
+      s0.cur.init(a, 0); s1.cur.init(a, 1);
       s0.pend = s1.pend = false;
       enter(s0); enter(s1);
       bool ok = true;
@@ -827,12 +920,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
         // next tile, loaded into the spare buffer long before it is wanted; the buffer the slot leaves becomes the
         // spare once the last Q K^T of its item has read it.  The MMA issuer rotates the buffers by the same rule.
-        ItemCursor<kTok> c0, c1;
-        c0.init(0); c1.init(1);
+        ItemCursor<kTok, kSplit> c0, c1;
+        c0.init(a, 0); c1.init(a, 1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t q_used = 0u, q_odd = 0u;  // per buffer (bit b): a tile was loaded; an odd number of tiles was loaded
         bool ok = true;
-        auto load_into = [&](const ItemCursor<kTok>& cur, const int b) -> bool {
+        auto load_into = [&](const ItemCursor<kTok, kSplit>& cur, const int b) -> bool {
           if (((q_used >> b) & 1u) &&
               !__all_sync(0xffffffffu, mbar_wait(bar(Smem::q_empty, b), ((q_odd >> b) & 1u) ^ 1u, ctx, kBarQEmpty)))
             return false;
@@ -873,12 +966,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             while (((q_used >> b) & 1u) && !mbar_try(bar(Smem::q_full, b), ((q_odd >> b) & 1u) ^ 1u) && globaltimer() - t1 < 4000000ull) {}
         }
       } else {
-        ItemCursor<kTok> c0, c1;
-        c0.init(0); c1.init(1);
+        ItemCursor<kTok, kSplit> c0, c1;
+        c0.init(a, 0); c1.init(a, 1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t ord0 = 0, ord1 = 0;
         // Loads the slot's next Q tile as soon as the last Q K^T of its previous item has read the buffer.
-        auto try_load = [&](ItemCursor<kTok>& cur, bool& has, uint32_t& ord, const int X) -> bool {
+        auto try_load = [&](ItemCursor<kTok, kSplit>& cur, bool& has, uint32_t& ord, const int X) -> bool {
           if (!has || !uni((int)mbar_test(bar(Smem::q_empty, X), (ord & 1) ^ 1))) return false;
           const int q_tok0 = kTok ? a.tok_a + cur.R * a.tok_tile : uni(a.rows.row_tok0[cur.R]);
           const int q_head = kTok ? cur.h * a.g : cur.h;
@@ -927,7 +1020,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {
-        LengthCursor<kTok> cur;
+        LengthCursor<kTok, kSplit> cur;
         int left;                      // blocks of the current item whose Q K^T is still to come (0: no item left)
         uint32_t st;                   // kPend: a P V is due, of its item's first (kFirst) / last (kLast) block;
                                        // kNewItem: the next Q K^T is the first of its item
@@ -1093,7 +1186,10 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   const int grid = std::min(p.n_items, p.sm_count);
   // Lists of up to a few hundred blocks: the spare Q tile (an item boundary then costs no wait for Q); the dense mode
   // and longer lists: the deeper K / V ring.
-  const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList;
+  // Grids of no more items than SMs leave the second slot of every CTA idle and are as long as one list: the two slots take
+  // half a list each (4K tokens, 2 heads, blocks of 64, lists of up to 16: the call goes from 28.7 to 26 us).
+  a.split = p.n_items <= p.sm_count ? 1 : 0;
+  const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList && !a.split;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

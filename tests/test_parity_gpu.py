@@ -270,3 +270,35 @@ def test_scoring_of_short_sequences(block, seqlens, hq, hkv, share):
     ties = compare_selection(idx_g, cnt_g, idx_ref, cnt_ref, M_g, nblk, w)
     assert len(ties) <= max(2, idx_g.shape[0] * idx_g.shape[1] // 200)
     plan.close()
+
+
+@pytest.mark.parametrize("rows", [74, 75])
+def test_lists_cut_in_halves_for_the_two_slots(rows):
+    # two heads: 148 items are one per SM (lists cut in halves), 150 are not; lists of 0, 1, 2, 3 and all causal blocks,
+    # with and without the diagonal block
+    w = wl.small("halves", seqlens=(rows * 64 - 7,), hq=2, hkv=1, block=64, permille=1000, seed=rows)
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w)
+    k_max = plan.info.k_max
+    r = np.random.default_rng(rows)
+    idx = np.full((2, rows, k_max), -1, np.int32)
+    cnt = np.zeros((2, rows), np.int32)
+    for h in range(2):
+        for row in range(rows):
+            n = min(int(r.choice([0, 1, 2, 3, 8, row + 1])), row + 1)
+            idx[h, row, :n] = np.sort(r.choice(row + 1, size=n, replace=False))
+            cnt[h, row] = n
+    n_tok = w.total_tokens
+    out = torch.full((n_tok, 2, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((2, n_tok), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_sparse_prefill(plan, q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out, lse)
+    assert binding.stem_check_status(plan)[0] == 0
+    O_ref, lse_ref = so.attention(data["q"], data["k"], data["v"], data["cu_seqlens"], 64, idx, cnt)
+    # tokens that no listed key precedes have no defined softmax (a list without the diagonal block always precedes)
+    check_attention(from_dev_bf16(out), O_ref, ~np.isnan(O_ref), label=f"{2 * rows} items")
+    got = lse.cpu().numpy()
+    assert np.isneginf(got[np.isneginf(lse_ref)]).all()
+    live = np.isfinite(lse_ref)
+    assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
+    plan.close()
