@@ -276,7 +276,7 @@ def test_scoring_of_short_sequences(block, seqlens, hq, hkv, share):
 def test_lists_cut_in_halves_for_the_two_slots(rows):
     # two heads: 148 items are one per SM (lists cut in halves), 150 are not; lists of 0, 1, 2, 3 and all causal blocks,
     # with and without the diagonal block
-    w = wl.small("halves", seqlens=(rows * 64 - 7,), hq=2, hkv=1, block=64, permille=1000, seed=rows)
+    w = wl.small("halves", seqlens=(rows * 64 - 7,), hq=2, hkv=1, block=64, permille=1000, mu_num=1, mu_den=1, seed=rows)
     data = wl.make_qkv(w)
     q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
     plan = StemPlan.from_workload(w)
