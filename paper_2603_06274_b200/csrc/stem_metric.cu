@@ -22,6 +22,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "stem_internal.h"
 #include "stem_ptx.cuh"
 
@@ -64,6 +66,7 @@ struct GemmArgs {
   int64_t m_tot, mt_tot;
   int Hq, Hkv, g, R_tot, KB_tot;  // Hq = heads of the metric (the list heads), g = of them per kv head
   float beta, scale;
+  int heads_per_cta;  // query heads of the group that one CTA takes (blockIdx.z: which)
   int as_keys;  // write bit planes of the metric's selection keys (for launch_select_planes) instead of floats
 };
 
@@ -81,7 +84,8 @@ metric_gemm_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // the Kbar parts stay in shared memory, the Qbar parts of the heads stream through, and two
   // accumulators in tensor memory let the epilogue of one head overlap the MMAs of the next.
   const int seq = a.tiles[3 * blockIdx.x], ti = a.tiles[3 * blockIdx.x + 1], tj = a.tiles[3 * blockIdx.x + 2];
-  const int kvh = blockIdx.y, g = a.g;
+  const int kvh = blockIdx.y, h_first = kvh * a.g + (int)blockIdx.z * a.heads_per_cta;
+  const int g = min(a.heads_per_cta, (kvh + 1) * a.g - h_first);  // heads of this CTA
   const int nb = a.rows.seq_nblk[seq];   // key blocks of the sequence
   const int r0 = a.rows.seq_r0[seq];     // first row of its query chunk
   const int R0 = a.rows.seq_row_off[seq] + ti * kTile;  // first query row of A (Qbar numbering)
@@ -125,7 +129,7 @@ metric_gemm_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
         for (int s = 0; s < 3; ++s)
           tma_load_3d(smem_base + kSmemA + (half * 3 + s) * kPartBytes, &map_q, a_full + 8 * half, 64 * half, R0,
-                      s * a.Hq + kvh * g + hh);
+                      s * a.Hq + h_first + hh);
       }
       __syncwarp();
     };
@@ -187,7 +191,7 @@ metric_gemm_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     bool ok = true;
 #pragma unroll 1
     for (int hh = 0; hh < g && ok; ++hh) {
-      const int h = kvh * g + hh;
+      const int h = h_first + hh;
       ok = __all_sync(0xffffffffu, mbar_wait(acc_full + 8 * (hh & 1), (hh >> 1) & 1, a.status));
       if (!ok) break;
       tc_fence_after();
@@ -284,7 +288,12 @@ cudaError_t launch_metric_gemm(const Plan& p, const void* qsplit, const void* ks
     attr_set[dev_slot] = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)a.Hkv);
+  // Few tiles leave most SMs idle while a CTA works through the group's heads one after the other: spread the heads then
+  // (32K tokens in two sequences, 32 / 8 heads: 32 CTAs of four heads 25 us, 128 of one 12).
+  const int ctas = p.n_gemm_tiles * a.Hkv;
+  const int split = std::min(a.g, std::max(1, p.sm_count / ctas));
+  a.heads_per_cta = (a.g + split - 1) / split;
+  cfg.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)a.Hkv, (unsigned)((a.g + a.heads_per_cta - 1) / a.heads_per_cta));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;
