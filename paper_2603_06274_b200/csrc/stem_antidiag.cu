@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const An
   const int ntok = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + r];
   const int j0 = (int)blockIdx.x * 32;
   if (ntok == BLK || r < r0 || j0 > r) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");  // as at the end
     return;
   }
   const int R = a.rows.seq_row_off[seq] + (r - r0);
@@ -323,8 +323,9 @@ __global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const An
       a.M[(int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)(r - r0) * nb + j] = val;
     }
   }
-  // This kernel is not complete before the contraction is: what follows on the stream reads both kernels' rows.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // This kernel is not complete before the contraction is: what follows on the stream reads both kernels' rows.  (One CTA
+  // waits for that; if all did, those that find no SM beside the contraction would start only behind it.)
+  if (blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace
