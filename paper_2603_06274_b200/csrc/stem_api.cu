@@ -395,8 +395,9 @@ static int enqueue_score_select(const Plan& p, const void* Q, const void* K, con
                                 int32_t* idx, int32_t* cnt, int first_word, cudaStream_t s) {
   const KSide ks = k_side(p, w, kcache);
   float* M = (float*)(w + p.ws.metric);  // holds the bit planes of the selection keys, not the floats
-  // (the anti-diagonal mode has no use for the pooled query vectors; the pooling kernel clears all status words)
-  int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, false,
+  // (the anti-diagonal mode has no use for the pooled query vectors; the pooling kernel clears the status words as well; with a
+  // cache, K and V are given when it is to be updated with the blocks that the chunk adds)
+  int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, kcache != nullptr,
                                (int32_t*)(w + p.ws.status) + first_word, kStatusWords - first_word, s));
   if (rc != STEM_OK) return rc;
   p.last_launches++;
@@ -520,14 +521,8 @@ static int enqueue_prefill(const Plan& p, const void* Q, const void* K, const vo
   int32_t* idx = sel_idx ? sel_idx : (int32_t*)(w + p.ws.sel_idx);
   int32_t* cnt = sel_cnt ? sel_cnt : (int32_t*)(w + p.ws.sel_cnt);
   p.last_launches = 0;
-  int rc = STEM_OK;
-  if (kcache && update_cache) {
-    const KSide ks = k_side(p, w, kcache);
-    rc = cuda_rc(launch_pool(p, nullptr, K, V, ks.mv, nullptr, ks.ksplit, true, nullptr, 0, s));
-    if (rc != STEM_OK) return rc;
-    p.last_launches++;
-  }
-  rc = enqueue_score_select(p, Q, kcache ? nullptr : K, kcache ? nullptr : V, kcache, w, idx, cnt, 0, s);
+  const bool pool_kv = !kcache || update_cache;
+  int rc = enqueue_score_select(p, Q, pool_kv ? K : nullptr, pool_kv ? V : nullptr, kcache, w, idx, cnt, 0, s);
   if (rc != STEM_OK) return rc;
   rc = cuda_rc(launch_sparse_attention(p, Q, K, V, idx, cnt, p.share_group, O, lse, (int32_t*)(w + p.ws.status), true, s));
   if (rc != STEM_OK) return rc;
