@@ -34,15 +34,47 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Rows of up to 16 384 tokens: W warps hold the row's keys in registers, 1024 a warp, 32 a lane, as bit planes (word k = bit
-// k of the lane's keys), and descend from the most significant bits, two at a time: how many undecided keys have the upper
-// bit, both, or only the lower one is a popcount per lane, a reduction per warp and one exchange between the warps.  No
-// histograms: shared-memory atomics take 14 cycles of the SM per warp instruction and bounded the byte-wise radix selection
-// below (8 lists of 8K tokens, top 2048: 1.24 ms, here 0.78).  The descent stops as soon as all the
-// undecided keys are taken.  Lane l of warp w owns the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are
+// Rows of up to 16 384 tokens: W warps hold the upper halves of the row's keys in registers, 1024 keys a warp, 32 a lane, as
+// 16 bit planes (word k = bit 16 + k of the lane's keys), and descend from the most significant bits, two at a time: how
+// many undecided keys have the upper bit, both, or only the lower one is a popcount per lane, a reduction per warp and one
+// exchange between the warps.  The descent ends when all undecided keys are taken, or when so few are left that ranking
+// them against each other is cheaper (kFinish); only rows with many keys in one bin of the upper halves go on with the
+// lower ones, read again.  No histograms: shared-memory atomics take 14 cycles of the SM per warp instruction and bounded the
+// byte-wise radix selection below.  The kernel is bound by its instructions.  In us, byte-wise / all 32 planes / this: 8
+// lists of 8K tokens, top 2048: 1240 / 780 / 588 (floor by its bytes 240); scores that are zero in half of the places
+// instead of normal: this 667.  Lane l of warp w owns the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are
 // coalesced 16-byte ones and the ascending list comes out q by q with a prefix sum over the lanes' nibbles.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPlanesMax = 16384;  // longest row
+constexpr int kFinish = 32;        // undecided keys that are ranked against each other (64: 597 us, 128: 654, 16: 587)
+
+// The planes of 16 bits of 32 keys: in, word k = the 16 bits of key k and, above them, of key k + 16; out, word k = bit k of
+// the 32 keys (the second to fifth stage of ptx::transpose32 on one half).
+__device__ __forceinline__ void transpose16(uint32_t (&w)[16]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {  // bytes
+    const uint32_t lo = __byte_perm(w[k], w[k + 8], 0x6240), hi = __byte_perm(w[k], w[k + 8], 0x7351);
+    w[k] = lo;
+    w[k + 8] = hi;
+  }
+#pragma unroll
+  for (int s = 2; s < 5; ++s) {
+    const int j = 16 >> s;
+    const uint32_t mhi = s == 2 ? 0xf0f0f0f0u : s == 3 ? 0xccccccccu : 0xaaaaaaaau;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      if (k & j) continue;
+      const uint32_t x = w[k], y = w[k + j];
+      w[k] = (x & ~mhi) | ((y << j) & mhi);
+      w[k + j] = ((x >> j) & ~mhi) | (y & mhi);
+    }
+  }
+}
+
+template <int W>
+__device__ __forceinline__ void row_sync() {  // among the warps of a row
+  if (W == 1) __syncwarp(); else __syncthreads();
+}
 
 template <int W>
 __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W, W == 1 ? 8 : 1024 / (32 * W))
@@ -50,6 +82,8 @@ token_select_planes_kernel(const float* __restrict__ scores, int N, int t_end, i
                            int local, int vec, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_cnt) {
   constexpr int kRows = W == 1 ? 4 : 1;  // rows per CTA
   __shared__ int xch[2][W][2];
+  __shared__ int fin_n[kRows];
+  __shared__ unsigned long long fin[kRows][kFinish];  // column, then key and column as one number, then whether it is taken
   // the kernel of the next shorter rows may start beside this one's last CTAs (it is complete only after this one)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = W == 1 ? 0 : (int)(threadIdx.x >> 5);
@@ -59,6 +93,8 @@ token_select_planes_kernel(const float* __restrict__ scores, int N, int t_end, i
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
+  const int sub = W == 1 ? (int)(threadIdx.x >> 5) : 0, tid = W == 1 ? lane : (int)threadIdx.x;
+  if (tid == 0) fin_n[sub] = 0;
   const int i = t + 1;
   const int n_stem = min(stem, i);
   const int c_lo = n_stem, c_hi = max(max(i - local, 0), n_stem);  // candidates [c_lo, c_hi)
@@ -85,59 +121,139 @@ token_select_planes_kernel(const float* __restrict__ scores, int N, int t_end, i
     if (!ranked) {
       sel = act;
     } else {
-      uint32_t w[32];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int col = col0 + 128 * q;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (vec) {
-          if (col < c_hi) v = __ldcs((const float4*)(row + col));
-        } else {
-          if (col < c_hi) v.x = __ldcs(row + col);
-          if (col + 1 < c_hi) v.y = __ldcs(row + col + 1);
-          if (col + 2 < c_hi) v.z = __ldcs(row + col + 2);
-          if (col + 3 < c_hi) v.w = __ldcs(row + col + 3);
-        }
-        // -0 -> +0, NaN -> -inf; the monotone map to unsigned is completed on the planes
-        w[4 * q] = __float_as_uint(fmaxf(v.x + 0.0f, __int_as_float(0xff800000)));
-        w[4 * q + 1] = __float_as_uint(fmaxf(v.y + 0.0f, __int_as_float(0xff800000)));
-        w[4 * q + 2] = __float_as_uint(fmaxf(v.z + 0.0f, __int_as_float(0xff800000)));
-        w[4 * q + 3] = __float_as_uint(fmaxf(v.w + 0.0f, __int_as_float(0xff800000)));
-      }
-      ptx::transpose32(w);
-      const uint32_t neg = w[31];
-#pragma unroll
-      for (int k = 0; k < 31; ++k) w[k] ^= neg;
-      w[31] = ~neg;
-
       uint32_t gt = 0u;      // known to be above the need-th largest key
+      uint32_t neg = 0u;     // the lane's negative keys
       int k = need;          // rank wanted among the undecided keys
       int n_act = n_cand;    // their number
+      bool fix = false;      // -0 -> +0 and NaN -> -inf are wanted
+      row_sync<W>();         // (fin_n)
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {  // upper, lower 16 bits
+        uint32_t w[16];
+#pragma unroll 1
+        for (;;) {
+          uint32_t v[32];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const uint32_t up = w[31 - 2 * r], low = w[30 - 2 * r];
-        const uint32_t h11 = act & up & low, h10 = act & up & ~low, h01 = act & ~up & low, h00 = act & ~(up | low);
-        int a = __popc(h11) | (__popc(h10) << 16), b = __popc(h01);
-        a = __reduce_add_sync(0xffffffffu, a);
-        b = __reduce_add_sync(0xffffffffu, b);
-        if (W > 1) {
-          if (lane == 0) { xch[r & 1][warp][0] = a; xch[r & 1][warp][1] = b; }
-          __syncthreads();
-          a = lane < W ? xch[r & 1][lane < W ? lane : 0][0] : 0;
-          b = lane < W ? xch[r & 1][lane < W ? lane : 0][1] : 0;
+          for (int q = 0; q < 8; ++q) {
+            const int col = col0 + 128 * q;
+            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vec) {
+              if (col < c_hi) f = *(const float4*)(row + col);
+            } else {
+              if (col < c_hi) f.x = row[col];
+              if (col + 1 < c_hi) f.y = row[col + 1];
+              if (col + 2 < c_hi) f.z = row[col + 2];
+              if (col + 3 < c_hi) f.w = row[col + 3];
+            }
+            v[4 * q] = __float_as_uint(f.x);
+            v[4 * q + 1] = __float_as_uint(f.y);
+            v[4 * q + 2] = __float_as_uint(f.z);
+            v[4 * q + 3] = __float_as_uint(f.w);
+          }
+          if (fix) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) v[c] = __float_as_uint(fmaxf(__uint_as_float(v[c]) + 0.0f, __int_as_float(0xff800000)));
+          }
+          const uint32_t pick = half ? 0x5410u : 0x7632u;
+#pragma unroll
+          for (int c = 0; c < 16; ++c) w[c] = __byte_perm(v[c], v[c + 16], pick);
+          transpose16(w);
+          if (fix) break;
+          // upper halves only: a negative key whose other 15 bits are zero may be -0, one whose exponent is all ones NaN
+          uint32_t some = w[14], ones = w[14];
+#pragma unroll
+          for (int c = 0; c < 14; ++c) {
+            some |= w[c];
+            if (c >= 7) ones &= w[c];
+          }
+          fix = true;
+          if (!__any_sync(0xffffffffu, (act & (ones | (w[15] & ~some))) != 0u)) break;
+        }
+        // the monotone map to unsigned, on the planes
+        if (half == 0) {
+          neg = w[15];
+          w[15] = ~0u;
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c) w[c] ^= neg;
+
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const uint32_t up = w[15 - 2 * r], low = w[14 - 2 * r];
+          const uint32_t h11 = act & up & low, h10 = act & up & ~low, h01 = act & ~up & low, h00 = act & ~(up | low);
+          int a = __popc(h11) | (__popc(h10) << 16), b = __popc(h01);
           a = __reduce_add_sync(0xffffffffu, a);
           b = __reduce_add_sync(0xffffffffu, b);
+          if (W > 1) {
+            if (lane == 0) { xch[r & 1][warp][0] = a; xch[r & 1][warp][1] = b; }
+            __syncthreads();
+            a = lane < W ? xch[r & 1][lane < W ? lane : 0][0] : 0;
+            b = lane < W ? xch[r & 1][lane < W ? lane : 0][1] : 0;
+            a = __reduce_add_sync(0xffffffffu, a);
+            b = __reduce_add_sync(0xffffffffu, b);
+          }
+          const int n11 = a & 0xffff, n10 = (int)((uint32_t)a >> 16), n01 = b;
+          // the pair of bits of the k-th largest key, straight-line
+          const bool in11 = n11 >= k, in10 = !in11 && n11 + n10 >= k, in01 = !in11 && !in10 && n11 + n10 + n01 >= k;
+          gt |= in11 ? 0u : in10 ? h11 : in01 ? (h11 | h10) : (h11 | h10 | h01);
+          k -= in11 ? 0 : in10 ? n11 : in01 ? n11 + n10 : n11 + n10 + n01;
+          act = in11 ? h11 : in10 ? h10 : in01 ? h01 : h00;
+          n_act = in11 ? n11 : in10 ? n10 : in01 ? n01 : n_act - n11 - n10 - n01;
+          if (n_act == k || n_act <= kFinish) break;
         }
-        const int n11 = a & 0xffff, n10 = (int)((uint32_t)a >> 16), n01 = b;
-        // the pair of bits of the k-th largest key, straight-line
-        const bool in11 = n11 >= k, in10 = !in11 && n11 + n10 >= k, in01 = !in11 && !in10 && n11 + n10 + n01 >= k;
-        gt |= in11 ? 0u : in10 ? h11 : in01 ? (h11 | h10) : (h11 | h10 | h01);
-        k -= in11 ? 0 : in10 ? n11 : in01 ? n11 + n10 : n11 + n10 + n01;
-        act = in11 ? h11 : in10 ? h10 : in01 ? h01 : h00;
-        n_act = in11 ? n11 : in10 ? n10 : in01 ? n01 : n_act - n11 - n10 - n01;
-        if (n_act == k) break;  // all of them are taken
+        if (n_act == k || n_act <= kFinish) break;
       }
-      if (n_act == k) {
+      if (n_act != k && n_act <= kFinish) {
+        // few are left: each is ranked against the others by (key descending, column ascending)
+        int at = 0;
+        if (act != 0u) {
+          at = atomicAdd(&fin_n[sub], __popc(act));
+          uint32_t m = act;
+          for (int p = at; m != 0u; ++p, m &= m - 1u) {
+            const int b = __ffs((int)m) - 1;
+            fin[sub][p] = (unsigned long long)(col0 + 128 * (b >> 2) + (b & 3));
+          }
+        }
+        row_sync<W>();
+        constexpr int kEach = kFinish > 32 * W ? kFinish / (32 * W) : 1;  // entries per thread
+        constexpr int kShare = kFinish < 32 * W ? 32 * W / kFinish : 1;   // threads per entry
+        const int e0 = tid / kShare, part = tid % kShare;
+        unsigned long long mine[kEach];
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+          const int e = e0 + 32 * W * u;
+          mine[u] = 0ull;
+          if (e < n_act) {
+            const uint32_t col = (uint32_t)fin[sub][e];
+            mine[u] = ((unsigned long long)score_key(row[col]) << 32) | (0xffffffffu - col);
+          }
+        }
+        row_sync<W>();
+#pragma unroll
+        for (int u = 0; u < kEach; ++u)
+          if (part == 0 && e0 + 32 * W * u < n_act) fin[sub][e0 + 32 * W * u] = mine[u];
+        row_sync<W>();
+        int rank[kEach];
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) rank[u] = 0;
+#pragma unroll 4
+        for (int o = part; o < n_act; o += kShare) {
+          const unsigned long long other = fin[sub][o];
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) rank[u] += other > mine[u] ? 1 : 0;
+        }
+#pragma unroll
+        for (int d = 1; d < kShare; d <<= 1) rank[0] += __shfl_xor_sync(0xffffffffu, rank[0], d);
+        row_sync<W>();
+#pragma unroll
+        for (int u = 0; u < kEach; ++u)
+          if (part == 0 && e0 + 32 * W * u < n_act) fin[sub][e0 + 32 * W * u] = rank[u] < k ? 1ull : 0ull;
+        row_sync<W>();
+        sel = gt;
+        uint32_t m = act;
+        for (int p = at; m != 0u; ++p, m &= m - 1u)
+          if (fin[sub][p] != 0ull) sel |= m & (0u - m);
+      } else if (n_act == k) {
         sel = gt | act;
       } else {
         // equal keys, of which the first k by column are taken: warp by warp, q by q, lane by lane
@@ -215,7 +331,6 @@ token_select_planes_kernel(const float* __restrict__ scores, int N, int t_end, i
     if (nib & 8u) *at = col + 3;
     base += (int)((tot >> sh) & 255u);
   }
-  const int tid = W == 1 ? lane : (int)threadIdx.x;
   constexpr int kStep = 32 * W;
   for (int j = tid; j < n_stem; j += kStep) out[j] = j;
   const int written = n_stem + need;

@@ -265,12 +265,18 @@ def test_token_attention_ignores_rows_no_list_names():
     (4097, 1, 2048, 0, 1, False),    # the first row of eight warps
     (8200, 1, 500, 4, 8, True),      # rows of sixteen warps
     (16388, 1, 700, 0, 1, True),     # longer than the registers hold: the other kernel for all rows
+    (1030, 2, 200, 0, 1, "low"),     # scores alike in their upper 16 bits, or in all but the last four
+    (4100, 1, 900, 2, 3, "low"),
+    (300, 2, 33, 0, 1, "low"),
 ])
 def test_token_selection_row_lengths(n, heads, k_start, stem, local, ties):
     g = torch.Generator(device="cuda")
     g.manual_seed(n)
     sc = torch.randn((heads, n, n), generator=g, device="cuda")
-    if ties:
+    if ties == "low":
+        last = torch.randint(0, 40000 if n % 4 else 16, (heads, n, n), generator=g, device="cuda", dtype=torch.int32)
+        sc = (torch.where(sc < 0.0, -1.5, 1.5).view(torch.int32) + last).view(torch.float32)
+    elif ties:
         sc = torch.round(sc * 2.0) / 2.0 * torch.where(torch.rand((heads, n, n), generator=g, device="cuda") < 0.5, 1.0, -1.0)
         sc[0, n - 1, 3:9] = float("nan")
         sc[0, n // 2, ::5] = float("inf")
