@@ -26,6 +26,13 @@
 // seven 32 KB tiles of shared memory are three Q tiles and a ring of four, the next tile is loaded into
 // the spare one while both current items run, and slot 1 starts half an item late so that the slots'
 // boundaries alternate; otherwise (dense mode, very long lists) two Q tiles and a ring of five.
+// Where two query heads of a group have the same list in every row (one list per kv head, or every causal block) the slots
+// work on such a pair in step (kPair): one stream of K / V tiles serves both, so a visit's tiles are filled once for two
+// visits (a visit's traffic on the 128 bytes a cycle of shared memory: operands 768 cycles, tiles 512, shared 256, beside
+// 1024 cycles of MMAs), half as much comes from the L2, which also saves power, and a ring of five reaches twice as far;
+// the next Q tiles have a whole round to land, so no spare is needed.  Two streams / one, TFLOP/s: dense 16K tokens, 32 / 8
+// heads 1237 / 1296; 128K, 64 / 8, lists of 42 blocks on average 1109 / 1189; 32K, 32 / 8, 22 blocks 1120 / 1211.  With the
+// spare Q tile and a ring of four: 1280, 1187, 1196.
 // Registers are re-balanced with setmaxnreg: the kernel must not spill, because with 227 KB of
 // shared memory in use almost no L1 is left for local memory.
 // Every mbarrier wait is bounded in time; a wait that gives up raises a CTA-wide abort flag,
@@ -355,6 +362,14 @@ __device__ __forceinline__ void tok_item(const AttnArgs& a, int i, int& kvh, int
   n = (min(a.tok_a + (tile + 1) * a.tok_tile, a.tok_b) - 1) / kTileM + 1;
 }
 
+// The first item of a slot; its items are 2 gridDim.x apart.  kPair: the slots have neighbours in the work order, two query
+// heads of a group in the same row; else slot 1 is gridDim.x items behind, or (split) has the other half of slot 0's item.
+template <bool kSplit, bool kPair>
+__device__ __forceinline__ int first_item_of(const AttnArgs& a, int slot) {
+  if (kPair) return 2 * (int)blockIdx.x + slot;
+  return (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x);
+}
+
 // A slot's part of a list of n entries that the two slots share.
 __device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
   const int first = (n + 1) >> 1;
@@ -367,14 +382,14 @@ __device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
 // their output rows).  Used by whole warps in lock step (values are broadcast from lane 0).
 // kSplit: with a.split both slots take the same item, slot 0 the first half of its list (rounded up), slot 1 the rest; `off` is
 // the first entry of the slot's part.
-template <bool kTok, bool kSplit>
+template <bool kTok, bool kSplit, bool kPair>
 struct ItemCursor {
   int idx, step, slot, off;
   int h, R, r, n;
   __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
     slot = slot_;
     off = 0;
-    idx = (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x) - 2 * (int)gridDim.x;
+    idx = first_item_of<kSplit, kPair>(a, slot) - 2 * (int)gridDim.x;
     step = 2 * (int)gridDim.x;
     n = 0;
   }
@@ -403,7 +418,7 @@ struct ItemCursor {
 
 // The list lengths of one slot's items, in the ItemCursor's order, for the MMA issuer: the loads that lead to the length
 // of the next item are started an item ahead (the work entry two items ahead), so that next() waits for none of them.
-template <bool kTok, bool kSplit>
+template <bool kTok, bool kSplit, bool kPair>
 struct LengthCursor {
   int idx, step, slot; // the item whose length `raw` is
   int raw, h2, R2;     // length of item idx as loaded; work entry of item idx + step
@@ -419,7 +434,7 @@ struct LengthCursor {
   __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
     slot = slot_;
     step = 2 * (int)gridDim.x;
-    idx = (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x);
+    idx = first_item_of<kSplit, kPair>(a, slot);
     if constexpr (kTok) return;
     entry(a, idx);
     raw = length(a, h2, R2);
@@ -494,7 +509,7 @@ __device__ __noinline__ void exact_token_row(float scale_log2, const __nv_bfloat
   if (lse) *lse = (m + log2f(l)) * 0.6931471805599453f;
 }
 
-template <int BLK, bool kSpareQ, bool kTok>
+template <int BLK, bool kSpareQ, bool kTok, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const AttnArgs a, const TokRows tok) {
@@ -511,7 +526,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // four K / V slots, for lists of tens of blocks, where an item boundary that waits for Q costs two blocks' time;
   // otherwise two Q tiles and a ring of five, for long lists (and the dense mode), where the deeper ring pays.
   static_assert(!kTok || (BLK == 128 && !kSpareQ), "the token-list form has two Q tiles and key blocks of 128");
-  constexpr bool kSplit = !kSpareQ && !kTok;  // the layout that may cut lists in halves (a.split)
+  static_assert(!kPair || !kSpareQ, "pairs have two Q tiles");
+  constexpr bool kSplit = !kSpareQ && !kTok && !kPair;  // the layout that may cut lists in halves (a.split)
   constexpr int kKvSlots = kSpareQ ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
@@ -543,7 +559,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   }
   if (!kTok && threadIdx.x < 2) {
     // the plan's tables do not depend on the kernels before this one: fetch what the first items need of them
-    const int item = (int)blockIdx.x + (kSplit && a.split ? 0 : (int)threadIdx.x * (int)gridDim.x);
+    const int item = first_item_of<kSplit, kPair>(a, (int)threadIdx.x);
     if (item < a.n_items) {
       const int R = a.work[2 * item + 1];
       const int seq = a.rows.row_seq[R];
@@ -602,7 +618,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
       return (uint32_t)n | (diag ? 0x80000000u : 0u) | halves;
     };
-    const int first_item = (int)blockIdx.x + (kSplit && a.split ? 0 : X * (int)gridDim.x);
+    const int first_item = first_item_of<kSplit, kPair>(a, X);
     uint32_t next_info = list_info(first_item);
     for (int item = first_item; item < a.n_items && ok; item += 2 * (int)gridDim.x) {
       const uint32_t info = next_info;
@@ -846,7 +862,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // ============================== K / V producer ==============================
       Ctx ctx{abort_flag, status, kRoleProducer, kTok ? 4 : 1};
       struct KvSlot {
-        ItemCursor<kTok, kSplit> cur;
+        ItemCursor<kTok, kSplit, kPair> cur;
         bool has, pend;
         int e, j_next, pend_tok, pend_kvh, seq_tok0;
         const int32_t* list;
@@ -895,14 +911,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       KvSlot s0, s1;
       s0.cur.init(a, 0); s1.cur.init(a, 1);
       s0.pend = s1.pend = false;
-      enter(s0); enter(s1);
+      enter(s0);
+      if (kPair) s1.has = false; else enter(s1);  // (pairs: one stream of K / V for both slots)
       bool ok = true;
       // With the spare Q tile slot 1 starts half an item behind slot 0, so that the two slots' item boundaries (and
       // their claims on the spare) do not fall together.  The MMA issuer skips the same visits.
       const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;
       for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
         ok = visit(s0);
-        if (ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
+        if (!kPair && ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
       }
       if (!ok && lane == 0) {
         // aborting: give copies already in flight a bounded time to land before the CTA exits
@@ -920,12 +937,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
         // next tile, loaded into the spare buffer long before it is wanted; the buffer the slot leaves becomes the
         // spare once the last Q K^T of its item has read it.  The MMA issuer rotates the buffers by the same rule.
-        ItemCursor<kTok, kSplit> c0, c1;
+        ItemCursor<kTok, kSplit, kPair> c0, c1;
         c0.init(a, 0); c1.init(a, 1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t q_used = 0u, q_odd = 0u;  // per buffer (bit b): a tile was loaded; an odd number of tiles was loaded
         bool ok = true;
-        auto load_into = [&](const ItemCursor<kTok, kSplit>& cur, const int b) -> bool {
+        auto load_into = [&](const ItemCursor<kTok, kSplit, kPair>& cur, const int b) -> bool {
           if (((q_used >> b) & 1u) &&
               !__all_sync(0xffffffffu, mbar_wait(bar(Smem::q_empty, b), ((q_odd >> b) & 1u) ^ 1u, ctx, kBarQEmpty)))
             return false;
@@ -966,12 +983,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             while (((q_used >> b) & 1u) && !mbar_try(bar(Smem::q_full, b), ((q_odd >> b) & 1u) ^ 1u) && globaltimer() - t1 < 4000000ull) {}
         }
       } else {
-        ItemCursor<kTok, kSplit> c0, c1;
+        ItemCursor<kTok, kSplit, kPair> c0, c1;
         c0.init(a, 0); c1.init(a, 1);
         bool has0 = c0.next(a), has1 = c1.next(a);
         uint32_t ord0 = 0, ord1 = 0;
         // Loads the slot's next Q tile as soon as the last Q K^T of its previous item has read the buffer.
-        auto try_load = [&](ItemCursor<kTok, kSplit>& cur, bool& has, uint32_t& ord, const int X) -> bool {
+        auto try_load = [&](ItemCursor<kTok, kSplit, kPair>& cur, bool& has, uint32_t& ord, const int X) -> bool {
           if (!has || !uni((int)mbar_test(bar(Smem::q_empty, X), (ord & 1) ^ 1))) return false;
           const int q_tok0 = kTok ? a.tok_a + cur.R * a.tok_tile : uni(a.rows.row_tok0[cur.R]);
           const int q_head = kTok ? cur.h * a.g : cur.h;
@@ -1020,7 +1037,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {
-        LengthCursor<kTok, kSplit> cur;
+        LengthCursor<kTok, kSplit, kPair> cur;
         int left;                      // blocks of the current item whose Q K^T is still to come (0: no item left)
         uint32_t st;                   // kPend: a P V is due, of its item's first (kFirst) / last (kLast) block;
                                        // kNewItem: the next Q K^T is the first of its item
@@ -1037,9 +1054,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const uint32_t s_tmem = tmem_base + X * 128;
         const uint32_t o_tmem = tmem_base + kOCol + X * 128;
         const uint32_t st = s.st;
+        const uint32_t ring0 = ring, ring_par0 = ring_par;
+        const bool shared = kPair && X == 0;  // slot 1's visit uses the same tiles and gives them back
         if (st & kPend) {
           const uint32_t v_addr = smem_base + kKvOff + ring * kSlotBytes;
-          mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
+          if (!kPair || X == 0) mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
           if (st & kFirst) mbar_wait_sticky(bar(Smem::o_free, X), s.o_par ^ 1, abort_addr, kBarOFree, failed);
           // P V starts on the leading key columns while the softmax still works on the last 32
           mbar_wait_sticky(bar(Smem::p_early, X), s.p_par, abort_addr, kBarPEarly, failed);
@@ -1057,7 +1076,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
 #pragma unroll
             for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
-            tc_commit(bar(Smem::kv_empty, ring));
+            if (!shared) tc_commit(bar(Smem::kv_empty, ring));
             if (st & kLast) tc_commit(bar(Smem::o_full, X));
           }
           __syncwarp();
@@ -1067,7 +1086,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           s.st = st & kNewItem;
         }
         if (s.left > 0) {
-          mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
+          if (!kPair || X == 0) mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
           if (st & kNewItem) mbar_wait_sticky(bar(Smem::q_full, s.qbuf), s.q_par, abort_addr, kBarQFull, failed);
           tc_fence_after();
           const bool last = --s.left == 0;
@@ -1078,7 +1097,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             for (int k = 0; k < kHeadDim / 16; ++k)  // 16 columns = 32 bytes on; the second four steps: the other 64-column half
               mma_ss(s_tmem, da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4), db + (((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4),
                      kIdescS, k > 0 ? 1u : 0u);
-            tc_commit(bar(Smem::kv_empty, ring));
+            if (!shared) tc_commit(bar(Smem::kv_empty, ring));
             tc_commit(bar(Smem::s_full, X));
             if (last) tc_commit(bar(Smem::q_empty, s.qbuf));
           }
@@ -1100,6 +1119,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
           }
         }
+        if (shared) { ring = ring0; ring_par = ring_par0; }
       };
       MmaSlot s0, s1;
       s0.cur.init(a, 0); s1.cur.init(a, 1);
@@ -1176,19 +1196,23 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   static bool attr_set[64] = {};
   const int dev_slot = p.device & 63;
   if (!attr_set[dev_slot]) {
-    e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[dev_slot] = true;
   }
-  const int grid = std::min(p.n_items, p.sm_count);
   // Lists of up to a few hundred blocks: the spare Q tile (an item boundary then costs no wait for Q); the dense mode
   // and longer lists: the deeper K / V ring.
   // Grids of no more items than SMs leave the second slot of every CTA idle and are as long as one list: the two slots take
   // half a list each (4K tokens, 2 heads, blocks of 64, lists of up to 16: the call goes from 28.7 to 26 us).
   a.split = p.n_items <= p.sm_count ? 1 : 0;
+  // Pairs wherever neighbours in the work order have the same list; the work order holds the heads of a group together.
+  const bool pair = a.g % 2 == 0 && (sel_idx == nullptr || list_group) && !a.split;
+  const int grid = std::min(pair ? p.n_items / 2 : p.n_items, p.sm_count);
   const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList && !a.split;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1202,8 +1226,9 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
   // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
   cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
-  auto kernel = B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false> : sparse_attn_kernel<128, false, false>)
-                         : (spare_q ? sparse_attn_kernel<64, true, false> : sparse_attn_kernel<64, false, false>);
+  auto kernel = pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
+              : B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false, false> : sparse_attn_kernel<128, false, false, false>)
+                         : (spare_q ? sparse_attn_kernel<64, true, false, false> : sparse_attn_kernel<64, false, false, false>);
   return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, a, TokRows{});
 }
 
@@ -1265,7 +1290,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
   const TokRows tok{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, q_st, q_sh, kv_st, kv_sh};
   static bool attr_set[64] = {};
   if (!attr_set[device & 63]) {
-    const cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    const cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[device & 63] = true;
   }
@@ -1281,7 +1306,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
     a.n_items = ((b - a.tok_a + tile - 1) / tile) * Hkv;
     cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, tile, O, a.mask_st, a.mask_sh, s);
     if (e != cudaSuccess) return e;
-    sparse_attn_kernel<128, false, true><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
+    sparse_attn_kernel<128, false, true, false><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -302,3 +302,50 @@ def test_lists_cut_in_halves_for_the_two_slots(rows):
     live = np.isfinite(lse_ref)
     assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
     plan.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv,dense", [
+    (128, (37 * 128 - 5,), 4, 2, False),        # 148 items: one per SM, lists cut in halves
+    (128, (38 * 128 - 5,), 4, 2, False),        # 152 items: two query heads of a group at a time on one stream of K / V
+    (64, (3000, 65, 1, 1900), 6, 1, False),
+    (64, (2500, 700), 16, 4, False),
+    (128, (2900, 129), 14, 2, False),           # an odd number of heads in a group: no pairs
+    (128, (38 * 128 - 5,), 4, 2, True),
+    (64, (3000, 65, 1, 1900), 6, 1, True),
+    (128, (2900, 129), 14, 2, True),
+])
+def test_heads_of_a_group_with_the_same_lists(block, seqlens, hq, hkv, dense):
+    # one list per kv head (lists of 0, 1, 2, 3 and up to all causal blocks, with and without the diagonal block), or dense
+    w = wl.small("pairs", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=1000, mu_num=1, mu_den=1, seed=sum(seqlens))
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w, share_group=True)
+    info = plan.info
+    n_blk = [(n + block - 1) // block for n in seqlens]
+    row_r = np.concatenate([np.arange(n) for n in n_blk])
+    r = np.random.default_rng(hq + sum(seqlens))
+    idx = np.full((hkv, info.total_q_blocks, info.k_max), -1, np.int32)
+    cnt = np.zeros((hkv, info.total_q_blocks), np.int32)
+    for h in range(hkv):
+        for R, row in enumerate(row_r):
+            n = row + 1 if dense else min(int(r.choice([0, 1, 2, 3, 8, row + 1])), row + 1)
+            idx[h, R, :n] = np.sort(r.choice(row + 1, size=n, replace=False))
+            cnt[h, R] = n
+    n_tok = w.total_tokens
+    outs = []
+    for _ in range(2):
+        out = torch.full((n_tok, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((hq, n_tok), float("nan"), dtype=torch.float32, device="cuda")
+        lists = (None, None) if dense else (torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda())
+        binding.stem_sparse_prefill(plan, q, k, v, *lists, out, lse)
+        assert binding.stem_check_status(plan)[0] == 0
+        outs.append((out, lse))
+    assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16)) and torch.equal(outs[0][1], outs[1][1])
+    ei, ec = so.expand_group_lists(idx, cnt, hq // hkv)
+    O_ref, lse_ref = so.attention(data["q"], data["k"], data["v"], data["cu_seqlens"], block, ei, ec)
+    check_attention(from_dev_bf16(outs[0][0]), O_ref, ~np.isnan(O_ref), label=f"{len(row_r) * hq} items")
+    got = outs[0][1].cpu().numpy()
+    assert np.isneginf(got[np.isneginf(lse_ref)]).all()
+    live = np.isfinite(lse_ref)
+    assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
+    plan.close()
