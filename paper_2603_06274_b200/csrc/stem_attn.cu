@@ -329,7 +329,8 @@ __host__ __device__ constexpr uint32_t make_idesc(int n, int b_mn_major) {
 }
 
 struct AttnArgs {
-  const int32_t* work;      // [n_items][2] (head, global row)
+  const int32_t* work;      // [n_items][2] (head, global row), by slot
+  const int32_t* slot_off;  // slot X of CTA c has the items slot_off[2 c + X] .. slot_off[2 c + X + 1] - 1
   const int32_t* sel_idx;   // null -> every causal block
   const int32_t* sel_cnt;
   __nv_bfloat16* O;
@@ -354,21 +355,50 @@ struct TokRows {
   int64_t q_st, q_sh, kv_st, kv_sh;
 };
 
-// kTok: item i is (kv head, tile of query tokens), the longest prefixes first; n = key blocks up to its last token.
+// kTok: item i is (kv head, tile of query tokens), the longest prefixes first; n = key blocks up to its last token.  kPair:
+// items 2 p and 2 p + 1 are neighbouring tiles with the key blocks of the later one, which may lie behind the last token.
+template <bool kPair>
 __device__ __forceinline__ void tok_item(const AttnArgs& a, int i, int& kvh, int& tile, int& n) {
-  const int q = i / a.n_kvh;
-  kvh = i - q * a.n_kvh;
-  tile = (a.tok_b - a.tok_a - 1) / a.tok_tile - q;
-  n = (min(a.tok_a + (tile + 1) * a.tok_tile, a.tok_b) - 1) / kTileM + 1;
+  const int p = kPair ? i >> 1 : i;
+  const int q = p / a.n_kvh;
+  kvh = p - q * a.n_kvh;
+  const int last = (a.tok_b - a.tok_a - 1) / a.tok_tile;
+  tile = kPair ? 2 * ((last >> 1) - q) + (i & 1) : last - q;
+  const int end = kPair ? tile | 1 : tile;
+  n = (min(a.tok_a + (end + 1) * a.tok_tile, a.tok_b) - 1) / kTileM + 1;
 }
 
-// The first item of a slot; its items are 2 gridDim.x apart.  kPair: the slots have neighbours in the work order, two query
-// heads of a group in the same row; else slot 1 is gridDim.x items behind, or (split) has the other half of slot 0's item.
-template <bool kSplit, bool kPair>
-__device__ __forceinline__ int first_item_of(const AttnArgs& a, int slot) {
-  if (kPair) return 2 * (int)blockIdx.x + slot;
-  return (int)blockIdx.x + (kSplit && a.split ? 0 : slot * (int)gridDim.x);
-}
+// The items of one slot of a CTA.  Plans assign them ahead of time (`slot_off`); where the items are computed (kTok) they are
+// dealt out longest first, in alternating directions so that every slot's sum of lengths is about the same (in one direction:
+// 8192 tokens, 32 / 8 heads 620 us, here 580; 12000, 8 / 2: 451, here 363; kPair: two neighbouring items at a time).  kSplit:
+// with a.split both slots of a CTA have its one item.
+template <bool kTok, bool kSplit, bool kPair>
+struct SlotWalk {
+  int idx, limit, step;
+  __device__ __forceinline__ void init(const AttnArgs& a, int slot) {
+    const int cta = (int)blockIdx.x, ctas = (int)gridDim.x;
+    if constexpr (kTok) {
+      idx = kPair ? 2 * cta + slot : cta + slot * ctas;
+      limit = a.n_items;
+      step = kPair ? 4 * (ctas - cta) - 2 : 2 * (2 * ctas - idx) - 1;
+    } else if (kSplit && a.split) {
+      idx = cta;
+      limit = cta + 1;
+    } else {
+      idx = a.slot_off[2 * cta + slot];
+      limit = a.slot_off[2 * cta + slot + 1];
+    }
+  }
+  __device__ __forceinline__ bool done() const { return idx >= limit; }
+  __device__ __forceinline__ void advance() {
+    if constexpr (kTok) {
+      idx += step;
+      step = 4 * (int)gridDim.x - step;
+    } else {
+      ++idx;
+    }
+  }
+};
 
 // A slot's part of a list of n entries that the two slots share.
 __device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
@@ -377,33 +407,31 @@ __device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
   n = slot ? n - first : first;
 }
 
-// Walks the items of one slot of this CTA: item i of the work order belongs to CTA i % gridDim.x,
-// slot (i / gridDim.x) % 2.  Items with an empty list are skipped (the slot's softmax warps zero
+// Walks the items of one slot of this CTA.  Items with an empty list are skipped (the slot's softmax warps zero
 // their output rows).  Used by whole warps in lock step (values are broadcast from lane 0).
 // kSplit: with a.split both slots take the same item, slot 0 the first half of its list (rounded up), slot 1 the rest; `off` is
 // the first entry of the slot's part.
 template <bool kTok, bool kSplit, bool kPair>
 struct ItemCursor {
-  int idx, step, slot, off;
+  SlotWalk<kTok, kSplit, kPair> walk;
+  int slot, off;
   int h, R, r, n;
   __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
     slot = slot_;
     off = 0;
-    idx = first_item_of<kSplit, kPair>(a, slot) - 2 * (int)gridDim.x;
-    step = 2 * (int)gridDim.x;
+    walk.init(a, slot);
     n = 0;
   }
   // Moves to the next item with a non-empty list; false when the slot has no more items.
   __device__ __forceinline__ bool next(const AttnArgs& a) {
-    if constexpr (kTok) {
-      idx += step;
-      n = 0;
-      if (idx >= a.n_items) return false;
-      tok_item(a, idx, h, R, n);
-      r = n - 1;
-      return true;
-    }
-    for (idx += step; idx < a.n_items; idx += step) {
+    for (; !walk.done();) {
+      const int idx = walk.idx;
+      walk.advance();
+      if constexpr (kTok) {
+        tok_item<kPair>(a, idx, h, R, n);
+        r = n - 1;
+        return true;
+      }
       h = uni(a.work[2 * idx]);
       R = uni(a.work[2 * idx + 1]);
       r = uni(a.rows.row_r[R]);
@@ -420,8 +448,9 @@ struct ItemCursor {
 // of the next item are started an item ahead (the work entry two items ahead), so that next() waits for none of them.
 template <bool kTok, bool kSplit, bool kPair>
 struct LengthCursor {
-  int idx, step, slot; // the item whose length `raw` is
-  int raw, h2, R2;     // length of item idx as loaded; work entry of item idx + step
+  SlotWalk<kTok, kSplit, kPair> walk;  // at the item whose length `raw` is
+  int slot;
+  int raw, h2, R2;  // length of that item as loaded; work entry of the next
   int n;
   __device__ __forceinline__ int length(const AttnArgs& a, int h, int R) const {
     return a.sel_idx ? a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R] : a.rows.row_r[R] + 1;
@@ -433,30 +462,29 @@ struct LengthCursor {
   }
   __device__ __forceinline__ void init(const AttnArgs& a, int slot_) {
     slot = slot_;
-    step = 2 * (int)gridDim.x;
-    idx = first_item_of<kSplit, kPair>(a, slot);
+    walk.init(a, slot);
     if constexpr (kTok) return;
-    entry(a, idx);
+    entry(a, walk.idx);
     raw = length(a, h2, R2);
-    entry(a, idx + step);
+    entry(a, walk.idx + 1);
   }
   // Moves to the next item with a non-empty list; false when the slot has no more items.
   __device__ __forceinline__ bool next(const AttnArgs& a) {
     do {
-      if (idx >= a.n_items) { n = 0; return false; }
+      if (walk.done()) { n = 0; return false; }
+      const int idx = walk.idx;
+      walk.advance();
       if constexpr (kTok) {
         int kvh, tile;
-        tok_item(a, idx, kvh, tile, n);
-        idx += step;
+        tok_item<kPair>(a, idx, kvh, tile, n);
         return true;
       }
       n = uni(raw);
       if (a.sel_idx) n = min(max(n, 0), a.k_max);
       int off;
       if (kSplit && a.split) part_of_list(slot, n, off);
-      idx += step;
       raw = length(a, h2, R2);
-      entry(a, idx + step);
+      entry(a, idx + 2);
     } while (n == 0);
     return true;
   }
@@ -559,8 +587,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   }
   if (!kTok && threadIdx.x < 2) {
     // the plan's tables do not depend on the kernels before this one: fetch what the first items need of them
-    const int item = first_item_of<kSplit, kPair>(a, (int)threadIdx.x);
-    if (item < a.n_items) {
+    SlotWalk<kTok, kSplit, kPair> first;
+    first.init(a, (int)threadIdx.x);
+    if (!first.done()) {
+      const int item = first.idx;
       const int R = a.work[2 * item + 1];
       const int seq = a.rows.row_seq[R];
       asm volatile("" ::"r"(a.work[2 * item]), "r"(a.rows.row_r[R]), "r"(a.rows.row_tok0[R]), "r"(a.rows.row_ntok[R]), "r"(a.rows.seq_tok0[seq]));
@@ -598,8 +628,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // chain of dependent global loads (work order -> row table -> length -> last entry).  The chain
     // of the next item is walked while the current item's blocks are processed, and its result kept
     // in one register (length, bit 31 = diagonal); the item's other fields are then cache hits.
+    SlotWalk<kTok, kSplit, kPair> walk;
+    walk.init(a, X);
     auto list_info = [&](const int item) -> uint32_t {
-      if (kTok || item >= a.n_items) return 0u;
+      if (kTok || item >= walk.limit) return 0u;
       const int h = a.work[2 * item], R = a.work[2 * item + 1];
       const int r = a.rows.row_r[R];
       int n = r + 1;
@@ -618,15 +650,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
       return (uint32_t)n | (diag ? 0x80000000u : 0u) | halves;
     };
-    const int first_item = first_item_of<kSplit, kPair>(a, X);
-    uint32_t next_info = list_info(first_item);
-    for (int item = first_item; item < a.n_items && ok; item += 2 * (int)gridDim.x) {
+    uint32_t next_info = list_info(walk.idx);
+    while (!walk.done() && ok) {
+      const int item = walk.idx;
+      walk.advance();
       const uint32_t info = next_info;
-      next_info = list_info(item + 2 * (int)gridDim.x);
+      next_info = list_info(walk.idx);
       int h, R, q_tok0, ntok, n;
       if constexpr (kTok) {
         int kvh, tile;
-        tok_item(a, item, kvh, tile, n);
+        tok_item<kPair>(a, item, kvh, tile, n);
         h = kvh * a.g + sub;
         R = kvh;
         q_tok0 = a.tok_a + tile * a.tok_tile + tokl - m;  // so that q_tok0 + m is the row's token
@@ -1179,7 +1212,8 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
     return cudaErrorInvalidValue;
 
   AttnArgs a{};
-  a.work = sel_idx ? p.d_work_sparse : p.d_work_dense;
+  const AttnWork& work = sel_idx ? p.work_sparse : p.work_dense;
+  a.work = work.d_items; a.slot_off = work.d_slot_off;
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt;
   a.O = (__nv_bfloat16*)O; a.lse = lse; a.status = status; a.rows = p.rows;
   a.n_items = p.n_items; a.Hq = p.cfg.num_q_heads; a.g = p.cfg.num_q_heads / p.cfg.num_kv_heads;
@@ -1210,9 +1244,8 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Grids of no more items than SMs leave the second slot of every CTA idle and are as long as one list: the two slots take
   // half a list each (4K tokens, 2 heads, blocks of 64, lists of up to 16: the call goes from 28.7 to 26 us).
   a.split = p.n_items <= p.sm_count ? 1 : 0;
-  // Pairs wherever neighbours in the work order have the same list; the work order holds the heads of a group together.
-  const bool pair = a.g % 2 == 0 && (sel_idx == nullptr || list_group) && !a.split;
-  const int grid = std::min(pair ? p.n_items / 2 : p.n_items, p.sm_count);
+  const bool pair = work.pair;
+  const int grid = work.ctas;
   const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList && !a.split;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1290,7 +1323,8 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
   const TokRows tok{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, q_st, q_sh, kv_st, kv_sh};
   static bool attr_set[64] = {};
   if (!attr_set[device & 63]) {
-    const cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[device & 63] = true;
   }
@@ -1303,10 +1337,16 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
     a.mask_sh = own_rows ? row_bytes : mask_bytes;
     a.mask_st = Hkv * a.mask_sh;
     a.tok_b = b;
-    a.n_items = ((b - a.tok_a + tile - 1) / tile) * Hkv;
-    cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, tile, O, a.mask_st, a.mask_sh, s);
+    const int tiles = (b - a.tok_a + tile - 1) / tile;
+    // Neighbouring tiles in pairs on one stream of K / V, where there are enough of them for every CTA.  Alone / in pairs, us:
+    // 8192 tokens, 32/8 heads (2048 tiles) 580 / 555; 9000, 28/4 (2000) 539 / 515; 1000, 64/8 (504) 35.5 / 34.1;
+    // 12000, 8/2 (750) 363 / 366; 1500, 32/8 (376) 37.9 / 39.3; 3000, 8/2 (188) 55.9 / 58.1.
+    const bool pair = tiles * Hkv > 3 * sm_count;
+    a.n_items = (pair ? (tiles + 1) / 2 * 2 : tiles) * Hkv;
+    cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, pair ? 2 * tile : tile, O, a.mask_st, a.mask_sh, s);
     if (e != cudaSuccess) return e;
-    sparse_attn_kernel<128, false, true, false><<<std::min(a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
+    auto kernel = pair ? sparse_attn_kernel<128, false, true, true> : sparse_attn_kernel<128, false, true, false>;
+    kernel<<<std::min(pair ? a.n_items / 2 : a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -53,6 +53,14 @@ struct WorkspaceLayout {
   size_t total = 0;
 };
 
+// The work of the attention kernel: which items each of the two slots of each CTA computes, in order.
+struct AttnWork {
+  const int32_t* d_items = nullptr;     // [n_items][2] (head, query row), by slot
+  const int32_t* d_slot_off = nullptr;  // [2 ctas + 1] first item of every slot
+  int ctas = 0;
+  bool pair = false;  // the slots of a CTA have two query heads of a group in the same rows, with the same lists
+};
+
 struct Plan {
   stem_config cfg{};
   std::vector<int32_t> cu;  // host copy of cu_seqlens (K / V packing)
@@ -80,8 +88,7 @@ struct Plan {
   RowTables rows{};
   const int32_t* d_gemm_tiles = nullptr;  // [n_gemm_tiles][3] (sequence, row tile, column tile) of the metric GEMM
   int32_t n_gemm_tiles = 0;
-  const int32_t* d_work_sparse = nullptr;  // [n_items][2] (head, query row), attention work order
-  const int32_t* d_work_dense = nullptr;
+  AttnWork work_sparse, work_dense;
   int32_t n_items = 0;
 
   WorkspaceLayout ws{};

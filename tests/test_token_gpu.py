@@ -206,6 +206,8 @@ def _plain_attention(q, k, v, idx, cnt, rows):
     (4300, 2, 2, 1501, "any", True, "masked, four launches, two windows of flags, entries read one at a time"),
     (897, 28, 4, 300, "ascending", True, "masked, 18-token tiles, lists that name a token twice"),
     (129, 64, 4, 128, "any", True, "masked, 8-token tiles, one token past a key block"),
+    (1000, 64, 8, 400, "ascending", True, "masked, an odd number of 16-token tiles in pairs"),
+    (2050, 28, 4, 512, "any", False, "masked, 18-token tiles in pairs that span two key blocks"),
     (3000, 2, 2, 20, "ascending", False, "gather: lists short against the prefix"),
     (300, 5, 1, 27, "any", True, "gather, lists in any order and with repeats"),
 ])
