@@ -64,13 +64,16 @@ static int validate(const stem_config* c) {
 // Neighbouring heads with the same lists go to the two slots of a CTA together, if there are more than `pairs_from` items:
 // few dense items do better one by one, as the longest of them share their CTAs with the shortest (3000 tokens, 8 / 2 heads
 // 43 us, in pairs 46; lists of a kv head are alike in length: 23 in pairs, 29).
+// Neighbours with lists of their own go to the two slots of a CTA as well, from more than `merge_from` items on, for the
+// blocks that both lists name.
 // Where there are no more items than SMs every CTA has one item (whose list its slots share).
-static void deal_items(const Plan& p, const std::vector<int32_t>& order, const std::vector<int32_t>& len, int pairs_from, AttnWork* w,
+static void deal_items(const Plan& p, const std::vector<int32_t>& order, const std::vector<int32_t>& len, int pairs_from, int merge_from, AttnWork* w,
                        std::vector<int32_t>& items, std::vector<int32_t>& slot_off) {
   const int Hq = p.cfg.num_q_heads, Hkv = p.cfg.num_kv_heads, g = Hq / Hkv;
   w->pair = g % 2 == 0 && p.n_items > pairs_from;
-  const int unit = w->pair ? 2 : 1;  // items dealt at a time
-  w->ctas = std::min(p.n_items / unit, p.sm_count);
+  w->merge = !w->pair && g > 1 && p.n_items > merge_from;
+  const int unit = w->pair || w->merge ? 2 : 1;  // items dealt at a time
+  w->ctas = std::min((p.n_items + unit - 1) / unit, p.sm_count);
   const int n_slots = 2 * w->ctas, n_queues = n_slots / unit;
   // slots by the time they are done at, first come first served; `next` links the slots done at the same time
   int64_t total = 0;
@@ -79,44 +82,46 @@ static void deal_items(const Plan& p, const std::vector<int32_t>& order, const s
     total += 2 * len[R] + 1;
     longest = std::max(longest, 2 * len[R] + 1);
   }
-  std::vector<int32_t> first((size_t)(total * (Hq / unit) / n_queues + longest + 2), -1), last(first.size(), -1), next(n_queues, -1);
+  std::vector<int32_t> first((size_t)(total * Hq / n_slots + (2 + Hkv / w->ctas) * longest + 2), -1), last(first.size(), -1), next(n_queues, -1);
   auto append = [&](size_t time, int32_t q) {
     next[q] = -1;
     if (first[time] < 0) first[time] = q; else next[last[time]] = q;
     last[time] = q;
   };
   // the second slots in reverse, so that the CTAs with the shortest first items are the first to get another one
-  if (w->pair) {
+  if (unit == 2) {
     for (int c = 0; c < w->ctas; ++c) append(0, c);
   } else {
     for (int c = 0; c < w->ctas; ++c) append(0, 2 * c);
     for (int c = w->ctas - 1; c >= 0; --c) append(0, 2 * c + 1);
   }
-  const size_t n_units = (size_t)p.n_items / unit;
-  std::vector<int32_t> owner(n_units), count(n_slots + 1, 0);
-  size_t time = 0, u = 0;
+  std::vector<int32_t> owner(p.n_items), count(n_slots + 1, 0);
+  size_t time = 0;
+  int i = 0;
+  int32_t queue = 0;
   for (int kvh = 0; kvh < Hkv; ++kvh)
     for (const int32_t R : order)
-      for (int q = 0; q < g; q += unit, ++u) {
-        while (first[time] < 0) ++time;
-        const int32_t s = first[time];
-        first[time] = next[s];
-        append(time + 2 * len[R] + 1, s);
-        owner[u] = s;
-        for (int x = 0; x < unit; ++x) ++count[unit * s + x + 1];
+      for (int q = 0; q < g; ++q, ++i) {
+        if (i % unit == 0) {
+          while (first[time] < 0) ++time;
+          queue = first[time];
+          first[time] = next[queue];
+          append(time + 2 * len[R] + 1, queue);
+        }
+        owner[i] = unit * queue + i % unit;
+        ++count[owner[i] + 1];
       }
   for (int s = 0; s < n_slots; ++s) count[s + 1] += count[s];
   slot_off = count;
   items.resize(2 * (size_t)p.n_items);
-  u = 0;
+  i = 0;
   for (int kvh = 0; kvh < Hkv; ++kvh)
     for (const int32_t R : order)
-      for (int q = 0; q < g; q += unit, ++u)
-        for (int x = 0; x < unit; ++x) {
-          const int32_t at = count[unit * owner[u] + x]++;
-          items[2 * at] = kvh * g + q + x;
-          items[2 * at + 1] = R;
-        }
+      for (int q = 0; q < g; ++q, ++i) {
+        const int32_t at = count[owner[i]]++;
+        items[2 * at] = kvh * g + q;
+        items[2 * at + 1] = R;
+      }
 }
 
 template <class T>
@@ -298,8 +303,9 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     std::stable_sort(by_r.begin(), by_r.end(), [&](int a, int b) { return row_r[a] > row_r[b]; });
     for (int R = 0; R < p.R_tot; ++R) len_dense[R] = row_r[R] + 1;
     p.n_items = p.R_tot * Hq;
-    deal_items(p, by_len, p.k_eff, p.share_group ? p.sm_count : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
-    deal_items(p, by_r, len_dense, 3 * p.sm_count, &p.work_dense, work_dense, slots_dense);
+    deal_items(p, by_len, p.k_eff, p.share_group ? p.sm_count : p.n_items,
+               p.k_max <= attention_merge_max_list() ? 2 * p.sm_count : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
+    deal_items(p, by_r, len_dense, 3 * p.sm_count, p.n_items, &p.work_dense, work_dense, slots_dense);
   }
 
   // Workspace layout.  With a caller-owned cache the K-side tensors are not part of the workspace.

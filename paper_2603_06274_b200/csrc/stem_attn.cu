@@ -12,10 +12,16 @@
 //                 the item's last block O / l -> bf16 -> global memory
 //     warps 4-7   the same for slot 1
 //     warp 8      TMA producer of the K / V ring (all lanes in lock step, one elected lane issues)
-//     warp 9      owns the TMEM allocation
+//     warp 9      owns the TMEM allocation; merges the lists of two items (kMerge)
 //     warp 10     TMA producer of the Q tiles (likewise)
 //     warp 11     MMA issuer (likewise): waits for K / V, Q, O and P of each visit and issues its MMAs; P V starts on
 //                 the leading key columns while the softmax still works on the last 32
+// Other query heads of a group have lists of their own, but choose many of the same blocks (always the first and the local
+// ones).  With kMerge the slots take neighbouring items, warp 9 finds a pair ahead which blocks both lists name, and each
+// slot walks its own blocks first and the common ones, the diagonal block last, in step with the other slot on one stream
+// of tiles.  Slots one by one / merged, TFLOP/s at 32 / 8 heads, lists of 22 blocks (32K tokens) and 42 (128K): 1128 / 1247 and
+// 1121 / 1262 with 9 of 10 blocks in common, 1120 / 1220 and 1110 / 1200 for independent random metrics; 64K tokens, 28 / 4:
+// 1135 / 1255; blocks of 64 at 32K 420 / 467.
 // TMEM columns: S/P of slot 0, S/P of slot 1, O of slot 0, O of slot 1 (128 columns each).
 // The MMA issuer visits the slots alternately; a visit issues P V of the slot's previous block and
 // then Q K^T of its next block (P overwrites S, so the order inside a visit is fixed).  The K / V
@@ -65,9 +71,13 @@ constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
 constexpr float kRescaleThreshold = 8.0f;                // log2 units
 constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after: 256 x 216 + 128 x 72
 
-enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4 };
+constexpr int kMergeMaxList = 208;                       // longest list (blocks) that is merged with its neighbour's
+constexpr int kMergeHeader = 32;                         // lengths, common blocks; kv head and first token of both slots
+constexpr int kMergeBytes = kMergeHeader + 2 * kMergeMaxList * 2;
+
+enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4, kRoleMerge = 5 };
 enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarPEarly, kBarHalves };
+                   kBarDrain, kBarPEarly, kBarHalves, kBarMergeFull, kBarMergeEmpty };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -86,7 +96,10 @@ struct Smem {
   static constexpr int drain = halves + 8;
   static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
-  static constexpr int total = abort_flag + 4;
+  static constexpr int merge_full = abort_flag + 4;       // kMerge: the merged lists of a pair of items, two buffers
+  static constexpr int merge_empty = merge_full + 16;
+  static constexpr int merge_buf = merge_empty + 16;
+  static constexpr int total = merge_buf + 2 * kMergeBytes;
 };
 constexpr int kSmemBytes = Smem::total + 1024;  // slack for manual 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
@@ -400,6 +413,12 @@ struct SlotWalk {
   }
 };
 
+// kMerge: the pairs of items of this CTA (slot 1's last one may be missing).
+__device__ __forceinline__ int pairs_of(const AttnArgs& a) {
+  const int32_t* off = a.slot_off + 2 * blockIdx.x;
+  return max(off[1] - off[0], off[2] - off[1]);
+}
+
 // A slot's part of a list of n entries that the two slots share.
 __device__ __forceinline__ void part_of_list(int slot, int& n, int& off) {
   const int first = (n + 1) >> 1;
@@ -537,7 +556,7 @@ __device__ __noinline__ void exact_token_row(float scale_log2, const __nv_bfloat
   if (lse) *lse = (m + log2f(l)) * 0.6931471805599453f;
 }
 
-template <int BLK, bool kSpareQ, bool kTok, bool kPair>
+template <int BLK, bool kSpareQ, bool kTok, bool kPair, bool kMerge = false>
 __global__ void __launch_bounds__(kThreads, 1)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const AttnArgs a, const TokRows tok) {
@@ -555,6 +574,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // otherwise two Q tiles and a ring of five, for long lists (and the dense mode), where the deeper ring pays.
   static_assert(!kTok || (BLK == 128 && !kSpareQ), "the token-list form has two Q tiles and key blocks of 128");
   static_assert(!kPair || !kSpareQ, "pairs have two Q tiles");
+  static_assert(!kMerge || (kSpareQ && !kTok && !kPair), "merged lists use the layout with the spare Q tile");
   constexpr bool kSplit = !kSpareQ && !kTok && !kPair;  // the layout that may cut lists in halves (a.split)
   constexpr int kKvSlots = kSpareQ ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
@@ -572,6 +592,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::p_early, i), 4);   // likewise
       mbar_init(bar(Smem::o_full, i), 1);
       mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
+    }
+    if constexpr (kMerge) {
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(bar(Smem::merge_full, i), 1);
+        mbar_init(bar(Smem::merge_empty, i), 2);  // the K / V producer and the MMA issuer
+      }
     }
     mbar_init(bar(Smem::halves, 0), 8);
     mbar_init(bar(Smem::drain, 0), 1);
@@ -941,18 +967,57 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         return true;
       };
-      KvSlot s0, s1;
-      s0.cur.init(a, 0); s1.cur.init(a, 1);
-      s0.pend = s1.pend = false;
-      enter(s0);
-      if (kPair) s1.has = false; else enter(s1);  // (pairs: one stream of K / V for both slots)
       bool ok = true;
-      // With the spare Q tile slot 1 starts half an item behind slot 0, so that the two slots' item boundaries (and
-      // their claims on the spare) do not fall together.  The MMA issuer skips the same visits.
-      const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;
-      for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
-        ok = visit(s0);
-        if (!kPair && ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
+      if constexpr (kMerge) {
+        // The merged lists: in each round a block of slot 0's own and one of slot 1's own, then those both have, one tile each.
+        int pend_tok[2] = {-1, -1}, pend_kvh[2] = {0, 0};  // V tile that is due; slot 0's alone if both have the block
+        auto pend = [&](const int X) -> bool {
+          if (pend_tok[X] < 0) return true;
+          const int tok = pend_tok[X];
+          pend_tok[X] = -1;
+          return load(&map_v, pend_kvh[X], tok);
+        };
+        const int pairs = pairs_of(a);
+        for (int k = 0; ok && k < pairs; ++k) {
+          const int b = k & 1;
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::merge_full, b), (k >> 1) & 1, ctx, kBarMergeFull));
+          if (!ok) break;
+          const volatile int* hdr = (const volatile int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
+          const volatile uint16_t* ent = (const volatile uint16_t*)(hdr + kMergeHeader / 4);
+          const int n0 = uni(hdr[0]), n1 = uni(hdr[1]), both = uni(hdr[2]);
+          const int kvh[2] = {uni(hdr[3]), uni(hdr[5])}, tok0[2] = {uni(hdr[4]), uni(hdr[6])};
+          const int c0 = n0 - both, c1 = n1 - both, own = max(c0, c1);
+          for (int it = 0; ok && it < own + both; ++it) {
+            ok = pend(0);
+            if (ok && it >= own - c0) {
+              pend_tok[0] = tok0[0] + uni((int)ent[it - (own - c0)]) * BLK;
+              pend_kvh[0] = kvh[0];
+              ok = load(&map_k, kvh[0], pend_tok[0]);
+            }
+            if (ok) ok = pend(1);
+            if (ok && it >= own - c1 && it < own) {
+              pend_tok[1] = tok0[1] + uni((int)ent[n0 + it - (own - c1)]) * BLK;
+              pend_kvh[1] = kvh[1];
+              ok = load(&map_k, kvh[1], pend_tok[1]);
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(Smem::merge_empty, b));
+        }
+        ok = ok && pend(0) && pend(1);
+      } else {
+        KvSlot s0, s1;
+        s0.cur.init(a, 0); s1.cur.init(a, 1);
+        s0.pend = s1.pend = false;
+        enter(s0);
+        if (kPair) s1.has = false; else enter(s1);  // (pairs: one stream of K / V for both slots)
+        // With the spare Q tile slot 1 starts half an item behind slot 0, so that the two slots' item boundaries (and
+        // their claims on the spare) do not fall together.  The MMA issuer skips the same visits.
+        const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;
+        for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
+          ok = visit(s0);
+          if (!kPair && ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
+        }
       }
       if (!ok && lane == 0) {
         // aborting: give copies already in flight a bounded time to land before the CTA exits
@@ -962,10 +1027,113 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           while (!mbar_try(bar(Smem::kv_full, c % kKvSlots), (c / kKvSlots) & 1) && globaltimer() - t0 < 2000000ull) {}
         }
       }
+    } else if (kMerge && warp == 9) {
+      // ============================== list merger ==============================
+      // For each pair of items, a pair ahead: the entries of slot 0's list that slot 1's does not have, then those both
+      // have; behind them the other entries of slot 1's.  Both lists have to be strictly ascending and to end on the same
+      // block (the last one is masked on the diagonal) in the same row of the same kv head; else they have nothing in common.
+      Ctx ctx{abort_flag, status, kRoleMerge, 1};
+      SlotWalk<kTok, kSplit, kPair> w[2];
+      w[0].init(a, 0); w[1].init(a, 1);
+      for (int k = 0; !w[0].done() || !w[1].done(); ++k) {
+        const int b = k & 1;
+        if (k >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar(Smem::merge_empty, b), ((k >> 1) & 1) ^ 1, ctx, kBarMergeEmpty))) break;
+        int n[2] = {0, 0}, R[2] = {-1, -1}, kvh[2] = {-1, -1}, r[2] = {0, 0}, tok0[2] = {0, 0};
+        const int32_t* list[2] = {nullptr, nullptr};
+#pragma unroll
+        for (int X = 0; X < 2; ++X) {
+          if (w[X].done()) continue;
+          const int h = a.work[2 * w[X].idx];
+          R[X] = a.work[2 * w[X].idx + 1];
+          w[X].advance();
+          const int64_t row = (int64_t)(h / a.list_div) * a.R_tot + R[X];
+          kvh[X] = h / a.g;
+          r[X] = a.rows.row_r[R[X]];
+          tok0[X] = a.rows.seq_tok0[a.rows.row_seq[R[X]]];
+          n[X] = min(max(a.sel_cnt[row], 0), a.k_max);
+          list[X] = a.sel_idx + row * a.k_max;
+        }
+        auto entry = [&](const int X, const int i) { return min(max(list[X][i], 0), r[X]); };
+        uint32_t both[2] = {0u, 0u};  // bit t: entry 32 t + lane is in the other list
+        if (R[0] == R[1] && kvh[0] == kvh[1] && n[0] > 0 && n[1] > 0) {
+          bool bad = entry(0, n[0] - 1) != entry(1, n[1] - 1);
+#pragma unroll
+          for (int X = 0; X < 2; ++X) {
+#pragma unroll 1
+            for (int i = lane, t = 0; i < n[X]; i += 32, ++t) {
+              const int v = entry(X, i);
+              bad = bad || (i > 0 && entry(X, i - 1) >= v);
+              int lo = 0, hi = n[X ^ 1] - 1;  // the first entry of the other list that is not below v, or the last
+              while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (entry(X ^ 1, mid) < v) lo = mid + 1; else hi = mid;
+              }
+              if (entry(X ^ 1, lo) == v) both[X] |= 1u << t;
+            }
+          }
+          if (__any_sync(0xffffffffu, bad)) both[0] = both[1] = 0u;
+        }
+        const int m = __reduce_add_sync(0xffffffffu, __popc(both[0]));
+        int* hdr = (int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
+        uint16_t* ent = (uint16_t*)(hdr + kMergeHeader / 4);
+        const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+        for (int X = 0; X < 2; ++X) {
+          int own_at = X ? n[0] : 0, both_at = n[0] - m;
+#pragma unroll 1
+          for (int i0 = 0, t = 0; i0 < n[X]; i0 += 32, ++t) {
+            const bool in = i0 + lane < n[X], shared = in && ((both[X] >> t) & 1u);
+            const uint32_t mo = __ballot_sync(0xffffffffu, in && !shared), mb = __ballot_sync(0xffffffffu, shared);
+            if (in && !(X == 1 && shared))
+              ent[shared ? both_at + __popc(mb & below) : own_at + __popc(mo & below)] = (uint16_t)entry(X, i0 + lane);
+            own_at += __popc(mo);
+            both_at += __popc(mb);
+          }
+        }
+        if (lane == 0) {
+          hdr[0] = n[0]; hdr[1] = n[1]; hdr[2] = m;
+          hdr[3] = kvh[0]; hdr[4] = tok0[0]; hdr[5] = kvh[1]; hdr[6] = tok0[1];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(Smem::merge_full, b));
+      }
     } else if (warp == 10) {
       // ============================== Q producer ==============================
       Ctx ctx{abort_flag, status, kRoleQProducer, kTok ? 4 : 1};
-      if constexpr (kSpareQ) {
+      if constexpr (kMerge) {
+        // The slots' items end in the same round: the tiles go through the three buffers in order, slot 0's first.
+        SlotWalk<kTok, kSplit, kPair> w[2];
+        w[0].init(a, 0); w[1].init(a, 1);
+        uint32_t tiles = 0, buf = 0, par = 0;
+        bool ok = true;
+        while (ok && (!w[0].done() || !w[1].done())) {
+#pragma unroll
+          for (int X = 0; X < 2; ++X) {
+            if (!ok || w[X].done()) continue;
+            const int h = uni(a.work[2 * w[X].idx]), R = uni(a.work[2 * w[X].idx + 1]);
+            w[X].advance();
+            if (uni(a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R]) <= 0) continue;
+            const int q_tok0 = uni(a.rows.row_tok0[R]);
+            if (tiles >= (uint32_t)kQBufs) ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::q_empty, buf), par ^ 1u, ctx, kBarQEmpty));
+            if (!ok) continue;
+            const uint32_t dst = smem_base + Smem::q + buf * kQBytes;
+            if (elect_one()) {
+              mbar_expect_tx(bar(Smem::q_full, buf), kQBytes);
+              tma_load_3d(dst, &map_q, bar(Smem::q_full, buf), 0, h, q_tok0);
+              tma_load_3d(dst + kTileM * 128, &map_q, bar(Smem::q_full, buf), 64, h, q_tok0);
+            }
+            __syncwarp();
+            ++tiles;
+            if (++buf == (uint32_t)kQBufs) { buf = 0; par ^= 1u; }
+          }
+        }
+        if (!ok && lane == 0) {
+          // aborting: bounded wait for the Q copies that may still be in flight
+          const uint64_t t1 = globaltimer();
+          for (uint32_t t = tiles > (uint32_t)kQBufs ? tiles - kQBufs : 0u; t < tiles; ++t)
+            while (!mbar_try(bar(Smem::q_full, t % kQBufs), (t / kQBufs) & 1) && globaltimer() - t1 < 4000000ull) {}
+        }
+      } else if constexpr (kSpareQ) {
         // The two slots advance one block per round of the MMA issuer, so the round at which a slot's item ends is the
         // running sum of its list lengths: the slot with the smaller sum finishes first (slot 0 on a tie) and gets the
         // next tile, loaded into the spare buffer long before it is wanted; the buffer the slot leaves becomes the
@@ -1083,60 +1251,74 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       constexpr int kEarlySteps = (BLK / 32 - 1) * 2;  // 16-key steps of P V covered by p_early
       const uint32_t abort_addr = smem_base + Smem::abort_flag;
       int failed = 0;
-      auto visit = [&](MmaSlot& s, const int X) {
+      auto next_tile = [&] {
+        if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
+      };
+      // O_X (+)= P V with the V tile in ring slot `tile`, which is given back with `release`.
+      auto issue_pv = [&](MmaSlot& s, const int X, const uint32_t tile, const bool release) {
         const uint32_t s_tmem = tmem_base + X * 128;
         const uint32_t o_tmem = tmem_base + kOCol + X * 128;
         const uint32_t st = s.st;
+        const uint32_t v_addr = smem_base + kKvOff + tile * kSlotBytes;
+        if (st & kFirst) mbar_wait_sticky(bar(Smem::o_free, X), s.o_par ^ 1, abort_addr, kBarOFree, failed);
+        // P V starts on the leading key columns while the softmax still works on the last 32
+        mbar_wait_sticky(bar(Smem::p_early, X), s.p_par, abort_addr, kBarPEarly, failed);
+        tc_fence_after();
+        if (leader) {
+          const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
+#pragma unroll
+          for (int k = 0; k < kEarlySteps; ++k)
+            mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, (k == 0 && (st & kFirst)) ? 0u : 1u);
+        }
+        __syncwarp();
+        mbar_wait_sticky(bar(Smem::p_ready, X), s.p_par, abort_addr, kBarPReady, failed);
+        tc_fence_after();
+        if (leader) {
+          const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
+#pragma unroll
+          for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
+          if (release) tc_commit(bar(Smem::kv_empty, tile));
+          if (st & kLast) tc_commit(bar(Smem::o_full, X));
+        }
+        __syncwarp();
+        s.p_par ^= 1;
+        if (st & kLast) s.o_par ^= 1;
+        s.st = st & kNewItem;
+      };
+      // S_X = Q K^T with the K tile in ring slot `tile`; true for the last block of the slot's item.
+      auto issue_qk = [&](MmaSlot& s, const int X, const uint32_t tile, const bool release) -> bool {
+        const uint32_t st = s.st;
+        if (st & kNewItem) mbar_wait_sticky(bar(Smem::q_full, s.qbuf), s.q_par, abort_addr, kBarQFull, failed);
+        tc_fence_after();
+        const bool last = --s.left == 0;
+        if (leader) {
+          const uint64_t da = smem_desc(smem_base + Smem::q + s.qbuf * kQBytes, 16, 1024);
+          const uint64_t db = smem_desc(smem_base + kKvOff + tile * kSlotBytes, 16, 1024);
+#pragma unroll
+          for (int k = 0; k < kHeadDim / 16; ++k)  // 16 columns = 32 bytes on; the second four steps: the other 64-column half
+            mma_ss(tmem_base + X * 128, da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4),
+                   db + (((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4), kIdescS, k > 0 ? 1u : 0u);
+          if (release) tc_commit(bar(Smem::kv_empty, tile));
+          tc_commit(bar(Smem::s_full, X));
+          if (last) tc_commit(bar(Smem::q_empty, s.qbuf));
+        }
+        __syncwarp();
+        s.st = kPend | ((st & kNewItem) ? kFirst : 0u) | (last ? kLast | kNewItem : 0u);
+        return last;
+      };
+      auto wait_tile = [&] { mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed); };
+      auto visit = [&](MmaSlot& s, const int X) {
         const uint32_t ring0 = ring, ring_par0 = ring_par;
         const bool shared = kPair && X == 0;  // slot 1's visit uses the same tiles and gives them back
-        if (st & kPend) {
-          const uint32_t v_addr = smem_base + kKvOff + ring * kSlotBytes;
-          if (!kPair || X == 0) mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
-          if (st & kFirst) mbar_wait_sticky(bar(Smem::o_free, X), s.o_par ^ 1, abort_addr, kBarOFree, failed);
-          // P V starts on the leading key columns while the softmax still works on the last 32
-          mbar_wait_sticky(bar(Smem::p_early, X), s.p_par, abort_addr, kBarPEarly, failed);
-          tc_fence_after();
-          if (leader) {
-            const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
-#pragma unroll
-            for (int k = 0; k < kEarlySteps; ++k)
-              mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, (k == 0 && (st & kFirst)) ? 0u : 1u);
-          }
-          __syncwarp();
-          mbar_wait_sticky(bar(Smem::p_ready, X), s.p_par, abort_addr, kBarPReady, failed);
-          tc_fence_after();
-          if (leader) {
-            const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
-#pragma unroll
-            for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
-            if (!shared) tc_commit(bar(Smem::kv_empty, ring));
-            if (st & kLast) tc_commit(bar(Smem::o_full, X));
-          }
-          __syncwarp();
-          if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
-          s.p_par ^= 1;
-          if (st & kLast) s.o_par ^= 1;
-          s.st = st & kNewItem;
+        if (s.st & kPend) {
+          if (!kPair || X == 0) wait_tile();
+          issue_pv(s, X, ring, !shared);
+          next_tile();
         }
         if (s.left > 0) {
-          if (!kPair || X == 0) mbar_wait_sticky(bar(Smem::kv_full, ring), ring_par, abort_addr, kBarKvFull, failed);
-          if (st & kNewItem) mbar_wait_sticky(bar(Smem::q_full, s.qbuf), s.q_par, abort_addr, kBarQFull, failed);
-          tc_fence_after();
-          const bool last = --s.left == 0;
-          if (leader) {
-            const uint64_t da = smem_desc(smem_base + Smem::q + s.qbuf * kQBytes, 16, 1024);
-            const uint64_t db = smem_desc(smem_base + kKvOff + ring * kSlotBytes, 16, 1024);
-#pragma unroll
-            for (int k = 0; k < kHeadDim / 16; ++k)  // 16 columns = 32 bytes on; the second four steps: the other 64-column half
-              mma_ss(s_tmem, da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4), db + (((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4),
-                     kIdescS, k > 0 ? 1u : 0u);
-            if (!shared) tc_commit(bar(Smem::kv_empty, ring));
-            tc_commit(bar(Smem::s_full, X));
-            if (last) tc_commit(bar(Smem::q_empty, s.qbuf));
-          }
-          __syncwarp();
-          if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
-          s.st = kPend | ((st & kNewItem) ? kFirst : 0u) | (last ? kLast | kNewItem : 0u);
+          if (!kPair || X == 0) wait_tile();
+          const bool last = issue_qk(s, X, ring, !shared);
+          next_tile();
           if (last) {
             s.left = s.cur.next(a) ? s.cur.n : 0;
             if constexpr (kSpareQ) {
@@ -1154,18 +1336,90 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         if (shared) { ring = ring0; ring_par = ring_par0; }
       };
-      MmaSlot s0, s1;
-      s0.cur.init(a, 0); s1.cur.init(a, 1);
-      s0.left = s0.cur.next(a) ? s0.cur.n : 0;
-      s1.left = s1.cur.next(a) ? s1.cur.n : 0;
-      s0.st = s1.st = kNewItem;
-      s0.p_par = s1.p_par = s0.q_par = s1.q_par = s0.o_par = s1.o_par = 0;
-      s0.qbuf = 0; s1.qbuf = 1;
-      const uint32_t delay1 = kSpareQ ? (uint32_t)s0.left / 2u : 0u;  // as in the K / V producer
-      for (uint32_t it = 0; s0.left > 0 || s1.left > 0 || ((s0.st | s1.st) & kPend); ++it) {
-        visit(s0, 0);
-        if (!kSpareQ || it >= delay1) visit(s1, 1);
-        if (__any_sync(0xffffffffu, failed != 0)) break;
+      if constexpr (kMerge) {
+        MmaSlot s0, s1;
+        s0.left = s1.left = 0;
+        s0.st = s1.st = kNewItem;
+        s0.p_par = s1.p_par = s0.o_par = s1.o_par = 0;
+        int q_tile = 0;
+        uint32_t q_phase = 0;
+        auto take_q = [&](MmaSlot& s) {
+          s.qbuf = q_tile;
+          s.q_par = q_phase;
+          if (++q_tile == kQBufs) { q_tile = 0; q_phase ^= 1; }
+        };
+        bool v_both = false;  // both slots' V tile that is due is the same
+        // A round: as in visit(), with the tiles of the blocks that both lists have used by slot 0, then by slot 1.
+        auto round = [&](const bool act0, const bool act1, const bool k_both) {
+          uint32_t v_tile = 0, k_tile = 0;
+          if (s0.st & kPend) {
+            v_tile = ring;
+            wait_tile();
+            issue_pv(s0, 0, ring, !v_both);
+            next_tile();
+          }
+          if (act0) {
+            k_tile = ring;
+            wait_tile();
+            issue_qk(s0, 0, ring, !k_both);
+            next_tile();
+          }
+          if (s1.st & kPend) {
+            if (!v_both) {
+              v_tile = ring;
+              wait_tile();
+              next_tile();
+            }
+            issue_pv(s1, 1, v_tile, true);
+          }
+          if (act1) {
+            if (!k_both) {
+              k_tile = ring;
+              wait_tile();
+              next_tile();
+            }
+            issue_qk(s1, 1, k_tile, true);
+          }
+          v_both = k_both;
+        };
+        const int pairs = pairs_of(a);
+        for (int k = 0; k < pairs; ++k) {
+          const int b = k & 1;
+          mbar_wait_sticky(bar(Smem::merge_full, b), (k >> 1) & 1, abort_addr, kBarMergeFull, failed);
+          if (__any_sync(0xffffffffu, failed != 0)) break;
+          const volatile int* hdr = (const volatile int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
+          s0.left = uni(hdr[0]);
+          s1.left = uni(hdr[1]);
+          const int both = uni(hdr[2]);
+          if (lane == 0) mbar_arrive(bar(Smem::merge_empty, b));
+          if (s0.left > 0) take_q(s0);
+          if (s1.left > 0) take_q(s1);
+          const int c0 = s0.left - both, c1 = s1.left - both, own = max(c0, c1);
+          for (int it = 0; it < own; ++it) {
+            round(it >= own - c0, it >= own - c1, false);
+            if (__any_sync(0xffffffffu, failed != 0)) break;
+          }
+          for (int it = 0; it < both; ++it) {
+            round(true, true, true);
+            if (__any_sync(0xffffffffu, failed != 0)) break;
+          }
+          if (__any_sync(0xffffffffu, failed != 0)) break;
+        }
+        if (!__any_sync(0xffffffffu, failed != 0)) round(false, false, false);
+      } else {
+        MmaSlot s0, s1;
+        s0.cur.init(a, 0); s1.cur.init(a, 1);
+        s0.left = s0.cur.next(a) ? s0.cur.n : 0;
+        s1.left = s1.cur.next(a) ? s1.cur.n : 0;
+        s0.st = s1.st = kNewItem;
+        s0.p_par = s1.p_par = s0.q_par = s1.q_par = s0.o_par = s1.o_par = 0;
+        s0.qbuf = 0; s1.qbuf = 1;
+        const uint32_t delay1 = kSpareQ ? (uint32_t)s0.left / 2u : 0u;  // as in the K / V producer
+        for (uint32_t it = 0; s0.left > 0 || s1.left > 0 || ((s0.st | s1.st) & kPend); ++it) {
+          visit(s0, 0);
+          if (!kSpareQ || it >= delay1) visit(s1, 1);
+          if (__any_sync(0xffffffffu, failed != 0)) break;
+        }
       }
       const bool ok = !__any_sync(0xffffffffu, failed != 0);
       if (failed != 0) raise_abort(ctx, failed);
@@ -1199,6 +1453,8 @@ bool make_map(CUtensorMap* map, const void* base, int64_t T, int H, int64_t stri
 }
 
 }  // namespace
+
+int attention_merge_max_list() { return kMergeMaxList; }
 
 cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K, const void* V, const int32_t* sel_idx,
                                     const int32_t* sel_cnt, bool list_group, void* O, float* lse, int32_t* status,
@@ -1236,6 +1492,8 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<128, true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_kernel<64, true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[dev_slot] = true;
   }
@@ -1244,7 +1502,7 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Grids of no more items than SMs leave the second slot of every CTA idle and are as long as one list: the two slots take
   // half a list each (4K tokens, 2 heads, blocks of 64, lists of up to 16: the call goes from 28.7 to 26 us).
   a.split = p.n_items <= p.sm_count ? 1 : 0;
-  const bool pair = work.pair;
+  const bool pair = work.pair, merge = work.merge;
   const int grid = work.ctas;
   const bool spare_q = sel_idx != nullptr && p.k_max <= kSpareQMaxList && !a.split;
   cudaLaunchAttribute attr[1];
@@ -1259,7 +1517,9 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
   // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
   cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
-  auto kernel = pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
+  // Two streams of tiles are for what is left: one query head per kv head, few items, very long lists.
+  auto kernel = merge ? (B == 128 ? sparse_attn_kernel<128, true, false, false, true> : sparse_attn_kernel<64, true, false, false, true>)
+              : pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
               : B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false, false> : sparse_attn_kernel<128, false, false, false>)
                          : (spare_q ? sparse_attn_kernel<64, true, false, false> : sparse_attn_kernel<64, false, false, false>);
   return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, a, TokRows{});

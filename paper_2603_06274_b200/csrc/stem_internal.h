@@ -59,6 +59,7 @@ struct AttnWork {
   const int32_t* d_slot_off = nullptr;  // [2 ctas + 1] first item of every slot
   int ctas = 0;
   bool pair = false;  // the slots of a CTA have two query heads of a group in the same rows, with the same lists
+  bool merge = false; // likewise, or a head and the next row's first, with lists of their own that may have blocks in common
 };
 
 struct Plan {
@@ -141,6 +142,8 @@ cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const v
 
 // dependent: launched as a programmatic dependent of the selection kernel enqueued just before, its status words cleared by
 // an earlier kernel; otherwise the launch clears them itself.
+// Longest list whose blocks the attention kernel looks up in another head's list.
+int attention_merge_max_list();
 // list_group: the lists are per kv head ([H_kv, R_tot, k_max]); every query head of a group walks its group's list.
 cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K, const void* V,
                                     const int32_t* sel_idx, const int32_t* sel_cnt, bool list_group, void* O, float* lse,

@@ -349,3 +349,58 @@ def test_heads_of_a_group_with_the_same_lists(block, seqlens, hq, hkv, dense):
     live = np.isfinite(lse_ref)
     assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
     plan.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (128, (37 * 128,), 8, 4),              # 296 items: each slot for itself
+    (128, (37 * 128 + 1,), 8, 4),          # 304: two heads of a group at a time, tiles that both lists name loaded once
+    (64, (2500, 700, 63), 14, 2),          # odd groups: pairs over two rows among them
+    (64, (64 * 20 + 9,), 15, 3),           # an odd number of items
+])
+def test_neighbouring_heads_with_lists_in_common(block, seqlens, hq, hkv):
+    # lists that are the same, share some blocks or only the last, differ in length, end on different blocks, are empty, in
+    # any order or name a block twice
+    w = wl.small("common", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=1000, mu_num=1, mu_den=1, seed=sum(seqlens))
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w)
+    info = plan.info
+    row_r = np.concatenate([np.arange((n + block - 1) // block) for n in seqlens])
+    r = np.random.default_rng(hq + sum(seqlens))
+    idx = np.full((hq, info.total_q_blocks, info.k_max), -1, np.int32)
+    cnt = np.zeros((hq, info.total_q_blocks), np.int32)
+    for R, row in enumerate(row_r):
+        kind = int(r.integers(0, 8))
+        base = np.sort(r.choice(row + 1, size=int(r.integers(1, row + 2)), replace=False))
+        for h in range(hq):
+            own = np.sort(r.choice(row + 1, size=int(r.integers(1, row + 2)), replace=False))
+            lst = base if kind < 2 else own
+            if kind in (0, 2, 3):
+                lst = np.union1d(lst, [row])                                # with the diagonal block
+            elif kind == 4:
+                lst = np.union1d(base[r.random(len(base)) < 0.8], [row])    # much in common
+            elif kind == 5:
+                lst = own[:0] if r.random() < 0.5 else np.union1d(own, [row])
+            elif kind == 6 and row > 0:
+                lst = np.append(r.permutation(own[own < row]), row)         # any order, the diagonal block last
+            elif kind == 7 and row > 0:
+                lst = np.sort(r.choice(row, size=min(row, 5)))              # repeats
+            lst = lst[-info.k_max:]
+            idx[h, R, :len(lst)] = lst
+            cnt[h, R] = len(lst)
+    n_tok = w.total_tokens
+    outs = []
+    for _ in range(2):
+        out = torch.full((n_tok, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((hq, n_tok), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_sparse_prefill(plan, q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out, lse)
+        assert binding.stem_check_status(plan)[0] == 0
+        outs.append((out, lse))
+    assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16)) and torch.equal(outs[0][1], outs[1][1])
+    O_ref, lse_ref = so.attention(data["q"], data["k"], data["v"], data["cu_seqlens"], block, idx, cnt)
+    check_attention(from_dev_bf16(outs[0][0]), O_ref, ~np.isnan(O_ref), label=f"{len(row_r) * hq} items")
+    got = outs[0][1].cpu().numpy()
+    assert np.isneginf(got[np.isneginf(lse_ref)]).all()
+    live = np.isfinite(lse_ref)
+    assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
+    plan.close()
