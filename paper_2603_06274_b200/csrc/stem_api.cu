@@ -62,16 +62,16 @@ static int validate(const stem_config* c) {
 // dense, us: 16K tokens, 32 / 8 heads 1735 / 1614; 4K, 28 / 4 127 / 114; 9000, 8 / 2 225 / 126 (the times of sparse layers
 // differ by less than their runs do).  An item counts half a block besides its blocks.
 // Neighbouring heads with the same lists go to the two slots of a CTA together, if there are more than `pairs_from` items:
-// few dense items do better one by one, as the longest of them share their CTAs with the shortest (3000 tokens, 8 / 2 heads
-// 43 us, in pairs 46; lists of a kv head are alike in length: 23 in pairs, 29).
+// few dense items do better one by one, as the longest of them share their CTAs with the shortest (3000 tokens, 8 / 2 heads,
+// 192 items: 43 us, in pairs 46); chosen lists are alike in length (29, in pairs 23).
 // Neighbours with lists of their own go to the two slots of a CTA as well, from more than `merge_from` items on, for the
-// blocks that both lists name.
+// blocks that both lists name (one by one / together, us: 160 items 21 / 23, 192 29 / 24, 256 29 / 25, 320 31 / 27).
 // Where there are no more items than SMs every CTA has one item (whose list its slots share).
 static void deal_items(const Plan& p, const std::vector<int32_t>& order, const std::vector<int32_t>& len, int pairs_from, int merge_from, AttnWork* w,
                        std::vector<int32_t>& items, std::vector<int32_t>& slot_off) {
   const int Hq = p.cfg.num_q_heads, Hkv = p.cfg.num_kv_heads, g = Hq / Hkv;
   w->pair = g % 2 == 0 && p.n_items > pairs_from;
-  w->merge = !w->pair && g > 1 && p.n_items > merge_from;
+  w->merge = !w->pair && p.n_items > merge_from;
   const int unit = w->pair || w->merge ? 2 : 1;  // items dealt at a time
   w->ctas = std::min((p.n_items + unit - 1) / unit, p.sm_count);
   const int n_slots = 2 * w->ctas, n_queues = n_slots / unit;
@@ -303,8 +303,9 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     std::stable_sort(by_r.begin(), by_r.end(), [&](int a, int b) { return row_r[a] > row_r[b]; });
     for (int R = 0; R < p.R_tot; ++R) len_dense[R] = row_r[R] + 1;
     p.n_items = p.R_tot * Hq;
-    deal_items(p, by_len, p.k_eff, p.share_group ? p.sm_count : p.n_items,
-               p.k_max <= attention_merge_max_list() ? 2 * p.sm_count : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
+    const int few = 5 * p.sm_count / 4;
+    deal_items(p, by_len, p.k_eff, p.share_group ? few : p.n_items,
+               p.k_max <= attention_merge_max_list() ? few : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
     deal_items(p, by_r, len_dense, 3 * p.sm_count, p.n_items, &p.work_dense, work_dense, slots_dense);
   }
 

@@ -21,7 +21,8 @@
 // slot walks its own blocks first and the common ones, the diagonal block last, in step with the other slot on one stream
 // of tiles.  Slots one by one / merged, TFLOP/s at 32 / 8 heads, lists of 22 blocks (32K tokens) and 42 (128K): 1128 / 1247 and
 // 1121 / 1262 with 9 of 10 blocks in common, 1120 / 1220 and 1110 / 1200 for independent random metrics; 64K tokens, 28 / 4:
-// 1135 / 1255; blocks of 64 at 32K 420 / 467.
+// 1135 / 1255; blocks of 64 at 32K 420 / 467.  Neighbours may be two rows of one head as well, whose last blocks differ: 64K
+// tokens, 2 / 2 heads 980 / 1150; 16K, 8 / 8, blocks of 64 350 / 420.
 // TMEM columns: S/P of slot 0, S/P of slot 1, O of slot 0, O of slot 1 (128 columns each).
 // The MMA issuer visits the slots alternately; a visit issues P V of the slot's previous block and
 // then Q K^T of its next block (P overwrites S, so the order inside a visit is fixed).  The K / V
@@ -72,7 +73,8 @@ constexpr float kRescaleThreshold = 8.0f;                // log2 units
 constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after: 256 x 216 + 128 x 72
 
 constexpr int kMergeMaxList = 208;                       // longest list (blocks) that is merged with its neighbour's
-constexpr int kMergeHeader = 32;                         // lengths, common blocks; kv head and first token of both slots
+constexpr int kMergeHeader = 32;                         // lengths, common blocks, whether the lists' last blocks come behind
+                                                         // those; kv head and first token of both slots
 constexpr int kMergeBytes = kMergeHeader + 2 * kMergeMaxList * 2;
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4, kRoleMerge = 5 };
@@ -985,9 +987,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const volatile int* hdr = (const volatile int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
           const volatile uint16_t* ent = (const volatile uint16_t*)(hdr + kMergeHeader / 4);
           const int n0 = uni(hdr[0]), n1 = uni(hdr[1]), both = uni(hdr[2]);
-          const int kvh[2] = {uni(hdr[3]), uni(hdr[5])}, tok0[2] = {uni(hdr[4]), uni(hdr[6])};
-          const int c0 = n0 - both, c1 = n1 - both, own = max(c0, c1);
-          for (int it = 0; ok && it < own + both; ++it) {
+          const int tail = uni(hdr[7]), kvh[2] = {uni(hdr[3]), uni(hdr[5])}, tok0[2] = {uni(hdr[4]), uni(hdr[6])};
+          const int c0 = n0 - both - tail, c1 = n1 - both - tail, own = max(c0, c1);
+          for (int it = 0; ok && it < own + both + tail; ++it) {
             ok = pend(0);
             if (ok && it >= own - c0) {
               pend_tok[0] = tok0[0] + uni((int)ent[it - (own - c0)]) * BLK;
@@ -995,8 +997,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
               ok = load(&map_k, kvh[0], pend_tok[0]);
             }
             if (ok) ok = pend(1);
-            if (ok && it >= own - c1 && it < own) {
-              pend_tok[1] = tok0[1] + uni((int)ent[n0 + it - (own - c1)]) * BLK;
+            if (ok && it >= own - c1 && (it < own || it == own + both)) {
+              pend_tok[1] = tok0[1] + uni((int)ent[n0 + (it < own ? it - (own - c1) : c1)]) * BLK;
               pend_kvh[1] = kvh[1];
               ok = load(&map_k, kvh[1], pend_tok[1]);
             }
@@ -1030,8 +1032,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     } else if (kMerge && warp == 9) {
       // ============================== list merger ==============================
       // For each pair of items, a pair ahead: the entries of slot 0's list that slot 1's does not have, then those both
-      // have; behind them the other entries of slot 1's.  Both lists have to be strictly ascending and to end on the same
-      // block (the last one is masked on the diagonal) in the same row of the same kv head; else they have nothing in common.
+      // have; behind them the other entries of slot 1's.  A list's last block stays its last (the diagonal is masked in it): if
+      // the lists end on different blocks, as those of different rows do, these follow behind the common ones (`tail`).
+      // Both lists have to be strictly ascending and of the same kv head and sequence; else they have nothing in common.
       Ctx ctx{abort_flag, status, kRoleMerge, 1};
       SlotWalk<kTok, kSplit, kPair> w[2];
       w[0].init(a, 0); w[1].init(a, 1);
@@ -1055,34 +1058,38 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         auto entry = [&](const int X, const int i) { return min(max(list[X][i], 0), r[X]); };
         uint32_t both[2] = {0u, 0u};  // bit t: entry 32 t + lane is in the other list
-        if (R[0] == R[1] && kvh[0] == kvh[1] && n[0] > 0 && n[1] > 0) {
-          bool bad = entry(0, n[0] - 1) != entry(1, n[1] - 1);
+        int tail = 0;
+        if (n[0] > 0 && n[1] > 0 && kvh[0] == kvh[1] && tok0[0] == tok0[1]) {
+          tail = entry(0, n[0] - 1) != entry(1, n[1] - 1) ? 1 : 0;
+          bool bad = false;
 #pragma unroll
           for (int X = 0; X < 2; ++X) {
 #pragma unroll 1
             for (int i = lane, t = 0; i < n[X]; i += 32, ++t) {
               const int v = entry(X, i);
               bad = bad || (i > 0 && entry(X, i - 1) >= v);
+              if (i >= n[X] - tail) continue;
               int lo = 0, hi = n[X ^ 1] - 1;  // the first entry of the other list that is not below v, or the last
               while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
                 if (entry(X ^ 1, mid) < v) lo = mid + 1; else hi = mid;
               }
-              if (entry(X ^ 1, lo) == v) both[X] |= 1u << t;
+              if (lo < n[X ^ 1] - tail && entry(X ^ 1, lo) == v) both[X] |= 1u << t;
             }
           }
           if (__any_sync(0xffffffffu, bad)) both[0] = both[1] = 0u;
         }
         const int m = __reduce_add_sync(0xffffffffu, __popc(both[0]));
+        if (m == 0) tail = 0;
         int* hdr = (int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
         uint16_t* ent = (uint16_t*)(hdr + kMergeHeader / 4);
         const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
         for (int X = 0; X < 2; ++X) {
-          int own_at = X ? n[0] : 0, both_at = n[0] - m;
+          int own_at = X ? n[0] : 0, both_at = n[0] - m - tail;
 #pragma unroll 1
           for (int i0 = 0, t = 0; i0 < n[X]; i0 += 32, ++t) {
-            const bool in = i0 + lane < n[X], shared = in && ((both[X] >> t) & 1u);
+            const bool in = i0 + lane < n[X] - tail, shared = in && ((both[X] >> t) & 1u);
             const uint32_t mo = __ballot_sync(0xffffffffu, in && !shared), mb = __ballot_sync(0xffffffffu, shared);
             if (in && !(X == 1 && shared))
               ent[shared ? both_at + __popc(mb & below) : own_at + __popc(mo & below)] = (uint16_t)entry(X, i0 + lane);
@@ -1091,6 +1098,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           }
         }
         if (lane == 0) {
+          if (tail) {
+            ent[n[0] - 1] = (uint16_t)entry(0, n[0] - 1);
+            ent[n[0] + n[1] - m - 1] = (uint16_t)entry(1, n[1] - 1);
+          }
+          hdr[7] = tail;
           hdr[0] = n[0]; hdr[1] = n[1]; hdr[2] = m;
           hdr[3] = kvh[0]; hdr[4] = tok0[0]; hdr[5] = kvh[1]; hdr[6] = tok0[1];
         }
@@ -1390,11 +1402,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const volatile int* hdr = (const volatile int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
           s0.left = uni(hdr[0]);
           s1.left = uni(hdr[1]);
-          const int both = uni(hdr[2]);
+          const int both = uni(hdr[2]), tail = uni(hdr[7]);
           if (lane == 0) mbar_arrive(bar(Smem::merge_empty, b));
           if (s0.left > 0) take_q(s0);
           if (s1.left > 0) take_q(s1);
-          const int c0 = s0.left - both, c1 = s1.left - both, own = max(c0, c1);
+          const int c0 = s0.left - both - tail, c1 = s1.left - both - tail, own = max(c0, c1);
           for (int it = 0; it < own; ++it) {
             round(it >= own - c0, it >= own - c1, false);
             if (__any_sync(0xffffffffu, failed != 0)) break;
@@ -1403,6 +1415,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             round(true, true, true);
             if (__any_sync(0xffffffffu, failed != 0)) break;
           }
+          if (tail) round(true, true, false);
           if (__any_sync(0xffffffffu, failed != 0)) break;
         }
         if (!__any_sync(0xffffffffu, failed != 0)) round(false, false, false);
@@ -1517,7 +1530,7 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
   // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
   cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
-  // Two streams of tiles are for what is left: one query head per kv head, few items, very long lists.
+  // Two streams of tiles are for what is left: few items, very long lists, the dense mode with an odd number of heads in a group.
   auto kernel = merge ? (B == 128 ? sparse_attn_kernel<128, true, false, false, true> : sparse_attn_kernel<64, true, false, false, true>)
               : pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
               : B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false, false> : sparse_attn_kernel<128, false, false, false>)

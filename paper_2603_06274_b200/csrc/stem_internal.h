@@ -59,7 +59,7 @@ struct AttnWork {
   const int32_t* d_slot_off = nullptr;  // [2 ctas + 1] first item of every slot
   int ctas = 0;
   bool pair = false;  // the slots of a CTA have two query heads of a group in the same rows, with the same lists
-  bool merge = false; // likewise, or a head and the next row's first, with lists of their own that may have blocks in common
+  bool merge = false; // the slots of a CTA have neighbours in the order of the items, whose lists may have blocks in common
 };
 
 struct Plan {

@@ -306,11 +306,12 @@ def test_lists_cut_in_halves_for_the_two_slots(rows):
 
 @pytest.mark.parametrize("block,seqlens,hq,hkv,dense", [
     (128, (37 * 128 - 5,), 4, 2, False),        # 148 items: one per SM, lists cut in halves
-    (128, (38 * 128 - 5,), 4, 2, False),        # 152 items: two query heads of a group at a time on one stream of K / V
+    (128, (38 * 128 - 5,), 4, 2, False),        # 152 items: one by one
+    (128, (48 * 128 - 5,), 4, 2, False),        # 192 items: two query heads of a group at a time on one stream of K / V
     (64, (3000, 65, 1, 1900), 6, 1, False),
     (64, (2500, 700), 16, 4, False),
-    (128, (2900, 129), 14, 2, False),           # an odd number of heads in a group: no pairs
-    (128, (38 * 128 - 5,), 4, 2, True),
+    (128, (2900, 129), 14, 2, False),           # an odd number of heads in a group: pairs by their lists
+    (128, (75 * 64,), 12, 6, True),             # 456 items: in pairs
     (64, (3000, 65, 1, 1900), 6, 1, True),
     (128, (2900, 129), 14, 2, True),
 ])
@@ -352,8 +353,9 @@ def test_heads_of_a_group_with_the_same_lists(block, seqlens, hq, hkv, dense):
 
 
 @pytest.mark.parametrize("block,seqlens,hq,hkv", [
-    (128, (37 * 128,), 8, 4),              # 296 items: each slot for itself
-    (128, (37 * 128 + 1,), 8, 4),          # 304: two heads of a group at a time, tiles that both lists name loaded once
+    (128, (23 * 128,), 8, 4),              # 184 items: each slot for itself
+    (128, (23 * 128 + 1,), 8, 4),          # 192: two heads of a group at a time, tiles that both lists name loaded once
+    (64, (64 * 40, 100), 7, 7),            # two rows of one head at a time
     (64, (2500, 700, 63), 14, 2),          # odd groups: pairs over two rows among them
     (64, (64 * 20 + 9,), 15, 3),           # an odd number of items
 ])
@@ -370,14 +372,14 @@ def test_neighbouring_heads_with_lists_in_common(block, seqlens, hq, hkv):
     idx = np.full((hq, info.total_q_blocks, info.k_max), -1, np.int32)
     cnt = np.zeros((hq, info.total_q_blocks), np.int32)
     for R, row in enumerate(row_r):
-        kind = int(r.integers(0, 8))
-        base = np.sort(r.choice(row + 1, size=int(r.integers(1, row + 2)), replace=False))
+        kind = int(r.integers(0, 9))
+        base = np.arange(1, row + 1) if kind == 8 else np.sort(r.choice(row + 1, size=int(r.integers(1, row + 2)), replace=False))
         for h in range(hq):
             own = np.sort(r.choice(row + 1, size=int(r.integers(1, row + 2)), replace=False))
             lst = base if kind < 2 else own
             if kind in (0, 2, 3):
                 lst = np.union1d(lst, [row])                                # with the diagonal block
-            elif kind == 4:
+            elif kind in (4, 8):
                 lst = np.union1d(base[r.random(len(base)) < 0.8], [row])    # much in common
             elif kind == 5:
                 lst = own[:0] if r.random() < 0.5 else np.union1d(own, [row])
