@@ -56,11 +56,15 @@ static int validate(const stem_config* c) {
   return STEM_OK;
 }
 
-// Deals the attention's items to the slots of its CTAs: in the order of `order` (rows, longest list first) for one kv head
+// Deals the attention's items to the slots of its CTAs: in the order of `order` (rows, longest list first), one kv head
 // after the other, each to the slot that is done first by the lengths of its lists, which the plan knows.  Dealt in turns,
 // the busiest of 148 SMs had 12.6 % more blocks than the mean in a dense layer of 16K tokens; so it has 1.2 %.  In turns / so,
 // dense, us: 16K tokens, 32 / 8 heads 1735 / 1614; 4K, 28 / 4 127 / 114; 9000, 8 / 2 225 / 126 (the times of sparse layers
 // differ by less than their runs do).  An item counts half a block besides its blocks.
+// Where a slot's whole work is less than three of the longest lists, the kv heads go row by row instead: the longest lists of
+// the last kv head would come too late (dense, us: 9000 tokens, 8 / 8 heads, blocks of 64 525 / 333; 4096, 28 / 4 110 / 105).
+// With more work per slot that balances itself, and a kv head at a time is better for the L2 (64K tokens, 32 / 8 heads, lists
+// of up to 51 blocks: 4.15 ms, row by row 4.45).
 // Neighbouring heads with the same lists go to the two slots of a CTA together, if there are more than `pairs_from` items:
 // few dense items do better one by one, as the longest of them share their CTAs with the shortest (3000 tokens, 8 / 2 heads,
 // 192 items: 43 us, in pairs 46); chosen lists are alike in length (29, in pairs 23).
@@ -95,33 +99,37 @@ static void deal_items(const Plan& p, const std::vector<int32_t>& order, const s
     for (int c = 0; c < w->ctas; ++c) append(0, 2 * c);
     for (int c = w->ctas - 1; c >= 0; --c) append(0, 2 * c + 1);
   }
+  // f(number, head, row) for every item: `rows` rows at a time of one kv head after the other
+  const bool by_row = total * Hq / n_slots < 3 * longest;
+  const int rows = !by_row ? p.R_tot : unit == 2 && g % 2 ? 2 : 1;
+  auto each = [&](auto f) {
+    int i = 0;
+    for (int r0 = 0; r0 < p.R_tot; r0 += rows)
+      for (int kvh = 0; kvh < Hkv; ++kvh)
+        for (int r = r0; r < std::min(r0 + rows, p.R_tot); ++r)
+          for (int q = 0; q < g; ++q, ++i) f(i, kvh * g + q, order[r]);
+  };
   std::vector<int32_t> owner(p.n_items), count(n_slots + 1, 0);
   size_t time = 0;
-  int i = 0;
   int32_t queue = 0;
-  for (int kvh = 0; kvh < Hkv; ++kvh)
-    for (const int32_t R : order)
-      for (int q = 0; q < g; ++q, ++i) {
-        if (i % unit == 0) {
-          while (first[time] < 0) ++time;
-          queue = first[time];
-          first[time] = next[queue];
-          append(time + 2 * len[R] + 1, queue);
-        }
-        owner[i] = unit * queue + i % unit;
-        ++count[owner[i] + 1];
-      }
+  each([&](int i, int, int32_t R) {
+    if (i % unit == 0) {
+      while (first[time] < 0) ++time;
+      queue = first[time];
+      first[time] = next[queue];
+      append(time + 2 * len[R] + 1, queue);
+    }
+    owner[i] = unit * queue + i % unit;
+    ++count[owner[i] + 1];
+  });
   for (int s = 0; s < n_slots; ++s) count[s + 1] += count[s];
   slot_off = count;
   items.resize(2 * (size_t)p.n_items);
-  i = 0;
-  for (int kvh = 0; kvh < Hkv; ++kvh)
-    for (const int32_t R : order)
-      for (int q = 0; q < g; ++q, ++i) {
-        const int32_t at = count[owner[i]]++;
-        items[2 * at] = kvh * g + q;
-        items[2 * at + 1] = R;
-      }
+  each([&](int i, int h, int32_t R) {
+    const int32_t at = count[owner[i]]++;
+    items[2 * at] = h;
+    items[2 * at + 1] = R;
+  });
 }
 
 template <class T>
@@ -306,7 +314,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     const int few = 5 * p.sm_count / 4;
     deal_items(p, by_len, p.k_eff, p.share_group ? few : p.n_items,
                p.k_max <= attention_merge_max_list() ? few : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
-    deal_items(p, by_r, len_dense, 3 * p.sm_count, p.n_items, &p.work_dense, work_dense, slots_dense);
+    deal_items(p, by_r, len_dense, 3 * p.sm_count, 3 * p.sm_count, &p.work_dense, work_dense, slots_dense);
   }
 
   // Workspace layout.  With a caller-owned cache the K-side tensors are not part of the workspace.

@@ -989,16 +989,21 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const int n0 = uni(hdr[0]), n1 = uni(hdr[1]), both = uni(hdr[2]);
           const int tail = uni(hdr[7]), kvh[2] = {uni(hdr[3]), uni(hdr[5])}, tok0[2] = {uni(hdr[4]), uni(hdr[6])};
           const int c0 = n0 - both - tail, c1 = n1 - both - tail, own = max(c0, c1);
+          // the i-th block of slot X: its own c, those both have, its last with `tail`; all causal blocks in the dense mode
+          auto block = [&](const int X, const int i, const int c) -> int {
+            if (dense) return i < c ? both + i : i < c + both ? i - c : c + both;
+            return uni((int)ent[X ? n0 + (i < c ? i : c) : i]);
+          };
           for (int it = 0; ok && it < own + both + tail; ++it) {
             ok = pend(0);
             if (ok && it >= own - c0) {
-              pend_tok[0] = tok0[0] + uni((int)ent[it - (own - c0)]) * BLK;
+              pend_tok[0] = tok0[0] + block(0, it - (own - c0), c0) * BLK;
               pend_kvh[0] = kvh[0];
               ok = load(&map_k, kvh[0], pend_tok[0]);
             }
             if (ok) ok = pend(1);
             if (ok && it >= own - c1 && (it < own || it == own + both)) {
-              pend_tok[1] = tok0[1] + uni((int)ent[n0 + (it < own ? it - (own - c1) : c1)]) * BLK;
+              pend_tok[1] = tok0[1] + block(1, it - (own - c1), c1) * BLK;
               pend_kvh[1] = kvh[1];
               ok = load(&map_k, kvh[1], pend_tok[1]);
             }
@@ -1053,13 +1058,18 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           kvh[X] = h / a.g;
           r[X] = a.rows.row_r[R[X]];
           tok0[X] = a.rows.seq_tok0[a.rows.row_seq[R[X]]];
-          n[X] = min(max(a.sel_cnt[row], 0), a.k_max);
-          list[X] = a.sel_idx + row * a.k_max;
+          n[X] = dense ? r[X] + 1 : min(max(a.sel_cnt[row], 0), a.k_max);
+          if (!dense) list[X] = a.sel_idx + row * a.k_max;
         }
         auto entry = [&](const int X, const int i) { return min(max(list[X][i], 0), r[X]); };
         uint32_t both[2] = {0u, 0u};  // bit t: entry 32 t + lane is in the other list
-        int tail = 0;
-        if (n[0] > 0 && n[1] > 0 && kvh[0] == kvh[1] && tok0[0] == tok0[1]) {
+        int tail = 0, m = 0;
+        if (dense) {
+          if (kvh[0] == kvh[1] && tok0[0] == tok0[1]) {  // (missing: slot 1's kv head is -1)
+            tail = r[0] != r[1] && min(r[0], r[1]) > 0 ? 1 : 0;
+            m = r[0] == r[1] ? n[0] : min(r[0], r[1]);
+          }
+        } else if (n[0] > 0 && n[1] > 0 && kvh[0] == kvh[1] && tok0[0] == tok0[1]) {
           tail = entry(0, n[0] - 1) != entry(1, n[1] - 1) ? 1 : 0;
           bool bad = false;
 #pragma unroll
@@ -1079,8 +1089,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           }
           if (__any_sync(0xffffffffu, bad)) both[0] = both[1] = 0u;
         }
-        const int m = __reduce_add_sync(0xffffffffu, __popc(both[0]));
-        if (m == 0) tail = 0;
+        if (!dense) {
+          m = __reduce_add_sync(0xffffffffu, __popc(both[0]));
+          if (m == 0) tail = 0;
+        }
         int* hdr = (int*)(smem_gen + Smem::merge_buf + b * kMergeBytes);
         uint16_t* ent = (uint16_t*)(hdr + kMergeHeader / 4);
         const uint32_t below = (1u << lane) - 1u;
@@ -1088,7 +1100,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int X = 0; X < 2; ++X) {
           int own_at = X ? n[0] : 0, both_at = n[0] - m - tail;
 #pragma unroll 1
-          for (int i0 = 0, t = 0; i0 < n[X]; i0 += 32, ++t) {
+          for (int i0 = 0, t = 0; !dense && i0 < n[X]; i0 += 32, ++t) {
             const bool in = i0 + lane < n[X] - tail, shared = in && ((both[X] >> t) & 1u);
             const uint32_t mo = __ballot_sync(0xffffffffu, in && !shared), mb = __ballot_sync(0xffffffffu, shared);
             if (in && !(X == 1 && shared))
@@ -1098,7 +1110,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           }
         }
         if (lane == 0) {
-          if (tail) {
+          if (tail && !dense) {
             ent[n[0] - 1] = (uint16_t)entry(0, n[0] - 1);
             ent[n[0] + n[1] - m - 1] = (uint16_t)entry(1, n[1] - 1);
           }
@@ -1124,7 +1136,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (!ok || w[X].done()) continue;
             const int h = uni(a.work[2 * w[X].idx]), R = uni(a.work[2 * w[X].idx + 1]);
             w[X].advance();
-            if (uni(a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R]) <= 0) continue;
+            if (!dense && uni(a.sel_cnt[(int64_t)(h / a.list_div) * a.R_tot + R]) <= 0) continue;
             const int q_tok0 = uni(a.rows.row_tok0[R]);
             if (tiles >= (uint32_t)kQBufs) ok = __all_sync(0xffffffffu, mbar_wait(bar(Smem::q_empty, buf), par ^ 1u, ctx, kBarQEmpty));
             if (!ok) continue;
@@ -1530,7 +1542,7 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
   // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
   cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
-  // Two streams of tiles are for what is left: few items, very long lists, the dense mode with an odd number of heads in a group.
+  // Two streams of tiles are for what is left: few items, and very long lists.
   auto kernel = merge ? (B == 128 ? sparse_attn_kernel<128, true, false, false, true> : sparse_attn_kernel<64, true, false, false, true>)
               : pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
               : B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false, false> : sparse_attn_kernel<128, false, false, false>)

@@ -312,8 +312,10 @@ def test_lists_cut_in_halves_for_the_two_slots(rows):
     (64, (2500, 700), 16, 4, False),
     (128, (2900, 129), 14, 2, False),           # an odd number of heads in a group: pairs by their lists
     (128, (75 * 64,), 12, 6, True),             # 456 items: in pairs
+    (64, (65 * 64, 130), 7, 7, True),           # 476 items: in pairs of rows of one head
     (64, (3000, 65, 1, 1900), 6, 1, True),
-    (128, (2900, 129), 14, 2, True),
+    (128, (2900, 129), 14, 2, True),            # 350 items: one by one
+    (128, (4300, 129), 14, 2, True),            # 504 items: pairs within and across rows
 ])
 def test_heads_of_a_group_with_the_same_lists(block, seqlens, hq, hkv, dense):
     # one list per kv head (lists of 0, 1, 2, 3 and up to all causal blocks, with and without the diagonal block), or dense
