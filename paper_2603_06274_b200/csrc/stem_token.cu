@@ -40,13 +40,13 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 // exchange between the warps.  The descent ends when all undecided keys are taken, or when so few are left that ranking
 // them against each other is cheaper (kFinish); only rows with many keys in one bin of the upper halves go on with the
 // lower ones, read again.  No histograms: shared-memory atomics take 14 cycles of the SM per warp instruction and bounded the
-// byte-wise radix selection below.  The kernel is bound by its instructions.  In us, byte-wise / all 32 planes / this: 8
-// lists of 8K tokens, top 2048: 1240 / 780 / 588 (floor by its bytes 240); scores that are zero in half of the places
-// instead of normal: this 667.  Lane l of warp w owns the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are
+// byte-wise radix selection below.  The kernel is bound by its integer instructions (pipe 78 % busy).  In us, byte-wise / all 32
+// planes / upper planes / with no idle warps (see the launch): 8 lists of 8K tokens, top 2048: 1240 / 780 / 588 / 497
+// (floor by its bytes 240); scores that are zero in half of the places instead of normal: 667 / 564.  Lane l of warp w owns the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are
 // coalesced 16-byte ones and the ascending list comes out q by q with a prefix sum over the lanes' nibbles.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPlanesMax = 16384;  // longest row
-constexpr int kFinish = 32;        // undecided keys that are ranked against each other (64: 597 us, 128: 654, 16: 587)
+constexpr int kFinish = 32;        // undecided keys that are ranked against each other (588 us; 64: 597, 128: 654, 16: 587)
 
 // The planes of 16 bits of 32 keys: in, word k = the 16 bits of key k and, above them, of key k + 16; out, word k = bit k of
 // the 32 keys (the second to fifth stage of ptx::transpose32 on one half).
@@ -216,7 +216,8 @@ token_select_planes_kernel(const float* __restrict__ scores, int N, int t_end, i
         }
         row_sync<W>();
         constexpr int kEach = kFinish > 32 * W ? kFinish / (32 * W) : 1;  // entries per thread
-        constexpr int kShare = kFinish < 32 * W ? 32 * W / kFinish : 1;   // threads per entry
+        constexpr int kShare = W >= 16 ? 16 : W >= 8 ? 8 : W >= 4 ? 4 : W >= 2 ? 2 : 1;  // threads per entry
+        static_assert(kFinish == 32, "kShare");
         const int e0 = tid / kShare, part = tid % kShare;
         unsigned long long mine[kEach];
 #pragma unroll
@@ -564,12 +565,13 @@ cudaError_t launch_token_masks(const int32_t* sel_idx, const int32_t* sel_cnt, i
 cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_max, const int32_t* k_tok, int stem, int local,
                                 int32_t* sel_idx, int32_t* sel_cnt, cudaStream_t s) {
   if (N <= kPlanesMax) {
-    // rows by length, the longest first: W warps for rows of more than 512 W (W > 1) and up to 1024 W tokens
+    // rows by length, the longest first: a warp for each 1024 tokens, two for each 2048 beyond 8192.  With powers of two alone a
+    // quarter of the warps had no keys: 8 lists of 8K tokens 588 us, so 497; 4K, top 512: 154 / 142; 2 of 12 000: 370 / 294.
     const int vec = N % 4 == 0 && ((uintptr_t)scores & 15u) == 0u;
     bool dependent = false;
-    for (int w = kPlanesMax / 1024; w >= 1; w >>= 1) {
-      const int hi = std::min(N, 1024 * w), lo = w == 1 ? 0 : 512 * w;
-      if (hi <= lo) continue;
+    auto launch = [&](auto kernel, int w, int lo) -> cudaError_t {
+      const int hi = std::min(N, 1024 * w);
+      if (hi <= lo) return cudaSuccess;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -579,12 +581,22 @@ cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_ma
       cfg.stream = s;
       cfg.attrs = attr;
       cfg.numAttrs = dependent ? 1 : 0;
-      auto kernel = w == 16 ? token_select_planes_kernel<16> : w == 8 ? token_select_planes_kernel<8>
-                    : w == 4 ? token_select_planes_kernel<4> : w == 2 ? token_select_planes_kernel<2> : token_select_planes_kernel<1>;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, scores, N, hi, k_max, k_tok, stem, local, vec, sel_idx, sel_cnt);
-      if (e != cudaSuccess) return e;
       dependent = true;
-    }
+      return cudaLaunchKernelEx(&cfg, kernel, scores, N, hi, k_max, k_tok, stem, local, vec, sel_idx, sel_cnt);
+    };
+    cudaError_t e = launch(token_select_planes_kernel<16>, 16, 14 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<14>, 14, 12 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<12>, 12, 10 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<10>, 10, 8 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<8>, 8, 7 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<7>, 7, 6 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<6>, 6, 5 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<5>, 5, 4 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<4>, 4, 3 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<3>, 3, 2 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<2>, 2, 1 * 1024);
+    if (e == cudaSuccess) e = launch(token_select_planes_kernel<1>, 1, 0);
+    if (e != cudaSuccess) return e;
     return cudaSuccess;
   }
   const dim3 grid((unsigned)N, (unsigned)H_list);

@@ -265,7 +265,8 @@ def test_token_attention_ignores_rows_no_list_names():
     (1025, 2, 1000, 0, 1, False),    # the first row of two warps; N not a multiple of four: scalar loads
     (2052, 1, 64, 1, 2, True),       # rows of two and of four warps
     (4097, 1, 2048, 0, 1, False),    # the first row of eight warps
-    (8200, 1, 500, 4, 8, True),      # rows of sixteen warps
+    (8200, 1, 500, 4, 8, True),      # rows of ten warps
+    (15000, 1, 2048, 0, 1, False),   # up to sixteen
     (16388, 1, 700, 0, 1, True),     # longer than the registers hold: the other kernel for all rows
     (1030, 2, 200, 0, 1, "low"),     # scores alike in their upper 16 bits, or in all but the last four
     (4100, 1, 900, 2, 3, "low"),
@@ -290,6 +291,7 @@ def test_token_selection_row_lengths(n, heads, k_start, stem, local, ties):
     binding.stem_token_select(sc, k_tok.cuda(), idx, cnt, stem, local)
     torch.cuda.synchronize()
     rows = sorted({0, 1, stem + local - 1, k_start - 1, k_start, n // 3, n // 2, n - 1, 1023, 1024, 2047, 2048, 4095, 4096, 8191, 8192}
+                  | {1024 * k + d for k in range(1, 17) for d in (-1, 0)}
                   | set(np.random.default_rng(n).integers(0, n, 40).tolist()))
     for h in range(heads):
         for t in [t for t in rows if 0 <= t < n]:
