@@ -79,15 +79,19 @@ static void deal_items(const Plan& p, const std::vector<int32_t>& order, const s
   const int unit = w->pair || w->merge ? 2 : 1;  // items dealt at a time
   w->ctas = std::min((p.n_items + unit - 1) / unit, p.sm_count);
   const int n_slots = 2 * w->ctas, n_queues = n_slots / unit;
-  // slots by the time they are done at, first come first served; `next` links the slots done at the same time
+  // slots by the time they are done at, first come first served, in a ring of buckets (all times lie within the longest item of
+  // the earliest); `next` links the slots done at the same time
   int64_t total = 0;
   int32_t longest = 0;
   for (int R = 0; R < p.R_tot; ++R) {
     total += 2 * len[R] + 1;
     longest = std::max(longest, 2 * len[R] + 1);
   }
-  std::vector<int32_t> first((size_t)(total * Hq / n_slots + (2 + Hkv / w->ctas) * longest + 2), -1), last(first.size(), -1), next(n_queues, -1);
-  auto append = [&](size_t time, int32_t q) {
+  uint32_t ring = 1;
+  while (ring <= (uint32_t)longest) ring <<= 1;
+  std::vector<int32_t> first(ring, -1), last(ring, -1), next(n_queues, -1);
+  auto append = [&](uint32_t time, int32_t q) {
+    time &= ring - 1;
     next[q] = -1;
     if (first[time] < 0) first[time] = q; else next[last[time]] = q;
     last[time] = q;
@@ -110,16 +114,16 @@ static void deal_items(const Plan& p, const std::vector<int32_t>& order, const s
           for (int q = 0; q < g; ++q, ++i) f(i, kvh * g + q, order[r]);
   };
   std::vector<int32_t> owner(p.n_items), count(n_slots + 1, 0);
-  size_t time = 0;
+  uint32_t time = 0;
   int32_t queue = 0;
   each([&](int i, int, int32_t R) {
-    if (i % unit == 0) {
-      while (first[time] < 0) ++time;
+    if ((i & (unit - 1)) == 0) {
+      while (first[time] < 0) time = (time + 1) & (ring - 1);
       queue = first[time];
       first[time] = next[queue];
       append(time + 2 * len[R] + 1, queue);
     }
-    owner[i] = unit * queue + i % unit;
+    owner[i] = unit * queue + (i & (unit - 1));
     ++count[owner[i] + 1];
   });
   for (int s = 0; s < n_slots; ++s) count[s + 1] += count[s];
