@@ -42,8 +42,9 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 // lower ones, read again.  No histograms: shared-memory atomics take 14 cycles of the SM per warp instruction and bounded the
 // byte-wise radix selection below.  The kernel is bound by its integer instructions (pipe 78 % busy).  In us, byte-wise / all 32
 // planes / upper planes / with no idle warps (see the launch): 8 lists of 8K tokens, top 2048: 1240 / 780 / 588 / 487
-// (floor by its bytes 240); scores that are zero in half of the places instead of normal: 667 / 553.  Lane l of warp w owns the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are
-// coalesced 16-byte ones and the ascending list comes out q by q with a prefix sum over the lanes' nibbles.
+// (floor by its bytes 240); scores that are zero in half of the places instead of normal: 667 / 553.  Lane l of warp w owns
+// the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are coalesced 16-byte ones and the ascending list comes out q
+// by q with a prefix sum over the lanes' nibbles.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPlanesMax = 16384;  // longest row
 constexpr int kFinish = 32;        // undecided keys that are ranked against each other (588 us; 64: 597, 128: 654, 16: 587)
