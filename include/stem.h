@@ -288,6 +288,11 @@ int stem_token_attention(const void* Q, const void* K, const void* V, int32_t n_
                          int64_t kv_stride_head, const int32_t* sel_idx, const int32_t* sel_cnt, int32_t k_max,
                          float softmax_scale, void* O, float* lse, void* stream);
 
+/* Which form stem_token_attention takes at these sizes on the current device: 0 gathers every list's rows, 1 computes
+ * every causal key block and masks what the lists do not name (k_max stands for the lists' lengths); negative: STEM_ERR_*.
+ * Host only. */
+int stem_token_attention_form(int32_t n_tokens, int32_t num_q_heads, int32_t num_kv_heads, int32_t k_max);
+
 /* Synchronises `stream`, then reads (and clears, if set) the status words of the gather-attention kernel on the
  * current device.  Returns STEM_OK, STEM_ERR_DEVICE_TIMEOUT (a bounded wait in stem_token_attention gave up; the
  * outputs of that call are undefined) or STEM_ERR_CUDA.  detail (optional, HOST int32[4]) receives

@@ -673,6 +673,17 @@ int stem_token_attention(const void* Q, const void* K, const void* V, int32_t n_
                                         num_kv_heads, k_max, sel_idx, sel_cnt, scale, O, lse, (cudaStream_t)stream));
 }
 
+int stem_token_attention_form(int32_t n_tokens, int32_t num_q_heads, int32_t num_kv_heads, int32_t k_max) {
+  if (n_tokens < 1 || num_q_heads < 1 || num_kv_heads < 1 || k_max < 1) return STEM_ERR_INVALID_ARG;
+  if (num_q_heads % num_kv_heads != 0 || num_q_heads / num_kv_heads > token_attn_max_group()) return STEM_ERR_UNSUPPORTED;
+  int device = 0, sms = 0;
+  if (cudaGetDevice(&device) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return STEM_ERR_CUDA;
+  }
+  return token_masked_is_cheaper(n_tokens, num_kv_heads, num_q_heads / num_kv_heads, k_max, sms) ? 1 : 0;
+}
+
 int stem_token_check_status(void* stream, int32_t* detail) {
   if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
   int32_t words[4] = {0, 0, 0, 0};

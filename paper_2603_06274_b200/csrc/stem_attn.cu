@@ -1565,7 +1565,7 @@ static int64_t mask_bytes_of(int b) { return (int64_t)((b + kTileM - 1) / kTileM
 // Measured gather / masked in us: 8192 tokens, 32/8 heads, top 2048: 6440 / 609; 12000, 32/2, 1024: 1877 / 1025;
 // 12000, 8/2, 256: 448 / 425; 12000, 8/2, 128: 337 / 422; 12000, 32/2, 256: 881 / 1004; 12000, 2/2, 128: 306 / 715 (ten
 // launches); 512, 4/1, 128: 15.5 / 21.8.
-static bool masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count) {
+bool token_masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count) {
   const double sms = sm_count, k = std::min(k_max, N);
   const double gather = 8.0 + (double)N * Hkv / sms * (0.7 + 0.14 * g + 1.05 * std::max(1.0, k / kTileM * (1.0 - 0.5 * k / N)));
   double masked = 0.0;
@@ -1594,7 +1594,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
                                 void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s) {
   *taken = false;
   const int g = Hq / Hkv, tile = kTileM / g;
-  if (!masked_is_cheaper(N, Hkv, g, k_max, sm_count)) return cudaSuccess;
+  if (!token_masked_is_cheaper(N, Hkv, g, k_max, sm_count)) return cudaSuccess;
   CUtensorMap mq, mk, mv;
   if (!make_map(&mq, Q, N, Hq, q_st, q_sh, tile, g) || !make_map(&mk, K, N, Hkv, kv_st, kv_sh, kTileM) ||
       !make_map(&mv, V, N, Hkv, kv_st, kv_sh, kTileM))

@@ -161,6 +161,7 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
 cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
                                 int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
                                 void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s);
+bool token_masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count);
 cudaError_t masked_status_words(int32_t* out4);
 // Bit masks of the token lists of query tokens t0 .. t1 - 1: bit x of the mask of (token t, kv head h), at
 // masks + (t - t0) st + h sh bytes, says whether the list names token x <= t; whole 128-key blocks up to that

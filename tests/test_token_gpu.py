@@ -212,6 +212,7 @@ def _plain_attention(q, k, v, idx, cnt, rows):
     (300, 5, 1, 27, "any", True, "gather, lists in any order and with repeats"),
 ])
 def test_token_attention_forms(n, hq, hkv, k_max, order, repeat, what):
+    assert what.startswith(binding.stem_token_attention_form(n, hq, hkv, k_max))
     r = np.random.default_rng(n + k_max)
     w = wl.small("token_forms", seqlens=(n,), hq=hq, hkv=hkv, block=64, permille=100, sink=True, seed=n)
     data = wl.make_qkv(w)
