@@ -361,13 +361,8 @@ struct AttnArgs {
   int tok_tile;             // query tokens of an item: as many as give at most 128 rows (tokens x query heads of a group)
   const unsigned char* masks;            // token t, kv head h: bit mask of its list at masks + (t - tok_a) mask_st + h mask_sh
   int64_t mask_st, mask_sh;
+  TokenRedo* redo;
   float scale_log2;
-};
-
-// kTok: the tensors themselves, for the rows that exact_token_row computes.
-struct TokRows {
-  const __nv_bfloat16 *Q, *K, *V;
-  int64_t q_st, q_sh, kv_st, kv_sh;
 };
 
 // kTok: item i is (kv head, tile of query tokens), the longest prefixes first; n = key blocks up to its last token.  kPair:
@@ -511,57 +506,10 @@ struct LengthCursor {
   }
 };
 
-// One output row of the token-list form straight from its definition, for the rows the masked form cannot do: a list
-// with the same token twice (a mask holds it once), or a row that met a non-finite value (0 times a V row that the list
-// does not name).  One thread, fp32; four passes over the output columns keep it small.
-__device__ __noinline__ void exact_token_row(float scale_log2, const __nv_bfloat16* K, const __nv_bfloat16* V, const __nv_bfloat16* q,
-                                             int64_t kv_st, const int32_t* list, int n, int t, __nv_bfloat16* o, float* lse) {
-  auto score = [&](int i) -> float {
-    const __nv_bfloat16* k = K + (int64_t)min(max(list[i], 0), t) * kv_st;
-    float acc = 0.f;
-#pragma unroll 1
-    for (int c = 0; c < kHeadDim; c += 8) {
-      const uint4 kv = *(const uint4*)(k + c), qv = *(const uint4*)(q + c);
-      const uint32_t kw[4] = {kv.x, kv.y, kv.z, kv.w}, qw[4] = {qv.x, qv.y, qv.z, qv.w};
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        acc = fmaf(__uint_as_float(qw[w] << 16), __uint_as_float(kw[w] << 16), acc);
-        acc = fmaf(__uint_as_float(qw[w] & 0xffff0000u), __uint_as_float(kw[w] & 0xffff0000u), acc);
-      }
-    }
-    return acc * scale_log2;
-  };
-  float m = -INFINITY, l = 0.f;
-#pragma unroll 1
-  for (int i = 0; i < n; ++i) m = fmaxf(m, score(i));
-#pragma unroll 1
-  for (int c0 = 0; c0 < kHeadDim; c0 += 32) {
-    float acc[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) acc[c] = 0.f;
-    l = 0.f;
-#pragma unroll 1
-    for (int i = 0; i < n; ++i) {
-      const float p = fast_exp2(score(i) - m);
-      l += p;
-      const __nv_bfloat16* v = V + (int64_t)min(max(list[i], 0), t) * kv_st + c0;
-#pragma unroll
-      for (int c = 0; c < 32; c += 2) {
-        const uint32_t w = *(const uint32_t*)(v + c);
-        acc[c] = fmaf(p, __uint_as_float(w << 16), acc[c]);
-        acc[c + 1] = fmaf(p, __uint_as_float(w & 0xffff0000u), acc[c + 1]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 32; c += 2) *(uint32_t*)(o + c0 + c) = pack_bf16(acc[c] / l, acc[c + 1] / l);
-  }
-  if (lse) *lse = (m + log2f(l)) * 0.6931471805599453f;
-}
-
 template <int BLK, bool kSpareQ, bool kTok, bool kPair, bool kMerge = false>
 __global__ void __launch_bounds__(kThreads, 1)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const AttnArgs a, const TokRows tok) {
+                   const __grid_constant__ CUtensorMap map_v, const AttnArgs a) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = ((uint32_t)__cvta_generic_to_shared(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem_gen = smem_raw + (smem_base - (uint32_t)__cvta_generic_to_shared(smem_raw));
@@ -627,6 +575,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   // Launched as a programmatic dependent of the selection, everything above overlaps its tail; lists, Q, K, V and O are
   // touched only below.  (Without that launch attribute this is a no-op.)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (kTok) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the gather kernel for the marked rows
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -700,13 +649,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         n = (int)(info & 0x3fffffffu);
       }
       const bool row_valid = m < ntok;
-      // kTok: the row's mask, its list's length, and how many tokens of it the mask has shown
+      // kTok: the row's mask, and how many tokens of its list the mask has not shown yet (kNoList: the list is empty)
       const int t_row = q_tok0 + m;
       const uint4* mask = nullptr;
-      int list_n = 0, seen = 0;
+      constexpr int kNoList = -1;
+      int unseen = kNoList;
       if constexpr (kTok) {
         if (row_valid) {
-          list_n = min(max(a.sel_cnt[(int64_t)R * a.T + t_row], 0), min(a.k_max, t_row + 1));
+          unseen = min(a.sel_cnt[(int64_t)R * a.T + t_row], min(a.k_max, t_row + 1));
+          if (unseen <= 0) unseen = kNoList;
           mask = (const uint4*)(a.masks + (t_row - a.tok_a) * a.mask_st + R * a.mask_sh);
         }
       }
@@ -724,8 +675,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       for (int e = 0; e < n; ++e, ++blk) {
         uint4 mask_w = make_uint4(0, 0, 0, 0);  // kTok: the block's mask words, here while S is still awaited
         if constexpr (kTok) {
-          if (row_valid) mask_w = mask[e];
-          seen += __popc(mask_w.x) + __popc(mask_w.y) + __popc(mask_w.z) + __popc(mask_w.w);
+          if (row_valid) mask_w = *mask++;
+          unseen -= __popc(mask_w.x) + __popc(mask_w.y) + __popc(mask_w.z) + __popc(mask_w.w);
         }
         // S of block e is complete; so is every earlier tensor-core operation of this slot,
         // P V of block e-1 included (the commit behind Q K^T covers all earlier operations)
@@ -865,8 +816,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           continue;
         }
       }
-      const float inv_l = (kTok && list_n == 0) ? 0.f : 1.f / l_run;
-      float finite = 0.f;  // kTok: turns NaN with the first value that is not finite
+      const float inv_l = (kTok && unseen == kNoList) ? 0.f : 1.f / l_run;
       const bool o_al32 = ((uintptr_t)a.O & 31u) == 0u;  // rows are multiples of 256 bytes apart
       __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
 #pragma unroll
@@ -886,7 +836,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           for (int q = 0; q < 16; ++q) w[q] = pack_bf16(o[2 * q] * inv_l, o[2 * q + 1] * inv_l);
           if constexpr (kTok) {
 #pragma unroll
-            for (int q = 0; q < 32; ++q) finite = fmaf(o[q], 0.f, finite);
+            for (int q = 0; q < 32; ++q) l_run = fmaf(o[q], 0.f, l_run);  // NaN from the first value on that is not finite
           }
           if (o_al32) {
             // whole 32-byte sectors per store: a thread writes its own 256-byte row, so the stores of
@@ -901,14 +851,18 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
       }
       if (a.lse && row_valid)
-        a.lse[(int64_t)h * a.T + q_tok0 + m] = (kTok && list_n == 0) ? -INFINITY : (m_run + log2f(l_run)) * 0.6931471805599453f;
+        a.lse[(int64_t)h * a.T + q_tok0 + m] = (kTok && unseen == kNoList) ? -INFINITY : (m_run + log2f(l_run)) * 0.6931471805599453f;
       if constexpr (kTok) {
-        if (row_valid && list_n > 0 && (seen != list_n || !(finite == 0.f && l_run < INFINITY)))
-          exact_token_row(a.scale_log2, tok.K + R * tok.kv_sh, tok.V + R * tok.kv_sh, tok.Q + (int64_t)t_row * tok.q_st + h * tok.q_sh, tok.kv_st, a.sel_idx + ((int64_t)R * a.T + t_row) * a.k_max,
-                          list_n, t_row, o_row, a.lse ? a.lse + (int64_t)h * a.T + t_row : nullptr);
-        else if (row_valid && list_n == 0)
+        // Rows that the masks cannot do are left to the gather kernel behind this one: a list that names a token twice (a mask
+        // holds it once), or a value that is not finite (0 times a V row that the list does not name).
+        const bool redo = row_valid && unseen != kNoList && (unseen != 0 || !(l_run < INFINITY));
+        if (redo) {
+          *(uint32_t*)o_row = kTokenRedoMark;
+          asm volatile("red.global.add.u64 [%0], 1;" ::"l"(&a.redo->marked) : "memory");
+        } else if (row_valid && unseen == kNoList) {
 #pragma unroll
           for (int c = 0; c < 16; ++c) *(uint4*)(o_row + c * 8) = make_uint4(0, 0, 0, 0);
+        }
         __syncwarp();
       }
       ++ord;
@@ -1547,7 +1501,7 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
               : pair ? (B == 128 ? sparse_attn_kernel<128, false, false, true> : sparse_attn_kernel<64, false, false, true>)
               : B == 128 ? (spare_q ? sparse_attn_kernel<128, true, false, false> : sparse_attn_kernel<128, false, false, false>)
                          : (spare_q ? sparse_attn_kernel<64, true, false, false> : sparse_attn_kernel<64, false, false, false>);
-  return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, a, TokRows{});
+  return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, a);
 }
 
 // The masks of the query tokens below b need mask_bytes each: from which token on they are computed in one launch.
@@ -1591,7 +1545,7 @@ bool token_masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count) {
 // room for their masks in the rows of the tokens before them.
 cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
                                 int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
-                                void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s) {
+                                void* O, float* lse, TokenRedo* redo, int device, int sm_count, bool* taken, cudaStream_t s) {
   *taken = false;
   const int g = Hq / Hkv, tile = kTileM / g;
   if (!token_masked_is_cheaper(N, Hkv, g, k_max, sm_count)) return cudaSuccess;
@@ -1603,9 +1557,8 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
   AttnArgs a{};
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt;
   a.O = (__nv_bfloat16*)O; a.lse = lse; a.status = nullptr;
-  a.Hq = Hq; a.g = g; a.k_max = k_max; a.T = N; a.list_div = g; a.n_kvh = Hkv; a.tok_tile = tile;
+  a.Hq = Hq; a.g = g; a.k_max = k_max; a.T = N; a.list_div = g; a.n_kvh = Hkv; a.tok_tile = tile; a.redo = redo;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
-  const TokRows tok{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, q_st, q_sh, kv_st, kv_sh};
   static bool attr_set[64] = {};
   if (!attr_set[device & 63]) {
     cudaError_t e = cudaFuncSetAttribute(sparse_attn_kernel<128, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
@@ -1631,7 +1584,7 @@ cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int
     cudaError_t e = launch_token_masks(sel_idx, sel_cnt, N, Hkv, k_max, a.tok_a, b, pair ? 2 * tile : tile, O, a.mask_st, a.mask_sh, s);
     if (e != cudaSuccess) return e;
     auto kernel = pair ? sparse_attn_kernel<128, false, true, true> : sparse_attn_kernel<128, false, true, false>;
-    kernel<<<std::min(pair ? a.n_items / 2 : a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a, tok);
+    kernel<<<std::min(pair ? a.n_items / 2 : a.n_items, sm_count), kThreads, kSmemBytes, s>>>(mq, mk, mv, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

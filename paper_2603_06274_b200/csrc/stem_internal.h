@@ -149,6 +149,15 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
                                     const int32_t* sel_idx, const int32_t* sel_cnt, bool list_group, void* O, float* lse,
                                     int32_t* status, bool dependent, cudaStream_t s);
 
+// Rows of O that the masked form of the token attention marked, and those of them that the gather kernel has taken up, over
+// all calls on a device.  Nothing resets them, so calls on several streams need no order: the rows of a call are counted in
+// `marked` before its gather kernel starts, so that equal counts, read in one access, tell it that none of them is its to do.
+struct alignas(16) TokenRedo {
+  unsigned long long marked, redone;
+};
+// Two bf16 NaNs with a payload that no conversion yields (those give 0x7fff).
+constexpr uint32_t kTokenRedoMark = 0xffa1ffa1u;
+
 // Token-level selection and gather attention (one sequence; lists per kv head).
 int token_attn_max_group();
 cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_max, const int32_t* k_tok, int stem, int local,
@@ -158,9 +167,11 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
                                    const int32_t* sel_cnt, float softmax_scale, void* O, float* lse, cudaStream_t s);
 // The same attention with every causal key block computed and masked by the lists (stem_attn.cu); *taken = false (and nothing
 // enqueued) where the gather form is the better one.
+// Rows that a mask cannot express carry kTokenRedoMark in their first four bytes afterwards and are counted in redo->marked;
+// launch_token_attention has the gather kernel compute them.
 cudaError_t launch_token_masked(const void* Q, const void* K, const void* V, int64_t q_st, int64_t q_sh, int64_t kv_st, int64_t kv_sh,
                                 int N, int Hq, int Hkv, int k_max, const int32_t* sel_idx, const int32_t* sel_cnt, float softmax_scale,
-                                void* O, float* lse, int device, int sm_count, bool* taken, cudaStream_t s);
+                                void* O, float* lse, TokenRedo* redo, int device, int sm_count, bool* taken, cudaStream_t s);
 bool token_masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count);
 cudaError_t masked_status_words(int32_t* out4);
 // Bit masks of the token lists of query tokens t0 .. t1 - 1: bit x of the mask of (token t, kv head h), at

@@ -53,7 +53,9 @@ constexpr int kPvBars = 4;
 constexpr int kNumBars = 3 * kStages + 3 * kSBuf + 2 + kPvBars + 1;
 constexpr int kOffTmem = kOffBars + kNumBars * 8;
 constexpr int kOffAbort = kOffTmem + 8;
-constexpr int kSmemBytes = kOffAbort + 8 + 1024;  // slack for manual 1024-byte alignment
+constexpr int kRedoItems = 8192;          // items of a CTA in a launch that looks for marked rows
+constexpr int kOffRedo = kOffAbort + 8;   // a bit for each
+constexpr int kSmemBytes = kOffRedo + kRedoItems / 8 + 1024;  // slack for manual 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 static_assert(kPvBars > kStages, "a P V completion barrier must never be a phase behind its waiter");
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;
@@ -65,6 +67,7 @@ constexpr int kRoleSoftmax = 0, kRoleCopy = 1, kRoleMma = 2;
 enum : int { kBarKFull = 0, kBarVFull, kBarEmpty, kBarSFull, kBarPReady, kBarRed, kBarSum, kBarPvDone, kBarOFree, kBarDrain /* the issuing warp's poll */ };
 
 __device__ int32_t g_token_status[4];
+__device__ TokenRedo g_token_redo;
 
 struct TokArgs {
   const __nv_bfloat16 *Q, *K, *V;
@@ -73,7 +76,9 @@ struct TokArgs {
   const int32_t* sel_idx;
   const int32_t* sel_cnt;
   int64_t q_st, q_sh, kv_st, kv_sh;
-  int N, Hq, Hkv, G, k_max, n_items;
+  int N, Hq, Hkv, G, k_max;
+  int item0, n_items;  // the items item0 .. n_items - 1
+  TokenRedo* redo;     // not null: of these, the ones with a row of O that carries kTokenRedoMark
   float scale_log2;
 };
 
@@ -161,6 +166,47 @@ token_attn_tc_kernel(const TokArgs a) {
   const uint32_t o_free = bars + 8 * (3 * kStages + 3 * kSBuf + 2 + kPvBars);
   volatile int* abort_flag = (volatile int*)(smem_gen + kOffAbort);
 
+  // Behind the masked form only the marked rows are wanted, as a rule none: then the launch is as long as one load (0.5 us of a
+  // call).  The bits are found once, by all threads together; an item is computed for all heads of its group.  With a row to
+  // a thread of the masked kernel instead, 1000 tokens at 64 / 8 heads with a repeat in every list took 18 ms, here 0.38 (in one
+  // list of 100: 4.5, 0.09), and long lists outlasted the bounded waits of that kernel's other warps.
+  uint32_t* const redo_bits = (uint32_t*)(smem_gen + kOffRedo);
+  if (a.redo) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int any = 0;
+    if (threadIdx.x == 0) {
+      unsigned long long marked, redone;  // in one access
+      asm volatile("{\n\t.reg .b128 c;\n\tld.relaxed.gpu.global.b128 c, [%2];\n\tmov.b128 {%0, %1}, c;\n\t}" : "=l"(marked), "=l"(redone) : "l"(a.redo) : "memory");
+      any = marked != redone;
+    }
+    for (int w = threadIdx.x; w < kRedoItems / 32; w += kThreads) redo_bits[w] = 0u;
+    if (!__syncthreads_or(any)) return;
+    int mine = 0;
+    for (int l = threadIdx.x; l < kRedoItems; l += kThreads) {
+      const int64_t i = (int64_t)a.item0 + blockIdx.x + (int64_t)l * gridDim.x;
+      if (i >= a.n_items) break;
+      const int64_t t = a.N - 1 - i / a.Hkv, kvh = i % a.Hkv;
+      int marked = 0;
+      for (int h = 0; h < a.G; ++h) marked += __ldcg((const uint32_t*)(a.O + (t * a.Hq + kvh * a.G + h) * kHeadDim)) == kTokenRedoMark ? 1 : 0;
+      if (marked) {
+        atomicOr(&redo_bits[l >> 5], 1u << (l & 31));
+        mine += marked;
+      }
+    }
+    if (mine) atomicAdd(&a.redo->redone, (unsigned long long)mine);
+    if (!__syncthreads_or(mine)) return;
+  }
+  // the first item of this CTA at or behind its item i that is to be computed
+  auto from_item = [&](int i) -> int {
+    if (!a.redo) return i;
+    for (uint32_t l = (uint32_t)(i - a.item0) / gridDim.x; l < kRedoItems; l = (l | 31u) + 1u) {
+      const uint32_t w = redo_bits[l >> 5] >> (l & 31u);
+      if (w != 0u) return a.item0 + (int)(blockIdx.x + (l + (uint32_t)__ffs((int)w) - 1u) * gridDim.x);
+    }
+    return a.n_items;
+  };
+  const int first = a.item0 + (int)blockIdx.x;
+
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(k_full(s), 128); mbar_init(v_full(s), 128); mbar_init(empty(s), 1); }  // full: an arrival per copying thread
     for (int b = 0; b < kSBuf; ++b) { mbar_init(s_full(b), 1); mbar_init(p_ready(b), 4); mbar_init(red_bar(b), 4); }
@@ -203,7 +249,7 @@ token_attn_tc_kernel(const TokArgs a) {
     uint32_t gs = 0;   // tiles so far
     uint32_t ord = 0;  // non-empty items so far
     bool ok = true;
-    for (int i = blockIdx.x; i < a.n_items && ok; i += gridDim.x) {
+    for (int i = from_item(first); i < a.n_items && ok; i = from_item(i + gridDim.x)) {
       int t, kvh, n;
       item_of(i, t, kvh, n);
       if (n == 0) {
@@ -323,20 +369,21 @@ token_attn_tc_kernel(const TokArgs a) {
     bool ok = true;
     // the list entry of this thread's row in the next tile is fetched one tile ahead
     auto first_item = [&](int from, int& t, int& kvh, int& n) -> int {
-      int i = from;
-      for (; i < a.n_items; i += gridDim.x) {
+      int i = from_item(from);
+      for (; i < a.n_items; i = from_item(i + gridDim.x)) {
         item_of(i, t, kvh, n);
         if (n > 0) break;
       }
       return i;
     };
     int t = 0, kvh = 0, n = 0;
-    int i = first_item(blockIdx.x, t, kvh, n);
+    int i = first_item(first, t, kvh, n);
     int ti = 0;
     auto row_of = [&](int t_, int kvh_, int n_, int ti_) -> int {
-      const int e = ti_ * kKeys + pw * 32 + lane;
-      // past the end of the list: the query token itself (a valid row; its probability is masked to zero)
-      return e < n_ ? min(max(a.sel_idx[((int64_t)kvh_ * a.N + t_) * a.k_max + e], 0), t_) : t_;
+      // past the end of the list: its last entry again (the probability is masked to zero, which a row that the list does not
+      // name could still turn into NaN)
+      const int e = min(ti_ * kKeys + pw * 32 + lane, n_ - 1);
+      return min(max(a.sel_idx[((int64_t)kvh_ * a.N + t_) * a.k_max + e], 0), t_);
     };
     int row = i < a.n_items ? row_of(t, kvh, n, 0) : 0;
     while (i < a.n_items && ok) {
@@ -398,7 +445,7 @@ token_attn_tc_kernel(const TokArgs a) {
       uint32_t g, ord;
     };
     auto seek = [&](Cursor& c) {  // to the first non-empty item at or behind c.i
-      for (; c.i < a.n_items; c.i += gridDim.x) {
+      for (c.i = from_item(c.i); c.i < a.n_items; c.i = from_item(c.i + gridDim.x)) {
         int t, kvh;
         item_of(c.i, t, kvh, c.n);
         if (c.n > 0) break;
@@ -414,7 +461,7 @@ token_attn_tc_kernel(const TokArgs a) {
         seek(c);
       }
     };
-    Cursor cq{(int)blockIdx.x, 0, 0, 0, 0u, 0u};
+    Cursor cq{first, 0, 0, 0, 0u, 0u};
     seek(cq);
     Cursor cp = cq;
     bool ok = true;
@@ -498,9 +545,6 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  bool taken = false;
-  e = launch_token_masked(Q, K, V, q_st, q_sh, kv_st, kv_sh, N, Hq, Hkv, k_max, sel_idx, sel_cnt, softmax_scale, O, lse, dev, sms, &taken, s);
-  if (e != cudaSuccess || taken) return e;
   if (!attr_set[dev & 63]) {
     e = cudaFuncSetAttribute(token_attn_tc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(token_attn_tc_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
@@ -508,6 +552,12 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
     if (e != cudaSuccess) return e;
     attr_set[dev & 63] = true;
   }
+  TokenRedo* redo = nullptr;
+  e = cudaGetSymbolAddress((void**)&redo, g_token_redo);
+  if (e != cudaSuccess) return e;
+  bool masked = false;
+  e = launch_token_masked(Q, K, V, q_st, q_sh, kv_st, kv_sh, N, Hq, Hkv, k_max, sel_idx, sel_cnt, softmax_scale, O, lse, redo, dev, sms, &masked, s);
+  if (e != cudaSuccess) return e;
   TokArgs a{};
   a.Q = (const __nv_bfloat16*)Q;
   a.K = (const __nv_bfloat16*)K;
@@ -518,13 +568,26 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
   a.sel_cnt = sel_cnt;
   a.q_st = q_st; a.q_sh = q_sh; a.kv_st = kv_st; a.kv_sh = kv_sh;
   a.N = N; a.Hq = Hq; a.Hkv = Hkv; a.G = Hq / Hkv; a.k_max = k_max;
-  a.n_items = N * Hkv;
   a.scale_log2 = softmax_scale * 1.4426950408889634f;
-  const int grid = std::min(a.n_items, sms);
-  if (a.G <= 4) token_attn_tc_kernel<4><<<grid, kThreads, kSmemBytes, s>>>(a);
-  else if (a.G <= 8) token_attn_tc_kernel<8><<<grid, kThreads, kSmemBytes, s>>>(a);
-  else token_attn_tc_kernel<16><<<grid, kThreads, kSmemBytes, s>>>(a);
-  return cudaGetLastError();
+  a.redo = masked ? redo : nullptr;
+  // all items, or behind the masked form those with marked rows, looked for among as many at a time as a CTA has bits for
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = masked ? 1 : 0;
+  const int64_t all = (int64_t)N * Hkv, step = masked ? (int64_t)kRedoItems * sms : all;
+  for (int64_t i = 0; i < all && e == cudaSuccess; i += step) {
+    a.item0 = (int)i;
+    a.n_items = (int)std::min(i + step, all);
+    cfg.gridDim = dim3((unsigned)std::min(a.n_items - a.item0, sms));
+    e = cudaLaunchKernelEx(&cfg, a.G <= 4 ? token_attn_tc_kernel<4> : a.G <= 8 ? token_attn_tc_kernel<8> : token_attn_tc_kernel<16>, a);
+  }
+  return e;
 }
 
 // Reads (and clears) the status words of the gather-attention kernel after the caller synchronised the stream.

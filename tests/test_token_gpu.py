@@ -307,3 +307,88 @@ def test_token_selection_row_lengths(n, heads, k_start, stem, local, ties):
             assert int(cnt[h, t]) == len(ref)
             assert np.array_equal(got[:len(ref)], ref), (h, t)
             assert (got[len(ref):] == -1).all()
+
+
+def _random_lists(r, n, hkv, k_max):
+    """Full lists (min(t + 1, k_max) tokens) in random order."""
+    idx = np.full((hkv, n, k_max), -1, np.int32)
+    for h in range(hkv):
+        for t in range(n):
+            m = min(t + 1, k_max)
+            idx[h, t, :m] = r.permutation(t + 1)[:m]
+    return idx, np.broadcast_to(np.minimum(np.arange(n) + 1, k_max).astype(np.int32), (hkv, n)).copy()
+
+
+# The masked form leaves the rows that a mask cannot express to the gather kernel: lists that name a token twice, and every
+# row behind a value that is not finite.  Long lists, where one thread to a row would outlast the bounded waits.
+@pytest.mark.parametrize("what", ["a token named twice by every 97th list", "by every list", "an infinite value row"])
+def test_rows_that_a_mask_cannot_express_at_long_lists(what):
+    n, hq, hkv, k_max = 8300, 4, 2, 8192
+    assert binding.stem_token_attention_form(n, hq, hkv, k_max) == "masked"
+    r = np.random.default_rng(83)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(83)
+    q, k, v = (torch.randn((n, h, 128), generator=g, device="cuda").to(torch.bfloat16) for h in (hq, hkv, hkv))
+    idx, cnt = _random_lists(r, n, hkv, k_max)
+    step = 97 if "97" in what else 1
+    bad = 5
+    if "infinite" in what:
+        v[bad, 0] = float("inf")                       # of kv head 0 alone
+        for t in range(8193, n, 2):                    # lists without this token, in its place one that they did not name
+            if (idx[0, t] == bad).any():
+                idx[0, t][idx[0, t] == bad] = np.setdiff1d(np.arange(t + 1), idx[0, t])[0]
+    else:
+        idx[:, 1::step, 0] = idx[:, 1::step, 1]
+    outs = []
+    for _ in range(2):
+        out = torch.full((n, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((hq, n), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_token_attention(q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out, lse)
+        st, detail = binding.stem_token_check_status()
+        assert st == 0, detail
+        outs.append((out, lse))
+    assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16))
+    got, got_lse = from_dev_bf16(outs[0][0]), outs[0][1].cpu().numpy()
+    toks = sorted({0, 1, 2, 96, 97, 98, 127, 128, 4095, 4096, 8191, 8192, n - 2, n - 1, *r.integers(0, n, 60).tolist(), *range(8193, n, 7)})
+    rows = [(h, t) for h in range(hq) for t in toks]
+    named = {(h, t): "infinite" in what and h < 2 and bool((idx[0, t, :cnt[0, t]] == bad).any()) for h, t in rows}
+    clean = [x for x in rows if not named[x]]
+    O_ref, lse_ref = _plain_attention(from_dev_bf16(q), from_dev_bf16(k), from_dev_bf16(v), idx, cnt, clean)
+    ref = np.stack([O_ref[x] for x in clean])
+    check_attention(np.stack([got[t, h] for h, t in clean]), ref, np.ones(ref.shape, bool), label=what)
+    assert max(abs(got_lse[h, t] - lse_ref[h, t]) for h, t in clean) < 1e-3
+    if "infinite" in what:
+        assert any(t > bad and h < 2 for h, t in clean) and any(named.values())
+        assert all(not np.isfinite(got[t, h]).any() for h, t in rows if named[h, t])
+    else:
+        assert np.isfinite(got).all()
+
+
+def test_marked_rows_over_several_launches_and_streams():
+    # masks in rows of earlier tokens (two launches) with repeats; calls without marked rows on another stream meanwhile
+    n, hq, hkv, k_max = 2049, 4, 4, 512
+    assert binding.stem_token_attention_form(n, hq, hkv, k_max) == "masked"
+    r = np.random.default_rng(12)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(12)
+    q, k, v = (torch.randn((n, h, 128), generator=g, device="cuda").to(torch.bfloat16) for h in (hq, hkv, hkv))
+    lists = {rep: _lists(r, n, hkv, k_max, "any", rep) for rep in (False, True)}
+    dev = {rep: tuple(torch.from_numpy(x).cuda() for x in lists[rep]) for rep in lists}
+    outs = {rep: [torch.full((n, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(6)] for rep in lists}
+    streams = {rep: torch.cuda.Stream() for rep in lists}
+    torch.cuda.synchronize()
+    for i in range(6):
+        for rep in lists:
+            with torch.cuda.stream(streams[rep]):
+                binding.stem_token_attention(q, k, v, *dev[rep], outs[rep][i])
+    torch.cuda.synchronize()
+    st, detail = binding.stem_token_check_status()
+    assert st == 0, detail
+    for rep, (idx, cnt) in lists.items():
+        rows = [(h, t) for h in range(hq) for t in sorted({0, 1, 127, 128, n - 1, *r.integers(0, n, 100).tolist()}) if cnt[h, t] > 0]
+        O_ref, _ = _plain_attention(from_dev_bf16(q), from_dev_bf16(k), from_dev_bf16(v), idx, cnt, rows)
+        ref = np.stack([O_ref[x] for x in rows])
+        got = from_dev_bf16(outs[rep][0])
+        check_attention(np.stack([got[t, h] for h, t in rows]), ref, np.ones(ref.shape, bool), label=f"repeats {rep}")
+        for o in outs[rep][1:]:
+            assert torch.equal(o.view(torch.int16), outs[rep][0].view(torch.int16))
