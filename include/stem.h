@@ -281,14 +281,15 @@ int stem_token_select(const float* scores, int32_t n_tokens, int32_t list_heads,
  * (STEM_ERR_UNSUPPORTED otherwise).  Strides in elements, multiples of 8; Q, K, V, O 16-byte aligned.
  * softmax_scale 0 means 1/sqrt(128).  O bf16 [n_tokens, num_q_heads, 128] (contiguous); lse fp32
  * [num_q_heads, n_tokens] or NULL.  Probabilities are rounded to bf16 before they meet V (as in stem_sparse_prefill).
- * The call only enqueues; O serves as scratch memory until its kernels are done.  A bounded device-side wait that gave up
- * is reported by stem_token_check_status. */
+ * The call only enqueues; O serves as scratch memory until its kernels are done.  O may be Q itself (contiguous), else it
+ * must not overlap Q, K or V; a call with O == Q always gathers (see stem_token_attention_form).  A bounded device-side
+ * wait that gave up is reported by stem_token_check_status. */
 int stem_token_attention(const void* Q, const void* K, const void* V, int32_t n_tokens, int32_t num_q_heads,
                          int32_t num_kv_heads, int64_t q_stride_tok, int64_t q_stride_head, int64_t kv_stride_tok,
                          int64_t kv_stride_head, const int32_t* sel_idx, const int32_t* sel_cnt, int32_t k_max,
                          float softmax_scale, void* O, float* lse, void* stream);
 
-/* Which form stem_token_attention takes at these sizes on the current device: 0 gathers every list's rows, 1 computes
+/* Which form stem_token_attention takes at these sizes, O apart from Q, on the current device: 0 gathers every list's rows, 1 computes
  * every causal key block and masks what the lists do not name (k_max stands for the lists' lengths); negative: STEM_ERR_*.
  * Host only. */
 int stem_token_attention_form(int32_t n_tokens, int32_t num_q_heads, int32_t num_kv_heads, int32_t k_max);

@@ -532,6 +532,14 @@ token_attn_tc_kernel(const TokArgs a) {
   }
 }
 
+// Whether a [n, heads, 128] bf16 tensor of these strides (elements) has an address among the `bytes` bytes at O.
+bool overlaps(const void* x, int64_t n, int64_t heads, int64_t st, int64_t sh, const void* O, int64_t bytes) {
+  const int64_t tok = (n - 1) * st, head = (heads - 1) * sh;
+  const char* lo = (const char*)x + 2 * (std::min<int64_t>(tok, 0) + std::min<int64_t>(head, 0));
+  const char* hi = (const char*)x + 2 * (std::max<int64_t>(tok, 0) + std::max<int64_t>(head, 0) + kHeadDim);
+  return lo < (const char*)O + bytes && (const char*)O < hi;
+}
+
 }  // namespace
 
 int token_attn_max_group() { return kNPad; }
@@ -555,8 +563,13 @@ cudaError_t launch_token_attention(const void* Q, const void* K, const void* V, 
   TokenRedo* redo = nullptr;
   e = cudaGetSymbolAddress((void**)&redo, g_token_redo);
   if (e != cudaSuccess) return e;
+  // The masked form keeps its masks in O, so O has to be a buffer of its own; the gather form reads a token's Q before it writes
+  // the token's O, which may take Q's place.
+  const int64_t o_bytes = (int64_t)N * Hq * kHeadDim * 2;
+  const bool own_o = !overlaps(Q, N, Hq, q_st, q_sh, O, o_bytes) && !overlaps(K, N, Hkv, kv_st, kv_sh, O, o_bytes) &&
+                     !overlaps(V, N, Hkv, kv_st, kv_sh, O, o_bytes);
   bool masked = false;
-  e = launch_token_masked(Q, K, V, q_st, q_sh, kv_st, kv_sh, N, Hq, Hkv, k_max, sel_idx, sel_cnt, softmax_scale, O, lse, redo, dev, sms, &masked, s);
+  if (own_o) e = launch_token_masked(Q, K, V, q_st, q_sh, kv_st, kv_sh, N, Hq, Hkv, k_max, sel_idx, sel_cnt, softmax_scale, O, lse, redo, dev, sms, &masked, s);
   if (e != cudaSuccess) return e;
   TokArgs a{};
   a.Q = (const __nv_bfloat16*)Q;

@@ -392,3 +392,35 @@ def test_marked_rows_over_several_launches_and_streams():
         check_attention(np.stack([got[t, h] for h, t in rows]), ref, np.ones(ref.shape, bool), label=f"repeats {rep}")
         for o in outs[rep][1:]:
             assert torch.equal(o.view(torch.int16), outs[rep][0].view(torch.int16))
+
+
+# O in the place of Q: served by the gather form at every size (the masked one keeps its masks in O).  Also the gather form
+# on lists of many tiles: its ring wraps, the row reference is raised more than once, all its completion barriers turn over.
+@pytest.mark.parametrize("n,hq,hkv,k_max,order,repeat", [
+    (600, 4, 2, 300, "ascending", False),
+    (2500, 8, 1, 2048, "ascending", False),     # up to 16 tiles
+    (4300, 16, 1, 1501, "any", True),
+    (3001, 3, 3, 2900, "any", False),           # up to 23 tiles, one head to a group
+    (1200, 28, 4, 900, "ascending", True),
+])
+def test_output_in_the_place_of_the_queries(n, hq, hkv, k_max, order, repeat):
+    assert binding.stem_token_attention_form(n, hq, hkv, k_max) == "masked"     # with an O of its own
+    r = np.random.default_rng(n)
+    w = wl.small("token_inplace", seqlens=(n,), hq=hq, hkv=hkv, block=64, permille=100, sink=True, seed=n)
+    data = wl.make_qkv(w)
+    idx, cnt = _lists(r, n, hkv, k_max, order, repeat)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    q_np = from_dev_bf16(q)
+    lse = torch.full((hq, n), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_token_attention(q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), q, lse)
+    st, detail = binding.stem_token_check_status()
+    assert st == 0, detail
+    g = hq // hkv
+    rows = [(h, t) for h in range(hq) for t in sorted({0, 1, 127, 128, n // 2, n - 1, *r.integers(0, n, 150).tolist()}) if cnt[h // g, t] > 0]
+    O_ref, lse_ref = _plain_attention(q_np, from_dev_bf16(k), from_dev_bf16(v), idx, cnt, rows)
+    got, got_lse = from_dev_bf16(q), lse.cpu().numpy()
+    ref = np.stack([O_ref[x] for x in rows])
+    check_attention(np.stack([got[t, h] for h, t in rows]), ref, np.ones(ref.shape, bool), label="O in the place of Q")
+    assert max(abs(got_lse[h, t] - lse_ref[h, t]) for h, t in rows) < 1e-3
+    empty = np.repeat(cnt == 0, g, axis=0)
+    assert (got.transpose(1, 0, 2)[empty] == 0).all() and np.isneginf(got_lse[empty]).all()
