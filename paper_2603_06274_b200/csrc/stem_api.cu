@@ -467,6 +467,22 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
   return rc;
 }
 
+// Alg. 1 steps 3a-3c from what step 1 left.  dependent: the pooling kernel was enqueued just before.
+static int enqueue_lists(const Plan& p, const void* Q, const void* K, uint8_t* w, const KSide& ks, bool dependent, int32_t* idx,
+                         int32_t* cnt, cudaStream_t s) {
+  int rc;
+  if (small_score_select(p)) {
+    rc = cuda_rc(launch_small_score_select(p, w + p.ws.qsplit, ks.ksplit, ks.mv, idx, cnt, s));
+  } else {
+    float* M = (float*)(w + p.ws.metric);  // holds the bit planes of the selection keys, not the floats
+    rc = enqueue_metric(p, Q, K, w, ks, M, true, dependent, s);
+    if (rc != STEM_OK) return rc;
+    rc = cuda_rc(launch_select_planes(p, (const uint32_t*)M, p.score_mode != 1, idx, cnt, s));
+  }
+  if (rc == STEM_OK) p.last_launches++;
+  return rc;
+}
+
 // Alg. 1 steps 1-3c on one stream: pooling (one pass over Q and, unless the K side comes from a cache, over K
 // and V; emits the pooled vectors as bf16 parts), the metric of every causal block on the tensor cores into
 // the workspace (stored as bit planes of the selection's order-preserving keys), and the row-wise selection
@@ -477,22 +493,13 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
 static int enqueue_score_select(const Plan& p, const void* Q, const void* K, const void* V, void* kcache, uint8_t* w,
                                 int32_t* idx, int32_t* cnt, int first_word, cudaStream_t s) {
   const KSide ks = k_side(p, w, kcache);
-  float* M = (float*)(w + p.ws.metric);  // holds the bit planes of the selection keys, not the floats
   // (the anti-diagonal mode has no use for the pooled query vectors; the pooling kernel clears the status words as well; with a
   // cache, K and V are given when it is to be updated with the blocks that the chunk adds)
   int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, kcache != nullptr,
                                (int32_t*)(w + p.ws.status) + first_word, kStatusWords - first_word, s));
   if (rc != STEM_OK) return rc;
   p.last_launches++;
-  if (small_score_select(p)) {
-    rc = cuda_rc(launch_small_score_select(p, w + p.ws.qsplit, ks.ksplit, ks.mv, idx, cnt, s));
-  } else {
-    rc = enqueue_metric(p, Q, K, w, ks, M, true, true, s);
-    if (rc != STEM_OK) return rc;
-    rc = cuda_rc(launch_select_planes(p, (const uint32_t*)M, p.score_mode != 1, idx, cnt, s));
-  }
-  if (rc == STEM_OK) p.last_launches++;
-  return rc;
+  return enqueue_lists(p, Q, K, w, ks, true, idx, cnt, s);
 }
 
 int stem_score(const stem_plan* plan, const void* Q, const void* K, const void* V, float* M, void* ws, size_t ws_bytes,
@@ -527,18 +534,12 @@ int stem_select(const stem_plan* plan, const float* M, int32_t* sel_idx, int32_t
   p.last_launches = 0;
   cudaStream_t s = (cudaStream_t)stream;
   if (!M) {
-    // recompute the metric (as selection keys) from the pooled vectors a previous stem_score left in the workspace
-    float* Mw = (float*)(w + p.ws.metric);
+    // the metric from the pooled vectors a previous stem_score left in the workspace, as stem_score_select has it
     rc = cuda_rc(cudaMemsetAsync(w + p.ws.status + 16, 0, 16, s));  // the metric kernel's status words
     if (rc != STEM_OK) return rc;
-    rc = cuda_rc(launch_metric_gemm(p, w + p.ws.qsplit, w + p.ws.ksplit, (const float*)(w + p.ws.mv), Mw, true, false,
-                                    (int32_t*)(w + p.ws.status), s));
-    if (rc != STEM_OK) return rc;
-    p.last_launches++;
-    rc = cuda_rc(launch_select_planes(p, (const uint32_t*)Mw, true, sel_idx, sel_cnt, s));
-  } else {
-    rc = cuda_rc(launch_select_rows(p, M, false, sel_idx, sel_cnt, s));
+    return enqueue_lists(p, nullptr, nullptr, w, k_side(p, w, nullptr), false, sel_idx, sel_cnt, s);
   }
+  rc = cuda_rc(launch_select_rows(p, M, false, sel_idx, sel_cnt, s));
   if (rc == STEM_OK) p.last_launches++;
   return rc;
 }

@@ -408,3 +408,53 @@ def test_neighbouring_heads_with_lists_in_common(block, seqlens, hq, hkv):
     live = np.isfinite(lse_ref)
     assert np.abs(got[live] - lse_ref[live]).max() < 1e-3
     plan.close()
+
+
+def _tied_inputs(seqlens, hq, hkv, block, seed):
+    """Q, K, V whose metric is decided by rounding: every key block holds the same keys in another order (means that differ
+    in the last bits alone) and values of the same norms."""
+    r = np.random.default_rng(seed)
+    T = sum(seqlens)
+    q = torch.from_numpy(r.standard_normal((T, hq, 128), dtype=np.float32)).to(torch.bfloat16)
+    base = torch.from_numpy(r.standard_normal((block, hkv, 128), dtype=np.float32)).to(torch.bfloat16)
+    k = torch.empty((T, hkv, 128), dtype=torch.bfloat16)
+    start = 0
+    for n in seqlens:
+        for a in range(0, n, block):
+            m = min(block, n - a)
+            k[start + a:start + a + m] = base[torch.from_numpy(r.permutation(block))][:m]
+        start += n
+    v = torch.from_numpy(r.standard_normal((1, hkv, 128), dtype=np.float32)).to(torch.bfloat16).expand(T, hkv, 128).contiguous()
+    return q.cuda(), k.cuda(), v.cuda()
+
+
+def _lists_of(plan, call):
+    info = plan.info
+    idx = torch.full((info.list_heads, info.total_q_blocks, info.k_max), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.full((info.list_heads, info.total_q_blocks), -7, dtype=torch.int32, device="cuda")
+    call(idx, cnt)
+    assert binding.stem_check_status(plan)[0] == 0
+    return idx, cnt
+
+
+# sequences of up to 64 blocks, longer ones, both beside each other; one list per query head and one per kv head
+LIST_SHAPES = [
+    (128, (2000, 8192, 1), 4, 2, False),
+    (64, (4096,), 8, 2, True),
+    (128, (8193,), 4, 2, False),
+    (64, (700, 4097, 64, 6000), 4, 2, False),
+    (128, (300, 9000, 8192), 8, 2, True),
+]
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv,share", LIST_SHAPES)
+def test_lists_in_two_steps_are_those_of_the_fused_call(block, seqlens, hq, hkv, share):
+    q, k, v = _tied_inputs(seqlens, hq, hkv, block, len(seqlens))
+    plan = StemPlan(seqlens, hq, hkv, block=block, budget_permille=300, share_group=share)
+    idx, cnt = _lists_of(plan, lambda i, c: binding.stem_score_select(plan, q, k, v, i, c))
+    binding.stem_score(plan, q, k, v)
+    idx2, cnt2 = _lists_of(plan, lambda i, c: binding.stem_select(plan, None, i, c))
+    assert torch.equal(cnt, cnt2) and torch.equal(idx, idx2)
+    out = torch.empty_like(q)
+    idx3, cnt3 = _lists_of(plan, lambda i, c: binding.stem_prefill(plan, q, k, v, out, i, c))
+    assert torch.equal(cnt, cnt3) and torch.equal(idx, idx3)
