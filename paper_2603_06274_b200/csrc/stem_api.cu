@@ -451,7 +451,7 @@ static KSide k_side(const Plan& p, uint8_t* w, void* kcache) {
   return {w + p.ws.ksplit, (float*)(w + p.ws.mv)};
 }
 
-// Alg. 1 step 3a from what step 1 left: the product of block means on the pooled vectors, or, in the anti-diagonal
+// Alg. 1 step 3a from what step 1 left, as floats or (as_keys) for launch_select_planes: the product of block means on the pooled vectors, or, in the anti-diagonal
 // scoring mode, the contraction of Q with K itself (MV comes from the pooling kernel in both).
 static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* w, const KSide& ks, float* M, bool as_keys,
                           bool dependent, cudaStream_t s) {
@@ -462,7 +462,8 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
     p.last_launches += launched;
     return rc;
   }
-  const int rc = cuda_rc(launch_metric_gemm(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, as_keys, dependent, status, s));
+  const int rc = cuda_rc(!as_keys && small_score_select(p) ? launch_small_metric(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, s)
+                                                           : launch_metric_gemm(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, as_keys, dependent, status, s));
   if (rc == STEM_OK) p.last_launches++;
   return rc;
 }

@@ -139,6 +139,8 @@ cudaError_t launch_select_planes(const Plan& p, const uint32_t* Mt, bool depende
 bool small_score_select(const Plan& p);
 cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
                                       int32_t* sel_cnt, cudaStream_t s);
+// The metric as that kernel ranks it (layout of stem_score's M; entries j > r are not written).
+cudaError_t launch_small_metric(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, float* M, cudaStream_t s);
 
 // dependent: launched as a programmatic dependent of the selection kernel enqueued just before, its status words cleared by
 // an earlier kernel; otherwise the launch clears them itself.

@@ -315,6 +315,8 @@ struct SmallArgs {
   const __nv_bfloat16 *q, *k;  // split pooled vectors [3, H_list, R_tot, d], [3, H_kv, KB_tot, d]
   const float* mv;
   int32_t *sel_idx, *sel_cnt;
+  float* M;  // kMetric: every causal entry (layout of stem_score's M) is written here, and no lists
+  int64_t m_tot;
   RowTables rows;
   int H_list, Hkv, R_tot, KB_tot, k_max, stem, local;
   float scale, beta;
@@ -334,6 +336,7 @@ __device__ __forceinline__ void load_split8(const __nv_bfloat16* p, int64_t plan
   }
 }
 
+template <bool kMetric>
 __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const SmallArgs a) {
   __shared__ float dots[kSmallBlocks];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -356,14 +359,15 @@ __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const
   uint64_t sel = all & ~cand;  // the forced blocks
   const bool ranked = need > 0 && need < n_cand;
   if (need > 0 && !ranked) sel = all;
+  const int cols = kMetric ? i : c_hi;  // columns whose metric is wanted
 
   // everything above overlaps the tail of the pooling kernel, whose results are read below
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (ranked) {
+  if (kMetric || ranked) {
     // warp w: the columns 16 w .. 16 w + 15, eight per half-warp, all of their loads in flight together
     const int64_t q_plane = (int64_t)a.H_list * a.R_tot * kHeadDim, k_plane = (int64_t)a.Hkv * a.KB_tot * kHeadDim;
     const int j0 = 16 * warp;
-    if (j0 < c_hi) {
+    if (j0 < cols) {
       const __nv_bfloat16* krow = a.k + ((int64_t)kvh * a.KB_tot + kb0) * kHeadDim + chunk * 8;
       float q[8], acc[8];
       load_split8(a.q + ((int64_t)h * a.R_tot + R) * kHeadDim + chunk * 8, q_plane, q);
@@ -385,9 +389,14 @@ __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const
     __syncthreads();
     if (warp == 0) {
       const float* mv = a.mv + (int64_t)kvh * a.KB_tot + kb0;
-      const float d0 = lane < c_hi ? dots[lane] : 0.f, d1 = lane + 32 < c_hi ? dots[lane + 32] : 0.f;
-      const uint32_t key0 = metric_key(fmaf(a.scale, d0, a.beta * mv[min(lane, r)]));
-      const uint32_t key1 = metric_key(fmaf(a.scale, d1, a.beta * mv[min(lane + 32, r)]));
+      const float d0 = lane < cols ? dots[lane] : 0.f, d1 = lane + 32 < cols ? dots[lane + 32] : 0.f;
+      const float m0 = fmaf(a.scale, d0, a.beta * mv[min(lane, r)]), m1 = fmaf(a.scale, d1, a.beta * mv[min(lane + 32, r)]);
+      if constexpr (kMetric) {
+        float* row = a.M + (int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)(r - a.rows.seq_r0[seq]) * a.rows.seq_nblk[seq];
+        if (lane < cols) row[lane] = m0;
+        if (lane + 32 < cols) row[lane + 32] = m1;
+      }
+      const uint32_t key0 = metric_key(m0), key1 = metric_key(m1);
       uint64_t act = cand, gt = 0ull;
       int k = need;
 #pragma unroll 1
@@ -406,7 +415,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const
       sel |= gt | act;
     }
   }
-  if (warp != 0) return;
+  if (kMetric || warp != 0) return;
   int32_t* out = a.sel_idx + ((int64_t)h * a.R_tot + R) * a.k_max;
   const int total = __popcll(sel);
 #pragma unroll
@@ -425,9 +434,10 @@ bool small_score_select(const Plan& p) {
   return p.score_mode == 0 && p.max_nblk <= kSmallBlocks && (int64_t)p.H_list * p.R_tot <= kSmallRowsMax;
 }
 
-cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
-                                      int32_t* sel_cnt, cudaStream_t s) {
+static cudaError_t launch_small(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, float* M, int32_t* sel_idx,
+                                int32_t* sel_cnt, cudaStream_t s) {
   SmallArgs a{};
+  a.M = M; a.m_tot = p.m_tot;
   a.q = (const __nv_bfloat16*)qsplit; a.k = (const __nv_bfloat16*)ksplit; a.mv = mv;
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt; a.rows = p.rows;
   a.H_list = p.H_list; a.Hkv = p.cfg.num_kv_heads; a.R_tot = p.R_tot; a.KB_tot = p.KB_tot; a.k_max = p.k_max;
@@ -441,7 +451,16 @@ cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const v
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, small_score_select_kernel, a);
+  return cudaLaunchKernelEx(&cfg, M ? small_score_select_kernel<true> : small_score_select_kernel<false>, a);
+}
+
+cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
+                                      int32_t* sel_cnt, cudaStream_t s) {
+  return launch_small(p, qsplit, ksplit, mv, nullptr, sel_idx, sel_cnt, s);
+}
+
+cudaError_t launch_small_metric(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, float* M, cudaStream_t s) {
+  return launch_small(p, qsplit, ksplit, mv, M, nullptr, nullptr, s);
 }
 
 int row_select_max_blocks() { return 2 * 1024; }

@@ -411,18 +411,18 @@ def test_neighbouring_heads_with_lists_in_common(block, seqlens, hq, hkv):
 
 
 def _tied_inputs(seqlens, hq, hkv, block, seed):
-    """Q, K, V whose metric is decided by rounding: every key block holds the same keys in another order (means that differ
-    in the last bits alone) and values of the same norms."""
+    """Q, K, V whose metric is decided by rounding: the queries are alike in every dimension and the key blocks hold the same
+    keys with their dimensions in another order, so all products are equal but for the order of their sums."""
     r = np.random.default_rng(seed)
     T = sum(seqlens)
-    q = torch.from_numpy(r.standard_normal((T, hq, 128), dtype=np.float32)).to(torch.bfloat16)
+    q = torch.from_numpy(r.standard_normal((T, hq, 1), dtype=np.float32)).to(torch.bfloat16).expand(T, hq, 128).contiguous()
     base = torch.from_numpy(r.standard_normal((block, hkv, 128), dtype=np.float32)).to(torch.bfloat16)
     k = torch.empty((T, hkv, 128), dtype=torch.bfloat16)
     start = 0
     for n in seqlens:
         for a in range(0, n, block):
             m = min(block, n - a)
-            k[start + a:start + a + m] = base[torch.from_numpy(r.permutation(block))][:m]
+            k[start + a:start + a + m] = base[:m][:, :, torch.from_numpy(r.permutation(128))]
         start += n
     v = torch.from_numpy(r.standard_normal((1, hkv, 128), dtype=np.float32)).to(torch.bfloat16).expand(T, hkv, 128).contiguous()
     return q.cuda(), k.cuda(), v.cuda()
@@ -458,3 +458,18 @@ def test_lists_in_two_steps_are_those_of_the_fused_call(block, seqlens, hq, hkv,
     out = torch.empty_like(q)
     idx3, cnt3 = _lists_of(plan, lambda i, c: binding.stem_prefill(plan, q, k, v, out, i, c))
     assert torch.equal(cnt, cnt3) and torch.equal(idx, idx3)
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv,share", LIST_SHAPES)
+def test_fused_lists_are_those_of_the_metric_handed_out(block, seqlens, hq, hkv, share):
+    q, k, v = _tied_inputs(seqlens, hq, hkv, block, 7 + len(seqlens))
+    plan = StemPlan(seqlens, hq, hkv, block=block, budget_permille=300, share_group=share)
+    idx, cnt = _lists_of(plan, lambda i, c: binding.stem_score_select(plan, q, k, v, i, c))
+    M = torch.full((plan.info.list_heads, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_score(plan, q, k, v, M)
+    idx2, cnt2 = _lists_of(plan, lambda i, c: binding.stem_select(plan, M, i, c))
+    assert torch.equal(cnt, cnt2) and torch.equal(idx, idx2)
+    M2 = torch.full_like(M, float("nan"))
+    binding.stem_score_static(plan, q, k, v, M2)
+    torch.cuda.synchronize()
+    assert torch.equal(M.view(torch.int32), M2.view(torch.int32))
