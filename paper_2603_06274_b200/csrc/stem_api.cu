@@ -219,6 +219,8 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   std::vector<int64_t> seq_m_off(batch), seq_mt_off(batch);
   int64_t m_off = 0, mt_off = 0;
   int32_t q_tok = 0, kb_off = 0;
+  std::vector<uint8_t> is_short(batch);
+  std::vector<int32_t> long_rows, short_rows;
   for (int b = 0; b < batch; ++b) {
     const int32_t n = p.cu[b + 1] - p.cu[b];           // tokens of the K / V prefix
     const int32_t nb = (n + B - 1) / B;                // its blocks
@@ -226,6 +228,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     const int32_t r0 = q0 / B;
     const int64_t n_tot = o.total_len_host ? o.total_len_host[b] : n;
     const int64_t nb_tot = (n_tot + B - 1) / B;        // blocks of the whole sequence: N of Eq. 3
+    is_short[b] = p.score_mode == 0 && nb_tot <= kShortBlocks;
     seq_tok0[b] = p.cu[b];
     seq_nblk[b] = nb;
     seq_r0[b] = r0;
@@ -247,6 +250,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
       kb_dst.push_back(seq_kb_off[b] + j);
     }
     for (int32_t r = r0; r < nb; ++r) {
+      (is_short[b] ? short_rows : long_rows).push_back((int32_t)row_seq.size());
       row_seq.push_back(b);
       row_r.push_back(r);
       row_tok0.push_back(q_tok + (r - r0) * B);
@@ -281,8 +285,13 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     return STEM_ERR_UNSUPPORTED;
   }
 
-  // Tiles of the metric GEMM: 128 query rows x 128 key blocks, the tiles of every sequence that hold a causal
-  // entry (j <= r for some row of the tile), long rows first.
+  std::reverse(long_rows.begin(), long_rows.end());  // the longest lists of a sequence first
+  std::reverse(short_rows.begin(), short_rows.end());
+  p.n_long_rows = (int32_t)long_rows.size();
+  p.n_short_rows = (int32_t)short_rows.size();
+
+  // Tiles of the metric GEMM: 128 query rows x 128 key blocks, the tiles of every sequence that is not short that hold a
+  // causal entry (j <= r for some row of the tile), long rows first.
   std::vector<int32_t> gemm_tiles;
   {
     int max_t = 0;
@@ -290,7 +299,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     for (int ti = max_t - 1; ti >= 0; --ti)
       for (int b = 0; b < batch; ++b) {
         const int rows_b = seq_nblk[b] - seq_r0[b];
-        if (ti >= (rows_b + 127) / 128) continue;
+        if (is_short[b] || ti >= (rows_b + 127) / 128) continue;
         const int r_last = seq_r0[b] + std::min(rows_b, (ti + 1) * 128) - 1;  // largest global row of the tile
         for (int tj = 0; tj <= r_last / 128; ++tj) { gemm_tiles.push_back(b); gemm_tiles.push_back(ti); gemm_tiles.push_back(tj); }
       }
@@ -344,7 +353,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
                o_seq_mt_off = push(blob, seq_mt_off), o_kb_tok0 = push(blob, kb_tok0), o_kb_ntok = push(blob, kb_ntok),
                o_kb_dst = push(blob, kb_dst), o_kb_new = push(blob, kb_new), o_gt = push(blob, gemm_tiles),
                o_ws = push(blob, work_sparse), o_wd = push(blob, work_dense), o_ss = push(blob, slots_sparse),
-               o_sd = push(blob, slots_dense);
+               o_sd = push(blob, slots_dense), o_lr = push(blob, long_rows), o_sr = push(blob, short_rows);
   if (cudaMalloc(&p.d_blob, blob.size()) != cudaSuccess ||
       cudaMemcpy(p.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
@@ -371,6 +380,8 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   p.rows.kb_dst = (const int32_t*)(d + o_kb_dst);
   p.rows.kb_new = (const int32_t*)(d + o_kb_new);
   p.d_gemm_tiles = (const int32_t*)(d + o_gt);
+  p.d_long_rows = (const int32_t*)(d + o_lr);
+  p.d_short_rows = (const int32_t*)(d + o_sr);
   p.work_sparse.d_items = (const int32_t*)(d + o_ws);
   p.work_sparse.d_slot_off = (const int32_t*)(d + o_ss);
   p.work_dense.d_items = (const int32_t*)(d + o_wd);
@@ -462,25 +473,35 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
     p.last_launches += launched;
     return rc;
   }
-  const int rc = cuda_rc(!as_keys && small_score_select(p) ? launch_small_metric(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, s)
-                                                           : launch_metric_gemm(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, as_keys, dependent, status, s));
-  if (rc == STEM_OK) p.last_launches++;
+  int rc = STEM_OK;
+  if (p.n_long_rows > 0) {
+    rc = cuda_rc(launch_metric_gemm(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, as_keys, dependent, status, s));
+    if (rc != STEM_OK) return rc;
+    p.last_launches++;
+  }
+  if (!as_keys && p.n_short_rows > 0) {
+    rc = cuda_rc(launch_small_metric(p, w + p.ws.qsplit, ks.ksplit, ks.mv, M, s));
+    if (rc == STEM_OK) p.last_launches++;
+  }
   return rc;
 }
 
 // Alg. 1 steps 3a-3c from what step 1 left.  dependent: the pooling kernel was enqueued just before.
 static int enqueue_lists(const Plan& p, const void* Q, const void* K, uint8_t* w, const KSide& ks, bool dependent, int32_t* idx,
                          int32_t* cnt, cudaStream_t s) {
-  int rc;
-  if (small_score_select(p)) {
-    rc = cuda_rc(launch_small_score_select(p, w + p.ws.qsplit, ks.ksplit, ks.mv, idx, cnt, s));
-  } else {
+  int rc = STEM_OK;
+  if (p.n_long_rows > 0) {
     float* M = (float*)(w + p.ws.metric);  // holds the bit planes of the selection keys, not the floats
     rc = enqueue_metric(p, Q, K, w, ks, M, true, dependent, s);
     if (rc != STEM_OK) return rc;
     rc = cuda_rc(launch_select_planes(p, (const uint32_t*)M, p.score_mode != 1, idx, cnt, s));
+    if (rc != STEM_OK) return rc;
+    p.last_launches++;
   }
-  if (rc == STEM_OK) p.last_launches++;
+  if (p.n_short_rows > 0) {
+    rc = cuda_rc(launch_small_score_select(p, w + p.ws.qsplit, ks.ksplit, ks.mv, idx, cnt, s));
+    if (rc == STEM_OK) p.last_launches++;
+  }
   return rc;
 }
 

@@ -87,8 +87,13 @@ struct Plan {
   // device blob
   void* d_blob = nullptr;
   RowTables rows{};
-  const int32_t* d_gemm_tiles = nullptr;  // [n_gemm_tiles][3] (sequence, row tile, column tile) of the metric GEMM
+  const int32_t* d_gemm_tiles = nullptr;  // [n_gemm_tiles][3] (sequence, row tile, column tile) of the metric GEMM (sequences that are not short)
   int32_t n_gemm_tiles = 0;
+  // Query rows, the last first, of the sequences that the tensor-core metric serves and of those that the kernel for short
+  // sequences does.  Which it is follows from the length of the whole sequence alone (total_len, with chunks): a row's list is
+  // the same whatever is batched beside it, however its sequence is cut in chunks and the heads in plans.
+  const int32_t *d_long_rows = nullptr, *d_short_rows = nullptr;
+  int32_t n_long_rows = 0, n_short_rows = 0;
   AttnWork work_sparse, work_dense;
   int32_t n_items = 0;
 
@@ -134,9 +139,9 @@ cudaError_t launch_select_rows(const Plan& p, const float* M, bool dependent, in
 cudaError_t launch_select_planes(const Plan& p, const uint32_t* Mt, bool dependent, int32_t* sel_idx, int32_t* sel_cnt,
                                  cudaStream_t s);
 
-// Metric and selection of short sequences in one kernel, straight from the split pooled vectors (Alg. 1 steps 3a-3c):
-// whether a plan is one for it, and its launch (a programmatic dependent of the pooling kernel).
-bool small_score_select(const Plan& p);
+// Metric and selection of the short sequences in one kernel, straight from the split pooled vectors (Alg. 1 steps 3a-3c),
+// launched as a programmatic dependent of the kernel before it.
+constexpr int kShortBlocks = 64;  // longest sequence for it
 cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, int32_t* sel_idx,
                                       int32_t* sel_cnt, cudaStream_t s);
 // The metric as that kernel ranks it (layout of stem_score's M; entries j > r are not written).

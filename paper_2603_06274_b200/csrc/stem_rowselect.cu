@@ -26,7 +26,6 @@ namespace stem {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int64_t kSmallRowsMax = 8192;  // (list head, row) pairs of the small kernel
 
 // Monotone map float -> uint32 with -0 == +0 and NaN below everything (as -inf).  Every key is >= 1.
 __device__ __forceinline__ uint32_t metric_key(float f) {
@@ -46,6 +45,8 @@ struct SelArgs {
   RowTables rows;
   int64_t m_tot, mt_tot;
   int Hq, R_tot, k_max, stem, local;
+  const int32_t* row_list;  // the rows of the launch (select_planes_kernel)
+  int n_rows;
 };
 
 // The mask of the n lowest set bits of m.
@@ -207,9 +208,9 @@ __global__ void __launch_bounds__(kThreads, SETS == 1 ? 4 : 2) select_planes_ker
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t item = (int64_t)blockIdx.x * (kThreads / 32) + warp;
-  if (item >= (int64_t)a.Hq * a.R_tot) return;
+  if (item >= (int64_t)a.Hq * a.n_rows) return;
   const int h = (int)(item % a.Hq);
-  const int R = a.R_tot - 1 - (int)(item / a.Hq);  // long rows first
+  const int R = a.row_list[item / a.Hq];
   const int seq = a.rows.row_seq[R];
   const int r = a.rows.row_r[R];
   const int nb = a.rows.seq_nblk[seq];
@@ -309,7 +310,9 @@ __global__ void __launch_bounds__(kThreads, SETS == 1 ? 4 : 2) select_planes_ker
 // a pooled key vector (its three parts, 256 bytes each) and multiplies it with the row's query vector; then one warp has
 // column j in lane j mod 32, a ballot per key bit gives that bit of all columns to every lane, and the radix descent needs
 // no reductions.  The tensor-core metric kernel and the selection behind it are bound by latency at these sizes (tensor
-// memory, tensor maps, a chain of copies and MMAs): 9.6 + 1.3 us at 12 blocks, where this takes 2.
+// memory, tensor maps, a chain of copies and MMAs): 9.6 + 1.3 us at 12 blocks, where this takes 2.  With many rows both are
+// as fast, so that the number of rows has no say (scoring stage, tensor cores / here, us: 1024 rows 22.9 / 17.0, 8192
+// 78 / 74, 16 384 142 / 138, 32 768 in sequences of 16, 32, 64 blocks 315 / 270, 284 / 271, 267 / 273, 65 536 310 / 324).
 // ------------------------------------------------------------------------------------------------
 struct SmallArgs {
   const __nv_bfloat16 *q, *k;  // split pooled vectors [3, H_list, R_tot, d], [3, H_kv, KB_tot, d]
@@ -318,11 +321,11 @@ struct SmallArgs {
   float* M;  // kMetric: every causal entry (layout of stem_score's M) is written here, and no lists
   int64_t m_tot;
   RowTables rows;
+  const int32_t* row_list;
   int H_list, Hkv, R_tot, KB_tot, k_max, stem, local;
   float scale, beta;
 };
 
-constexpr int kSmallBlocks = 64;
 constexpr int kSmallThreads = 128;
 
 // Eight pooled values of one lane: the sum of the three bf16 parts is the fp32 value exactly.
@@ -338,12 +341,12 @@ __device__ __forceinline__ void load_split8(const __nv_bfloat16* p, int64_t plan
 
 template <bool kMetric>
 __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const SmallArgs a) {
-  __shared__ float dots[kSmallBlocks];
+  __shared__ float dots[kShortBlocks];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int half = lane >> 4, chunk = lane & 15;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int item = blockIdx.x;
-  const int h = item % a.H_list, R = a.R_tot - 1 - item / a.H_list;  // long rows first
+  const int h = item % a.H_list, R = a.row_list[item / a.H_list];
   const int kvh = h / (a.H_list / a.Hkv);
   const int seq = a.rows.row_seq[R], r = a.rows.row_r[R];
   const int kb0 = a.rows.seq_kb_off[seq];
@@ -429,11 +432,6 @@ __global__ void __launch_bounds__(kSmallThreads) small_score_select_kernel(const
 
 }  // namespace
 
-// Sequences of up to 64 blocks, and not so many rows that the tensor cores pay.
-bool small_score_select(const Plan& p) {
-  return p.score_mode == 0 && p.max_nblk <= kSmallBlocks && (int64_t)p.H_list * p.R_tot <= kSmallRowsMax;
-}
-
 static cudaError_t launch_small(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, float* M, int32_t* sel_idx,
                                 int32_t* sel_cnt, cudaStream_t s) {
   SmallArgs a{};
@@ -441,12 +439,13 @@ static cudaError_t launch_small(const Plan& p, const void* qsplit, const void* k
   a.q = (const __nv_bfloat16*)qsplit; a.k = (const __nv_bfloat16*)ksplit; a.mv = mv;
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt; a.rows = p.rows;
   a.H_list = p.H_list; a.Hkv = p.cfg.num_kv_heads; a.R_tot = p.R_tot; a.KB_tot = p.KB_tot; a.k_max = p.k_max;
+  a.row_list = p.d_short_rows;
   a.stem = p.cfg.stem_blocks; a.local = p.cfg.local_blocks; a.scale = p.score_scale; a.beta = p.cfg.beta;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.H_list * p.R_tot));
+  cfg.gridDim = dim3((unsigned)((int64_t)p.H_list * p.n_short_rows));
   cfg.blockDim = dim3(kSmallThreads);
   cfg.stream = s;
   cfg.attrs = attr;
@@ -468,13 +467,13 @@ int row_select_max_blocks() { return 2 * 1024; }
 static SelArgs make_args(const Plan& p, int32_t* sel_idx, int32_t* sel_cnt) {
   SelArgs a{};
   a.sel_idx = sel_idx; a.sel_cnt = sel_cnt; a.rows = p.rows; a.m_tot = p.m_tot; a.mt_tot = p.mt_tot;
-  a.Hq = p.H_list; a.R_tot = p.R_tot; a.k_max = p.k_max;
+  a.Hq = p.H_list; a.R_tot = p.R_tot; a.n_rows = p.R_tot; a.k_max = p.k_max;
   a.stem = p.cfg.stem_blocks; a.local = p.cfg.local_blocks;
   return a;
 }
 
 static cudaLaunchConfig_t make_config(const SelArgs& a, size_t smem, cudaStream_t s, cudaLaunchAttribute* attr, bool dependent) {
-  const int64_t items = (int64_t)a.Hq * a.R_tot;
+  const int64_t items = (int64_t)a.Hq * a.n_rows;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((items + kThreads / 32 - 1) / (kThreads / 32)));
   cfg.blockDim = dim3(kThreads);
@@ -513,6 +512,7 @@ cudaError_t launch_select_planes(const Plan& p, const uint32_t* Mt, bool depende
                                  cudaStream_t s) {
   SelArgs a = make_args(p, sel_idx, sel_cnt);
   a.Mt = Mt;
+  a.row_list = p.d_long_rows; a.n_rows = p.n_long_rows;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = make_config(a, 0, s, attr, dependent);
   if (p.max_nblk <= 1024) return cudaLaunchKernelEx(&cfg, select_planes_kernel<1>, a);

@@ -84,8 +84,13 @@ extern "C" int stem_score_static(const stem_plan* plan, const void* Q, const voi
   if (cudaMemsetAsync(status, 0, kStatusWords * sizeof(int32_t), s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
   if (launch_pool(p, Q, K, V, mv, qsplit, ksplit, false, nullptr, 0, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
   p.last_launches++;
-  if ((small_score_select(p) ? launch_small_metric(p, qsplit, ksplit, mv, M, s)
-                             : launch_metric_gemm(p, qsplit, ksplit, mv, M, false, true, status, s)) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
-  p.last_launches++;
+  if (p.n_long_rows > 0) {
+    if (launch_metric_gemm(p, qsplit, ksplit, mv, M, false, true, status, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
+    p.last_launches++;
+  }
+  if (p.n_short_rows > 0) {
+    if (launch_small_metric(p, qsplit, ksplit, mv, M, s) != cudaSuccess) { cudaGetLastError(); return STEM_ERR_CUDA; }
+    p.last_launches++;
+  }
   return STEM_OK;
 }

@@ -473,3 +473,50 @@ def test_fused_lists_are_those_of_the_metric_handed_out(block, seqlens, hq, hkv,
     binding.stem_score_static(plan, q, k, v, M2)
     torch.cuda.synchronize()
     assert torch.equal(M.view(torch.int32), M2.view(torch.int32))
+
+
+def _same_lists(idx, cnt, idx2, cnt2):
+    k = min(idx.shape[2], idx2.shape[2])  # padded to the longest list of each plan
+    return torch.equal(cnt, cnt2) and torch.equal(idx[:, :, :k], idx2[:, :, :k]) and int(cnt.max()) <= k
+
+
+@pytest.mark.parametrize("total,chunk_blocks,hq,hkv,block", [
+    (100 * 128 - 5, 40, 28, 4, 128),   # chunks of a sequence of 100 blocks, the first ones of up to 64
+    (64 * 128, 33, 4, 2, 128),         # a whole sequence of 64 blocks
+    (70 * 64, 64, 8, 2, 64),
+])
+def test_lists_of_a_sequence_are_the_same_in_any_chunks_batch_and_head_split(total, chunk_blocks, hq, hkv, block):
+    lens = (total, 3 * block + 1, 90 * block, 64 * block)
+    q, k, v = _tied_inputs(lens, hq, hkv, block, total)
+    kw = dict(block=block, budget_permille=200)
+    plan = StemPlan(lens, hq, hkv, **kw)
+    out = torch.empty_like(q)
+    idx, cnt = _lists_of(plan, lambda i, c: binding.stem_prefill(plan, q, k, v, out, i, c))
+    n = (total + block - 1) // block
+    # the first sequence alone, in chunks (their K / V the prefix), the pooled keys from the chunks before
+    cache = None
+    for r0 in range(0, n, chunk_blocks):
+        a, b = r0 * block, min(total, (r0 + chunk_blocks) * block)
+        part = StemPlan((b,), hq, hkv, q_starts=[a], total_lens=[total], kcache_blocks_per_seq=n, **kw)
+        if cache is None:
+            cache = torch.zeros(int(part.info.kcache_bytes), dtype=torch.uint8, device="cuda")
+        o = torch.full((b - a, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        i, c = _lists_of(part, lambda i, c: binding.stem_prefill_cached(part, q[a:b], k[:b], v[:b], o, cache, True, i, c))
+        r1 = (b + block - 1) // block
+        assert _same_lists(idx[:, r0:r1], cnt[:, r0:r1], i, c)
+        # O: the blocks of a list are added up in another order, their probabilities rounded against another reference
+        check_attention(from_dev_bf16(o), from_dev_bf16(out[a:b]), label=f"chunk at block {r0}")
+    # each sequence alone, and each kv head alone
+    row = tok = 0
+    for m in lens:
+        nb = (m + block - 1) // block
+        one = StemPlan((m,), hq, hkv, **kw)
+        i, c = _lists_of(one, lambda i, c: binding.stem_score_select(one, q[tok:tok + m], k[tok:tok + m], v[tok:tok + m], i, c))
+        assert _same_lists(idx[:, row:row + nb], cnt[:, row:row + nb], i, c)
+        row += nb
+        tok += m
+    g = hq // hkv
+    for h in range(hkv):
+        one = StemPlan(lens, g, 1, q_strides=(hq * 128, 128), kv_strides=(hkv * 128, 128), **kw)
+        i, c = _lists_of(one, lambda i, c: binding.stem_score_select(one, q[:, h * g:(h + 1) * g], k[:, h:h + 1], v[:, h:h + 1], i, c))
+        assert _same_lists(idx[h * g:(h + 1) * g], cnt[h * g:(h + 1) * g], i, c)
