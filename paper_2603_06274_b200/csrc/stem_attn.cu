@@ -18,8 +18,9 @@
 //                 the leading key columns while the softmax still works on the last 32
 // Other query heads of a group have lists of their own, but choose many of the same blocks (always the first and the local
 // ones).  With kMerge the slots take neighbouring items, warp 9 finds a pair ahead which blocks both lists name, and each
-// slot walks its own blocks first and the common ones, the diagonal block last, in step with the other slot on one stream
-// of tiles.  Slots one by one / merged, TFLOP/s at 32 / 8 heads, lists of 22 blocks (32K tokens) and 42 (128K): 1128 / 1247 and
+// slot walks the common blocks first, in step with the other slot on one stream of tiles, then its own, the diagonal block last.
+// (The first block, which draws most of the attention, is a common one and sets the row's reference as it does in list order:
+// with the common blocks last, O's error against 64 bits was up to 4 % larger at 128K tokens, and the layers 1 % slower.)  Slots one by one / merged, TFLOP/s at 32 / 8 heads, lists of 22 blocks (32K tokens) and 42 (128K): 1128 / 1247 and
 // 1121 / 1262 with 9 of 10 blocks in common, 1120 / 1220 and 1110 / 1200 for independent random metrics; 64K tokens, 28 / 4:
 // 1135 / 1255; blocks of 64 at 32K 420 / 467.  Neighbours may be two rows of one head as well, whose last blocks differ: 64K
 // tokens, 2 / 2 heads 980 / 1150; 16K, 8 / 8, blocks of 64 350 / 420.
@@ -925,7 +926,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       };
       bool ok = true;
       if constexpr (kMerge) {
-        // The merged lists: in each round a block of slot 0's own and one of slot 1's own, then those both have, one tile each.
+        // The merged lists: the blocks both have, one tile each, then in each round a block of slot 0's own and one of slot 1's
+        // own, then the last ones.
         int pend_tok[2] = {-1, -1}, pend_kvh[2] = {0, 0};  // V tile that is due; slot 0's alone if both have the block
         auto pend = [&](const int X) -> bool {
           if (pend_tok[X] < 0) return true;
@@ -943,25 +945,26 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const int n0 = uni(hdr[0]), n1 = uni(hdr[1]), both = uni(hdr[2]);
           const int tail = uni(hdr[7]), kvh[2] = {uni(hdr[3]), uni(hdr[5])}, tok0[2] = {uni(hdr[4]), uni(hdr[6])};
           const int c0 = n0 - both - tail, c1 = n1 - both - tail, own = max(c0, c1);
-          // the i-th block of slot X: its own c, those both have, its last with `tail`; all causal blocks in the dense mode
-          auto block = [&](const int X, const int i, const int c) -> int {
-            if (dense) return i < c ? both + i : i < c + both ? i - c : c + both;
-            return uni((int)ent[X ? n0 + (i < c ? i : c) : i]);
+          const int lead = both - (tail == 0 && both > 0 ? 1 : 0);  // the common last block stays the last
+          // the i-th block that both have, the i-th of slot X's own, slot X's last; all causal blocks in the dense mode
+          auto common = [&](const int i) -> int { return dense ? i : uni((int)ent[c0 + i]); };
+          auto alone = [&](const int X, const int i) -> int { return dense ? both + i : uni((int)ent[X ? n0 + i : i]); };
+          auto last = [&](const int X) -> int { return dense ? (X ? n1 : n0) - 1 : uni((int)ent[X ? n0 + c1 : n0 - 1]); };
+          auto key = [&](const int X, const int j) -> bool {
+            pend_tok[X] = tok0[X] + j * BLK;
+            pend_kvh[X] = kvh[X];
+            return load(&map_k, kvh[X], pend_tok[X]);
           };
-          for (int it = 0; ok && it < own + both + tail; ++it) {
+          auto shared_round = [&](const int i) -> bool { return pend(0) && key(0, common(i)) && pend(1); };
+          for (int it = 0; ok && it < lead; ++it) ok = shared_round(it);
+          for (int it = 0; ok && it < own; ++it) {
             ok = pend(0);
-            if (ok && it >= own - c0) {
-              pend_tok[0] = tok0[0] + block(0, it - (own - c0), c0) * BLK;
-              pend_kvh[0] = kvh[0];
-              ok = load(&map_k, kvh[0], pend_tok[0]);
-            }
+            if (ok && it >= own - c0) ok = key(0, alone(0, it - (own - c0)));
             if (ok) ok = pend(1);
-            if (ok && it >= own - c1 && (it < own || it == own + both)) {
-              pend_tok[1] = tok0[1] + block(1, it - (own - c1), c1) * BLK;
-              pend_kvh[1] = kvh[1];
-              ok = load(&map_k, kvh[1], pend_tok[1]);
-            }
+            if (ok && it >= own - c1) ok = key(1, alone(1, it - (own - c1)));
           }
+          if (ok && tail) ok = pend(0) && key(0, last(0)) && pend(1) && key(1, last(1));
+          else if (ok && both > 0) ok = shared_round(lead);
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(Smem::merge_empty, b));
         }
@@ -1373,15 +1376,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           if (s0.left > 0) take_q(s0);
           if (s1.left > 0) take_q(s1);
           const int c0 = s0.left - both - tail, c1 = s1.left - both - tail, own = max(c0, c1);
+          const int lead = both - (tail == 0 && both > 0 ? 1 : 0);  // as in the K / V producer
+          for (int it = 0; it < lead; ++it) {
+            round(true, true, true);
+            if (__any_sync(0xffffffffu, failed != 0)) break;
+          }
           for (int it = 0; it < own; ++it) {
             round(it >= own - c0, it >= own - c1, false);
             if (__any_sync(0xffffffffu, failed != 0)) break;
           }
-          for (int it = 0; it < both; ++it) {
-            round(true, true, true);
-            if (__any_sync(0xffffffffu, failed != 0)) break;
-          }
-          if (tail) round(true, true, false);
+          if (tail || both > 0) round(true, true, tail == 0);
           if (__any_sync(0xffffffffu, failed != 0)) break;
         }
         if (!__any_sync(0xffffffffu, failed != 0)) round(false, false, false);
