@@ -294,10 +294,11 @@ int stem_token_attention(const void* Q, const void* K, const void* V, int32_t n_
  * Host only. */
 int stem_token_attention_form(int32_t n_tokens, int32_t num_q_heads, int32_t num_kv_heads, int32_t k_max);
 
-/* Synchronises `stream`, then reads (and clears, if set) the status words of the gather-attention kernel on the
+/* Synchronises `stream`, then reads (and clears, if set) the status words of the token-attention kernels on the
  * current device.  Returns STEM_OK, STEM_ERR_DEVICE_TIMEOUT (a bounded wait in stem_token_attention gave up; the
  * outputs of that call are undefined) or STEM_ERR_CUDA.  detail (optional, HOST int32[4]) receives
- * {4, CTA index, role, barrier id}. */
+ * {4, CTA index, role, barrier id} of the kernel that gathers, or {5, CTA index, role, barrier id} of the one that masks
+ * (each kernel numbers its roles and barriers itself).  If both gave up, the second is reported by the next call. */
 int stem_token_check_status(void* stream, int32_t* detail_host);
 
 /* Synchronises `stream`, then reads the device status words of `workspace` (workspace == NULL: of

@@ -342,7 +342,7 @@ def stem_token_attention_form(n_tokens: int, num_q_heads: int, num_kv_heads: int
 
 
 def stem_token_check_status():
-    """Synchronise the current stream and return (status, detail[4]) of the gather-attention kernel."""
+    """Synchronise the current stream and return (status, detail[4]) of the token-attention kernels."""
     detail = (ctypes.c_int32 * 4)()
     st = load().stem_token_check_status(_stream(), ctypes.cast(detail, ctypes.POINTER(ctypes.c_int32)))
     return int(st), [int(x) for x in detail]

@@ -67,7 +67,7 @@ struct AntiArgs {
 // Bounded wait; false when the time limit ran out (the status words then say so).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* status) {
   if (mbar_wait_bounded(bar, parity, kWaitLimitNs)) return true;
-  if (atomicCAS(status + 4, 0, 3) == 0) { status[5] = (int32_t)blockIdx.x; status[6] = (int32_t)blockIdx.y; }
+  if (atomicCAS(status + 4, 0, kGaveUpAntidiag) == 0) { status[5] = (int32_t)blockIdx.x; status[6] = (int32_t)blockIdx.y; }
   return false;
 }
 

@@ -157,7 +157,7 @@ struct Ctx {
   volatile int* abort_flag;  // shared memory
   int32_t* status;           // global memory status words
   int role;
-  int code;                  // what the first of them says: 1, or 4 for the token-list form
+  int code;                  // what the first of them says
 };
 
 __device__ __forceinline__ void raise_abort(const Ctx& c, int bar_id) {
@@ -587,12 +587,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   constexpr uint32_t kIdescS = make_idesc(BLK, 0);
   constexpr uint32_t kIdescPV = make_idesc(kHeadDim, 1);
   const bool dense = kTok || a.sel_idx == nullptr;
+  constexpr int kGaveUp = kTok ? kGaveUpTokenMasked : kGaveUpAttention;
 
   if (warp < 8) {
     // ============================== softmax of slot X ==============================
     set_max_regs_inc<kRegsSoftmax>();
     const int X = warp >> 2;
-    Ctx ctx{abort_flag, status, kRoleSoftmax, kTok ? 4 : 1};
+    Ctx ctx{abort_flag, status, kRoleSoftmax, kGaveUp};
     const int m = (warp & 3) * 32 + lane;  // query row inside the tile == TMEM lane
     const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_addr = lane_addr + X * 128;
@@ -876,7 +877,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     set_max_regs_dec<kRegsOther>();
     if (warp == 8) {
       // ============================== K / V producer ==============================
-      Ctx ctx{abort_flag, status, kRoleProducer, kTok ? 4 : 1};
+      Ctx ctx{abort_flag, status, kRoleProducer, kGaveUp};
       struct KvSlot {
         ItemCursor<kTok, kSplit, kPair> cur;
         bool has, pend;
@@ -997,7 +998,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // have; behind them the other entries of slot 1's.  A list's last block stays its last (the diagonal is masked in it): if
       // the lists end on different blocks, as those of different rows do, these follow behind the common ones (`tail`).
       // Both lists have to be strictly ascending and of the same kv head and sequence; else they have nothing in common.
-      Ctx ctx{abort_flag, status, kRoleMerge, 1};
+      Ctx ctx{abort_flag, status, kRoleMerge, kGaveUp};
       SlotWalk<kTok, kSplit, kPair> w[2];
       w[0].init(a, 0); w[1].init(a, 1);
       for (int k = 0; !w[0].done() || !w[1].done(); ++k) {
@@ -1080,7 +1081,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
     } else if (warp == 10) {
       // ============================== Q producer ==============================
-      Ctx ctx{abort_flag, status, kRoleQProducer, kTok ? 4 : 1};
+      Ctx ctx{abort_flag, status, kRoleQProducer, kGaveUp};
       if constexpr (kMerge) {
         // The slots' items end in the same round: the tiles go through the three buffers in order, slot 0's first.
         SlotWalk<kTok, kSplit, kPair> w[2];
@@ -1215,7 +1216,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       // a branch when there is nothing to wait for, a wait that gave up is looked at once per round, the MMA loops are
       // unrolled and the list lengths are fetched an item ahead (LengthCursor).  Dense 16K tokens: 1234 TFLOP/s; rolled
       // loops 1200; waits that return a flag and vote 1053; a second warp that checks ahead and queues commands 1197.
-      Ctx ctx{abort_flag, status, kRoleMma, kTok ? 4 : 1};
+      Ctx ctx{abort_flag, status, kRoleMma, kGaveUp};
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
       struct MmaSlot {

@@ -16,6 +16,8 @@ constexpr int kHeadDim = 128;
 //   [0] code (0 = ok, 1 = a bounded wait of the attention kernel gave up)   [1] CTA index   [2] role   [3] barrier id
 //   [4] code (2 = a bounded wait of the metric kernel gave up)   [5] tile   [6] head
 constexpr int kStatusWords = 8;
+// First status word of a kernel whose bounded wait gave up: which kernel.
+enum StatusCode : int32_t { kGaveUpAttention = 1, kGaveUpMetric, kGaveUpAntidiag, kGaveUpTokenGather, kGaveUpTokenMasked };
 constexpr int kRoleSelfTest = 99;  // role recorded by stem_selftest_wait_timeout
 
 // Device-side tables, built once per plan.  Query-block rows and key blocks are numbered separately:
@@ -186,8 +188,8 @@ cudaError_t masked_status_words(int32_t* out4);
 // of the last token of t's tile of `tile` tokens.
 cudaError_t launch_token_masks(const int32_t* sel_idx, const int32_t* sel_cnt, int N, int Hkv, int k_max, int t0, int t1, int tile, void* masks,
                                int64_t st, int64_t sh, cudaStream_t s);
-// The status words {4, CTA, role, barrier} of the gather-attention kernel on the current device, read to the host
-// and cleared when set (the caller has synchronised).
+// The status words {4, CTA, role, barrier} of the gather-attention kernel on the current device or, if that has none to
+// report, {5, CTA, role, barrier} of the masked form, read to the host and cleared when set (the caller has synchronised).
 cudaError_t token_status_words(int32_t* out4);
 
 // One thread waits 1 ms on a barrier nobody arrives at and records the time-out in status words 0..3.

@@ -18,7 +18,7 @@ __global__ void selftest_wait_kernel(int32_t* status) {
   ptx::mbar_init_fence();
   // phase 0 of a barrier that expects one arrival and never gets it
   if (!ptx::mbar_wait_bounded(bar_addr, 0, kSelfTestLimitNs)) {
-    if (atomicCAS(status, 0, 1) == 0) {
+    if (atomicCAS(status, 0, kGaveUpAttention) == 0) {
       status[1] = (int32_t)blockIdx.x;
       status[2] = kRoleSelfTest;
       status[3] = 0;

@@ -91,7 +91,7 @@ struct Ctx {
 __device__ __forceinline__ void give_up(const Ctx& c, int which) {
   if (!*c.abort) {
     *c.abort = 1;
-    if (atomicCAS(&g_token_status[0], 0, 4) == 0) {
+    if (atomicCAS(&g_token_status[0], 0, kGaveUpTokenGather) == 0) {
       g_token_status[1] = (int32_t)blockIdx.x;
       g_token_status[2] = c.role;
       g_token_status[3] = which;
