@@ -309,10 +309,10 @@ int stem_token_check_status(void* stream, int32_t* detail_host);
  * the wait that gave up was in the metric kernel ({3, tile, query head, 0}: its anti-diagonal form). */
 int stem_check_status(const stem_plan* plan, void* workspace, void* stream, int32_t* detail_host);
 
-/* Self-test of the time-out reporting (the paper has no counterpart).  Enqueues a one-thread kernel
- * that waits 1 ms, with the same bounded-wait routine the attention and metric kernels use, on a
- * barrier nothing ever arrives at, records {1, 0, 99, 0} in the workspace status words and returns
- * normally.  A following stem_check_status must report STEM_ERR_DEVICE_TIMEOUT; the CUDA context
+/* Self-test of the time-out reporting (the paper has no counterpart).  Enqueues two small kernels
+ * that wait 1 ms, with each of the bounded-wait routines the attention and metric kernels use, on a
+ * barrier nothing ever arrives at, record {1, 0, 99, 0} in the workspace status words (a number other
+ * than 0 at the end: the check that failed) and return normally.  A following stem_check_status must report STEM_ERR_DEVICE_TIMEOUT; the CUDA context
  * stays usable.  Never needed in production. */
 int stem_selftest_wait_timeout(const stem_plan* plan, void* workspace, size_t workspace_bytes, void* stream);
 

@@ -193,7 +193,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const C
 // The issuer's form of the bounded wait: nothing but the probe and one branch when the phase is complete.  A wait that
 // gives up raises the CTA's abort flag and leaves `id` in `failed`, which the caller looks at when it is cheap to; what
 // it issues in between works on undefined data inside the CTA's own shared and tensor memory.
-__device__ __forceinline__ void mbar_wait_sticky(uint32_t bar, uint32_t parity, uint32_t abort_addr, int id, int& failed) {
+__device__ __forceinline__ void mbar_wait_sticky(uint32_t bar, uint32_t parity, uint32_t abort_addr, int id, int& failed,
+                                                 uint64_t limit_ns = kWaitLimitNs) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 f;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -216,7 +217,7 @@ __device__ __forceinline__ void mbar_wait_sticky(uint32_t bar, uint32_t parity, 
       "st.volatile.shared::cta.u32 [%3], 1;\n\t"
       "DONE_%=:\n\t}"
       : "+r"(failed)
-      : "r"(bar), "r"(parity), "r"(abort_addr), "r"(id), "l"(kWaitLimitNs)
+      : "r"(bar), "r"(parity), "r"(abort_addr), "r"(id), "l"(limit_ns)
       : "memory");
 }
 
@@ -1426,6 +1427,44 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   }
 }
 
+// Both waits of this file run out, with a limit of 1 ms, on a barrier that nothing arrives at: the issuer's has to leave its id
+// and raise the abort flag, after which another of either kind gives up at once; the other has to record the status words.
+// What does not behave is recorded as its number in the place of the barrier.
+__global__ void selftest_waits_kernel(int32_t* status) {
+  __shared__ __align__(8) uint64_t bar_mem;
+  __shared__ int abort_mem;
+  constexpr uint64_t kLimitNs = 1000ull * 1000;
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&bar_mem), abort_addr = (uint32_t)__cvta_generic_to_shared(&abort_mem);
+  volatile int* const abort_flag = &abort_mem;
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    abort_mem = 0;
+  }
+  __syncthreads();
+  const Ctx ctx{abort_flag, status, kRoleSelfTest, kGaveUpAttention};
+  int bad = 0;  // the last check that failed
+  auto expect = [&](const bool good, const int what) {
+    if (!__all_sync(0xffffffffu, good)) bad = what;
+  };
+  int failed = 0;
+  const uint64_t t0 = globaltimer();
+  mbar_wait_sticky(bar, 1, abort_addr, 41, failed, kLimitNs);  // the phase before the first counts as complete
+  expect(failed == 0 && *abort_flag == 0, 1);
+  mbar_wait_sticky(bar, 0, abort_addr, 42, failed, kLimitNs);
+  expect(failed == 42 && *abort_flag != 0 && globaltimer() - t0 >= kLimitNs, 2);
+  const uint64_t t1 = globaltimer();
+  mbar_wait_sticky(bar, 0, abort_addr, 43, failed);
+  expect(failed == 43 && !mbar_wait(bar, 0, ctx, 44) && globaltimer() - t1 < kWaitLimitNs / 4, 3);
+  __syncthreads();
+  if (threadIdx.x == 0) *abort_flag = 0;
+  __syncthreads();
+  const bool gave_up = !mbar_wait(bar, 0, ctx, bad, kLimitNs);
+  bad = 0;
+  expect(gave_up && *abort_flag != 0, 4);
+  if (bad != 0 && threadIdx.x == 0) atomicMax(status + 3, bad);
+}
+
 // ------------------------------------------------------------------------------------------------
 // host side: tensor maps and launch
 // ------------------------------------------------------------------------------------------------
@@ -1437,6 +1476,11 @@ bool make_map(CUtensorMap* map, const void* base, int64_t T, int H, int64_t stri
 }
 
 }  // namespace
+
+cudaError_t launch_selftest_waits(int32_t* status, cudaStream_t s) {
+  selftest_waits_kernel<<<1, 32, 0, s>>>(status);
+  return cudaGetLastError();
+}
 
 int attention_merge_max_list() { return kMergeMaxList; }
 

@@ -192,8 +192,9 @@ cudaError_t launch_token_masks(const int32_t* sel_idx, const int32_t* sel_cnt, i
 // report, {5, CTA, role, barrier} of the masked form, read to the host and cleared when set (the caller has synchronised).
 cudaError_t token_status_words(int32_t* out4);
 
-// One thread waits 1 ms on a barrier nobody arrives at and records the time-out in status words 0..3.
+// All kinds of bounded waits run out on a barrier nobody arrives at; the time-out is recorded in status words 0..3.
 cudaError_t launch_selftest_wait(int32_t* status, cudaStream_t s);
+cudaError_t launch_selftest_waits(int32_t* status, cudaStream_t s);  // those of the attention kernel
 
 // Status words of the scratch built into the library (stem_score_static) on the current device.
 int static_scratch_status_words(int device, int32_t** out);

@@ -1,8 +1,8 @@
 // stem_selftest_wait_timeout: exercises the bounded-wait machinery of the library without touching
-// the production kernels.  One thread waits, with a 1 ms limit, on an mbarrier that nothing ever
-// arrives at, using the same helper the attention and metric kernels wait with; when the limit runs
-// out it records a status code the way those kernels do and returns normally.  The context stays
-// usable; stem_check_status then reports STEM_ERR_DEVICE_TIMEOUT.
+// the production kernels.  The waits of the attention kernel and then the helper that the metric and
+// gather kernels wait with run out, with a 1 ms limit, on an mbarrier that nothing ever arrives at; a
+// status code is recorded the way those kernels do and the kernels return normally.  The context
+// stays usable; stem_check_status then reports STEM_ERR_DEVICE_TIMEOUT.
 #include "stem_internal.h"
 #include "stem_ptx.cuh"
 
@@ -17,18 +17,14 @@ __global__ void selftest_wait_kernel(int32_t* status) {
   ptx::mbar_init(bar_addr, 1);
   ptx::mbar_init_fence();
   // phase 0 of a barrier that expects one arrival and never gets it
-  if (!ptx::mbar_wait_bounded(bar_addr, 0, kSelfTestLimitNs)) {
-    if (atomicCAS(status, 0, kGaveUpAttention) == 0) {
-      status[1] = (int32_t)blockIdx.x;
-      status[2] = kRoleSelfTest;
-      status[3] = 0;
-    }
-  }
+  if (ptx::mbar_wait_bounded(bar_addr, 0, kSelfTestLimitNs)) atomicMax(status + 3, 5);  // it must not succeed
 }
 
 }  // namespace
 
 cudaError_t launch_selftest_wait(int32_t* status, cudaStream_t s) {
+  cudaError_t e = launch_selftest_waits(status, s);
+  if (e != cudaSuccess) return e;
   selftest_wait_kernel<<<1, 1, 0, s>>>(status);
   return cudaGetLastError();
 }

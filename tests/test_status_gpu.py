@@ -3,9 +3,10 @@
 A bounded device-side wait that gives up records a code in the status words at the start of the
 workspace; stem_check_status turns it into STEM_ERR_DEVICE_TIMEOUT, hands out the detail words and
 clears them.  Two forms: (i) the words are written from the host, as the attention kernel and the
-metric kernel would write them; (ii) the library's self-test kernel really waits (1 ms limit) on a
-barrier nothing arrives at, with the routine the production kernels wait with, and records the
-time-out itself.  Neither hangs, traps or faults; the context stays usable, which the tests check
+metric kernel would write them; (ii) the library's self-test kernels really wait (1 ms limit) on a
+barrier nothing arrives at, with the routines the production kernels wait with (the attention
+kernel's two, one of which only leaves an id and raises the abort flag, and the shared one), and
+record the time-out themselves; the last word is the number of the check that failed, if any.  Neither hangs, traps or faults; the context stays usable, which the tests check
 by running the real path afterwards and comparing bit for bit."""
 import pytest
 import torch
