@@ -20,6 +20,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "stem_internal.h"
 #include "stem_ptx.cuh"
@@ -261,31 +262,40 @@ __global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const An
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[q][c] = 0.f;
       }
-#pragma unroll 2
-      for (int s = s_lo + 2 * which + half; s < BLK; s += 4) {
-        uint4 kv[4], qv[4];
+      // kDiag: one of the columns is block r itself, which has no key for some of the queries (0 for the key is not enough: the
+      // query may be infinite)
+      auto products = [&](auto diag) {
+        constexpr bool kDiag = decltype(diag)::value;
+#pragma unroll(kDiag ? 1 : 2)
+        for (int s = s_lo + 2 * which + half; s < BLK; s += 4) {
+          uint4 kv[4], qv[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) kv[c] = s < s_hi[c] ? *(const uint4*)(kcol[c] + (int64_t)s * a.kv_st) : make_uint4(0, 0, 0, 0);
+          for (int c = 0; c < 4; ++c) kv[c] = s < s_hi[c] ? *(const uint4*)(kcol[c] + (int64_t)s * a.kv_st) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) qv[q] = *(const uint4*)(qh[q] + (int64_t)(BLK - 1 - s) * a.q_st);
+          for (int q = 0; q < 4; ++q) qv[q] = *(const uint4*)(qh[q] + (int64_t)(BLK - 1 - s) * a.q_st);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float kl[4], kh[4];
+          for (int i = 0; i < 4; ++i) {
+            float kl[4], kh[4];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t w = i == 0 ? kv[c].x : i == 1 ? kv[c].y : i == 2 ? kv[c].z : kv[c].w;
-            kl[c] = __uint_as_float(w << 16);
-            kh[c] = __uint_as_float(w & 0xffff0000u);
-          }
+            for (int c = 0; c < 4; ++c) {
+              const uint32_t w = i == 0 ? kv[c].x : i == 1 ? kv[c].y : i == 2 ? kv[c].z : kv[c].w;
+              kl[c] = __uint_as_float(w << 16);
+              kh[c] = __uint_as_float(w & 0xffff0000u);
+            }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t w = i == 0 ? qv[q].x : i == 1 ? qv[q].y : i == 2 ? qv[q].z : qv[q].w;
-            const float ql = __uint_as_float(w << 16), qu = __uint_as_float(w & 0xffff0000u);
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t w = i == 0 ? qv[q].x : i == 1 ? qv[q].y : i == 2 ? qv[q].z : qv[q].w;
+              const float ql = __uint_as_float(w << 16), qu = __uint_as_float(w & 0xffff0000u);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[q][c] = fmaf(qu, kh[c], fmaf(ql, kl[c], acc[q][c]));
+              for (int c = 0; c < 4; ++c) {
+                const float sum = fmaf(qu, kh[c], fmaf(ql, kl[c], acc[q][c]));
+                acc[q][c] = kDiag && s >= s_hi[c] ? acc[q][c] : sum;
+              }
+            }
           }
         }
-      }
+      };
+      if (j0 + c0 + 3 >= r) products(std::true_type{}); else products(std::false_type{});
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
 #pragma unroll

@@ -138,3 +138,24 @@ def test_antidiagonal_metric_row_of_a_partial_last_block(block, seqlens, hq, hkv
     assert np.array_equal(np.isnan(M_g), ~defined)
     assert np.all(np.abs(M_g[defined] - M_ref[defined]) <= METRIC_ABS + METRIC_REL * np.abs(M_ref[defined]))
     plan.close()
+
+
+def test_a_query_without_a_partner_in_the_last_block_leaves_its_own_entry_alone():
+    # 40 of 64 tokens: token t of the last block meets key 63 - t of block j; of the block itself only the keys 24 .. 39 exist
+    w = wl.small("ad_inf", seqlens=(64 * 5 + 40,), hq=2, hkv=1, block=64, permille=200, seed=3)
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w, score_mode=1)
+    nb = 6
+    rows = []
+    for bad in (False, True):
+        if bad:
+            q[5 * 64 + 5, 0] = float("inf")
+        M = torch.full((2, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_score(plan, q, k, v, M)
+        assert binding.stem_check_status(plan)[0] == 0
+        rows.append(M.cpu().numpy()[:, -nb:])
+    assert not np.isfinite(rows[1][0, :nb - 1]).any()
+    assert rows[1][0, nb - 1] == rows[0][0, nb - 1] and np.isfinite(rows[0][0, nb - 1])
+    assert np.array_equal(rows[1][1], rows[0][1])
+    plan.close()
