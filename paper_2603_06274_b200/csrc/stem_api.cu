@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <numeric>
 
@@ -71,8 +72,9 @@ static int validate(const stem_config* c) {
 // Neighbours with lists of their own go to the two slots of a CTA as well, from more than `merge_from` items on, for the
 // blocks that both lists name (one by one / together, us: 160 items 21 / 23, 192 29 / 24, 256 29 / 25, 320 31 / 27).
 // Where there are no more items than SMs every CTA has one item (whose list its slots share).
+// items: [n_items][2]; slot_off: room for 2 sm_count + 1; owner: scratch, an entry for each item.
 static void deal_items(const Plan& p, const std::vector<int32_t>& order, const std::vector<int32_t>& len, int pairs_from, int merge_from, AttnWork* w,
-                       std::vector<int32_t>& items, std::vector<int32_t>& slot_off) {
+                       int32_t* items, int32_t* slot_off, int32_t* owner) {
   const int Hq = p.cfg.num_q_heads, Hkv = p.cfg.num_kv_heads, g = Hq / Hkv;
   w->pair = g % 2 == 0 && p.n_items > pairs_from;
   w->merge = !w->pair && p.n_items > merge_from;
@@ -103,46 +105,71 @@ static void deal_items(const Plan& p, const std::vector<int32_t>& order, const s
     for (int c = 0; c < w->ctas; ++c) append(0, 2 * c);
     for (int c = w->ctas - 1; c >= 0; --c) append(0, 2 * c + 1);
   }
-  // f(number, head, row) for every item: `rows` rows at a time of one kv head after the other
+  // f(kv head, row) for the items of the query heads of a group: `rows` rows at a time of one kv head after the other
   const bool by_row = total * Hq / n_slots < 3 * longest;
   const int rows = !by_row ? p.R_tot : unit == 2 && g % 2 ? 2 : 1;
   auto each = [&](auto f) {
-    int i = 0;
     for (int r0 = 0; r0 < p.R_tot; r0 += rows)
       for (int kvh = 0; kvh < Hkv; ++kvh)
-        for (int r = r0; r < std::min(r0 + rows, p.R_tot); ++r)
-          for (int q = 0; q < g; ++q, ++i) f(i, kvh * g + q, order[r]);
+        for (int r = r0; r < std::min(r0 + rows, p.R_tot); ++r) f(kvh, order[r]);
   };
-  std::vector<int32_t> owner(p.n_items), count(n_slots + 1, 0);
+  std::vector<int32_t> at(n_slots + 1, 0);
   uint32_t time = 0;
   int32_t queue = 0;
-  each([&](int i, int, int32_t R) {
-    if ((i & (unit - 1)) == 0) {
-      while (first[time] < 0) time = (time + 1) & (ring - 1);
-      queue = first[time];
-      first[time] = next[queue];
-      append(time + 2 * len[R] + 1, queue);
+  int i = 0;
+  each([&](int, int32_t R) {
+    const uint32_t weight = 2 * len[R] + 1;
+    for (const int end = i + g; i < end; ++i) {
+      const int second = i & (unit - 1);
+      if (second == 0) {
+        while (first[time] < 0) time = (time + 1) & (ring - 1);
+        queue = first[time];
+        first[time] = next[queue];
+        append(time + weight, queue);
+      }
+      owner[i] = unit * queue + second;
+      ++at[owner[i] + 1];
     }
-    owner[i] = unit * queue + (i & (unit - 1));
-    ++count[owner[i] + 1];
   });
-  for (int s = 0; s < n_slots; ++s) count[s + 1] += count[s];
-  slot_off = count;
-  items.resize(2 * (size_t)p.n_items);
-  each([&](int i, int h, int32_t R) {
-    const int32_t at = count[owner[i]]++;
-    items[2 * at] = h;
-    items[2 * at + 1] = R;
+  for (int s = 0; s < n_slots; ++s) at[s + 1] += at[s];
+  std::copy(at.begin(), at.end(), slot_off);
+  i = 0;
+  each([&](int kvh, int32_t R) {
+    for (int h = kvh * g; h < (kvh + 1) * g; ++h, ++i) {
+      int32_t* item = items + 2 * (size_t)at[owner[i]]++;
+      item[0] = h;
+      item[1] = R;
+    }
   });
 }
 
-template <class T>
-static size_t push(std::vector<uint8_t>& blob, const std::vector<T>& v) {
-  size_t off = align_up(blob.size(), 256);
-  blob.resize(off + std::max<size_t>(v.size() * sizeof(T), 1));
-  if (!v.empty()) std::memcpy(blob.data() + off, v.data(), v.size() * sizeof(T));
-  return off;
-}
+// A plan's tables as they lie in its device memory: room is taken for all of them first, then they are written in place.
+struct Blob {
+  size_t size = 0;
+  std::unique_ptr<uint8_t[]> bytes;
+  struct Part {
+    size_t off;
+    const void* src;
+    size_t n;
+  };
+  std::vector<Part> parts;
+  size_t take(size_t n) {
+    const size_t off = align_up(size, 256);
+    size = off + std::max<size_t>(n, 1);
+    return off;
+  }
+  template <class T>
+  size_t add(const std::vector<T>& v) {
+    const size_t n = v.size() * sizeof(T);
+    parts.push_back({take(n), v.data(), n});
+    return parts.back().off;
+  }
+  void write() {
+    bytes.reset(new uint8_t[size]);
+    for (const Part& x : parts)
+      if (x.n) std::memcpy(bytes.get() + x.off, x.src, x.n);
+  }
+};
 
 // Frees everything a plan owns (also a half-built one).
 static void release_plan(stem_plan* sp) {
@@ -151,32 +178,7 @@ static void release_plan(stem_plan* sp) {
   delete sp;
 }
 
-}  // namespace stem
-
-using namespace stem;
-
-extern "C" {
-
-int stem_version(void) { return 100; }
-
-const char* stem_status_string(int s) {
-  switch (s) {
-    case STEM_OK: return "ok";
-    case STEM_ERR_INVALID_ARG: return "invalid argument";
-    case STEM_ERR_UNSUPPORTED: return "unsupported configuration";
-    case STEM_ERR_WORKSPACE: return "workspace missing or too small";
-    case STEM_ERR_CUDA: return "CUDA error";
-    case STEM_ERR_DEVICE_TIMEOUT: return "a bounded device-side wait gave up";
-    case STEM_ERR_STATIC_SCRATCH: return "problem exceeds the built-in scratch of the allocation-free entry point";
-    default: return "unknown status";
-  }
-}
-
-int stem_plan_create(const stem_config* cfg, stem_plan** out) { return stem_plan_create_ex(cfg, nullptr, out); }
-
-int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_plan** out) {
-  if (!out) return STEM_ERR_INVALID_ARG;
-  *out = nullptr;
+static int create_plan(const stem_config* cfg, const stem_options* opts, stem_plan** out) {
   int rc = validate(cfg);
   if (rc != STEM_OK) return rc;
   stem_options o{};
@@ -198,8 +200,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     if (o.kcache_blocks_per_seq > 0 && (kv_len + B - 1) / B > o.kcache_blocks_per_seq) return STEM_ERR_INVALID_ARG;
   }
 
-  stem_plan* sp = new (std::nothrow) stem_plan();
-  if (!sp) return STEM_ERR_CUDA;
+  std::unique_ptr<stem_plan, void (*)(stem_plan*)> sp(new stem_plan(), release_plan);
   Plan& p = sp->p;
   p.cfg = *cfg;
   p.cu.assign(cfg->cu_seqlens_host, cfg->cu_seqlens_host + cfg->batch + 1);
@@ -281,7 +282,6 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   p.causal_pairs *= Hq;
 
   if (p.max_nblk > row_select_max_blocks()) {
-    delete sp;
     return STEM_ERR_UNSUPPORTED;
   }
 
@@ -309,13 +309,25 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   if (cudaGetDevice(&p.device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p.sm_count, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) {
     cudaGetLastError();
-    delete sp;
     return STEM_ERR_CUDA;
   }
 
-  // Attention work order: kv-head-major so that the K/V of one kv head stay hot in L2; inside a
-  // kv head, rows by descending list length (longest first), the g heads of a row together.
-  std::vector<int32_t> work_sparse, work_dense, slots_sparse, slots_dense;
+  p.n_items = p.R_tot * Hq;
+
+  Blob blob;
+  const size_t o_row_seq = blob.add(row_seq), o_row_r = blob.add(row_r), o_row_tok0 = blob.add(row_tok0),
+               o_row_ntok = blob.add(row_ntok), o_keff = blob.add(p.k_eff), o_seq_tok0 = blob.add(seq_tok0),
+               o_seq_nblk = blob.add(seq_nblk), o_seq_r0 = blob.add(seq_r0), o_seq_row_off = blob.add(seq_row_off),
+               o_seq_kb_off = blob.add(seq_kb_off), o_seq_kb_first = blob.add(seq_kb_first), o_seq_m_off = blob.add(seq_m_off),
+               o_seq_mt_off = blob.add(seq_mt_off), o_kb_tok0 = blob.add(kb_tok0), o_kb_ntok = blob.add(kb_ntok),
+               o_kb_dst = blob.add(kb_dst), o_kb_new = blob.add(kb_new), o_gt = blob.add(gemm_tiles),
+               o_lr = blob.add(long_rows), o_sr = blob.add(short_rows);
+  const size_t item_bytes = 2 * (size_t)p.n_items * sizeof(int32_t), slot_bytes = (2 * (size_t)p.sm_count + 1) * sizeof(int32_t);
+  const size_t o_ws = blob.take(item_bytes), o_wd = blob.take(item_bytes), o_ss = blob.take(slot_bytes), o_sd = blob.take(slot_bytes);
+  blob.write();
+
+  // Attention work order: rows by descending list length (longest first), the g heads of a row together; kv-head-major so
+  // that the K / V of one kv head stay hot in L2, or row by row where a slot has few items (deal_items).
   {
     std::vector<int32_t> by_len(p.R_tot), by_r(p.R_tot), len_dense(p.R_tot);
     std::iota(by_len.begin(), by_len.end(), 0);
@@ -323,11 +335,12 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
     std::stable_sort(by_len.begin(), by_len.end(), [&](int a, int b) { return p.k_eff[a] > p.k_eff[b]; });
     std::stable_sort(by_r.begin(), by_r.end(), [&](int a, int b) { return row_r[a] > row_r[b]; });
     for (int R = 0; R < p.R_tot; ++R) len_dense[R] = row_r[R] + 1;
-    p.n_items = p.R_tot * Hq;
     const int few = 5 * p.sm_count / 4;
-    deal_items(p, by_len, p.k_eff, p.share_group ? few : p.n_items,
-               p.k_max <= attention_merge_max_list() ? few : p.n_items, &p.work_sparse, work_sparse, slots_sparse);
-    deal_items(p, by_r, len_dense, 3 * p.sm_count, 3 * p.sm_count, &p.work_dense, work_dense, slots_dense);
+    const std::unique_ptr<int32_t[]> owner(new int32_t[p.n_items]);
+    auto ints = [&](size_t off) { return (int32_t*)(blob.bytes.get() + off); };
+    deal_items(p, by_len, p.k_eff, p.share_group ? few : p.n_items, p.k_max <= attention_merge_max_list() ? few : p.n_items,
+               &p.work_sparse, ints(o_ws), ints(o_ss), owner.get());
+    deal_items(p, by_r, len_dense, 3 * p.sm_count, 3 * p.sm_count, &p.work_dense, ints(o_wd), ints(o_sd), owner.get());
   }
 
   // Workspace layout.  With a caller-owned cache the K-side tensors are not part of the workspace.
@@ -345,20 +358,9 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   }
 
   // Upload tables.
-  std::vector<uint8_t> blob;
-  const size_t o_row_seq = push(blob, row_seq), o_row_r = push(blob, row_r), o_row_tok0 = push(blob, row_tok0),
-               o_row_ntok = push(blob, row_ntok), o_keff = push(blob, p.k_eff), o_seq_tok0 = push(blob, seq_tok0),
-               o_seq_nblk = push(blob, seq_nblk), o_seq_r0 = push(blob, seq_r0), o_seq_row_off = push(blob, seq_row_off),
-               o_seq_kb_off = push(blob, seq_kb_off), o_seq_kb_first = push(blob, seq_kb_first), o_seq_m_off = push(blob, seq_m_off),
-               o_seq_mt_off = push(blob, seq_mt_off), o_kb_tok0 = push(blob, kb_tok0), o_kb_ntok = push(blob, kb_ntok),
-               o_kb_dst = push(blob, kb_dst), o_kb_new = push(blob, kb_new), o_gt = push(blob, gemm_tiles),
-               o_ws = push(blob, work_sparse), o_wd = push(blob, work_dense), o_ss = push(blob, slots_sparse),
-               o_sd = push(blob, slots_dense), o_lr = push(blob, long_rows), o_sr = push(blob, short_rows);
-  if (cudaMalloc(&p.d_blob, blob.size()) != cudaSuccess ||
-      cudaMemcpy(p.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (cudaMalloc(&p.d_blob, blob.size) != cudaSuccess ||
+      cudaMemcpy(p.d_blob, blob.bytes.get(), blob.size, cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaGetLastError();
-    if (p.d_blob) cudaFree(p.d_blob);
-    delete sp;
     return STEM_ERR_CUDA;
   }
   const uint8_t* d = (const uint8_t*)p.d_blob;
@@ -386,8 +388,41 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   p.work_sparse.d_slot_off = (const int32_t*)(d + o_ss);
   p.work_dense.d_items = (const int32_t*)(d + o_wd);
   p.work_dense.d_slot_off = (const int32_t*)(d + o_sd);
-  *out = sp;
+  *out = sp.release();
   return STEM_OK;
+}
+
+}  // namespace stem
+
+using namespace stem;
+
+extern "C" {
+
+int stem_version(void) { return 100; }
+
+const char* stem_status_string(int s) {
+  switch (s) {
+    case STEM_OK: return "ok";
+    case STEM_ERR_INVALID_ARG: return "invalid argument";
+    case STEM_ERR_UNSUPPORTED: return "unsupported configuration";
+    case STEM_ERR_WORKSPACE: return "workspace missing or too small";
+    case STEM_ERR_CUDA: return "CUDA error";
+    case STEM_ERR_DEVICE_TIMEOUT: return "a bounded device-side wait gave up";
+    case STEM_ERR_STATIC_SCRATCH: return "problem exceeds the built-in scratch of the allocation-free entry point";
+    default: return "unknown status";
+  }
+}
+
+int stem_plan_create(const stem_config* cfg, stem_plan** out) { return stem_plan_create_ex(cfg, nullptr, out); }
+
+int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_plan** out) {
+  if (!out) return STEM_ERR_INVALID_ARG;
+  *out = nullptr;
+  try {
+    return create_plan(cfg, opts, out);
+  } catch (const std::bad_alloc&) {  // no exception leaves a C entry
+    return STEM_ERR_CUDA;
+  }
 }
 
 int stem_plan_destroy(stem_plan* plan) {
