@@ -52,6 +52,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cfloat>
 
 #include "stem_internal.h"
 #include "stem_ptx.cuh"
@@ -709,7 +710,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         const float mx_c = fmaxf(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], max3(mx[5], mx[6], mx[7]))) * a.scale_log2;
         if (e == 0) {
-          m_run = kTok ? fmaxf(mx_c, -1e30f) : mx_c;  // finite: a block may hold no token of the row's list
+          m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
         } else {
           const bool grow = mx_c > m_run + kRescaleThreshold;
           if (__any_sync(0xffffffffu, grow)) {

@@ -553,3 +553,25 @@ def test_blocks_shared_by_two_heads_cost_no_precision(block, blocks, hq, hkv, pe
         err.append(num ** 0.5)
     print(f"error against 64 bits: common blocks together {err[0]:.5e}, in list order {err[1]:.5e}")
     assert abs(err[0] / err[1] - 1.0) <= 3e-3
+
+
+@pytest.mark.parametrize("seqlen", [6 * 64, 80 * 64])
+def test_a_block_of_keys_at_minus_infinity_draws_nothing(seqlen):
+    # positive queries, so that such a key's scores are -inf; of the dense lists of up to 6 blocks (12 items, cut in halves for
+    # the two slots) and of 80 (in list order) any block but the first may be one, also where a half begins
+    r = np.random.default_rng(seqlen)
+    n = seqlen // 64
+    q = torch.from_numpy(np.abs(r.standard_normal((seqlen, 2, 128), dtype=np.float32)) + 0.1).to(torch.bfloat16).cuda()
+    k = torch.from_numpy(r.standard_normal((seqlen, 1, 128), dtype=np.float32)).to(torch.bfloat16).cuda()
+    v = torch.from_numpy(r.standard_normal((seqlen, 1, 128), dtype=np.float32)).to(torch.bfloat16).cuda()
+    plan = StemPlan((seqlen,), 2, 1, block=64, budget_permille=1000, mu=(1, 1))
+    for bad in (1, 2, 3, n - 2):
+        kb = k.clone()
+        kb[bad * 64:(bad + 1) * 64] = float("-inf")
+        out = torch.full_like(q, float("nan"))
+        binding.stem_sparse_prefill(plan, q, kb, v, None, None, out)
+        assert binding.stem_check_status(plan)[0] == 0
+        s = torch.einsum("thd,sd->hts", q.double(), kb[:, 0].double()) / 128.0 ** 0.5
+        s = s.masked_fill(torch.ones((seqlen, seqlen), dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+        ref = torch.einsum("hts,sd->thd", torch.softmax(s, 2), v[:, 0].double())
+        check_attention(from_dev_bf16(out), ref.cpu().numpy(), label=f"{n} blocks, keys of block {bad} at -inf")
