@@ -137,3 +137,14 @@ def test_token_level_budget_is_the_schedule_with_one_token_per_block():
     uncapped = np.floor(k_s - k_s * 0.3 * np.arange(1, n + 1) / n)
     assert abs(uncapped.mean() / k_s - 0.85) < 1e-3
     assert got[-1] == int(0.7 * k_s) and got[0] == 1 and got[k_s + 500] == uncapped[k_s + 500]
+
+
+def test_current_stream_handle_without_the_private_function(monkeypatch):
+    # torch's raw-handle function is private: where it is missing the public Stream object serves
+    import types
+    monkeypatch.setattr(binding.torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 100 + device)
+    assert binding._stream() == 103
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    assert binding._stream() == 77
