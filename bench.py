@@ -493,8 +493,8 @@ def main():
         score_bytes = hkv * n * (n + 1) // 2 * 4
         res["token_level_top2048_8k"] = {"select_ms": t["select"][0], "attention_ms": t["attention"][0],
                                          "select_gbs_on_causal_scores": score_bytes / (t["select"][0] * 1e-3) / 1e9,
-                                         "gathered_gb_per_launch": listed * 512 / 1e9,
-                                         "gather_gbs": listed * 512 / (t["attention"][0] * 1e-3) / 1e9,
+                                         "attention_form": pkg.stem_token_attention_form(n, wt.num_q_heads, hkv, k_max),
+                                         "listed_kv_gb": listed * 512 / 1e9,   # K and V rows of all lists, once per list
                                          "attention_tflops": 4.0 * 128 * listed * (wt.num_q_heads // hkv) / (t["attention"][0] * 1e-3) / 1e12}
         return res
 
