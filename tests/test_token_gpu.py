@@ -235,9 +235,11 @@ def test_token_attention_forms(n, hq, hkv, k_max, order, repeat, what):
     assert np.isfinite(got).all()
 
 
-def test_token_attention_ignores_rows_no_list_names():
-    # a value row that is not finite reaches only the queries whose lists name it, and so does a key row
-    n, hq, hkv, k_max = 400, 4, 2, 100
+@pytest.mark.parametrize("shape,form", [((1500, 4, 2, 100), "masked"), ((400, 4, 2, 100), None), ((200, 4, 2, 100), "gather")])
+def test_token_attention_ignores_rows_no_list_names(shape, form):
+    # a value row that is not finite reaches only the queries whose lists name it, and so does a key row, in either form
+    n, hq, hkv, k_max = shape
+    assert form in (None, binding.stem_token_attention_form(n, hq, hkv, k_max))
     w = wl.small("token_nan", seqlens=(n,), hq=hq, hkv=hkv, block=64, permille=100, sink=False, seed=5)
     data = wl.make_qkv(w)
     r = np.random.default_rng(5)
