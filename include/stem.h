@@ -215,15 +215,19 @@ int stem_select(const stem_plan* plan, const float* M, int32_t* sel_idx, int32_t
 
 /* Alg. 1 steps 1-3c in one call: block-wise representations, Output-Aware Metric (Eq. 7), Token
  * Position-Decay budget (Eq. 3) and top-k selection; the metric is kept in the workspace (as bit
- *   planes of its order-preserving selection keys, part of workspace_bytes), never handed to the caller.
- *   Same results as stem_score(M = NULL) followed by stem_select(M = NULL).
+ *   planes of its order-preserving selection keys, part of workspace_bytes) or, for sequences of up to 64 blocks, in
+ *   registers, never handed to the caller.  Same lists, bit for bit, as stem_score(M) and stem_select(M), M = NULL or not.
+ *   A sequence's lists depend on that sequence alone: they are the same in any batch, in any split into chunks (with
+ *   total_len given) and with the heads in any number of plans.
  *   Writes sel_idx / sel_cnt; leaves the pooled tensors in the workspace. */
 int stem_score_select(const stem_plan* plan, const void* Q, const void* K, const void* V, int32_t* sel_idx,
                       int32_t* sel_cnt, void* workspace, size_t workspace_bytes, void* stream);
 
 /* Alg. 1 step 3d.
  *   O[t,h,:] = softmax_k( Q[t,h].K[k,kv(h)] * softmax_scale ) V over the keys k of the listed
- *   blocks of t's row with position <= t.  sel_idx == NULL (with sel_cnt == NULL) means every
+ *   blocks of t's row with position <= t.  The blocks' contributions are added up in an order that depends on what else
+ *   the plan holds, so O is the same from plan to plan up to the rounding of its sums and of P to bf16 (about 2e-3 of its
+ *   norm), and bit for bit from call to call.  sel_idx == NULL (with sel_cnt == NULL) means every
  *   causal block, i.e. dense causal attention.  Lists must be ascending and within [0, r];
  *   out-of-range ids are clamped, never dereferenced.  lse (fp32 [num_q_heads, T], natural-log
  *   sum-exp of the scaled scores) is optional (NULL to skip). */
@@ -275,12 +279,14 @@ int stem_token_budget(int32_t n_tokens, int32_t k_start, int32_t mu_num, int32_t
 int stem_token_select(const float* scores, int32_t n_tokens, int32_t list_heads, const int32_t* k_tok, int32_t stem_tokens,
                       int32_t local_tokens, int32_t k_max, int32_t* sel_idx, int32_t* sel_cnt, void* stream);
 
-/* Gather-style attention over token lists: O[t,h] = softmax_s( Q[t,h].K[s,kv(h)] * softmax_scale ) V over the tokens
+/* Attention over token lists: O[t,h] = softmax_s( Q[t,h].K[s,kv(h)] * softmax_scale ) V over the tokens
  * s of list (kv(h), t) (ids are clamped to [0, t], never dereferenced out of range; at most min(k_max, t+1) entries
  * of a list are used).  Lists are per kv head ([num_kv_heads, n_tokens, k_max]); at most 16 query heads per kv head
  * (STEM_ERR_UNSUPPORTED otherwise).  Strides in elements, multiples of 8; Q, K, V, O 16-byte aligned.
  * softmax_scale 0 means 1/sqrt(128).  O bf16 [n_tokens, num_q_heads, 128] (contiguous); lse fp32
  * [num_q_heads, n_tokens] or NULL.  Probabilities are rounded to bf16 before they meet V (as in stem_sparse_prefill).
+ * Each list's K and V rows are gathered, or every causal key block is computed and the tokens that a list does not name
+ * masked out, whichever is estimated to be faster for lists of k_max tokens: let k_max be the length of the longest list.
  * The call only enqueues; O serves as scratch memory until its kernels are done.  O may be Q itself (contiguous), else it
  * must not overlap Q, K or V; a call with O == Q always gathers (see stem_token_attention_form).  A bounded device-side
  * wait that gave up is reported by stem_token_check_status. */

@@ -332,7 +332,7 @@ def stem_token_select(scores: torch.Tensor, k_tok: torch.Tensor, sel_idx: torch.
 
 def stem_token_attention(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, sel_idx: torch.Tensor, sel_cnt: torch.Tensor,
                          out: torch.Tensor, lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0) -> None:
-    """Gather-style attention over per-kv-head token lists; q [N, H_q, 128], k / v [N, H_kv, 128]."""
+    """Attention over per-kv-head token lists; q [N, H_q, 128], k / v [N, H_kv, 128]."""
     n, hq, _ = q.shape
     hkv = k.shape[1]
     _check(load().stem_token_attention(_ptr(q), _ptr(k), _ptr(v), n, hq, hkv, q.stride(0), q.stride(1), k.stride(0), k.stride(1),

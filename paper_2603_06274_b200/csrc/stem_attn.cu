@@ -19,11 +19,11 @@
 // Other query heads of a group have lists of their own, but choose many of the same blocks (always the first and the local
 // ones).  With kMerge the slots take neighbouring items, warp 9 finds a pair ahead which blocks both lists name, and each
 // slot walks the common blocks first, in step with the other slot on one stream of tiles, then its own, the diagonal block last.
-// (The first block, which draws most of the attention, is a common one and sets the row's reference as it does in list order:
-// with the common blocks last, O's error against 64 bits was up to 4 % larger at 128K tokens, and the layers 1 % slower.)  Slots one by one / merged, TFLOP/s at 32 / 8 heads, lists of 22 blocks (32K tokens) and 42 (128K): 1128 / 1247 and
-// 1121 / 1262 with 9 of 10 blocks in common, 1120 / 1220 and 1110 / 1200 for independent random metrics; 64K tokens, 28 / 4:
-// 1135 / 1255; blocks of 64 at 32K 420 / 467.  Neighbours may be two rows of one head as well, whose last blocks differ: 64K
-// tokens, 2 / 2 heads 980 / 1150; 16K, 8 / 8, blocks of 64 350 / 420.
+// The first block, which draws most of the attention, is a common one and sets the row's reference as it does in list order:
+// with the common blocks last, O's error against 64 bits was up to 4 % larger at 128K tokens, and the layers 1 % slower.
+// Slots one by one / merged, TFLOP/s (back to back for seconds, under the power cap): 128K tokens, 32 / 8 heads 1034 / 1121;
+// blocks of 64 at 32K 403 / 474.  Neighbours may be two rows of one head as well, whose last blocks differ: 64K tokens, 2 / 2
+// heads 831 / 900.
 // TMEM columns: S/P of slot 0, S/P of slot 1, O of slot 0, O of slot 1 (128 columns each).
 // The MMA issuer visits the slots alternately; a visit issues P V of the slot's previous block and
 // then Q K^T of its next block (P overwrites S, so the order inside a visit is fixed).  The K / V
@@ -38,9 +38,8 @@
 // work on such a pair in step (kPair): one stream of K / V tiles serves both, so a visit's tiles are filled once for two
 // visits (a visit's traffic on the 128 bytes a cycle of shared memory: operands 768 cycles, tiles 512, shared 256, beside
 // 1024 cycles of MMAs), half as much comes from the L2, which also saves power, and a ring of five reaches twice as far;
-// the next Q tiles have a whole round to land, so no spare is needed.  Two streams / one, TFLOP/s: dense 16K tokens, 32 / 8
-// heads 1237 / 1296; 128K, 64 / 8, lists of 42 blocks on average 1109 / 1189; 32K, 32 / 8, 22 blocks 1120 / 1211.  With the
-// spare Q tile and a ring of four: 1280, 1187, 1196.
+// the next Q tiles have a whole round to land, so no spare is needed.  Two streams / one, TFLOP/s (likewise): dense 16K tokens,
+// 32 / 8 heads 1102 / 1152; 128K, 64 / 8, one list per kv head 1044 / 1117.
 // Registers are re-balanced with setmaxnreg: the kernel must not spill, because with 227 KB of
 // shared memory in use almost no L1 is left for local memory.
 // Every mbarrier wait is bounded in time; a wait that gives up raises a CTA-wide abort flag,
@@ -1544,7 +1543,8 @@ cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K,
   cfg.stream = s;
   cfg.attrs = attr;
   // Started early only where a call is short: CTAs that take the SMs in the order in which the selection leaves them run the
-  // long layers 3 % slower than a plain launch (32K tokens: 1275 -> 1315 us), while it saves a short one 3 us of 27.
+  // long layers 3-12 % slower than a plain launch, while it saves a short one 1-4 us.  Plain / early, us of a call: 128 items
+  // 23.4 / 21.5, 592 (4 per SM) 47.9 / 45.7, 768 66.9 / 64.4, 1024 78.9 / 78.8 and 189 / 206, 2048 168 / 188, 8192 1318 / 1373.
   cfg.numAttrs = dependent && p.n_items <= 4 * p.sm_count ? 1 : 0;
   // Two streams of tiles are for what is left: few items, and very long lists.
   auto kernel = merge ? (B == 128 ? sparse_attn_kernel<128, true, false, false, true> : sparse_attn_kernel<64, true, false, false, true>)
@@ -1562,13 +1562,14 @@ static int first_token_of_launch(int b, int64_t mask_bytes, int64_t row_bytes) {
 static int64_t mask_bytes_of(int b) { return (int64_t)((b + kTileM - 1) / kTileM) * (kTileM / 8); }
 
 // Whether computing every causal key block is cheaper than gathering the lists, by estimates in microseconds that were
-// fitted to both (148 SMs, within 25 % from 0.02 to 7 ms):
+// fitted to both (148 SMs, within 25 % from 0.02 to 7 ms; k_max stands for the lists' lengths, which only the device knows):
 //   gather   a list entry tile of 128 costs 1.05, an item (token, kv head) 0.7 + 0.14 g on top, spread over the SMs
 //   masked   a launch 12, then a block of 128 keys x 128 rows 2.1 on a CTA whose two slots are busy, 1.7 on one whose
 //            first alone is, along the items of the CTA that gets the longest ones; reading the lists 5 TB/s
 // Measured gather / masked in us: 8192 tokens, 32/8 heads, top 2048: 6440 / 609; 12000, 32/2, 1024: 1877 / 1025;
 // 12000, 8/2, 256: 448 / 425; 12000, 8/2, 128: 337 / 422; 12000, 32/2, 256: 881 / 1004; 12000, 2/2, 128: 306 / 715 (ten
-// launches); 512, 4/1, 128: 15.5 / 21.8.
+// launches); 512, 4/1, 128: 15.5 / 21.8.  Beyond the fit it still chose the faster one in each of twelve: 32K tokens, 32/8, 2048:
+// 29 900 / 8100; 64K 62 950 / 34 500; 128K 134 400 / 139 000; 32K, 32/8, 512: 8880 / 7630; 64K, 16/1, 2048: 9480 / 13 600.
 bool token_masked_is_cheaper(int N, int Hkv, int g, int k_max, int sm_count) {
   const double sms = sm_count, k = std::min(k_max, N);
   const double gather = 8.0 + (double)N * Hkv / sms * (0.7 + 0.14 * g + 1.05 * std::max(1.0, k / kTileM * (1.0 - 0.5 * k / N)));

@@ -149,10 +149,10 @@ cudaError_t launch_small_score_select(const Plan& p, const void* qsplit, const v
 // The metric as that kernel ranks it (layout of stem_score's M; entries j > r are not written).
 cudaError_t launch_small_metric(const Plan& p, const void* qsplit, const void* ksplit, const float* mv, float* M, cudaStream_t s);
 
-// dependent: launched as a programmatic dependent of the selection kernel enqueued just before, its status words cleared by
-// an earlier kernel; otherwise the launch clears them itself.
 // Longest list whose blocks the attention kernel looks up in another head's list.
 int attention_merge_max_list();
+// dependent: launched as a programmatic dependent of the selection kernel enqueued just before, its status words cleared by
+// an earlier kernel; otherwise the launch clears them itself.
 // list_group: the lists are per kv head ([H_kv, R_tot, k_max]); every query head of a group walks its group's list.
 cudaError_t launch_sparse_attention(const Plan& p, const void* Q, const void* K, const void* V,
                                     const int32_t* sel_idx, const int32_t* sel_cnt, bool list_group, void* O, float* lse,
@@ -167,7 +167,7 @@ struct alignas(16) TokenRedo {
 // Two bf16 NaNs with a payload that no conversion yields (those give 0x7fff).
 constexpr uint32_t kTokenRedoMark = 0xffa1ffa1u;
 
-// Token-level selection and gather attention (one sequence; lists per kv head).
+// Token-level selection and attention (one sequence; lists per kv head).
 int token_attn_max_group();
 cudaError_t launch_token_select(const float* scores, int N, int H_list, int k_max, const int32_t* k_tok, int stem, int local,
                                 int32_t* sel_idx, int32_t* sel_cnt, cudaStream_t s);

@@ -2,17 +2,18 @@
 // model whose indexer keeps the top 2048 tokens per query; there k_start = 2048 and mu = 0.7).  Selection
 // granularity is one token: query token t keeps k(t) of its t+1 causal tokens, k(t) from Eq. 3 at token
 // positions, ranked by an indexer score the caller supplies (one score matrix per kv head: the heads of a
-// group share the selection), and attends over exactly those tokens.  This file holds the selection:
+// group share the selection), and attends over exactly those tokens.  This file holds the selection, the exact top-k of a
+// row's candidates by (score descending, token id ascending), the forced tokens (the first `stem` and the last `local`,
+// the token itself included) kept outside the ranking, the list ascending; and the lists as bit masks:
 //
-//   token_select_kernel   one CTA per (list head, query token): exact top-k of the row's candidates by
-//                         (score descending, token id ascending) with a radix selection, a byte per pass, on
-//                         order-preserving keys through shared-memory histograms (it stops as soon as the bin that
-//                         holds the rank is taken whole); the forced tokens (the first
-//                         `stem` and the last `local`, the token itself included) are kept outside the
-//                         ranking; the list comes out ascending.  The row's keys are converted once into
-//                         shared memory (rows of up to 51 200 tokens; longer rows are re-read from the L2).
+//   token_select_planes_kernel  rows of up to 16 384 tokens: a warp to each 1024 keys, which it holds as bit planes
+//   token_select_kernel         longer rows: one CTA per (list head, query token), a radix selection, a byte per pass, on
+//                               order-preserving keys through shared-memory histograms (it stops as soon as the bin that
+//                               holds the rank is taken whole); the row's keys are converted once into shared memory
+//                               (rows of up to 51 200 tokens; longer rows are re-read from the L2)
+//   token_mask_kernel           bit masks of the lists for the attention that computes every causal key block
 //
-// The attention over the lists is in stem_token_attn.cu.
+// The attention over the lists is in stem_attn.cu (every causal key block, masked) and stem_token_attn.cu (gathered).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -41,7 +42,7 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 // them against each other is cheaper (kFinish); only rows with many keys in one bin of the upper halves go on with the
 // lower ones, read again.  No histograms: shared-memory atomics take 14 cycles of the SM per warp instruction and bounded the
 // byte-wise radix selection below.  The kernel is bound by its integer instructions (pipe 78 % busy).  In us, byte-wise / all 32
-// planes / upper planes / with no idle warps (see the launch): 8 lists of 8K tokens, top 2048: 1240 / 780 / 588 / 487
+// planes / upper planes / with no idle warps (see the launch): 8 lists of 8K tokens, top 2048: 1240 / 780 / 588 / 497
 // (floor by its bytes 240); scores that are zero in half of the places instead of normal: 667 / 553.  Lane l of warp w owns
 // the columns 1024 w + 128 q + 4 l + c (bit 4 q + c), so loads are coalesced 16-byte ones and the ascending list comes out q
 // by q with a prefix sum over the lanes' nibbles.
