@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <new>
 #include <numeric>
@@ -420,7 +421,7 @@ int stem_plan_create_ex(const stem_config* cfg, const stem_options* opts, stem_p
   *out = nullptr;
   try {
     return create_plan(cfg, opts, out);
-  } catch (const std::bad_alloc&) {  // no exception leaves a C entry
+  } catch (const std::exception&) {  // out of host memory; no exception leaves a C entry
     return STEM_ERR_CUDA;
   }
 }
