@@ -8,7 +8,7 @@
 //     O += P V_j           TS form, P (bf16) read from TMEM, V MN-major from shared memory
 // Warp roles (384 threads):
 //     warps 0-3   softmax and epilogue of slot 0: one thread per query row; tcgen05.ld S, online
-//                 softmax in the log2 domain with lazy rescaling of O, tcgen05.st P over S; after
+//                 softmax in the log2 domain with lazy rescaling of O, tcgen05.st P; after
 //                 the item's last block O / l -> bf16 -> global memory
 //     warps 4-7   the same for slot 1
 //     warp 8      TMA producer of the K / V ring (all lanes in lock step, one elected lane issues)
@@ -24,12 +24,17 @@
 // Slots one by one / merged, TFLOP/s (back to back for seconds, under the power cap): 128K tokens, 32 / 8 heads 1034 / 1121;
 // blocks of 64 at 32K 403 / 474.  Neighbours may be two rows of one head as well, whose last blocks differ: 64K tokens, 2 / 2
 // heads 831 / 900.
-// TMEM columns: S/P of slot 0, S/P of slot 1, O of slot 0, O of slot 1 (128 columns each).
-// The MMA issuer visits the slots alternately; a visit issues P V of the slot's previous block and
-// then Q K^T of its next block (P overwrites S, so the order inside a visit is fixed).  The K / V
-// producer walks the same visit sequence, so one shared ring serves both slots in order.  A slot's
-// items follow each other without a gap: Q K^T of the next item's first block is issued right
-// behind P V of the previous item's last block while the slot's softmax warps drain O.
+// TMEM columns: S of one slot at a time (128), P of slot 0, P of slot 1 (64 each), O of slot 0, O of slot 1 (128 each).
+// S is only passed through: the softmax takes it into registers at once (170 cycles) and the columns are free for Q K^T of the
+// other slot's next block, which so runs while this slot's exponentials do; P has columns of its own, and Q K^T of a
+// slot's next block need not wait for P V of the one before.  (With S and P of a slot in the same 128 columns every block was a
+// chain softmax -> P V -> Q K^T -> softmax, 3460 cycles for a block of both slots against 2800 now; tensor pipe 59 % -> 70 %.
+// The clock gives part of it back under the power cap, 1650 -> 1570 MHz: 32K tokens, 32 / 8 heads 1314 -> 1214 us of a call,
+// dense 16K 1840 -> 1717, 128K 10170 -> 9430.)  Blocks of 64 keys leave room for an S of each slot.
+// The MMA issuer visits the slots alternately; a visit issues Q K^T of the slot's next block (as soon as the other slot's S has
+// been read) and then P V of its previous block.  The K / V producer walks the same visit sequence, so one shared ring serves
+// both slots in order.  A slot's items follow each other without a gap: S of the next item's first block is taken into
+// registers before O of the old one is written.
 // For that the next item's Q tile has to be there already: with lists of tens of blocks (kSpareQ) the
 // seven 32 KB tiles of shared memory are three Q tiles and a ring of four, the next tile is loaded into
 // the spare one while both current items run, and slot 1 starts half an item late so that the slots'
@@ -68,9 +73,14 @@ constexpr int kSlotBytes = 32 * 1024;
 constexpr int kQBytes = 32 * 1024;
 constexpr int kTmemCols = 512;
 constexpr int kSpareQMaxList = 256;                      // longest list (blocks) served with the spare Q tile
-constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X; S/P at 128 X
+constexpr int kPCol = 128;                               // P of slot X at kPCol + 64 X (S at 0, or 64 X for blocks of 64)
+constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
-constexpr float kRescaleThreshold = 8.0f;                // log2 units
+// O is rescaled when a row's maximum grows past its reference by more than this (log2 units).  Floating point does not care
+// which power of two P carries (it is at most 2^24 here, O at most 2^24 times keys times |V|, far from the 2^127 of bf16 and fp32),
+// while a rescale costs a block 550 cycles, and with 8 every other one of the first blocks had one in some of its 32 rows
+// (2 % of the keys four times as long): 32K tokens 1305 / 1262 us, dense 16K 1792 / 1734.
+constexpr float kRescaleThreshold = 24.0f;
 constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after: 256 x 216 + 128 x 72
 
 constexpr int kMergeMaxList = 208;                       // longest list (blocks) that is merged with its neighbour's
@@ -79,8 +89,8 @@ constexpr int kMergeHeader = 32;                         // lengths, common bloc
 constexpr int kMergeBytes = kMergeHeader + 2 * kMergeMaxList * 2;
 
 enum Role : int { kRoleSoftmax = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQProducer = 4, kRoleMerge = 5 };
-enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarOFree,
-                   kBarDrain, kBarPEarly, kBarHalves, kBarMergeFull, kBarMergeEmpty };
+enum BarId : int { kBarKvFull = 1, kBarKvEmpty, kBarQFull, kBarQEmpty, kBarSFull, kBarPReady, kBarOFull, kBarSRead,
+                   kBarDrain, kBarPEarly, kBarHalves, kBarMergeFull, kBarMergeEmpty, kBarPvDone };
 
 struct Smem {
   // offsets from the 1024-aligned base
@@ -93,9 +103,10 @@ struct Smem {
   static constexpr int s_full = q_empty + 8 * kQBufsMax;
   static constexpr int p_ready = s_full + 16;
   static constexpr int p_early = p_ready + 16;            // all of P but its last 32 key columns stored
-  static constexpr int o_full = p_early + 16;
-  static constexpr int o_free = o_full + 16;
-  static constexpr int halves = o_free + 16;              // both slots' parts of a list that was cut in halves
+  static constexpr int pv_done = p_early + 16;            // P V of a block complete
+  static constexpr int s_read = pv_done + 16;             // S is in registers: the next Q K^T may overwrite it
+  static constexpr int o_full = s_read + 16;              // lists cut in halves: the slot's last P V is complete
+  static constexpr int halves = o_full + 16;              // both slots' parts of such a list
   static constexpr int drain = halves + 8;
   static constexpr int tmem_ptr = drain + 8;
   static constexpr int abort_flag = tmem_ptr + 4;
@@ -531,6 +542,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   constexpr int kKvSlots = kSpareQ ? 4 : 5;
   constexpr int kQBufs = kSpareQ ? 3 : 2;
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
+  constexpr bool kOwnS = BLK == 64;  // S of a block of 64 keys takes half of the 128 columns: one half for each slot
+  // The slots' visits of a round go together, Q K^T of both before P V of both: with an S each neither waits for the other's P,
+  // which counts where they run side by side through half a list each (4K tokens, 2 heads: 25.3 us of a call, so 24.6).
+  constexpr bool kTogether = kOwnS && kSplit;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kKvSlots; ++i) { mbar_init(bar(Smem::kv_full, i), 1); mbar_init(bar(Smem::kv_empty, i), 1); }
@@ -542,8 +557,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(bar(Smem::s_full, i), 1);
       mbar_init(bar(Smem::p_ready, i), 4);   // one arrival per softmax warp
       mbar_init(bar(Smem::p_early, i), 4);   // likewise
+      mbar_init(bar(Smem::pv_done, i), 1);
+      mbar_init(bar(Smem::s_read, i), 4);    // likewise
       mbar_init(bar(Smem::o_full, i), 1);
-      mbar_init(bar(Smem::o_free, i), 4);    // one arrival per softmax warp
     }
     if constexpr (kMerge) {
       for (int i = 0; i < 2; ++i) {
@@ -597,11 +613,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     Ctx ctx{abort_flag, status, kRoleSoftmax, kGaveUp};
     const int m = (warp & 3) * 32 + lane;  // query row inside the tile == TMEM lane
     const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t s_addr = lane_addr + X * 128;
+    const uint32_t s_addr = lane_addr + (kOwnS ? X * 64 : 0);
+    const uint32_t p_addr = lane_addr + kPCol + X * 64;
     const uint32_t o_addr = lane_addr + kOCol + X * 128;
-    uint32_t blk = 0;   // blocks of this slot so far (phase of s_full / p_ready)
-    uint32_t ord = 0;   // non-empty items of this slot so far (phase of o_full / o_free)
+    uint32_t blk = 0;   // blocks of this slot so far (phase of s_full / s_read / p_ready / pv_done)
     bool ok = true;
+    // P V of the slot's block before this one is complete (its P may be overwritten, its O read and rescaled)
+    auto wait_pv = [&] { return __all_sync(0xffffffffu, mbar_wait(bar(Smem::pv_done, X), (blk & 1) ^ 1, ctx, kBarPvDone)); };
+    // Where a CTA runs one item, each barrier is probed ahead of its wait: the answer takes 150 cycles to come.  (18.8 us of a
+    // call for two ragged prompts, 19.3 without; with both slots busy the probes cost more than they save: 32K tokens 1231 / 1214.)
+    constexpr bool kProbeAhead = kSplit;
+    uint32_t s_seen = 0, pv_seen = 0;
     // kTok: row m is query head m % g of the tile's token m / g
     const int tokl = kTok ? m / a.g : 0, sub = kTok ? m - tokl * a.g : 0;
     // The list length of an item and whether its list ends on the diagonal block sit at the end of a
@@ -631,6 +653,49 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       return (uint32_t)n | (diag ? 0x80000000u : 0u) | halves;
     };
     uint32_t next_info = list_info(walk.idx);
+    float m_run = -INFINITY, l_run = 0.f;
+    // O / l of an item whose last P V is complete -> bf16 -> global memory
+    auto write_rows = [&](const int h, const int q_tok0, const bool row_valid, const float inv_l) {
+      const bool o_al32 = ((uintptr_t)a.O & 31u) == 0u;  // rows are multiples of 256 bytes apart
+      __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
+#pragma unroll 1
+      for (int c = 0; c < kHeadDim / 32; ++c) {
+        float o[32];
+        tmem_ld32(o_addr + c * 32, o);
+        tmem_ld_wait();
+        if (row_valid) {
+          uint32_t w[16];
+#pragma unroll
+          for (int q = 0; q < 16; ++q) w[q] = pack_bf16(o[2 * q] * inv_l, o[2 * q + 1] * inv_l);
+          if constexpr (kTok) {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) l_run = fmaf(o[q], 0.f, l_run);  // NaN from the first value on that is not finite
+          }
+          if (o_al32) {
+            // whole 32-byte sectors per store: a thread writes its own 256-byte row, so the stores of
+            // a warp are 32 separate sectors either way, and this halves their number
+            st_global_v8(o_row + c * 32, w);
+            st_global_v8(o_row + c * 32 + 16, w + 8);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              *(uint4*)(o_row + c * 32 + q * 8) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+          }
+        }
+      }
+    };
+    // kDefer: the item before this one, whose O is written once S of this one's first block is in registers
+    constexpr bool kDefer = kSpareQ;
+    bool d_has = false, d_valid = false;
+    int d_h = 0, d_tok0 = 0;
+    auto write_deferred = [&]() -> bool {
+      if (!wait_pv()) return false;
+      tc_fence_after();
+      write_rows(d_h, d_tok0, d_valid, 1.f / l_run);
+      if (a.lse && d_valid) a.lse[(int64_t)d_h * a.T + d_tok0 + m] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+      d_has = false;
+      return true;
+    };
     while (!walk.done() && ok) {
       const int item = walk.idx;
       walk.advance();
@@ -674,23 +739,26 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         continue;
       }
       const bool has_diag = (info >> 31) != 0u;
-      float m_run = -INFINITY, l_run = 0.f;
       for (int e = 0; e < n; ++e, ++blk) {
         uint4 mask_w = make_uint4(0, 0, 0, 0);  // kTok: the block's mask words, here while S is still awaited
         if constexpr (kTok) {
           if (row_valid) mask_w = *mask++;
           unseen -= __popc(mask_w.x) + __popc(mask_w.y) + __popc(mask_w.z) + __popc(mask_w.w);
         }
-        // S of block e is complete; so is every earlier tensor-core operation of this slot,
-        // P V of block e-1 included (the commit behind Q K^T covers all earlier operations)
-        ok = mbar_wait(bar(Smem::s_full, X), blk & 1, ctx, kBarSFull);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
+        if (!kProbeAhead || !__all_sync(0xffffffffu, s_seen)) {
+          ok = mbar_wait(bar(Smem::s_full, X), blk & 1, ctx, kBarSFull);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+        }
         tc_fence_after();
         float s[BLK];
 #pragma unroll
         for (int c = 0; c < BLK / 32; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
         tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(Smem::s_read, kOwnS ? X : 0));
+        if (kProbeAhead) pv_seen = mbar_test(bar(Smem::pv_done, X), (blk & 1) ^ 1);
         if constexpr (kTok) {
           const uint32_t w[4] = {mask_w.x, mask_w.y, mask_w.z, mask_w.w};
 #pragma unroll
@@ -709,12 +777,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         const float mx_c = fmaxf(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], max3(mx[5], mx[6], mx[7]))) * a.scale_log2;
         if (e == 0) {
+          if (kDefer && d_has && !(ok = write_deferred())) break;
+          l_run = 0.f;
           m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
         } else {
           const bool grow = mx_c > m_run + kRescaleThreshold;
           if (__any_sync(0xffffffffu, grow)) {
             const float alpha = grow ? fast_exp2(m_run - mx_c) : 1.f;
             if (grow) { m_run = mx_c; l_run *= alpha; }
+            ok = wait_pv();
+            if (!ok) break;
+            tc_fence_after();
 #pragma unroll
             for (int c = 0; c < kHeadDim / 32; ++c) {
               float o[32];
@@ -744,7 +817,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             pk[c / 2] = pack_bf16(p0.x, p0.y);
             pk[c / 2 + 1] = pack_bf16(p1.x, p1.y);
           }
-          tmem_st16(s_addr + g * 16, pk);
+          if (g == 0) {
+            if (!kProbeAhead || !__all_sync(0xffffffffu, pv_seen)) ok = wait_pv();  // (if it gave up, what follows works on this CTA's own tensor memory, and the loop ends below)
+            tc_fence_after();
+          }
+          tmem_st16(p_addr + g * 16, pk);
+          if (kProbeAhead && g == BLK / 32 - 2) s_seen = mbar_test(bar(Smem::s_full, X), (blk & 1) ^ 1);
           if (g == BLK / 32 - 2) {
             // all but the last 32 key columns of P are stored: their share of P V may start
             tmem_st_wait();
@@ -760,9 +838,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (lane == 0) mbar_arrive(bar(Smem::p_ready, X));
       }
       if (!ok) break;
-      // ---- epilogue: the item's last P V is complete -> O / l -> bf16 -> global memory
-      ok = mbar_wait(bar(Smem::o_full, X), ord & 1, ctx, kBarOFull);
-      ok = __all_sync(0xffffffffu, ok);
+      if constexpr (kDefer) {
+        d_has = true; d_valid = row_valid; d_h = h; d_tok0 = q_tok0;
+        continue;
+      }
+      ok = wait_pv();
       if (!ok) break;
       tc_fence_after();
       if constexpr (kSplit) {
@@ -815,49 +895,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
           }
           if (a.lse && row_valid && X == 0) a.lse[(int64_t)h * a.T + q_tok0 + m] = (m_both + log2f(l_both)) * 0.6931471805599453f;
-          ++ord;
           continue;
         }
       }
       const float inv_l = (kTok && unseen == kNoList) ? 0.f : 1.f / l_run;
-      const bool o_al32 = ((uintptr_t)a.O & 31u) == 0u;  // rows are multiples of 256 bytes apart
-      __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
-#pragma unroll
-      for (int c = 0; c < kHeadDim / 32; ++c) {
-        float o[32];
-        tmem_ld32(o_addr + c * 32, o);
-        tmem_ld_wait();
-        if (c == kHeadDim / 32 - 1) {
-          // O is in registers: P V of the slot's next item may overwrite it
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(Smem::o_free, X));
-        }
-        if (row_valid) {
-          uint32_t w[16];
-#pragma unroll
-          for (int q = 0; q < 16; ++q) w[q] = pack_bf16(o[2 * q] * inv_l, o[2 * q + 1] * inv_l);
-          if constexpr (kTok) {
-#pragma unroll
-            for (int q = 0; q < 32; ++q) l_run = fmaf(o[q], 0.f, l_run);  // NaN from the first value on that is not finite
-          }
-          if (o_al32) {
-            // whole 32-byte sectors per store: a thread writes its own 256-byte row, so the stores of
-            // a warp are 32 separate sectors either way, and this halves their number
-            st_global_v8(o_row + c * 32, w);
-            st_global_v8(o_row + c * 32 + 16, w + 8);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              *(uint4*)(o_row + c * 32 + q * 8) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-          }
-        }
-      }
+      write_rows(h, q_tok0, row_valid, inv_l);
       if (a.lse && row_valid)
         a.lse[(int64_t)h * a.T + q_tok0 + m] = (kTok && unseen == kNoList) ? -INFINITY : (m_run + log2f(l_run)) * 0.6931471805599453f;
       if constexpr (kTok) {
         // Rows that the masks cannot do are left to the gather kernel behind this one: a list that names a token twice (a mask
         // holds it once), or a value that is not finite (0 times a V row that the list does not name).
+        __nv_bfloat16* o_row = a.O + ((int64_t)(q_tok0 + m) * a.Hq + h) * kHeadDim;
         const bool redo = row_valid && unseen != kNoList && (unseen != 0 || !(l_run < INFINITY));
         if (redo) {
           *(uint32_t*)o_row = kTokenRedoMark;
@@ -868,8 +916,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         __syncwarp();
       }
-      ++ord;
     }
+    if (kDefer && ok && d_has) write_deferred();
   } else {
     // The issuing roles run with all 32 lanes in lock step on warp-uniform values (loads are
     // broadcast through lane 0), so that descriptors, coordinates and barrier addresses live in
@@ -909,12 +957,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         ++kv_prod;
         return true;
       };
-      // One visit: V of the block whose K went out on the slot's previous visit, then K of the next block.
+      // One visit: K of the next block, then V of the block whose K went out on the slot's previous visit.
       auto visit = [&](KvSlot& s) -> bool {
-        if (s.pend) {
-          s.pend = false;
-          if (!load(&map_v, s.pend_kvh, s.pend_tok)) return false;
-        }
+        const bool due = s.pend;
+        const int due_tok = s.pend_tok, due_kvh = s.pend_kvh;
+        s.pend = false;
         if (s.has) {
           const int j = min(max(s.j_next, 0), s.cur.r);
           const int kvh = kTok ? s.cur.h : s.cur.h / a.g;
@@ -924,18 +971,23 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           if (++s.e < s.cur.n) s.j_next = dense ? s.cur.off + s.e : uni(s.list[s.e]);  // consumed on the slot's next visit
           else enter(s);
         }
-        return true;
+        return !due || load(&map_v, due_kvh, due_tok);
       };
       bool ok = true;
       if constexpr (kMerge) {
         // The merged lists: the blocks both have, one tile each, then in each round a block of slot 0's own and one of slot 1's
         // own, then the last ones.
         int pend_tok[2] = {-1, -1}, pend_kvh[2] = {0, 0};  // V tile that is due; slot 0's alone if both have the block
-        auto pend = [&](const int X) -> bool {
-          if (pend_tok[X] < 0) return true;
-          const int tok = pend_tok[X];
+        // slot X's part of a round: K of block j (none if negative), then V of the slot's block before it
+        auto part = [&](const int X, const int j, const int kvh, const int tok0) -> bool {
+          const int due_tok = pend_tok[X], due_kvh = pend_kvh[X];
           pend_tok[X] = -1;
-          return load(&map_v, pend_kvh[X], tok);
+          if (j >= 0) {
+            pend_tok[X] = tok0 + j * BLK;
+            pend_kvh[X] = kvh;
+            if (!load(&map_k, kvh, pend_tok[X])) return false;
+          }
+          return due_tok < 0 || load(&map_v, due_kvh, due_tok);
         };
         const int pairs = pairs_of(a);
         for (int k = 0; ok && k < pairs; ++k) {
@@ -952,25 +1004,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           auto common = [&](const int i) -> int { return dense ? i : uni((int)ent[c0 + i]); };
           auto alone = [&](const int X, const int i) -> int { return dense ? both + i : uni((int)ent[X ? n0 + i : i]); };
           auto last = [&](const int X) -> int { return dense ? (X ? n1 : n0) - 1 : uni((int)ent[X ? n0 + c1 : n0 - 1]); };
-          auto key = [&](const int X, const int j) -> bool {
-            pend_tok[X] = tok0[X] + j * BLK;
-            pend_kvh[X] = kvh[X];
-            return load(&map_k, kvh[X], pend_tok[X]);
-          };
-          auto shared_round = [&](const int i) -> bool { return pend(0) && key(0, common(i)) && pend(1); };
-          for (int it = 0; ok && it < lead; ++it) ok = shared_round(it);
-          for (int it = 0; ok && it < own; ++it) {
-            ok = pend(0);
-            if (ok && it >= own - c0) ok = key(0, alone(0, it - (own - c0)));
-            if (ok) ok = pend(1);
-            if (ok && it >= own - c1) ok = key(1, alone(1, it - (own - c1)));
-          }
-          if (ok && tail) ok = pend(0) && key(0, last(0)) && pend(1) && key(1, last(1));
-          else if (ok && both > 0) ok = shared_round(lead);
+          auto round = [&](const int j0, const int j1) -> bool { return part(0, j0, kvh[0], tok0[0]) && part(1, j1, kvh[1], tok0[1]); };
+          for (int it = 0; ok && it < lead; ++it) ok = round(common(it), -1);
+          for (int it = 0; ok && it < own; ++it)
+            ok = round(it >= own - c0 ? alone(0, it - (own - c0)) : -1, it >= own - c1 ? alone(1, it - (own - c1)) : -1);
+          if (ok && tail) ok = round(last(0), last(1));
+          else if (ok && both > 0) ok = round(common(lead), -1);
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(Smem::merge_empty, b));
         }
-        ok = ok && pend(0) && pend(1);
+        ok = ok && part(0, -1, 0, 0) && part(1, -1, 0, 0);
       } else {
         KvSlot s0, s1;
         s0.cur.init(a, 0); s1.cur.init(a, 1);
@@ -981,8 +1024,15 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // their claims on the spare) do not fall together.  The MMA issuer skips the same visits.
         const uint32_t delay1 = (kSpareQ && s0.has) ? (uint32_t)s0.cur.n / 2u : 0u;
         for (uint32_t it = 0; ok && (s0.has || s1.has || s0.pend || s1.pend); ++it) {
-          ok = visit(s0);
-          if (!kPair && ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
+          if constexpr (kTogether) {
+            const bool due0 = s0.pend, due1 = s1.pend;
+            const int tok0 = s0.pend_tok, tok1 = s1.pend_tok, kvh0 = s0.pend_kvh, kvh1 = s1.pend_kvh;
+            s0.pend = s1.pend = false;
+            ok = visit(s0) && visit(s1) && (!due0 || load(&map_v, kvh0, tok0)) && (!due1 || load(&map_v, kvh1, tok1));
+          } else {
+            ok = visit(s0);
+            if (!kPair && ok && (!kSpareQ || it >= delay1)) ok = visit(s1);
+          }
         }
       }
       if (!ok && lane == 0) {
@@ -1225,10 +1275,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int left;                      // blocks of the current item whose Q K^T is still to come (0: no item left)
         uint32_t st;                   // kPend: a P V is due, of its item's first (kFirst) / last (kLast) block;
                                        // kNewItem: the next Q K^T is the first of its item
-        uint32_t p_par, q_par, o_par;  // phase parities of p_early / p_ready, q_full, o_full / o_free
+        uint32_t p_par, q_par;         // phase parities of p_early / p_ready, q_full
+        uint32_t f_par;                // kOwnS: of s_read
         int qbuf;                      // Q buffer of the slot's current item
       };
       uint32_t ring = 0, ring_par = 0;  // next K / V ring slot to consume and its phase
+      uint32_t f_par = 1;               // phase parity of s_read
       int q_spare = 2;      // kSpareQ: the buffer that receives the next item's tile, and per buffer (bit b) whether an
       uint32_t q_odd = 3u;  // odd number of items was assigned to it so far - the Q producer's rule, step for step
       constexpr int kEarlySteps = (BLK / 32 - 1) * 2;  // 16-key steps of P V covered by p_early
@@ -1238,12 +1290,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (++ring == kKvSlots) { ring = 0; ring_par ^= 1; }
       };
       // O_X (+)= P V with the V tile in ring slot `tile`, which is given back with `release`.
-      auto issue_pv = [&](MmaSlot& s, const int X, const uint32_t tile, const bool release) {
-        const uint32_t s_tmem = tmem_base + X * 128;
+      auto issue_pv = [&](MmaSlot& s, const int X, const uint32_t st, const uint32_t tile, const bool release) {
+        const uint32_t p_tmem = tmem_base + kPCol + X * 64;
         const uint32_t o_tmem = tmem_base + kOCol + X * 128;
-        const uint32_t st = s.st;
         const uint32_t v_addr = smem_base + kKvOff + tile * kSlotBytes;
-        if (st & kFirst) mbar_wait_sticky(bar(Smem::o_free, X), s.o_par ^ 1, abort_addr, kBarOFree, failed);
         // P V starts on the leading key columns while the softmax still works on the last 32
         mbar_wait_sticky(bar(Smem::p_early, X), s.p_par, abort_addr, kBarPEarly, failed);
         tc_fence_after();
@@ -1251,7 +1301,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
 #pragma unroll
           for (int k = 0; k < kEarlySteps; ++k)
-            mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, (k == 0 && (st & kFirst)) ? 0u : 1u);
+            mma_ts(o_tmem, p_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, (k == 0 && (st & kFirst)) ? 0u : 1u);
         }
         __syncwarp();
         mbar_wait_sticky(bar(Smem::p_ready, X), s.p_par, abort_addr, kBarPReady, failed);
@@ -1259,19 +1309,21 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (leader) {
           const uint64_t db = smem_desc(v_addr, kHalfBytes, 1024);
 #pragma unroll
-          for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, s_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
+          for (int k = kEarlySteps; k < BLK / 16; ++k) mma_ts(o_tmem, p_tmem + k * 8, db + k * (2048 >> 4), kIdescPV, 1u);
           if (release) tc_commit(bar(Smem::kv_empty, tile));
-          if (st & kLast) tc_commit(bar(Smem::o_full, X));
+          tc_commit(bar(Smem::pv_done, X));
+          if (kSplit && (st & kLast)) tc_commit(bar(Smem::o_full, X));
         }
         __syncwarp();
         s.p_par ^= 1;
-        if (st & kLast) s.o_par ^= 1;
-        s.st = st & kNewItem;
       };
       // S_X = Q K^T with the K tile in ring slot `tile`; true for the last block of the slot's item.
       auto issue_qk = [&](MmaSlot& s, const int X, const uint32_t tile, const bool release) -> bool {
         const uint32_t st = s.st;
         if (st & kNewItem) mbar_wait_sticky(bar(Smem::q_full, s.qbuf), s.q_par, abort_addr, kBarQFull, failed);
+        uint32_t& f = kOwnS ? s.f_par : f_par;
+        mbar_wait_sticky(bar(Smem::s_read, kOwnS ? X : 0), f, abort_addr, kBarSRead, failed);
+        f ^= 1;
         tc_fence_after();
         const bool last = --s.left == 0;
         if (leader) {
@@ -1279,7 +1331,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           const uint64_t db = smem_desc(smem_base + kKvOff + tile * kSlotBytes, 16, 1024);
 #pragma unroll
           for (int k = 0; k < kHeadDim / 16; ++k)  // 16 columns = 32 bytes on; the second four steps: the other 64-column half
-            mma_ss(tmem_base + X * 128, da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4),
+            mma_ss(tmem_base + (kOwnS ? X * 64 : 0), da + (((k >> 2) * kTileM * 128 + (k & 3) * 32) >> 4),
                    db + (((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4), kIdescS, k > 0 ? 1u : 0u);
           if (release) tc_commit(bar(Smem::kv_empty, tile));
           tc_commit(bar(Smem::s_full, X));
@@ -1293,11 +1345,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       auto visit = [&](MmaSlot& s, const int X) {
         const uint32_t ring0 = ring, ring_par0 = ring_par;
         const bool shared = kPair && X == 0;  // slot 1's visit uses the same tiles and gives them back
-        if (s.st & kPend) {
-          if (!kPair || X == 0) wait_tile();
-          issue_pv(s, X, ring, !shared);
+        const uint32_t due = s.st;
+        // Without a spare the Q tile of a new item is the last thing to arrive: P V, which the end of the old item waits for,
+        // goes first (its V tile is behind the K tile in the ring all the same).
+        const bool swap = !kSpareQ && (due & kNewItem) && (due & kPend) && s.left > 0;
+        if (swap) {
           next_tile();
+          if (!kPair || X == 0) wait_tile();
+          issue_pv(s, X, due, ring, !shared);
+          ring = ring0; ring_par = ring_par0;
         }
+        s.st = due & kNewItem;
         if (s.left > 0) {
           if (!kPair || X == 0) wait_tile();
           const bool last = issue_qk(s, X, ring, !shared);
@@ -1317,13 +1375,21 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
           }
         }
+        if (swap) {
+          next_tile();
+        } else if (due & kPend) {
+          if (!kPair || X == 0) wait_tile();
+          issue_pv(s, X, due, ring, !shared);
+          next_tile();
+        }
         if (shared) { ring = ring0; ring_par = ring_par0; }
       };
       if constexpr (kMerge) {
         MmaSlot s0, s1;
         s0.left = s1.left = 0;
         s0.st = s1.st = kNewItem;
-        s0.p_par = s1.p_par = s0.o_par = s1.o_par = 0;
+        s0.p_par = s1.p_par = 0;
+        s0.f_par = s1.f_par = 1;
         int q_tile = 0;
         uint32_t q_phase = 0;
         auto take_q = [&](MmaSlot& s) {
@@ -1335,25 +1401,20 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // A round: as in visit(), with the tiles of the blocks that both lists have used by slot 0, then by slot 1.
         auto round = [&](const bool act0, const bool act1, const bool k_both) {
           uint32_t v_tile = 0, k_tile = 0;
-          if (s0.st & kPend) {
-            v_tile = ring;
-            wait_tile();
-            issue_pv(s0, 0, ring, !v_both);
-            next_tile();
-          }
+          const uint32_t due0 = s0.st, due1 = s1.st;
+          s0.st = due0 & kNewItem;
+          s1.st = due1 & kNewItem;
           if (act0) {
             k_tile = ring;
             wait_tile();
             issue_qk(s0, 0, ring, !k_both);
             next_tile();
           }
-          if (s1.st & kPend) {
-            if (!v_both) {
-              v_tile = ring;
-              wait_tile();
-              next_tile();
-            }
-            issue_pv(s1, 1, v_tile, true);
+          if (due0 & kPend) {
+            v_tile = ring;
+            wait_tile();
+            issue_pv(s0, 0, due0, ring, !v_both);
+            next_tile();
           }
           if (act1) {
             if (!k_both) {
@@ -1362,6 +1423,14 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
               next_tile();
             }
             issue_qk(s1, 1, k_tile, true);
+          }
+          if (due1 & kPend) {
+            if (!v_both) {
+              v_tile = ring;
+              wait_tile();
+              next_tile();
+            }
+            issue_pv(s1, 1, due1, v_tile, true);
           }
           v_both = k_both;
         };
@@ -1397,12 +1466,23 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         s0.left = s0.cur.next(a) ? s0.cur.n : 0;
         s1.left = s1.cur.next(a) ? s1.cur.n : 0;
         s0.st = s1.st = kNewItem;
-        s0.p_par = s1.p_par = s0.q_par = s1.q_par = s0.o_par = s1.o_par = 0;
+        s0.p_par = s1.p_par = s0.q_par = s1.q_par = 0;
+        s0.f_par = s1.f_par = 1;
         s0.qbuf = 0; s1.qbuf = 1;
         const uint32_t delay1 = kSpareQ ? (uint32_t)s0.left / 2u : 0u;  // as in the K / V producer
         for (uint32_t it = 0; s0.left > 0 || s1.left > 0 || ((s0.st | s1.st) & kPend); ++it) {
-          visit(s0, 0);
-          if (!kSpareQ || it >= delay1) visit(s1, 1);
+          if constexpr (kTogether) {
+            const uint32_t due0 = s0.st, due1 = s1.st;
+            s0.st = due0 & kNewItem;
+            s1.st = due1 & kNewItem;
+            visit(s0, 0);
+            visit(s1, 1);
+            if (due0 & kPend) { wait_tile(); issue_pv(s0, 0, due0, ring, true); next_tile(); }
+            if (due1 & kPend) { wait_tile(); issue_pv(s1, 1, due1, ring, true); next_tile(); }
+          } else {
+            visit(s0, 0);
+            if (!kSpareQ || it >= delay1) visit(s1, 1);
+          }
           if (__any_sync(0xffffffffu, failed != 0)) break;
         }
       }

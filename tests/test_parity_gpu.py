@@ -575,3 +575,44 @@ def test_a_block_of_keys_at_minus_infinity_draws_nothing(seqlen):
         s = s.masked_fill(torch.ones((seqlen, seqlen), dtype=torch.bool, device="cuda").triu(1), float("-inf"))
         ref = torch.einsum("hts,sd->thd", torch.softmax(s, 2), v[:, 0].double())
         check_attention(from_dev_bf16(out), ref.cpu().numpy(), label=f"{n} blocks, keys of block {bad} at -inf")
+
+
+@pytest.mark.parametrize("block,seqlen,hq,hkv,dense", [
+    (128, 6 * 128 - 5, 2, 1, False),    # each slot half of a list
+    (64, 9 * 64, 2, 1, False),
+    (128, 38 * 128 - 5, 4, 2, False),   # item by item
+    (128, 25 * 128, 8, 4, False),       # neighbouring items, merged lists
+    (64, 50 * 64 + 7, 4, 2, False),
+    (128, 25 * 128, 8, 4, True),        # pairs of heads on one stream of K / V
+    (64, 50 * 64 + 7, 4, 2, True),
+])
+def test_row_maxima_that_grow_from_block_to_block(block, seqlen, hq, hkv, dense):
+    # The scores of block j are about step[j] powers of two: rows whose maximum grows by less than the rescale threshold (24)
+    # keep the reference of an earlier block, at 23 with probabilities up to 2^23; larger steps rescale O, once or again.
+    w = wl.small("grow", seqlens=(seqlen,), hq=hq, hkv=hkv, block=block, permille=1000, mu_num=1, mu_den=1, seed=seqlen)
+    data = dict(wl.make_qkv(w))
+    r = np.random.default_rng(seqlen + hq)
+    step = np.array([0, 10, 23, 22, 48, 40, 71, 95, 95, 60] + list(r.integers(0, 120, size=60)))[:(seqlen + block - 1) // block]
+    u = r.standard_normal(128)
+    u /= np.linalg.norm(u)
+    scale = np.sqrt(128) / np.log2(np.e) / 8  # q = 8 u, so that k = scale * step * u scores `step` powers of two
+    k = np.repeat(step, block)[:seqlen, None, None] * scale * u + 0.3 * r.standard_normal((seqlen, hkv, 128))
+    q = 8 * u + 0.3 * r.standard_normal((seqlen, hq, 128))
+    bits = lambda t: torch.from_numpy(t.astype(np.float32)).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    data["q"], data["k"] = bits(q), bits(k)
+    plan = StemPlan.from_workload(w)
+    info = plan.info
+    n_blk = info.total_q_blocks
+    idx = np.full((hq, n_blk, info.k_max), -1, np.int32)
+    for row in range(n_blk):
+        idx[:, row, :row + 1] = np.arange(row + 1)
+    cnt = np.broadcast_to(np.arange(1, n_blk + 1, dtype=np.int32), (hq, n_blk)).copy()
+    out = torch.full((seqlen, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((hq, seqlen), float("nan"), dtype=torch.float32, device="cuda")
+    lists = (None, None) if dense else (torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda())
+    binding.stem_sparse_prefill(plan, to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"]), *lists, out, lse)
+    assert binding.stem_check_status(plan)[0] == 0
+    O_ref, lse_ref = so.attention(data["q"], data["k"], data["v"], data["cu_seqlens"], block, idx, cnt)
+    check_attention(from_dev_bf16(out), O_ref, ~np.isnan(O_ref), label="growing maxima")
+    assert np.abs(lse.cpu().numpy() - lse_ref).max() < 1e-3
+    plan.close()
