@@ -29,8 +29,8 @@
 // other slot's next block, which so runs while this slot's exponentials do; P has columns of its own, and Q K^T of a
 // slot's next block need not wait for P V of the one before.  (With S and P of a slot in the same 128 columns every block was a
 // chain softmax -> P V -> Q K^T -> softmax, 3460 cycles for a block of both slots against 2800 now; tensor pipe 59 % -> 70 %.
-// The clock gives part of it back under the power cap, 1650 -> 1570 MHz: 32K tokens, 32 / 8 heads 1314 -> 1214 us of a call,
-// dense 16K 1840 -> 1717, 128K 10170 -> 9430.)  Blocks of 64 keys leave room for an S of each slot.
+// The clock gives part of it back under the power cap, 1650 -> 1570 MHz: 32K tokens, 32 / 8 heads 1314 -> 1240 us of a call,
+// dense 16K 1840 -> 1740.)  Blocks of 64 keys leave room for an S of each slot.
 // The MMA issuer visits the slots alternately; a visit issues Q K^T of the slot's next block (as soon as the other slot's S has
 // been read) and then P V of its previous block.  The K / V producer walks the same visit sequence, so one shared ring serves
 // both slots in order.  A slot's items follow each other without a gap: S of the next item's first block is taken into
@@ -76,11 +76,11 @@ constexpr int kSpareQMaxList = 256;                      // longest list (blocks
 constexpr int kPCol = 128;                               // P of slot X at kPCol + 64 X (S at 0, or 64 X for blocks of 64)
 constexpr int kOCol = 256;                               // O of slot X at kOCol + 128 X
 constexpr uint64_t kWaitLimitNs = 400ull * 1000 * 1000;  // per wait
-// O is rescaled when a row's maximum grows past its reference by more than this (log2 units).  Floating point does not care
-// which power of two P carries (it is at most 2^24 here, O at most 2^24 times keys times |V|, far from the 2^127 of bf16 and fp32),
-// while a rescale costs a block 550 cycles, and with 8 every other one of the first blocks had one in some of its 32 rows
-// (2 % of the keys four times as long): 32K tokens 1305 / 1262 us, dense 16K 1792 / 1734.
-constexpr float kRescaleThreshold = 24.0f;
+// O is rescaled when a row's maximum has grown past its reference by more than this (log2 units).  All rows of the warp then
+// move to their own maximum: a reference that is the maximum makes the largest P exactly 1, whose rounding to bf16 costs
+// nothing, so O's error against 64 bits is smaller (32K tokens 1.84e-3, 1.94e-3 where only the rows that grew move; thresholds of
+// 12 / 24 with all rows: 1.96e-3 / 2.09e-3), and fewer blocks rescale.
+constexpr float kRescaleThreshold = 8.0f;
 constexpr int kRegsSoftmax = 216, kRegsOther = 72;  // launch: 384 x 168; after: 256 x 216 + 128 x 72
 
 constexpr int kMergeMaxList = 208;                       // longest list (blocks) that is merged with its neighbour's
@@ -684,6 +684,25 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
       }
     };
+    // O of the blocks so far, whose P V are complete, times alpha.  Before the exponentials this costs a block 550 cycles; once most
+    // of its scores are gone, and P V is long complete, less (32K tokens 1273 / 1263 us, dense 16K 1785 / 1764).  Where a CTA runs
+    // one item (kSplit) that would spill: two ragged short prompts 20.5 us of a call, 18.6 before the exponentials.
+    constexpr bool kRescaleLate = !kSplit;
+    auto rescale_o = [&](const float alpha) {
+      constexpr int kAtOnce = kSpareQ ? 64 : 32;  // columns
+#pragma unroll(kSplit ? 4 : 1)
+      for (int c = 0; c < kHeadDim; c += kAtOnce) {
+        float o[kAtOnce];
+#pragma unroll
+        for (int u = 0; u < kAtOnce; u += 32) tmem_ld32(o_addr + c + u, o + u);
+        tmem_ld_wait();
+        uint32_t w[kAtOnce];
+#pragma unroll
+        for (int q = 0; q < kAtOnce; ++q) w[q] = __float_as_uint(o[q] * alpha);
+#pragma unroll
+        for (int u = 0; u < kAtOnce; u += 32) tmem_st32(o_addr + c + u, w + u);
+      }
+    };
     // kDefer: the item before this one, whose O is written once S of this one's first block is in registers
     constexpr bool kDefer = kSpareQ;
     bool d_has = false, d_valid = false;
@@ -776,27 +795,25 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           for (int q = 0; q < 8; ++q) mx[q] = max3(mx[q], s[c + 2 * q], s[c + 2 * q + 1]);
         }
         const float mx_c = fmaxf(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], max3(mx[5], mx[6], mx[7]))) * a.scale_log2;
+        bool rescale = false;  // some row of the warp
+        float alpha = 1.f;
         if (e == 0) {
           if (kDefer && d_has && !(ok = write_deferred())) break;
           l_run = 0.f;
           m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
         } else {
           const bool grow = mx_c > m_run + kRescaleThreshold;
-          if (__any_sync(0xffffffffu, grow)) {
-            const float alpha = grow ? fast_exp2(m_run - mx_c) : 1.f;
-            if (grow) { m_run = mx_c; l_run *= alpha; }
-            ok = wait_pv();
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll
-            for (int c = 0; c < kHeadDim / 32; ++c) {
-              float o[32];
-              tmem_ld32(o_addr + c * 32, o);
-              tmem_ld_wait();
-              uint32_t w[32];
-#pragma unroll
-              for (int q = 0; q < 32; ++q) w[q] = __float_as_uint(o[q] * alpha);
-              tmem_st32(o_addr + c * 32, w);
+          rescale = __any_sync(0xffffffffu, grow);
+          if (rescale) {
+            const float m_new = fmaxf(m_run, mx_c);
+            alpha = fast_exp2(m_run - m_new);
+            m_run = m_new;
+            l_run *= alpha;
+            if (!kRescaleLate) {
+              ok = wait_pv();
+              if (!ok) break;
+              tc_fence_after();
+              rescale_o(alpha);
             }
           }
         }
@@ -806,6 +823,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
         for (int g = 0; g < BLK / 32; ++g) {
           uint32_t pk[16];  // 32 probabilities as bf16 pairs = 16 TMEM columns
+          constexpr int kEarly = BLK / 32 - 2;  // after these 32 keys P V may start
 #pragma unroll
           for (int c = 0; c < 32; c += 4) {
             const float2 x0 = __ffma2_rn(make_float2(s[g * 32 + c], s[g * 32 + c + 1]), sc2, nm2);
@@ -818,12 +836,13 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             pk[c / 2 + 1] = pack_bf16(p1.x, p1.y);
           }
           if (g == 0) {
-            if (!kProbeAhead || !__all_sync(0xffffffffu, pv_seen)) ok = wait_pv();  // (if it gave up, what follows works on this CTA's own tensor memory, and the loop ends below)
+            if (!kProbeAhead || !__all_sync(0xffffffffu, pv_seen)) ok = wait_pv();
             tc_fence_after();
           }
           tmem_st16(p_addr + g * 16, pk);
-          if (kProbeAhead && g == BLK / 32 - 2) s_seen = mbar_test(bar(Smem::s_full, X), (blk & 1) ^ 1);
-          if (g == BLK / 32 - 2) {
+          if (kProbeAhead && g == kEarly) s_seen = mbar_test(bar(Smem::s_full, X), (blk & 1) ^ 1);
+          if (kRescaleLate && g == kEarly && rescale) rescale_o(alpha);
+          if (g == kEarly) {
             // all but the last 32 key columns of P are stored: their share of P V may start
             tmem_st_wait();
             tc_fence_before();

@@ -587,12 +587,12 @@ def test_a_block_of_keys_at_minus_infinity_draws_nothing(seqlen):
     (64, 50 * 64 + 7, 4, 2, True),
 ])
 def test_row_maxima_that_grow_from_block_to_block(block, seqlen, hq, hkv, dense):
-    # The scores of block j are about step[j] powers of two: rows whose maximum grows by less than the rescale threshold (24)
-    # keep the reference of an earlier block, at 23 with probabilities up to 2^23; larger steps rescale O, once or again.
+    # The scores of block j are about step[j] powers of two: rows whose maximum grows by less than the rescale threshold (8)
+    # keep the reference of an earlier block; larger steps rescale O, once or again.
     w = wl.small("grow", seqlens=(seqlen,), hq=hq, hkv=hkv, block=block, permille=1000, mu_num=1, mu_den=1, seed=seqlen)
     data = dict(wl.make_qkv(w))
     r = np.random.default_rng(seqlen + hq)
-    step = np.array([0, 10, 23, 22, 48, 40, 71, 95, 95, 60] + list(r.integers(0, 120, size=60)))[:(seqlen + block - 1) // block]
+    step = np.array([0, 7, 14, 22, 21, 48, 71, 95, 95, 60] + list(r.integers(0, 120, size=60)))[:(seqlen + block - 1) // block]
     u = r.standard_normal(128)
     u /= np.linalg.norm(u)
     scale = np.sqrt(128) / np.log2(np.e) / 8  # q = 8 u, so that k = scale * step * u scores `step` powers of two
