@@ -10,9 +10,13 @@
 // block, block) lets one TMA box fetch "64 columns of token t of 128 consecutive blocks" as a 128-row
 // K-major operand tile; the query map is walked with t = B-1-s, the key map with t = s.
 //
-// One CTA per (128 x 128 tile of one sequence's causal triangle, query head): warp 4 issues the copies
-// through a ring of stages, warp 5 the MMAs into one TMEM accumulator, warps 0-3 write the tile as floats
-// (the public M) or as bit planes of the selection keys (the fused path's workspace form).  Only FULL
+// One CTA per (128 x 128 tile of one sequence's causal triangle, two query heads of a group or one where a group's size is odd,
+// part of the inner dimension): warp 4 issues the copies through a ring of stages, warp 5 the MMAs into a TMEM accumulator for
+// each head, warps 0-3 write the tile as floats (the public M) or as bit planes of the selection keys (the fused path's
+// workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
+// heads share the key tile, 48 KB for two heads' step instead of 64, and short sequences, whose tiles are fewer than the SMs,
+// are computed in parts (antidiag_parts), which a small kernel adds up in order.  Lists of a call at 32 / 8 heads, a head and a whole
+// sum each / two heads, in parts: 16K tokens 89.8 / 63.2 us, 32K 119.5 / 102.5, 128K 877 / 780.  Only FULL
 // blocks go through the contraction (the maps end at the last full block, so nothing is read past a
 // sequence); a sequence's partial last block, whose anti-diagonal is truncated (the mean is over the
 // pairs whose two tokens exist), is one metric row that a small second kernel computes with plain FMAs.
@@ -33,13 +37,12 @@ using namespace ptx;
 
 constexpr int kThreads = 192;
 constexpr int kTile = 128;
-constexpr int kStages = 6;
+constexpr int kRingTiles = 12;           // operand tiles in the ring: six stages of two, or four of three with two heads
 constexpr int kPartBytes = kTile * 128;  // one operand tile of a step: 128 rows x 64 columns bf16
-constexpr int kSmemA = 0;
-constexpr int kSmemB = kSmemA + kStages * kPartBytes;
-constexpr int kSmemBias = kSmemB + kStages * kPartBytes;
-constexpr int kSmemBars = kSmemBias + kTile * 4;  // full[kStages], empty[kStages], acc_full
-constexpr int kSmemTmem = kSmemBars + (2 * kStages + 1) * 8;
+constexpr int kSmemBias = kRingTiles * kPartBytes;
+constexpr int kSmemBars = kSmemBias + kTile * 4;  // full[stages], empty[stages], acc_full
+constexpr int kStagesMax = kRingTiles / 2;
+constexpr int kSmemTmem = kSmemBars + (2 * kStagesMax + 1) * 8;
 constexpr int kSmemBytes = kSmemTmem + 16 + 1024;  // slack for manual 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 constexpr uint64_t kWaitLimitNs = 200ull * 1000 * 1000;
@@ -63,12 +66,19 @@ struct AntiArgs {
   const __nv_bfloat16 *Q, *K;
   int64_t q_st, q_sh, kv_st, kv_sh;
   int batch;
+  // sums over parts of the inner dimension, [max_parts][n_tiles][Hq][column][row] of the tile, of the sequences in parts
+  float* sums;
+  int parts[kMaxSeqs];
 };
 
+__device__ __forceinline__ float* part_sums(const AntiArgs& a, int part, int tile, int n_tiles, int h) {
+  return a.sums + (((int64_t)part * n_tiles + tile) * a.Hq + h) * (kTile * kTile);
+}
+
 // Bounded wait; false when the time limit ran out (the status words then say so).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* status) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* status, int head) {
   if (mbar_wait_bounded(bar, parity, kWaitLimitNs)) return true;
-  if (atomicCAS(status + 4, 0, kGaveUpAntidiag) == 0) { status[5] = (int32_t)blockIdx.x; status[6] = (int32_t)blockIdx.y; }
+  if (atomicCAS(status + 4, 0, kGaveUpAntidiag) == 0) { status[5] = (int32_t)blockIdx.x; status[6] = head; }
   return false;
 }
 
@@ -80,7 +90,32 @@ __device__ __forceinline__ uint32_t metric_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-template <int BLK>
+// 32 columns of one row of a tile, v = the sums of its anti-diagonals: the metric as floats, or as bit planes of its keys.
+__device__ __forceinline__ void store_columns(const AntiArgs& a, int seq, int h, int r0, int nb, int rl, int col, const float (&v)[32],
+                                              const float* bias) {
+  const int stride = (nb + 31) & ~31;
+  if (a.as_keys) {
+    if (col >= stride) return;
+    uint32_t* dst = (uint32_t*)a.M + (int64_t)h * a.mt_tot + a.rows.seq_mt_off[seq] + (int64_t)rl * stride + col;
+    uint32_t w[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) w[c] = __float_as_uint(fmaxf(fmaf(a.scale, v[c], bias[c]) + 0.0f, __int_as_float(0xff800000)));
+    transpose32(w);
+    const uint32_t neg = w[31];  // bit t: value t is negative
+#pragma unroll
+    for (int k = 0; k < 31; ++k) w[k] ^= neg;
+    w[31] = ~neg;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) *(uint4*)(dst + q * 4) = make_uint4(w[q * 4], w[q * 4 + 1], w[q * 4 + 2], w[q * 4 + 3]);
+  } else {
+    float* mrow = a.M + (int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)rl * nb;
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+      if (col + c <= r0 + rl) mrow[col + c] = fmaf(a.scale, v[c], bias[c]);
+  }
+}
+
+template <int BLK, int kHeads>
 __global__ void __launch_bounds__(kThreads, 1)
 antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -88,20 +123,23 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   unsigned char* smem_gen = smem_raw + (smem_base - (uint32_t)__cvta_generic_to_shared(smem_raw));
   const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const uint32_t bars = smem_base + kSmemBars;
+  constexpr int kStages = kRingTiles / (kHeads + 1);
+  constexpr int kStageBytes = (kHeads + 1) * kPartBytes;  // the key tile, then the heads' query tiles
   auto full = [&](int s) { return bars + 8 * s; };
   auto empty = [&](int s) { return bars + 8 * (kStages + s); };
   const uint32_t acc_full = bars + 8 * 2 * kStages;
   float* bias = (float*)(smem_gen + kSmemBias);
 
   const int seq = a.tiles[3 * blockIdx.x], ti = a.tiles[3 * blockIdx.x + 1], tj = a.tiles[3 * blockIdx.x + 2];
-  const int h = blockIdx.y, kvh = h / a.g;
+  const int h = (int)blockIdx.y * kHeads, kvh = h / a.g;
+  const int parts = a.parts[seq], part = blockIdx.z;
   const int nb = a.rows.seq_nblk[seq];
   const int r0 = a.rows.seq_r0[seq];
   // full blocks of the sequence: all of them, or all but the last when that one is partial
   const int last_ntok = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1];
   const int nfull = last_ntok == BLK ? nb : nb - 1;
-  // nothing to do when the tile holds no full row or no full column
-  if (r0 + ti * kTile >= nfull || tj * kTile >= nfull) {
+  // nothing to do when the tile holds no full row or no full column, or is computed in fewer parts
+  if (r0 + ti * kTile >= nfull || tj * kTile >= nfull || part >= parts) {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // before it counts as done: see the partial-row kernel
     return;
   }
@@ -112,39 +150,34 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
     mbar_init_fence();
   }
   if (warp == 5) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_base + kSmemTmem), "n"(128)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_base + kSmemTmem), "n"(128 * kHeads)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  // Launched as a programmatic dependent of the pooling kernel (which writes MV), everything above overlaps
-  // its tail.  (Without that launch attribute both are no-ops.)
-  // The partial-row kernel may start behind the wait: it needs MV as well, and nothing of this kernel's.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x < kTile) {
-    const int c = threadIdx.x;
-    bias[c] = (tj * kTile + c < nb) ? a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + tj * kTile + c] : 0.f;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *(volatile uint32_t*)(smem_gen + kSmemTmem);
   constexpr int kIters = 2 * BLK;  // (token of the block, half of the head dimension)
+  const int first = part * kIters / parts, n_iters = (part + 1) * kIters / parts - first;
 
   if (warp == 4) {
     // ============================== copies ==============================
     const bool leader = elect_one();
     bool ok = true;
 #pragma unroll 1
-    for (int it = 0; it < kIters && ok; ++it) {
-      const int st = it % kStages, s = it >> 1, half = it & 1;
-      if (it >= kStages) ok = __all_sync(0xffffffffu, mbar_wait(empty(st), ((it / kStages) - 1) & 1, a.status));
+    for (int it = 0; it < n_iters && ok; ++it) {
+      const int st = it % kStages, s = (first + it) >> 1, half = (first + it) & 1;
+      if (it >= kStages) ok = __all_sync(0xffffffffu, mbar_wait(empty(st), ((it / kStages) - 1) & 1, a.status, h));
       if (!ok) break;
       if (leader) {
-        mbar_expect_tx(full(st), 2 * kPartBytes);
+        const uint32_t stage = smem_base + st * kStageBytes;
+        mbar_expect_tx(full(st), kStageBytes);
         // query tokens in reverse order, key tokens in order: step s pairs q[B-1-s] with k[s]
-        tma_load_4d(smem_base + kSmemA + st * kPartBytes, &maps.q[seq], full(st), 64 * half, h, BLK - 1 - s, ti * kTile);
-        tma_load_4d(smem_base + kSmemB + st * kPartBytes, &maps.k[seq], full(st), 64 * half, kvh, s, tj * kTile);
+        tma_load_4d(stage, &maps.k[seq], full(st), 64 * half, kvh, s, tj * kTile);
+#pragma unroll
+        for (int x = 0; x < kHeads; ++x)
+          tma_load_4d(stage + (x + 1) * kPartBytes, &maps.q[seq], full(st), 64 * half, h + x, BLK - 1 - s, ti * kTile);
       }
       __syncwarp();
     }
@@ -153,57 +186,54 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
     const bool leader = elect_one();
     bool ok = true;
 #pragma unroll 1
-    for (int it = 0; it < kIters && ok; ++it) {
+    for (int it = 0; it < n_iters && ok; ++it) {
       const int st = it % kStages;
-      ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status));
+      ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status, h));
       if (!ok) break;
       tc_fence_after();
       if (leader) {
-        const uint32_t a_addr = smem_base + kSmemA + st * kPartBytes, b_addr = smem_base + kSmemB + st * kPartBytes;
+        const uint32_t b_addr = smem_base + st * kStageBytes;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) mma_ss(tmem, smem_desc(a_addr + k * 32), smem_desc(b_addr + k * 32), kIdesc, (it | k) ? 1u : 0u);
+        for (int x = 0; x < kHeads; ++x) {
+          const uint32_t a_addr = b_addr + (x + 1) * kPartBytes;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_ss(tmem + x * kTile, smem_desc(a_addr + k * 32), smem_desc(b_addr + k * 32), kIdesc, (it | k) ? 1u : 0u);
+        }
         tc_commit(empty(st));
-        if (it == kIters - 1) tc_commit(acc_full);
+        if (it == n_iters - 1) tc_commit(acc_full);
       }
       __syncwarp();
     }
   } else {
     // ============================== epilogue ==============================
+    // Launched as a programmatic dependent of the pooling kernel, of which only these warps need anything (MV): the contraction
+    // itself starts beside its last CTAs, on Q and K as they were before it.  The partial-row kernel may start behind the wait:
+    // it needs MV as well, and nothing of this kernel's.  (Without that launch attribute both are no-ops.)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (threadIdx.x < kTile) {
+      const int c = threadIdx.x;
+      bias[c] = (tj * kTile + c < nb) ? a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + tj * kTile + c] : 0.f;
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");  // these four warps
     const int m = warp * 32 + lane;       // row of the tile == TMEM lane
     const int rl = ti * kTile + m;        // row inside the chunk
     const int r = r0 + rl;                // row inside the sequence
-    const int stride = (nb + 31) & ~31;
-    if (__all_sync(0xffffffffu, mbar_wait(acc_full, 0, a.status))) {
+    if (__all_sync(0xffffffffu, mbar_wait(acc_full, 0, a.status, h))) {
       tc_fence_after();
       const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-      uint32_t* dst_planes = (uint32_t*)a.M + (int64_t)h * a.mt_tot + a.rows.seq_mt_off[seq] + (int64_t)rl * stride + tj * kTile;
-      float* mrow = a.M + (int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)rl * nb;
 #pragma unroll 1
-      for (int gq = 0; gq < 4; ++gq) {
+      for (int gq = 0; gq < 4 * kHeads; ++gq) {
         float v[32];
         tmem_ld32_sync(taddr + gq * 32, v);
-        if (r >= nfull) continue;  // rows of the partial block (or past the end) belong to the other kernel
-        if (a.as_keys) {
-          uint32_t w[32];
+        const int x = gq >> 2, c0 = (gq & 3) * 32;
+        if (parts > 1) {
+          float* dst = part_sums(a, part, blockIdx.x, gridDim.x, h + x) + c0 * kTile + m;
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
-            w[c] = __float_as_uint(fmaxf(fmaf(a.scale, v[c], bias[gq * 32 + c]) + 0.0f, __int_as_float(0xff800000)));
-          transpose32(w);
-          const uint32_t neg = w[31];  // bit t: value t is negative
-#pragma unroll
-          for (int k = 0; k < 31; ++k) w[k] ^= neg;
-          w[31] = ~neg;
-          if (tj * kTile + gq * 32 < stride) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *(uint4*)(dst_planes + gq * 32 + q * 4) = make_uint4(w[q * 4], w[q * 4 + 1], w[q * 4 + 2], w[q * 4 + 3]);
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const int cg = tj * kTile + gq * 32 + c;
-            if (cg <= r) mrow[cg] = fmaf(a.scale, v[c], bias[gq * 32 + c]);
-          }
+          for (int c = 0; c < 32; ++c) dst[c * kTile] = v[c];
+        } else if (r < nfull) {  // rows of the partial block (or past the end) belong to the other kernel
+          store_columns(a, seq, h + x, r0, nb, rl, tj * kTile + c0, v, bias + c0);
         }
       }
     }
@@ -212,8 +242,33 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   __syncthreads();
   if (warp == 5) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(128) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(128 * kHeads) : "memory");
   }
+}
+
+// Adds up the parts of a tile of a sequence in parts, in order, 32 columns a CTA: the metric of its full rows.
+template <int BLK>
+__global__ void __launch_bounds__(kTile) antidiag_sum_kernel(const AntiArgs a, int n_tiles) {
+  const int tile = blockIdx.x, h = blockIdx.y, c0 = blockIdx.z * 32, m = threadIdx.x;
+  const int seq = a.tiles[3 * tile], ti = a.tiles[3 * tile + 1], tj = a.tiles[3 * tile + 2];
+  const int nb = a.rows.seq_nblk[seq], r0 = a.rows.seq_r0[seq], parts = a.parts[seq];
+  const int nfull = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1] == BLK ? nb : nb - 1;
+  const int rl = ti * kTile + m;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (parts == 1 || r0 + rl >= nfull || tj * kTile >= nfull) return;
+  float v[32], bias[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] = part_sums(a, 0, tile, n_tiles, h)[(c0 + c) * kTile + m];
+#pragma unroll 1
+  for (int p = 1; p < parts; ++p) {
+    const float* src = part_sums(a, p, tile, n_tiles, h) + c0 * kTile + m;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) v[c] += src[c * kTile];
+  }
+  const float* mv = a.mv + (int64_t)(h / a.g) * a.KB_tot + a.rows.seq_kb_off[seq];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) bias[c] = tj * kTile + c0 + c < nb ? a.beta * mv[tj * kTile + c0 + c] : 0.f;
+  store_columns(a, seq, h, r0, nb, rl, tj * kTile + c0, v, bias);
 }
 
 // The metric row of a sequence's partial last block (when it belongs to the query chunk): for every j <= r the
@@ -221,7 +276,8 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
 // reads 256-byte rows with 16-byte loads and multiplies the key rows of four columns with the matching query rows of
 // four heads of the group, 8 loads for 16 products (with a column at a time the L1 traffic of the query rows bounds the
 // kernel, with one row in flight the latency: a 60-token block against 255 full blocks at 32 / 8 heads took 0.76 ms);
-// two warps share four columns, each taking every other pair of rows.
+// two warps share four columns, each taking every other pair of rows.  (CTAs of 256 threads, which fit beside one of the
+// contraction on its SM, take longer than they save: 133 us of a call for a ragged 32K prompt, 116.)
 constexpr int kPartThreads = 512;
 constexpr int kPartMaxGroup = 32;
 template <int BLK>
@@ -342,7 +398,16 @@ __global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const An
 
 int antidiag_max_sequences() { return kMaxSeqs; }
 
-cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys,
+// In how many parts the inner dimension is summed for a sequence of n blocks: by its whole length alone, so that its lists do
+// not depend on the batch, its chunks or the heads of a plan.  Up to 128 blocks are one tile, 16 CTAs at 32 / 8 heads; up to 256
+// three, 48 CTAs; up to 384 six, 96 CTAs, in three parts two waves of a third each.  Beyond, the tiles fill the SMs.
+int antidiag_parts(int n) { return n <= kTile ? 8 : n <= 3 * kTile ? 3 : 1; }
+
+size_t antidiag_sums_bytes(int max_parts, int n_tiles, int Hq) {
+  return max_parts > 1 ? (size_t)max_parts * n_tiles * Hq * kTile * kTile * sizeof(float) : 0;
+}
+
+cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s) {
   *launched = 0;
   const int B = p.cfg.block, batch = p.cfg.batch;
@@ -375,13 +440,17 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   a.Q = (const __nv_bfloat16*)Q; a.K = (const __nv_bfloat16*)K;
   a.q_st = p.cfg.q_stride_tok; a.q_sh = p.cfg.q_stride_head; a.kv_st = p.cfg.kv_stride_tok; a.kv_sh = p.cfg.kv_stride_head;
   a.batch = batch;
+  a.sums = sums;
+  for (int b = 0; b < batch; ++b) a.parts[b] = p.antidiag_parts[b];
+  const bool two = a.g % 2 == 0;
 
   static bool attr_set[64] = {};
   const int dev_slot = p.device & 63;
   if (!attr_set[dev_slot]) {
-    cudaError_t e = cudaFuncSetAttribute(antidiag_metric_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(antidiag_metric_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(antidiag_metric_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr_set[dev_slot] = true;
   }
@@ -389,26 +458,40 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)a.Hq);
+  cfg.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)(two ? a.Hq / 2 : a.Hq), (unsigned)p.antidiag_max_parts);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = B == 128 ? cudaLaunchKernelEx(&cfg, antidiag_metric_kernel<128>, maps, a)
-                           : cudaLaunchKernelEx(&cfg, antidiag_metric_kernel<64>, maps, a);
+  auto kernel = B == 128 ? (two ? antidiag_metric_kernel<128, 2> : antidiag_metric_kernel<128, 1>)
+                         : (two ? antidiag_metric_kernel<64, 2> : antidiag_metric_kernel<64, 1>);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, maps, a);
   if (e != cudaSuccess) return e;
   ++*launched;
-  if (!any_partial) return e;
-  // the metric rows of partial last blocks, beside the contraction (the rows are not those the contraction writes, and
-  // MV is complete once every CTA of the contraction is past its wait or gone)
-  cudaLaunchConfig_t cfg2 = {};
-  cfg2.gridDim = dim3((unsigned)((p.max_nblk + 31) / 32), (unsigned)(batch * p.cfg.num_kv_heads));
-  cfg2.blockDim = dim3(kPartThreads);
-  cfg2.stream = s;
-  cfg2.attrs = attr;
-  cfg2.numAttrs = 1;
-  e = B == 128 ? cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<128>, a) : cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<64>, a);
+  if (any_partial) {
+    // the metric rows of partial last blocks, beside the contraction (the rows are not those the contraction writes, and
+    // MV is complete once every CTA of the contraction is past its wait or gone)
+    cudaLaunchConfig_t cfg2 = {};
+    cfg2.gridDim = dim3((unsigned)((p.max_nblk + 31) / 32), (unsigned)(batch * p.cfg.num_kv_heads));
+    cfg2.blockDim = dim3(kPartThreads);
+    cfg2.stream = s;
+    cfg2.attrs = attr;
+    cfg2.numAttrs = 1;
+    e = B == 128 ? cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<128>, a) : cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<64>, a);
+    if (e != cudaSuccess) return e;
+    ++*launched;
+  }
+  if (p.antidiag_max_parts == 1) return e;
+  // behind the partial-row kernel, which is complete only after the contraction is, or behind the contraction itself
+  cudaLaunchConfig_t cfg3 = {};
+  cfg3.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)a.Hq, kTile / 32);
+  cfg3.blockDim = dim3(kTile);
+  cfg3.stream = s;
+  cfg3.attrs = attr;
+  cfg3.numAttrs = 1;
+  e = B == 128 ? cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<128>, a, p.n_gemm_tiles)
+               : cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<64>, a, p.n_gemm_tiles);
   if (e == cudaSuccess) ++*launched;
   return e;
 }

@@ -231,6 +231,8 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     const int64_t n_tot = o.total_len_host ? o.total_len_host[b] : n;
     const int64_t nb_tot = (n_tot + B - 1) / B;        // blocks of the whole sequence: N of Eq. 3
     is_short[b] = p.score_mode == 0 && nb_tot <= kShortBlocks;
+    p.antidiag_parts.push_back(p.score_mode == 1 ? antidiag_parts((int)std::min<int64_t>(nb_tot, INT32_MAX)) : 1);
+    p.antidiag_max_parts = std::max(p.antidiag_max_parts, p.antidiag_parts.back());
     seq_tok0[b] = p.cu[b];
     seq_nblk[b] = nb;
     seq_r0[b] = r0;
@@ -353,6 +355,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     p.ws.qsplit = off; off = align_up(off + (size_t)3 * p.H_list * p.R_tot * kHeadDim * 2, 256);
     p.ws.ksplit = off; off = align_up(off + (own_k ? (size_t)3 * Hkv * p.KB_tot * kHeadDim * 2 : 0), 256);
     p.ws.metric = off; off = align_up(off + (size_t)p.H_list * (size_t)p.mt_tot * 4, 256);
+    p.ws.sums = off; off = align_up(off + (p.score_mode == 1 ? antidiag_sums_bytes(p.antidiag_max_parts, p.n_gemm_tiles, p.cfg.num_q_heads) : 0), 256);
     p.ws.sel_idx = off; off = align_up(off + (size_t)p.H_list * p.R_tot * p.k_max * 4, 256);
     p.ws.sel_cnt = off; off = align_up(off + (size_t)p.H_list * p.R_tot * 4, 256);
     p.ws.total = off;
@@ -505,7 +508,7 @@ static int enqueue_metric(const Plan& p, const void* Q, const void* K, uint8_t* 
   int32_t* status = (int32_t*)(w + p.ws.status);
   if (p.score_mode == 1) {
     int launched = 0;
-    const int rc = cuda_rc(launch_antidiag_metric(p, Q, K, ks.mv, M, as_keys, status, &launched, s));
+    const int rc = cuda_rc(launch_antidiag_metric(p, Q, K, ks.mv, M, as_keys, (float*)(w + p.ws.sums), status, &launched, s));
     p.last_launches += launched;
     return rc;
   }
@@ -551,9 +554,9 @@ static int enqueue_lists(const Plan& p, const void* Q, const void* K, uint8_t* w
 static int enqueue_score_select(const Plan& p, const void* Q, const void* K, const void* V, void* kcache, uint8_t* w,
                                 int32_t* idx, int32_t* cnt, int first_word, cudaStream_t s) {
   const KSide ks = k_side(p, w, kcache);
-  // (the anti-diagonal mode has no use for the pooled query vectors; the pooling kernel clears the status words as well; with a
+  // (the anti-diagonal mode has no use for the pooled vectors, only for MV; the pooling kernel clears the status words as well; with a
   // cache, K and V are given when it is to be updated with the blocks that the chunk adds)
-  int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, kcache != nullptr,
+  int rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, p.score_mode == 1 ? nullptr : K, V, ks.mv, w + p.ws.qsplit, ks.ksplit, kcache != nullptr,
                                (int32_t*)(w + p.ws.status) + first_word, kStatusWords - first_word, s));
   if (rc != STEM_OK) return rc;
   p.last_launches++;
@@ -572,7 +575,7 @@ int stem_score(const stem_plan* plan, const void* Q, const void* K, const void* 
   cudaStream_t s = (cudaStream_t)stream;
   p.last_launches = 0;
   float* mv = (float*)(w + p.ws.mv);
-  rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, K, V, mv, w + p.ws.qsplit, w + p.ws.ksplit, false,
+  rc = cuda_rc(launch_pool(p, p.score_mode == 1 ? nullptr : Q, p.score_mode == 1 ? nullptr : K, V, mv, w + p.ws.qsplit, w + p.ws.ksplit, false,
                            (int32_t*)(w + p.ws.status) + 4, 4, s));  // ... and the metric kernel's status words
   if (rc != STEM_OK) return rc;
   p.last_launches++;

@@ -50,6 +50,7 @@ struct WorkspaceLayout {
   size_t qsplit = 0;   // bf16 [3, H_list, R_tot, d]: Qbar as hi + mid + lo parts
   size_t ksplit = 0;   // bf16 [3, H_kv, KB_tot, d]: Kbar likewise
   size_t metric = 0;   // uint32 [H_list, mt_tot]: the metric of the fused path as bit planes of its selection keys
+  size_t sums = 0;     // fp32: anti-diagonal scoring, the sums over parts of the inner dimension (antidiag_sums_bytes)
   size_t sel_idx = 0;  // int32 [H_list, R_tot, k_max]
   size_t sel_cnt = 0;  // int32 [H_list, R_tot]
   size_t total = 0;
@@ -77,6 +78,8 @@ struct Plan {
   int32_t k_max = 0, max_nblk = 0;
   int32_t kcache_blocks = 0;  // per-sequence capacity of a caller-owned pooled-K cache (0: none)
   bool share_group = false;   // one index list per (kv head, row)
+  std::vector<int32_t> antidiag_parts;  // anti-diagonal scoring: parts in which a sequence's contraction is summed
+  int32_t antidiag_max_parts = 1;
   int32_t score_mode = 0;     // 0: product of block means (Eq. 7 on pooled blocks); 1: anti-diagonal scoring
   std::vector<int32_t> h_seq_r0, h_seq_qtok0;  // host copies: first chunk row, first packed Q token of every sequence
   int32_t H_list = 0;         // heads of the metric and of the lists: H_q, or H_kv with share_group
@@ -111,8 +114,8 @@ inline size_t kcache_bytes(const Plan& p) { return kcache_mv_offset(p) + (size_t
 
 // Kernel launchers (each returns the cudaError_t of the launch).
 // Alg. 1 step 1.  Q side (Q != null): Qbar of every query row as hi + mid + lo bf16 parts into qsplit
-// [3, H_list, R_tot, d] (the mean over the heads of a kv group as well, with share_group).  K side (K, V != null):
-// Kbar parts into ksplit [3, H_kv, KB_tot, d] and MV into mv [H_kv, KB_tot], for every key block of the plan or,
+// [3, H_list, R_tot, d] (the mean over the heads of a kv group as well, with share_group).  K side (V != null):
+// Kbar parts into ksplit [3, H_kv, KB_tot, d] (K null: none) and MV into mv [H_kv, KB_tot], for every key block of the plan or,
 // with only_new, for the blocks the chunk adds.  The n_clear status words at `clear` are set to zero.
 cudaError_t launch_pool(const Plan& p, const void* Q, const void* K, const void* V, float* mv, void* qsplit, void* ksplit,
                         bool only_new, int32_t* clear, int n_clear, cudaStream_t s);
@@ -130,7 +133,9 @@ cudaError_t launch_metric_gemm(const Plan& p, const void* qsplit, const void* ks
 // contraction over the full blocks plus, where a sequence ends in a partial block, a small kernel for that row.
 // *launched receives the number of kernels enqueued.
 int antidiag_max_sequences();
-cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys,
+int antidiag_parts(int n_blocks);
+size_t antidiag_sums_bytes(int max_parts, int n_tiles, int Hq);
+cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s);
 
 // Selection from a stored metric (layout of stem_score's M), one warp per (head, row).

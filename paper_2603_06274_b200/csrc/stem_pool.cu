@@ -33,7 +33,7 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
 // (16 lanes x 16 bytes); a warp covers kTok / 4 consecutive tokens, two per step.
 // CTAs 0 .. n_q - 1 pool Q: one per (query row, list head); with heads_per_list > 1 (one index list per kv
 // group) a CTA averages the block over the group's query heads as well.  The CTAs after them pool K and V:
-// one per (key block, kv head, K or V), over every key block of the plan or only the blocks a chunk adds.
+// one per (key block, kv head, K if it is given or V), over every key block of the plan or only the blocks a chunk adds.
 struct PoolArgs {
   const __nv_bfloat16 *Q, *K, *V;
   int64_t q_st, q_sh, kv_st, kv_sh;
@@ -71,11 +71,12 @@ __global__ void __launch_bounds__(128) pool_kernel(const PoolArgs a) {
     ntok = a.rows.row_ntok[R];
     dst_row = R;
   } else {
-    const int i = ((int)blockIdx.x - a.n_q) / (2 * a.Hkv);
-    const int slot = ((int)blockIdx.x - a.n_q) - i * 2 * a.Hkv;
+    const int heads_k = a.K ? a.Hkv : 0, per = heads_k + a.Hkv;
+    const int i = ((int)blockIdx.x - a.n_q) / per;
+    const int slot = ((int)blockIdx.x - a.n_q) - i * per;
     const int kb = a.only_new ? a.rows.kb_new[i] : i;
-    kind = slot < a.Hkv ? 1 : 2;
-    h = kind == 1 ? slot : slot - a.Hkv;
+    kind = slot < heads_k ? 1 : 2;
+    h = kind == 1 ? slot : slot - heads_k;
     base = (kind == 1 ? a.K : a.V) + (int64_t)h * a.kv_sh;
     st = a.kv_st; sh = a.kv_sh;
     tok0 = a.rows.kb_tok0[kb];
@@ -180,7 +181,7 @@ cudaError_t launch_pool(const Plan& p, const void* Q, const void* K, const void*
   a.n_q = Q ? p.R_tot * p.H_list : 0;
   a.only_new = only_new ? 1 : 0;
   a.rows = p.rows; a.mv = mv; a.qsplit = (__nv_bfloat16*)qsplit; a.ksplit = (__nv_bfloat16*)ksplit;
-  const int64_t n_k = K ? (int64_t)(only_new ? p.n_kb_new : p.n_kb_all) * 2 * p.cfg.num_kv_heads : 0;
+  const int64_t n_k = V ? (int64_t)(only_new ? p.n_kb_new : p.n_kb_all) * (K ? 2 : 1) * p.cfg.num_kv_heads : 0;
   const dim3 grid((unsigned)(a.n_q + n_k));
   if (grid.x == 0) return cudaSuccess;
   const bool group_mean = a.heads_per_list > 1;

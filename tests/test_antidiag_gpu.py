@@ -159,3 +159,36 @@ def test_a_query_without_a_partner_in_the_last_block_leaves_its_own_entry_alone(
     assert rows[1][0, nb - 1] == rows[0][0, nb - 1] and np.isfinite(rows[0][0, nb - 1])
     assert np.array_equal(rows[1][1], rows[0][1])
     plan.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (64, (64 * 385, 64 * 130 + 7, 64 * 128), 4, 2),   # a sequence summed at once, one in three parts, one in eight; two heads a tile
+    (64, (64 * 384 + 1, 64 * 3), 3, 1),               # just above the limit with the last block, and tiny; an odd group
+    (128, (128 * 129, 128 * 128 + 100), 6, 1),        # one block above 128; two heads a tile
+])
+def test_metric_of_sequences_summed_in_parts(block, seqlens, hq, hkv):
+    w = wl.small("ad_parts", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=100, seed=sum(seqlens))
+    data = wl.make_qkv(w)
+    M_ref, _ = so.score_antidiag(data["q"], data["k"], data["v"], data["cu_seqlens"], oracle_params(w))
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+
+    def metric(plan, q, k, v):
+        M = torch.full((hq, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_score(plan, q, k, v, M)
+        assert binding.stem_check_status(plan)[0] == 0
+        plan.close()
+        return M.cpu().numpy()
+
+    M_g = metric(StemPlan.from_workload(w, score_mode=1), q, k, v)
+    defined = ~np.isnan(M_ref)
+    assert np.array_equal(np.isnan(M_g), ~defined)
+    assert np.all(np.abs(M_g[defined] - M_ref[defined]) <= METRIC_ABS + METRIC_REL * np.abs(M_ref[defined]))
+    # each sequence alone has the same values: the parts follow from its own length
+    tok = off = 0
+    for n in seqlens:
+        nb = (n + block - 1) // block
+        one = wl.small("ad_one", seqlens=(n,), hq=hq, hkv=hkv, block=block, permille=100)
+        alone = metric(StemPlan.from_workload(one, score_mode=1), q[tok:tok + n], k[tok:tok + n], v[tok:tok + n])
+        assert np.array_equal(alone, M_g[:, off:off + nb * nb], equal_nan=True)
+        tok += n
+        off += nb * nb
