@@ -689,7 +689,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     };
     // O of the blocks so far, whose P V are complete, times alpha.  Before the exponentials this costs a block 550 cycles; once most
     // of its scores are gone, and P V is long complete, less (32K tokens 1273 / 1263 us, dense 16K 1785 / 1764).  Where a CTA runs
-    // one item (kSplit) that would spill: two ragged short prompts 20.5 us of a call, 18.6 before the exponentials.
+    // one item (kSplit) that would spill: two ragged short prompts 20.5 us of a call, 19.1 before the exponentials.
     constexpr bool kRescaleLate = !kSplit;
     auto rescale_o = [&](const float alpha) {
       constexpr int kAtOnce = kSpareQ ? 64 : 32;  // columns
