@@ -805,7 +805,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           l_run = 0.f;
           m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
         } else {
-          const bool grow = mx_c > m_run + kRescaleThreshold;
+          // (Rows behind the sequence's last token hold what is packed behind it: they have no vote on the others' references.)
+          const bool grow = row_valid && mx_c > m_run + kRescaleThreshold;
           rescale = __any_sync(0xffffffffu, grow);
           if (rescale) {
             const float m_new = fmaxf(m_run, mx_c);

@@ -616,3 +616,35 @@ def test_row_maxima_that_grow_from_block_to_block(block, seqlen, hq, hkv, dense)
     check_attention(from_dev_bf16(out), O_ref, ~np.isnan(O_ref), label="growing maxima")
     assert np.abs(lse.cpu().numpy() - lse_ref).max() < 1e-3
     plan.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv,dense", [
+    (128, (6 * 128 - 80, 100), 2, 1, False),      # each slot half of a list; the last block's second warp has 16 rows
+    (64, (9 * 64 - 19, 64), 2, 1, False),
+    (128, (38 * 128 - 5, 300), 4, 2, False),      # item by item
+    (128, (25 * 128 - 70, 500), 8, 4, False),     # neighbouring items, merged lists
+    (64, (50 * 64 + 7, 200), 4, 2, False),
+    (128, (25 * 128 - 70, 500), 8, 4, True),      # pairs of heads on one stream of K / V
+    (64, (50 * 64 + 7, 200), 4, 2, True),
+])
+def test_a_sequence_does_not_see_what_is_packed_behind_it(block, seqlens, hq, hkv, dense):
+    # The rows of a tile behind a sequence's last token hold the next sequence's queries.  Nothing of them may reach the rows
+    # before: the same bits, whether their scores are about 1 or about 2^60 (which outgrows every reference).
+    w = wl.small("behind", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=400, seed=sum(seqlens))
+    data, plan, q, k, v = _setup(w)
+    n = seqlens[0]
+    idx, cnt = _alloc_lists(plan)
+    binding.stem_score_select(plan, q, k, v, idx, cnt)
+    lists = (None, None) if dense else (idx, cnt)
+    got = []
+    for scale in (1.0, 2.0 ** 30):
+        q[n:] *= scale
+        k[n:] *= scale
+        out = torch.full((w.total_tokens, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((hq, w.total_tokens), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_sparse_prefill(plan, q, k, v, *lists, out, lse)
+        _ok(plan)
+        got.append((out[:n].clone(), lse[:, :n].clone()))
+    assert torch.isfinite(got[0][0].float()).all()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    plan.close()
