@@ -15,7 +15,7 @@
 // each head, warps 0-3 write the tile as floats (the public M) or as bit planes of the selection keys (the fused path's
 // workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
 // heads share the key tile, 48 KB for two heads' step instead of 64, and short sequences, whose tiles are fewer than the SMs,
-// are computed in parts (antidiag_parts), which a small kernel adds up in order.  Lists of a call at 32 / 8 heads, a head and a whole
+// are computed in parts (antidiag_class), which a small kernel adds up in order.  Lists of a call at 32 / 8 heads, a head and a whole
 // sum each / two heads, in parts: 16K tokens 89.8 / 63.2 us, 32K 119.5 / 102.5, 128K 877 / 780.  Only FULL
 // blocks go through the contraction (the maps end at the last full block, so nothing is read past a
 // sequence); a sequence's partial last block, whose anti-diagonal is truncated (the mean is over the
@@ -53,7 +53,9 @@ struct MapSet {
 };
 
 struct AntiArgs {
-  const int32_t* tiles;  // [n_tiles][3] (sequence, row tile, column tile)
+  const AntidiagTile* tiles;
+  int n_tiles[kAntidiagClasses];
+  int parts;             // if all tiles are of one class; else 0
   const float* mv;       // [H_kv, KB_tot]
   float* M;
   int32_t* status;
@@ -66,19 +68,17 @@ struct AntiArgs {
   const __nv_bfloat16 *Q, *K;
   int64_t q_st, q_sh, kv_st, kv_sh;
   int batch;
-  // sums over parts of the inner dimension, [max_parts][n_tiles][Hq][column][row] of the tile, of the sequences in parts
-  float* sums;
-  int parts[kMaxSeqs];
+  float* sums;  // over parts of the inner dimension, [slot][Hq][column][row] of the tile; slots: class, part, tile
 };
 
-__device__ __forceinline__ float* part_sums(const AntiArgs& a, int part, int tile, int n_tiles, int h) {
-  return a.sums + (((int64_t)part * n_tiles + tile) * a.Hq + h) * (kTile * kTile);
+__device__ __forceinline__ float* part_sums(const AntiArgs& a, int slot, int h) {
+  return a.sums + ((int64_t)slot * a.Hq + h) * (kTile * kTile);
 }
 
 // Bounded wait; false when the time limit ran out (the status words then say so).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* status, int head) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* status, int tile, int head) {
   if (mbar_wait_bounded(bar, parity, kWaitLimitNs)) return true;
-  if (atomicCAS(status + 4, 0, kGaveUpAntidiag) == 0) { status[5] = (int32_t)blockIdx.x; status[6] = head; }
+  if (atomicCAS(status + 4, 0, kGaveUpAntidiag) == 0) { status[5] = tile; status[6] = head; }
   return false;
 }
 
@@ -90,16 +90,15 @@ __device__ __forceinline__ uint32_t metric_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// 32 columns of one row of a tile, v = the sums of its anti-diagonals: the metric as floats, or as bit planes of its keys.
-__device__ __forceinline__ void store_columns(const AntiArgs& a, int seq, int h, int r0, int nb, int rl, int col, const float (&v)[32],
-                                              const float* bias) {
+// 32 columns of one row of a tile: the metric v as floats, or as bit planes of its keys.
+__device__ __forceinline__ void store_columns(const AntiArgs& a, int seq, int h, int r0, int nb, int rl, int col, const float (&v)[32]) {
   const int stride = (nb + 31) & ~31;
   if (a.as_keys) {
     if (col >= stride) return;
     uint32_t* dst = (uint32_t*)a.M + (int64_t)h * a.mt_tot + a.rows.seq_mt_off[seq] + (int64_t)rl * stride + col;
     uint32_t w[32];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) w[c] = __float_as_uint(fmaxf(fmaf(a.scale, v[c], bias[c]) + 0.0f, __int_as_float(0xff800000)));
+    for (int c = 0; c < 32; ++c) w[c] = __float_as_uint(fmaxf(v[c] + 0.0f, __int_as_float(0xff800000)));
     transpose32(w);
     const uint32_t neg = w[31];  // bit t: value t is negative
 #pragma unroll
@@ -111,7 +110,7 @@ __device__ __forceinline__ void store_columns(const AntiArgs& a, int seq, int h,
     float* mrow = a.M + (int64_t)h * a.m_tot + a.rows.seq_m_off[seq] + (int64_t)rl * nb;
 #pragma unroll
     for (int c = 0; c < 32; ++c)
-      if (col + c <= r0 + rl) mrow[col + c] = fmaf(a.scale, v[c], bias[c]);
+      if (col + c <= r0 + rl) mrow[col + c] = v[c];
   }
 }
 
@@ -130,19 +129,37 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   const uint32_t acc_full = bars + 8 * 2 * kStages;
   float* bias = (float*)(smem_gen + kSmemBias);
 
-  const int seq = a.tiles[3 * blockIdx.x], ti = a.tiles[3 * blockIdx.x + 1], tj = a.tiles[3 * blockIdx.x + 2];
-  const int h = (int)blockIdx.y * kHeads, kvh = h / a.g;
-  const int parts = a.parts[seq], part = blockIdx.z;
+  // The CTAs in order: whole sums first; in a class all tiles and heads of the first part before those of the next, so that the
+  // CTAs that run together read the same tokens of all heads, whole rows of Q and K (part by part of a tile and head: eight
+  // prompts of 16K tokens 374 us of a call, so 361).
+  int tile = (int)blockIdx.x, y = (int)blockIdx.y, part = (int)blockIdx.z, parts = a.parts, slot = part * (int)gridDim.x + tile;
+  if (parts == 0) {  // tiles of several classes: a grid of one dimension
+    int n_tiles = 0, tile0 = 0, rest = tile;
+    slot = 0;
+#pragma unroll 1
+    for (int c = 0; c < kAntidiagClasses; ++c) {
+      tile0 += n_tiles;
+      n_tiles = a.n_tiles[c];
+      parts = antidiag_parts(c);
+      const int per_part = n_tiles * (a.Hq / kHeads);
+      for (part = 0; part < parts && rest >= per_part; ++part) {
+        rest -= per_part;
+        if (parts > 1) slot += n_tiles;
+      }
+      if (part < parts) break;
+    }
+    y = rest / n_tiles;
+    tile = tile0 + rest - y * n_tiles;
+    slot += rest - y * n_tiles;
+  }
+  const AntidiagTile at = a.tiles[tile];
+  const int seq = at.seq, ti = at.ti, tj = at.tj;
+  const int h = y * kHeads, kvh = h / a.g;
   const int nb = a.rows.seq_nblk[seq];
   const int r0 = a.rows.seq_r0[seq];
   // full blocks of the sequence: all of them, or all but the last when that one is partial
   const int last_ntok = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1];
   const int nfull = last_ntok == BLK ? nb : nb - 1;
-  // nothing to do when the tile holds no full row or no full column, or is computed in fewer parts
-  if (r0 + ti * kTile >= nfull || tj * kTile >= nfull || part >= parts) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // before it counts as done: see the partial-row kernel
-    return;
-  }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
@@ -168,7 +185,7 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
 #pragma unroll 1
     for (int it = 0; it < n_iters && ok; ++it) {
       const int st = it % kStages, s = (first + it) >> 1, half = (first + it) & 1;
-      if (it >= kStages) ok = __all_sync(0xffffffffu, mbar_wait(empty(st), ((it / kStages) - 1) & 1, a.status, h));
+      if (it >= kStages) ok = __all_sync(0xffffffffu, mbar_wait(empty(st), ((it / kStages) - 1) & 1, a.status, tile, h));
       if (!ok) break;
       if (leader) {
         const uint32_t stage = smem_base + st * kStageBytes;
@@ -188,7 +205,7 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
 #pragma unroll 1
     for (int it = 0; it < n_iters && ok; ++it) {
       const int st = it % kStages;
-      ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status, h));
+      ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status, tile, h));
       if (!ok) break;
       tc_fence_after();
       if (leader) {
@@ -220,7 +237,7 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
     const int m = warp * 32 + lane;       // row of the tile == TMEM lane
     const int rl = ti * kTile + m;        // row inside the chunk
     const int r = r0 + rl;                // row inside the sequence
-    if (__all_sync(0xffffffffu, mbar_wait(acc_full, 0, a.status, h))) {
+    if (__all_sync(0xffffffffu, mbar_wait(acc_full, 0, a.status, tile, h))) {
       tc_fence_after();
       const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
@@ -229,11 +246,13 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
         tmem_ld32_sync(taddr + gq * 32, v);
         const int x = gq >> 2, c0 = (gq & 3) * 32;
         if (parts > 1) {
-          float* dst = part_sums(a, part, blockIdx.x, gridDim.x, h + x) + c0 * kTile + m;
+          float* dst = part_sums(a, slot, h + x) + c0 * kTile + m;
 #pragma unroll
           for (int c = 0; c < 32; ++c) dst[c * kTile] = v[c];
         } else if (r < nfull) {  // rows of the partial block (or past the end) belong to the other kernel
-          store_columns(a, seq, h + x, r0, nb, rl, tj * kTile + c0, v, bias + c0);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = fmaf(a.scale, v[c], bias[c0 + c]);
+          store_columns(a, seq, h + x, r0, nb, rl, tj * kTile + c0, v);
         }
       }
     }
@@ -246,29 +265,50 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   }
 }
 
-// Adds up the parts of a tile of a sequence in parts, in order, 32 columns a CTA: the metric of its full rows.
+// Adds up the parts of a tile of a sequence in parts, in order, 32 columns a CTA: the metric of its full rows.  What bounds it is
+// latency for short sequences and the memory for many: a thread adds 16 columns, whose parts are in flight together, and passes
+// them on through shared memory to the threads that have all 32.  (Us of a call at 32 / 8 heads, 32 / 16 columns a thread: 1500
+// tokens 34.8 / 32.8, 16K 63.5 / 61.2; 8 columns 57.5 there, but 117.2 for a ragged 32K prompt, which takes 116.8 so.)
+constexpr int kSumCols = 16;
+constexpr int kSumThreads = kTile * (32 / kSumCols);
 template <int BLK>
-__global__ void __launch_bounds__(kTile) antidiag_sum_kernel(const AntiArgs a, int n_tiles) {
-  const int tile = blockIdx.x, h = blockIdx.y, c0 = blockIdx.z * 32, m = threadIdx.x;
-  const int seq = a.tiles[3 * tile], ti = a.tiles[3 * tile + 1], tj = a.tiles[3 * tile + 2];
-  const int nb = a.rows.seq_nblk[seq], r0 = a.rows.seq_r0[seq], parts = a.parts[seq];
+__global__ void __launch_bounds__(kSumThreads, 1024 / kSumThreads) antidiag_sum_kernel(const AntiArgs a) {
+  __shared__ float metric[32][kTile];
+  const int n1 = a.n_tiles[1], i = (int)blockIdx.x;
+  const AntidiagTile tile = a.tiles[a.n_tiles[0] + i];
+  const int h = blockIdx.y, c0 = blockIdx.z * 32, m = threadIdx.x % kTile, first = threadIdx.x / kTile * kSumCols;
+  const int seq = tile.seq, ti = tile.ti, tj = tile.tj;
+  const int nb = a.rows.seq_nblk[seq], r0 = a.rows.seq_r0[seq];
   const int nfull = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1] == BLK ? nb : nb - 1;
   const int rl = ti * kTile + m;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (parts == 1 || r0 + rl >= nfull || tj * kTile >= nfull) return;
-  float v[32], bias[32];
-#pragma unroll
-  for (int c = 0; c < 32; ++c) v[c] = part_sums(a, 0, tile, n_tiles, h)[(c0 + c) * kTile + m];
-#pragma unroll 1
-  for (int p = 1; p < parts; ++p) {
-    const float* src = part_sums(a, p, tile, n_tiles, h) + c0 * kTile + m;
-#pragma unroll
-    for (int c = 0; c < 32; ++c) v[c] += src[c * kTile];
-  }
+  const bool row = r0 + rl < nfull;
+  const float* src = part_sums(a, i < n1 ? i : antidiag_parts(1) * n1 + i - n1, h) + (c0 + first) * kTile + m;
   const float* mv = a.mv + (int64_t)(h / a.g) * a.KB_tot + a.rows.seq_kb_off[seq];
+  const int64_t step = (int64_t)(i < n1 ? n1 : a.n_tiles[2]) * a.Hq * (kTile * kTile);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  auto add_up = [&](auto parts) {
+    float v[kSumCols];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) bias[c] = tj * kTile + c0 + c < nb ? a.beta * mv[tj * kTile + c0 + c] : 0.f;
-  store_columns(a, seq, h, r0, nb, rl, tj * kTile + c0, v, bias);
+    for (int p = 0; p < decltype(parts)::value; ++p) {
+#pragma unroll
+      for (int c = 0; c < kSumCols; ++c) v[c] = p == 0 ? src[c * kTile] : v[c] + src[p * step + c * kTile];
+    }
+#pragma unroll
+    for (int c = 0; c < kSumCols; ++c) {
+      const int col = tj * kTile + c0 + first + c;
+      metric[first + c][m] = fmaf(a.scale, v[c], col < nb ? a.beta * mv[col] : 0.f);
+    }
+  };
+  if (row) {
+    if (i < n1) add_up(std::integral_constant<int, antidiag_parts(1)>{});
+    else add_up(std::integral_constant<int, antidiag_parts(2)>{});
+  }
+  __syncthreads();
+  if (!row || first > 0) return;
+  float v[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] = metric[c][m];
+  store_columns(a, seq, h, r0, nb, rl, tj * kTile + c0, v);
 }
 
 // The metric row of a sequence's partial last block (when it belongs to the query chunk): for every j <= r the
@@ -401,11 +441,9 @@ int antidiag_max_sequences() { return kMaxSeqs; }
 // In how many parts the inner dimension is summed for a sequence of n blocks: by its whole length alone, so that its lists do
 // not depend on the batch, its chunks or the heads of a plan.  Up to 128 blocks are one tile, 16 CTAs at 32 / 8 heads; up to 256
 // three, 48 CTAs; up to 384 six, 96 CTAs, in three parts two waves of a third each.  Beyond, the tiles fill the SMs.
-int antidiag_parts(int n) { return n <= kTile ? 8 : n <= 3 * kTile ? 3 : 1; }
+int antidiag_class(int64_t n) { return n <= kTile ? 2 : n <= 3 * kTile ? 1 : 0; }
 
-size_t antidiag_sums_bytes(int max_parts, int n_tiles, int Hq) {
-  return max_parts > 1 ? (size_t)max_parts * n_tiles * Hq * kTile * kTile * sizeof(float) : 0;
-}
+size_t antidiag_sums_bytes(int slots, int Hq) { return (size_t)slots * Hq * kTile * kTile * sizeof(float); }
 
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s) {
@@ -434,14 +472,20 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   for (int b = batch; b < kMaxSeqs; ++b) { maps.q[b] = maps.q[0]; maps.k[b] = maps.k[0]; }
 
   AntiArgs a{};
-  a.tiles = p.d_gemm_tiles; a.mv = mv; a.M = M; a.status = status; a.rows = p.rows; a.m_tot = p.m_tot; a.mt_tot = p.mt_tot;
+  a.tiles = p.d_antidiag_tiles; a.mv = mv; a.M = M; a.status = status; a.rows = p.rows; a.m_tot = p.m_tot; a.mt_tot = p.mt_tot;
   a.Hq = p.cfg.num_q_heads; a.g = a.Hq / p.cfg.num_kv_heads; a.KB_tot = p.KB_tot; a.block = B;
   a.beta = p.cfg.beta; a.scale = p.score_scale / (float)B; a.as_keys = as_keys ? 1 : 0;
   a.Q = (const __nv_bfloat16*)Q; a.K = (const __nv_bfloat16*)K;
   a.q_st = p.cfg.q_stride_tok; a.q_sh = p.cfg.q_stride_head; a.kv_st = p.cfg.kv_stride_tok; a.kv_sh = p.cfg.kv_stride_head;
   a.batch = batch;
   a.sums = sums;
-  for (int b = 0; b < batch; ++b) a.parts[b] = p.antidiag_parts[b];
+  int n_tiles = 0, n_shares = 0;
+  for (int c = 0; c < kAntidiagClasses; ++c) {
+    a.n_tiles[c] = p.n_antidiag_tiles[c];
+    n_tiles += a.n_tiles[c];
+    n_shares += a.n_tiles[c] * antidiag_parts(c);
+  }
+  const int n_sum = n_tiles - a.n_tiles[0];
   const bool two = a.g % 2 == 0;
 
   static bool attr_set[64] = {};
@@ -457,41 +501,49 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)(two ? a.Hq / 2 : a.Hq), (unsigned)p.antidiag_max_parts);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  auto kernel = B == 128 ? (two ? antidiag_metric_kernel<128, 2> : antidiag_metric_kernel<128, 1>)
-                         : (two ? antidiag_metric_kernel<64, 2> : antidiag_metric_kernel<64, 1>);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, maps, a);
-  if (e != cudaSuccess) return e;
-  ++*launched;
+  cudaError_t e = cudaSuccess;
+  if (n_tiles > 0) {
+    cudaLaunchConfig_t cfg = {};
+    const unsigned heads = (unsigned)(two ? a.Hq / 2 : a.Hq);
+    cfg.gridDim = dim3((unsigned)n_shares * heads);
+    for (int c = 0; c < kAntidiagClasses; ++c)
+      if (a.n_tiles[c] == n_tiles) {
+        a.parts = antidiag_parts(c);
+        cfg.gridDim = dim3((unsigned)n_tiles, heads, (unsigned)a.parts);
+      }
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto kernel = B == 128 ? (two ? antidiag_metric_kernel<128, 2> : antidiag_metric_kernel<128, 1>)
+                           : (two ? antidiag_metric_kernel<64, 2> : antidiag_metric_kernel<64, 1>);
+    e = cudaLaunchKernelEx(&cfg, kernel, maps, a);
+    if (e != cudaSuccess) return e;
+    ++*launched;
+  }
   if (any_partial) {
     // the metric rows of partial last blocks, beside the contraction (the rows are not those the contraction writes, and
-    // MV is complete once every CTA of the contraction is past its wait or gone)
+    // MV is complete once every CTA of the contraction is past its wait or gone; without one, a plain launch waits for the pooling)
     cudaLaunchConfig_t cfg2 = {};
     cfg2.gridDim = dim3((unsigned)((p.max_nblk + 31) / 32), (unsigned)(batch * p.cfg.num_kv_heads));
     cfg2.blockDim = dim3(kPartThreads);
     cfg2.stream = s;
     cfg2.attrs = attr;
-    cfg2.numAttrs = 1;
+    cfg2.numAttrs = n_tiles > 0 ? 1 : 0;
     e = B == 128 ? cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<128>, a) : cudaLaunchKernelEx(&cfg2, antidiag_partial_kernel<64>, a);
     if (e != cudaSuccess) return e;
     ++*launched;
   }
-  if (p.antidiag_max_parts == 1) return e;
+  if (n_sum == 0) return e;
   // behind the partial-row kernel, which is complete only after the contraction is, or behind the contraction itself
   cudaLaunchConfig_t cfg3 = {};
-  cfg3.gridDim = dim3((unsigned)p.n_gemm_tiles, (unsigned)a.Hq, kTile / 32);
-  cfg3.blockDim = dim3(kTile);
+  cfg3.gridDim = dim3((unsigned)n_sum, (unsigned)a.Hq, kTile / 32);
+  cfg3.blockDim = dim3(kSumThreads);
   cfg3.stream = s;
   cfg3.attrs = attr;
   cfg3.numAttrs = 1;
-  e = B == 128 ? cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<128>, a, p.n_gemm_tiles)
-               : cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<64>, a, p.n_gemm_tiles);
+  e = B == 128 ? cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<128>, a) : cudaLaunchKernelEx(&cfg3, antidiag_sum_kernel<64>, a);
   if (e == cudaSuccess) ++*launched;
   return e;
 }

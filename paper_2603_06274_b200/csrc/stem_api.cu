@@ -217,7 +217,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
   p.T_kv = p.cu[batch];
 
   std::vector<int32_t> row_seq, row_r, row_tok0, row_ntok, seq_tok0(batch), seq_nblk(batch), seq_r0(batch),
-      seq_row_off(batch), seq_kb_off(batch), seq_kb_first(batch), kb_tok0, kb_ntok, kb_dst, kb_new;
+      seq_row_off(batch), seq_kb_off(batch), seq_kb_first(batch), seq_class(batch), kb_tok0, kb_ntok, kb_dst, kb_new;
   std::vector<int64_t> seq_m_off(batch), seq_mt_off(batch);
   int64_t m_off = 0, mt_off = 0;
   int32_t q_tok = 0, kb_off = 0;
@@ -231,8 +231,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     const int64_t n_tot = o.total_len_host ? o.total_len_host[b] : n;
     const int64_t nb_tot = (n_tot + B - 1) / B;        // blocks of the whole sequence: N of Eq. 3
     is_short[b] = p.score_mode == 0 && nb_tot <= kShortBlocks;
-    p.antidiag_parts.push_back(p.score_mode == 1 ? antidiag_parts((int)std::min<int64_t>(nb_tot, INT32_MAX)) : 1);
-    p.antidiag_max_parts = std::max(p.antidiag_max_parts, p.antidiag_parts.back());
+    seq_class[b] = antidiag_class(nb_tot);
     seq_tok0[b] = p.cu[b];
     seq_nblk[b] = nb;
     seq_r0[b] = r0;
@@ -306,8 +305,23 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
         const int r_last = seq_r0[b] + std::min(rows_b, (ti + 1) * 128) - 1;  // largest global row of the tile
         for (int tj = 0; tj <= r_last / 128; ++tj) { gemm_tiles.push_back(b); gemm_tiles.push_back(ti); gemm_tiles.push_back(tj); }
       }
-    p.n_gemm_tiles = (int32_t)(gemm_tiles.size() / 3);
   }
+  // Anti-diagonal scoring has work only where a tile holds a full row and a full column.  What a tile costs and what it keeps
+  // in the workspace follow from its own sequence, whatever is batched beside it.
+  std::vector<AntidiagTile> anti_tiles;
+  int antidiag_slots = 0;
+  if (p.score_mode == 1) {
+    for (int c = 0; c < kAntidiagClasses; ++c)
+      for (size_t i = 0; i < gemm_tiles.size(); i += 3) {
+        const int32_t b = gemm_tiles[i], ti = gemm_tiles[i + 1], tj = gemm_tiles[i + 2], n_full = (p.cu[b + 1] - p.cu[b]) / B;
+        if (seq_class[b] != c || seq_r0[b] + ti * 128 >= n_full || tj * 128 >= n_full) continue;
+        anti_tiles.push_back({b, ti, tj});
+        ++p.n_antidiag_tiles[c];
+        antidiag_slots += c > 0 ? antidiag_parts(c) : 0;
+      }
+    gemm_tiles.clear();
+  }
+  p.n_gemm_tiles = (int32_t)(gemm_tiles.size() / 3);
 
   if (cudaGetDevice(&p.device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p.sm_count, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) {
@@ -324,7 +338,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
                o_seq_kb_off = blob.add(seq_kb_off), o_seq_kb_first = blob.add(seq_kb_first), o_seq_m_off = blob.add(seq_m_off),
                o_seq_mt_off = blob.add(seq_mt_off), o_kb_tok0 = blob.add(kb_tok0), o_kb_ntok = blob.add(kb_ntok),
                o_kb_dst = blob.add(kb_dst), o_kb_new = blob.add(kb_new), o_gt = blob.add(gemm_tiles),
-               o_lr = blob.add(long_rows), o_sr = blob.add(short_rows);
+               o_lr = blob.add(long_rows), o_sr = blob.add(short_rows), o_at = blob.add(anti_tiles);
   const size_t item_bytes = 2 * (size_t)p.n_items * sizeof(int32_t), slot_bytes = (2 * (size_t)p.sm_count + 1) * sizeof(int32_t);
   const size_t o_ws = blob.take(item_bytes), o_wd = blob.take(item_bytes), o_ss = blob.take(slot_bytes), o_sd = blob.take(slot_bytes);
   blob.write();
@@ -355,7 +369,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     p.ws.qsplit = off; off = align_up(off + (size_t)3 * p.H_list * p.R_tot * kHeadDim * 2, 256);
     p.ws.ksplit = off; off = align_up(off + (own_k ? (size_t)3 * Hkv * p.KB_tot * kHeadDim * 2 : 0), 256);
     p.ws.metric = off; off = align_up(off + (size_t)p.H_list * (size_t)p.mt_tot * 4, 256);
-    p.ws.sums = off; off = align_up(off + (p.score_mode == 1 ? antidiag_sums_bytes(p.antidiag_max_parts, p.n_gemm_tiles, p.cfg.num_q_heads) : 0), 256);
+    p.ws.sums = off; off = align_up(off + antidiag_sums_bytes(antidiag_slots, Hq), 256);
     p.ws.sel_idx = off; off = align_up(off + (size_t)p.H_list * p.R_tot * p.k_max * 4, 256);
     p.ws.sel_cnt = off; off = align_up(off + (size_t)p.H_list * p.R_tot * 4, 256);
     p.ws.total = off;
@@ -388,6 +402,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
   p.d_gemm_tiles = (const int32_t*)(d + o_gt);
   p.d_long_rows = (const int32_t*)(d + o_lr);
   p.d_short_rows = (const int32_t*)(d + o_sr);
+  p.d_antidiag_tiles = (const AntidiagTile*)(d + o_at);
   p.work_sparse.d_items = (const int32_t*)(d + o_ws);
   p.work_sparse.d_slot_off = (const int32_t*)(d + o_ss);
   p.work_dense.d_items = (const int32_t*)(d + o_wd);

@@ -43,6 +43,14 @@ struct RowTables {
   const int32_t* kb_new;       // [n_kb_new] indices into the three arrays above of the blocks that the chunk adds
 };
 
+// A tile of the anti-diagonal contraction: sequence, row tile, column tile.
+struct AntidiagTile {
+  int32_t seq, ti, tj;
+};
+// In how many parts the inner dimension is summed: the classes of antidiag_class.
+constexpr int kAntidiagClasses = 3;
+__host__ __device__ constexpr int antidiag_parts(int c) { return c == 0 ? 1 : c == 1 ? 3 : 8; }
+
 // Where things live inside the caller's workspace (byte offsets, 256-aligned).
 struct WorkspaceLayout {
   size_t status = 0;
@@ -50,7 +58,7 @@ struct WorkspaceLayout {
   size_t qsplit = 0;   // bf16 [3, H_list, R_tot, d]: Qbar as hi + mid + lo parts
   size_t ksplit = 0;   // bf16 [3, H_kv, KB_tot, d]: Kbar likewise
   size_t metric = 0;   // uint32 [H_list, mt_tot]: the metric of the fused path as bit planes of its selection keys
-  size_t sums = 0;     // fp32: anti-diagonal scoring, the sums over parts of the inner dimension (antidiag_sums_bytes)
+  size_t sums = 0;     // fp32 [slots, H_q, 128, 128]: anti-diagonal scoring, the sums over parts of the inner dimension
   size_t sel_idx = 0;  // int32 [H_list, R_tot, k_max]
   size_t sel_cnt = 0;  // int32 [H_list, R_tot]
   size_t total = 0;
@@ -78,8 +86,9 @@ struct Plan {
   int32_t k_max = 0, max_nblk = 0;
   int32_t kcache_blocks = 0;  // per-sequence capacity of a caller-owned pooled-K cache (0: none)
   bool share_group = false;   // one index list per (kv head, row)
-  std::vector<int32_t> antidiag_parts;  // anti-diagonal scoring: parts in which a sequence's contraction is summed
-  int32_t antidiag_max_parts = 1;
+  // Anti-diagonal scoring: the tiles with a full row and a full column, class by class.
+  const AntidiagTile* d_antidiag_tiles = nullptr;
+  int32_t n_antidiag_tiles[kAntidiagClasses] = {0, 0, 0};
   int32_t score_mode = 0;     // 0: product of block means (Eq. 7 on pooled blocks); 1: anti-diagonal scoring
   std::vector<int32_t> h_seq_r0, h_seq_qtok0;  // host copies: first chunk row, first packed Q token of every sequence
   int32_t H_list = 0;         // heads of the metric and of the lists: H_q, or H_kv with share_group
@@ -92,7 +101,8 @@ struct Plan {
   // device blob
   void* d_blob = nullptr;
   RowTables rows{};
-  const int32_t* d_gemm_tiles = nullptr;  // [n_gemm_tiles][3] (sequence, row tile, column tile) of the metric GEMM (sequences that are not short)
+  // [n_gemm_tiles][3] (sequence, row tile, column tile) of the metric GEMM (product of block means, sequences that are not short)
+  const int32_t* d_gemm_tiles = nullptr;
   int32_t n_gemm_tiles = 0;
   // Query rows, the last first, of the sequences that the tensor-core metric serves and of those that the kernel for short
   // sequences does.  Which it is follows from the length of the whole sequence alone (total_len, with chunks): a row's list is
@@ -133,8 +143,8 @@ cudaError_t launch_metric_gemm(const Plan& p, const void* qsplit, const void* ks
 // contraction over the full blocks plus, where a sequence ends in a partial block, a small kernel for that row.
 // *launched receives the number of kernels enqueued.
 int antidiag_max_sequences();
-int antidiag_parts(int n_blocks);
-size_t antidiag_sums_bytes(int max_parts, int n_tiles, int Hq);
+int antidiag_class(int64_t n_blocks);
+size_t antidiag_sums_bytes(int slots, int Hq);
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s);
 

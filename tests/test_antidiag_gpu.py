@@ -192,3 +192,21 @@ def test_metric_of_sequences_summed_in_parts(block, seqlens, hq, hkv):
         assert np.array_equal(alone, M_g[:, off:off + nb * nb], equal_nan=True)
         tok += n
         off += nb * nb
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (128, (131072, 1500), 32, 8),              # a sequence that is summed at once beside one of 12 blocks in eight parts
+    (64, (131072, 64 * 100), 64, 8),
+    (64, (64 * 300, 64 * 1000 + 1, 70), 4, 2),  # three parts, at once, eight parts
+])
+def test_a_batch_needs_no_more_memory_than_its_sequences_alone(block, seqlens, hq, hkv):
+    def bytes_of(lens):
+        plan = StemPlan.from_workload(wl.small("ad_ws", seqlens=lens, hq=hq, hkv=hkv, block=block, permille=50), score_mode=1)
+        info = plan.info
+        plan.close()
+        return info.workspace_bytes, info.total_q_blocks * info.k_max * hq * 4
+
+    # (there is room for lists as long as the longest in every row)
+    total, lists = bytes_of(seqlens)
+    alone = [bytes_of((n,)) for n in seqlens]
+    assert total - lists <= sum(n - l for n, l in alone)
