@@ -127,8 +127,9 @@ typedef struct {
  * is the mean of the token scores along the main anti-diagonal of the B x B score block,
  *   (1/n) sum_s q[rB + B-1-s] . k[jB + s]  over the s whose two tokens exist (n = B for full blocks),
  * in place of Qbar[h,r] . Kbar[kv(h),j]; the magnitude term, the budget and the selection are unchanged.
- * Computed as one tensor-core contraction of Q with K (inner dimension B * d).  Not combinable with the
- * pooled-K cache or share_group; at most 8 sequences per plan (STEM_ERR_UNSUPPORTED otherwise). */
+ * Computed as one tensor-core contraction of Q with K (inner dimension B * d); of the pooled tensors of step 1 only MV is
+ * computed and kept.  Not combinable with the pooled-K cache or share_group; at most 8 sequences per plan
+ * (STEM_ERR_UNSUPPORTED otherwise). */
 typedef struct {
   const int32_t* q_start_host;    /* HOST [batch]: first query token of every sequence's chunk, a multiple of
                                      block, < kv_len(b); NULL = 0 (no chunking)                               */

@@ -360,14 +360,15 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     deal_items(p, by_r, len_dense, 3 * p.sm_count, 3 * p.sm_count, &p.work_dense, ints(o_wd), ints(o_sd), owner.get());
   }
 
-  // Workspace layout.  With a caller-owned cache the K-side tensors are not part of the workspace.
+  // Workspace layout.  With a caller-owned cache the K-side tensors are not part of the workspace; the anti-diagonal mode has no
+  // pooled vectors, only MV.
   {
-    const bool own_k = p.kcache_blocks == 0;
+    const bool own_k = p.kcache_blocks == 0, vectors = p.score_mode != 1;
     size_t off = 0;
     p.ws.status = off; off = align_up(off + kStatusWords * 4, 256);
     p.ws.mv = off;     off = align_up(off + (own_k ? (size_t)Hkv * p.KB_tot * 4 : 0), 256);
-    p.ws.qsplit = off; off = align_up(off + (size_t)3 * p.H_list * p.R_tot * kHeadDim * 2, 256);
-    p.ws.ksplit = off; off = align_up(off + (own_k ? (size_t)3 * Hkv * p.KB_tot * kHeadDim * 2 : 0), 256);
+    p.ws.qsplit = off; off = align_up(off + (vectors ? (size_t)3 * p.H_list * p.R_tot * kHeadDim * 2 : 0), 256);
+    p.ws.ksplit = off; off = align_up(off + (own_k && vectors ? (size_t)3 * Hkv * p.KB_tot * kHeadDim * 2 : 0), 256);
     p.ws.metric = off; off = align_up(off + (size_t)p.H_list * (size_t)p.mt_tot * 4, 256);
     p.ws.sums = off; off = align_up(off + antidiag_sums_bytes(antidiag_slots, Hq), 256);
     p.ws.sel_idx = off; off = align_up(off + (size_t)p.H_list * p.R_tot * p.k_max * 4, 256);
