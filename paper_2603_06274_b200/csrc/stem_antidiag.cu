@@ -10,7 +10,7 @@
 // block, block) lets one TMA box fetch "64 columns of token t of 128 consecutive blocks" as a 128-row
 // K-major operand tile; the query map is walked with t = B-1-s, the key map with t = s.
 //
-// One CTA per (128 x 128 tile of one sequence's causal triangle, two query heads of a group or one where a group's size is odd,
+// One CTA per (128 x 128 tile of one sequence's causal triangle, two query heads of a group or one (antidiag_heads),
 // part of the inner dimension): warp 4 issues the copies through a ring of stages, warp 5 the MMAs into a TMEM accumulator for
 // each head, warps 0-3 write the tile as floats (the public M) or as bit planes of the selection keys (the fused path's
 // workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <map>
 #include <type_traits>
 
 #include "stem_internal.h"
@@ -439,9 +440,33 @@ __global__ void __launch_bounds__(kPartThreads) antidiag_partial_kernel(const An
 int antidiag_max_sequences() { return kMaxSeqs; }
 
 // In how many parts the inner dimension is summed for a sequence of n blocks: by its whole length alone, so that its lists do
-// not depend on the batch, its chunks or the heads of a plan.  Up to 128 blocks are one tile, 16 CTAs at 32 / 8 heads; up to 256
-// three, 48 CTAs; up to 384 six, 96 CTAs, in three parts two waves of a third each.  Beyond, the tiles fill the SMs.
+// not depend on the batch, its chunks or the heads of a plan.  Chosen for 32 / 8 heads: up to 128 blocks are one tile, 16 CTAs of
+// two heads; up to 256 three, 48 CTAs; up to 384 six, 96 CTAs, in three parts two waves of a third each.  From ten tiles on the
+// CTAs of 32 heads are a wave of the SMs or more; with fewer heads SMs stay idle there.
 int antidiag_class(int64_t n) { return n <= kTile ? 2 : n <= 3 * kTile ? 1 : 0; }
+
+// How many query heads a CTA computes (two or one of an even group; a head's sums are the same either way).  A step of two heads
+// moves 48 KB into the SM where one moves 32, so two are taken where the last CTA is then done in less than 2/3 of the shares.
+// Us of a call, two heads / one, by the waves of CTAs: 1 against 1: 4 / 2 heads, 400 blocks 124 / 82, 8 / 2, 640 132 / 104; 2 against
+// 3: 16 / 4, 768 290 / 282, 32 / 8, 512 307 / 289; 1 against 2: 8 / 2, 1024 183 / 205, 16 / 4, 512 149 / 169; 3 against 5: 32 / 8, 768
+// 502 / 514; 4 against 8: 32 / 8, 1024 780 / 856.
+int antidiag_heads(const int32_t* n_tiles, int Hq, int g, int sms) {
+  // when the last CTA is done, in 24ths of a tile's sum; CTAs start in order, each on the SM that is free first
+  auto done = [&](int heads) {
+    std::map<int64_t, int64_t> free_at{{0, sms}};  // SMs by the time they are free
+    for (int c = 0; c < kAntidiagClasses; ++c)
+      for (int64_t left = (int64_t)n_tiles[c] * antidiag_parts(c) * (Hq / heads); left > 0;) {
+        const auto first = *free_at.begin();
+        const int64_t n = std::min(left, first.second);
+        free_at.erase(free_at.begin());
+        if (first.second > n) free_at[first.first] = first.second - n;
+        free_at[first.first + 24 / antidiag_parts(c)] += n;
+        left -= n;
+      }
+    return free_at.rbegin()->first;
+  };
+  return g % 2 == 0 && 3 * done(2) < 2 * done(1) ? 2 : 1;
+}
 
 size_t antidiag_sums_bytes(int slots, int Hq) { return (size_t)slots * Hq * kTile * kTile * sizeof(float); }
 
@@ -486,7 +511,7 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
     n_shares += a.n_tiles[c] * antidiag_parts(c);
   }
   const int n_sum = n_tiles - a.n_tiles[0];
-  const bool two = a.g % 2 == 0;
+  const bool two = p.antidiag_heads == 2;
 
   static bool attr_set[64] = {};
   const int dev_slot = p.device & 63;

@@ -219,3 +219,29 @@ def test_the_workspace_has_no_pooled_vectors():
     sizes = (32, hkv * nb * 4, hq * nb * ((nb + 31) // 32 * 32) * 4, hq * nb * plan.info.k_max * 4, hq * nb * 4)
     assert plan.info.workspace_bytes == sum((n + 255) // 256 * 256 for n in sizes)
     plan.close()
+
+
+@pytest.mark.parametrize("seqlens", [(64 * 700 + 5,), (64 * 200,), (64 * 400, 64 * 90 + 60)])
+def test_heads_in_pairs_and_alone_have_the_same_metric(seqlens):
+    # 32 heads fill the SMs with two to a CTA, the four of one kv head do not
+    hq, hkv, n = 32, 8, sum(seqlens)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn((n, h, 128), generator=gen, device="cuda").to(torch.bfloat16) for h in (hq, hkv, hkv))
+
+    def metric(heads, kv_heads, q, k, v):
+        plan = StemPlan(seqlens, heads, kv_heads, block=64, budget_permille=50, score_mode=1)
+        M = torch.full((heads, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+        idx = torch.full((heads, plan.info.total_q_blocks, plan.info.k_max), -7, dtype=torch.int32, device="cuda")
+        cnt = torch.full((heads, plan.info.total_q_blocks), -7, dtype=torch.int32, device="cuda")
+        binding.stem_score(plan, q, k, v, M)
+        binding.stem_score_select(plan, q, k, v, idx, cnt)
+        assert binding.stem_check_status(plan)[0] == 0
+        plan.close()
+        return M, idx, cnt
+
+    M, idx, cnt = metric(hq, hkv, q, k, v)
+    for kvh in (0, 5):
+        rows = slice(4 * kvh, 4 * kvh + 4)
+        one = metric(4, 1, q[:, rows].contiguous(), k[:, kvh:kvh + 1].contiguous(), v[:, kvh:kvh + 1].contiguous())
+        assert torch.equal(one[0].nan_to_num(7e30), M[rows].nan_to_num(7e30))
+        assert torch.equal(one[1], idx[rows]) and torch.equal(one[2], cnt[rows])
