@@ -841,6 +841,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           }
           if (g == 0) {
             if (!kProbeAhead || !__all_sync(0xffffffffu, pv_seen)) ok = wait_pv();
+            if (!ok) break;
             tc_fence_after();
           }
           tmem_st16(p_addr + g * 16, pk);
@@ -854,6 +855,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (lane == 0) mbar_arrive(bar(Smem::p_early, X));
           }
         }
+        if (!ok) break;
         l_run += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
         tmem_st_wait();
         tc_fence_before();
