@@ -245,3 +245,64 @@ def test_heads_in_pairs_and_alone_have_the_same_metric(seqlens):
         one = metric(4, 1, q[:, rows].contiguous(), k[:, kvh:kvh + 1].contiguous(), v[:, kvh:kvh + 1].contiguous())
         assert torch.equal(one[0].nan_to_num(7e30), M[rows].nan_to_num(7e30))
         assert torch.equal(one[1], idx[rows]) and torch.equal(one[2], cnt[rows])
+
+
+def _lists_of(plan, q, k, v):
+    info = plan.info
+    idx = torch.full((plan.num_q_heads, info.total_q_blocks, info.k_max), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.full((plan.num_q_heads, info.total_q_blocks), -7, dtype=torch.int32, device="cuda")
+    binding.stem_score_select(plan, q, k, v, idx, cnt)
+    assert binding.stem_check_status(plan)[0] == 0
+    return idx.cpu().numpy(), cnt.cpu().numpy()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (64, (64 * 385, 64 * 130 + 7, 64 * 128), 4, 2),   # bit planes of the contraction itself and of the sums in three and eight parts
+    (64, (64 * 400 + 9, 64 * 200), 3, 1),             # the same with an odd group
+    (128, (128 * 390, 128 * 20 + 100), 2, 1),
+    (128, (128 * 386 + 1,), 3, 3),
+])
+def test_fused_lists_are_those_of_the_metric(block, seqlens, hq, hkv):
+    w = wl.small("ad_planes", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=100, seed=sum(seqlens))
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    plan = StemPlan.from_workload(w, score_mode=1)
+    info = plan.info
+    idx, cnt = _lists_of(plan, q, k, v)
+    M = torch.full((hq, info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_score(plan, q, k, v, M)
+    idx_m = torch.full((hq, info.total_q_blocks, info.k_max), -7, dtype=torch.int32, device="cuda")
+    cnt_m = torch.full((hq, info.total_q_blocks), -7, dtype=torch.int32, device="cuda")
+    binding.stem_select(plan, M, idx_m, cnt_m)
+    assert binding.stem_check_status(plan)[0] == 0
+    assert np.array_equal(idx, idx_m.cpu().numpy()) and np.array_equal(cnt, cnt_m.cpu().numpy())
+    plan.close()
+
+
+@pytest.mark.parametrize("block,n,q_start,hq,hkv", [
+    (128, 128 * 200 + 50, 128 * 70, 4, 2),    # three parts; the chunk's tiles start inside the sequence's
+    (64, 64 * 100, 64 * 33, 4, 2),            # eight parts
+    (64, 64 * 390 + 5, 64 * 130, 2, 1),       # at once
+    (128, 128 * 3 + 60, 128 * 3, 3, 1),       # the chunk is the partial block alone
+])
+def test_lists_of_a_chunk_are_those_of_the_whole_sequence(block, n, q_start, hq, hkv):
+    w = wl.small("ad_chunk", seqlens=(n,), hq=hq, hkv=hkv, block=block, permille=100, seed=n)
+    data = wl.make_qkv(w)
+    q, k, v = to_dev(data["q"]), to_dev(data["k"]), to_dev(data["v"])
+    whole = StemPlan.from_workload(w, score_mode=1)
+    idx, cnt = _lists_of(whole, q, k, v)
+    # the first chunk sees the tokens before q_start alone, the second one all keys
+    parts = [(q[:q_start], q_start, 0), (q[q_start:], n, q_start)]
+    row = 0
+    for q_chunk, kv_len, start in parts:
+        wc = wl.small("ad_chunk", seqlens=(kv_len,), hq=hq, hkv=hkv, block=block, permille=100)
+        plan = StemPlan.from_workload(wc, score_mode=1, q_starts=[start], total_lens=[n])
+        idx_c, cnt_c = _lists_of(plan, q_chunk, k[:kv_len], v[:kv_len])
+        rows = slice(row, row + plan.info.total_q_blocks)
+        assert np.array_equal(cnt_c, cnt[:, rows])
+        width = plan.info.k_max
+        assert np.array_equal(idx_c, idx[:, rows, :width]) and (idx[:, rows, width:] == -1).all()
+        row = rows.stop
+        plan.close()
+    assert row == whole.info.total_q_blocks
+    whole.close()

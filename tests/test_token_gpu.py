@@ -426,3 +426,43 @@ def test_output_in_the_place_of_the_queries(n, hq, hkv, k_max, order, repeat):
     assert max(abs(got_lse[h, t] - lse_ref[h, t]) for h, t in rows) < 1e-3
     empty = np.repeat(cnt == 0, g, axis=0)
     assert (got.transpose(1, 0, 2)[empty] == 0).all() and np.isneginf(got_lse[empty]).all()
+
+
+@pytest.mark.parametrize("n,hq,hkv", [(1500, 4, 2), (1400, 7, 1)])
+def test_row_maxima_that_grow_from_block_to_block_in_the_masked_form(n, hq, hkv):
+    # The scores of key block j are about step[j] powers of two: a row's reference stays (growth of less than 8), moves once or
+    # moves with every block; some lists name nothing in the blocks that outgrow it.
+    k_max = 150
+    assert binding.stem_token_attention_form(n, hq, hkv, k_max) == "masked"
+    r = np.random.default_rng(n + hq)
+    step = np.array([0, 7, 14, 22, 21, 48, 71, 95, 95, 60, 90, 120])[:(n + 127) // 128]
+    u = r.standard_normal(128)
+    u /= np.linalg.norm(u)
+    scale = np.sqrt(128) / np.log2(np.e) / 8  # q = 8 u, so that k = scale * step * u scores `step` powers of two
+    dev = lambda t: torch.from_numpy(t).to(device="cuda", dtype=torch.bfloat16)
+    k = dev(np.repeat(step, 128)[:n, None, None] * scale * u + 0.3 * r.standard_normal((n, hkv, 128)))
+    q = dev(8 * u + 0.3 * r.standard_normal((n, hq, 128)))
+    v = dev(r.standard_normal((n, hkv, 128)))
+    idx = np.full((hkv, n, k_max), -1, np.int32)
+    cnt = np.zeros((hkv, n), np.int32)
+    for h in range(hkv):
+        for t in range(n):
+            tokens = np.arange(t + 1)
+            if t % 3 == 1:
+                tokens = tokens[tokens // 128 != t // 128] if t >= 128 else tokens
+            pick = np.sort(r.choice(tokens, min(len(tokens), k_max), replace=False))
+            idx[h, t, :len(pick)] = pick
+            cnt[h, t] = len(pick)
+    out = torch.full((n, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((hq, n), float("nan"), dtype=torch.float32, device="cuda")
+    binding.stem_token_attention(q, k, v, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), out, lse)
+    st, detail = binding.stem_token_check_status()
+    assert st == 0, detail
+    g = hq // hkv
+    named = torch.zeros((hkv, n, n + 1), dtype=torch.bool, device="cuda")
+    named.scatter_(2, torch.from_numpy(np.where(idx < 0, n, idx)).cuda().long(), True)
+    s = torch.einsum("thd,shd->hts", q.double(), k.double().repeat_interleave(g, 1)) / np.sqrt(128)
+    s = s.masked_fill(~named[:, :, :n].repeat_interleave(g, 0), float("-inf"))
+    ref = torch.einsum("hts,shd->thd", torch.softmax(s, 2), v.double().repeat_interleave(g, 1))
+    check_attention(from_dev_bf16(out), ref.cpu().numpy(), label=f"growing maxima, token lists, {hq}/{hkv} heads")
+    assert (lse - torch.logsumexp(s, 2)).abs().max() < 1e-3
