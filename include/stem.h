@@ -230,7 +230,7 @@ int stem_score_select(const stem_plan* plan, const void* Q, const void* K, const
  *   the plan holds, so O is the same from plan to plan up to the rounding of its sums and of P to bf16 (about 2e-3 of its
  *   norm), and bit for bit from call to call.  P is rounded relative to a reference that the up to 32 tokens of a sequence
  *   which share a warp move together: that rounding of a token's O may change with the queries of the others, never with
- *   another sequence's tensors.  sel_idx == NULL (with sel_cnt == NULL) means every
+ *   another sequence's queries and keys.  sel_idx == NULL (with sel_cnt == NULL) means every
  *   causal block, i.e. dense causal attention.  Lists must be ascending and within [0, r];
  *   out-of-range ids are clamped, never dereferenced.  lse (fp32 [num_q_heads, T], natural-log
  *   sum-exp of the scaled scores) is optional (NULL to skip). */

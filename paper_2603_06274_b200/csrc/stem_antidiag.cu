@@ -16,7 +16,7 @@
 // workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
 // heads share the key tile, 48 KB for two heads' step instead of 64, and short sequences, whose tiles are fewer than the SMs,
 // are computed in parts (antidiag_class), which a small kernel adds up in order.  Lists of a call at 32 / 8 heads, a head and a whole
-// sum each / two heads, in parts: 16K tokens 89.8 / 63.2 us, 32K 119.5 / 102.5, 128K 877 / 780.  Only FULL
+// sum each / two heads, in parts: 16K tokens 89.8 / 61.2 us, 32K 119.5 / 101.0, 128K 877 / 780.  Only FULL
 // blocks go through the contraction (the maps end at the last full block, so nothing is read past a
 // sequence); a sequence's partial last block, whose anti-diagonal is truncated (the mean is over the
 // pairs whose two tokens exist), is one metric row that a small second kernel computes with plain FMAs.

@@ -28,13 +28,13 @@
 // S is only passed through: the softmax takes it into registers at once (170 cycles) and the columns are free for Q K^T of the
 // other slot's next block, which so runs while this slot's exponentials do; P has columns of its own, and Q K^T of a
 // slot's next block need not wait for P V of the one before.  (With S and P of a slot in the same 128 columns every block was a
-// chain softmax -> P V -> Q K^T -> softmax, 3460 cycles for a block of both slots against 2800 now; tensor pipe 59 % -> 70 %.
-// The clock gives part of it back under the power cap, 1650 -> 1570 MHz: 32K tokens, 32 / 8 heads 1314 -> 1240 us of a call,
-// dense 16K 1840 -> 1740.)  Blocks of 64 keys leave room for an S of each slot.
+// chain softmax -> P V -> Q K^T -> softmax: 3330 cycles of an SM for a block of both slots, tensor pipe 61.5 % of them; now 3010
+// and 68.1 % (32K tokens, 32 / 8 heads, under the profiler).  The clock gives part of it back under the power cap, 1650 -> 1570
+// MHz: that layer 1314 -> 1240 us of a call, dense 16K 1840 -> 1740.)  Blocks of 64 keys leave room for an S of each slot.
 // The MMA issuer visits the slots alternately; a visit issues Q K^T of the slot's next block (as soon as the other slot's S has
 // been read) and then P V of its previous block.  The K / V producer walks the same visit sequence, so one shared ring serves
 // both slots in order.  A slot's items follow each other without a gap: S of the next item's first block is taken into
-// registers before O of the old one is written.
+// registers before O of the old one is written (with kSpareQ).
 // For that the next item's Q tile has to be there already: with lists of tens of blocks (kSpareQ) the
 // seven 32 KB tiles of shared memory are three Q tiles and a ring of four, the next tile is loaded into
 // the spare one while both current items run, and slot 1 starts half an item late so that the slots'
@@ -544,7 +544,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   constexpr int kKvOff = Smem::q + kQBufs * kQBytes;
   constexpr bool kOwnS = BLK == 64;  // S of a block of 64 keys takes half of the 128 columns: one half for each slot
   // The slots' visits of a round go together, Q K^T of both before P V of both: with an S each neither waits for the other's P,
-  // which counts where they run side by side through half a list each (4K tokens, 2 heads: 25.3 us of a call, so 24.6).
+  // which counts where they run side by side through half a list each (4K tokens, 2 heads: 25.0 us of a call, so 24.6).
   constexpr bool kTogether = kOwnS && kSplit;
   // A query block of 64 tokens fills half of a tile's rows: the warps of the other half have nothing to do (they used to compute
   // undefined rows; 32K tokens, 32 / 8 heads 2885 us of a call, so 2670).
@@ -623,8 +623,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     bool ok = true;
     // P V of the slot's block before this one is complete (its P may be overwritten, its O read and rescaled)
     auto wait_pv = [&] { return __all_sync(0xffffffffu, mbar_wait(bar(Smem::pv_done, X), (blk & 1) ^ 1, ctx, kBarPvDone)); };
-    // Where a CTA runs one item, each barrier is probed ahead of its wait: the answer takes 150 cycles to come.  (18.8 us of a
-    // call for two ragged prompts, 19.3 without; with both slots busy the probes cost more than they save: 32K tokens 1231 / 1214.)
+    // Where a CTA runs one item, each barrier is probed ahead of its wait: the answer takes 150 cycles to come.  (19.2 us of a
+    // call for two ragged prompts, 20.2 without; with both slots busy the probes cost more than they save: 32K tokens 1281, without
+    // 1269, dense 16K 1800 / 1776.)
     constexpr bool kProbeAhead = kSplit;
     uint32_t s_seen = 0, pv_seen = 0;
     // kTok: row m is query head m % g of the tile's token m / g
@@ -688,8 +689,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
     };
     // O of the blocks so far, whose P V are complete, times alpha.  Before the exponentials this costs a block 550 cycles; once most
-    // of its scores are gone, and P V is long complete, less (32K tokens 1273 / 1263 us, dense 16K 1785 / 1764).  Where a CTA runs
-    // one item (kSplit) that would spill: two ragged short prompts 20.5 us of a call, 19.1 before the exponentials.
+    // of its scores are gone, and P V is long complete, less (dense 16K 1790 / 1776 us of a call, 32K tokens 1264 / 1269).  Where a
+    // CTA runs one item (kSplit) that would spill: two ragged short prompts 20.5 us of a call, 19.1 before the exponentials.
     constexpr bool kRescaleLate = !kSplit;
     auto rescale_o = [&](const float alpha) {
       constexpr int kAtOnce = kSpareQ ? 64 : 32;  // columns
@@ -1285,13 +1286,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       }
     } else if (warp == 11) {
       // ============================== MMA issuer ==============================
-      // Visits the slots in turn.  A visit issues O_X (+)= P V of the slot's previous block, then S_X = Q K^T of its
-      // next block (which overwrites the P just consumed), with the commits that publish them.
+      // Visits the slots in turn.  A visit issues S = Q K^T of the slot's next block, once the softmax has read the S that
+      // was in the columns before, then O_X (+)= P V of the slot's previous block, with the commits that publish them.
+      // Q K^T needs nothing of that P V: P has columns of its own.  Two exceptions: without a spare Q tile, P V of an old
+      // item's last block goes before Q K^T of the new one's first, whose Q tile comes last (swap in visit()); and where each
+      // slot has an S of its own and half a list, Q K^T of both slots go before P V of both (kTogether).
       // This warp is what the tensor core waits for: a visit's 16 MMAs run 1024 cycles, only a few of them can be
       // queued, and every instruction here competes with two softmax warps for issue.  So the waits cost a probe and
       // a branch when there is nothing to wait for, a wait that gave up is looked at once per round, the MMA loops are
-      // unrolled and the list lengths are fetched an item ahead (LengthCursor).  Dense 16K tokens: 1234 TFLOP/s; rolled
-      // loops 1200; waits that return a flag and vote 1053; a second warp that checks ahead and queues commands 1197.
+      // unrolled and the list lengths are fetched an item ahead (LengthCursor).  Dense 16K tokens 1776 us of a call, with
+      // rolled loops 1985.  (With S and P in the same columns, TFLOP/s: so 1234, waits that return a flag and vote 1053, a
+      // second warp that checks ahead and queues commands 1197.)
       Ctx ctx{abort_flag, status, kRoleMma, kGaveUp};
       const bool leader = elect_one();  // one lane issues every MMA and commit (a commit covers its own thread's MMAs)
       enum : uint32_t { kPend = 1u, kFirst = 2u, kLast = 4u, kNewItem = 8u };
