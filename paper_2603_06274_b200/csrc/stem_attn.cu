@@ -762,6 +762,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         continue;
       }
       const bool has_diag = (info >> 31) != 0u;
+      // Rows behind the sequence's last token hold what is packed behind it: they have no vote on the others' references.  (Rows
+      // without a token list are all -inf.)
+      const float threshold = kTok || row_valid ? kRescaleThreshold : INFINITY;
       for (int e = 0; e < n; ++e, ++blk) {
         uint4 mask_w = make_uint4(0, 0, 0, 0);  // kTok: the block's mask words, here while S is still awaited
         if constexpr (kTok) {
@@ -806,8 +809,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
           l_run = 0.f;
           m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
         } else {
-          // (Rows behind the sequence's last token hold what is packed behind it: they have no vote on the others' references.)
-          const bool grow = row_valid && mx_c > m_run + kRescaleThreshold;
+          const bool grow = mx_c > m_run + threshold;
           rescale = __any_sync(0xffffffffu, grow);
           if (rescale) {
             const float m_new = fmaxf(m_run, mx_c);
