@@ -69,11 +69,12 @@ struct AntiArgs {
   const __nv_bfloat16 *Q, *K;
   int64_t q_st, q_sh, kv_st, kv_sh;
   int batch;
-  float* sums;  // over parts of the inner dimension, [slot][Hq][column][row] of the tile; slots: class, part, tile
+  float* sums;  // over parts of the inner dimension (AntidiagTile)
 };
 
-__device__ __forceinline__ float* part_sums(const AntiArgs& a, int slot, int h) {
-  return a.sums + ((int64_t)slot * a.Hq + h) * (kTile * kTile);
+// A part's sums of a square of the tile, [column][row].
+__device__ __forceinline__ float* part_sums(const AntiArgs& a, const AntidiagTile& t, int part, int h, int row32, int col32) {
+  return a.sums + ((int64_t)t.sums_at * a.Hq + ((int64_t)part * a.Hq + h) * (t.rows * t.cols) + col32 * t.rows + row32) * 1024;
 }
 
 // Bounded wait; false when the time limit ran out (the status words then say so).
@@ -133,25 +134,20 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   // The CTAs in order: whole sums first; in a class all tiles and heads of the first part before those of the next, so that the
   // CTAs that run together read the same tokens of all heads, whole rows of Q and K (part by part of a tile and head: eight
   // prompts of 16K tokens 374 us of a call, so 361).
-  int tile = (int)blockIdx.x, y = (int)blockIdx.y, part = (int)blockIdx.z, parts = a.parts, slot = part * (int)gridDim.x + tile;
+  int tile = (int)blockIdx.x, y = (int)blockIdx.y, part = (int)blockIdx.z, parts = a.parts;
   if (parts == 0) {  // tiles of several classes: a grid of one dimension
     int n_tiles = 0, tile0 = 0, rest = tile;
-    slot = 0;
 #pragma unroll 1
     for (int c = 0; c < kAntidiagClasses; ++c) {
       tile0 += n_tiles;
       n_tiles = a.n_tiles[c];
       parts = antidiag_parts(c);
       const int per_part = n_tiles * (a.Hq / kHeads);
-      for (part = 0; part < parts && rest >= per_part; ++part) {
-        rest -= per_part;
-        if (parts > 1) slot += n_tiles;
-      }
+      for (part = 0; part < parts && rest >= per_part; ++part) rest -= per_part;
       if (part < parts) break;
     }
     y = rest / n_tiles;
     tile = tile0 + rest - y * n_tiles;
-    slot += rest - y * n_tiles;
   }
   const AntidiagTile at = a.tiles[tile];
   const int seq = at.seq, ti = at.ti, tj = at.tj;
@@ -247,9 +243,10 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
         tmem_ld32_sync(taddr + gq * 32, v);
         const int x = gq >> 2, c0 = (gq & 3) * 32;
         if (parts > 1) {
-          float* dst = part_sums(a, slot, h + x) + c0 * kTile + m;
+          if (warp >= at.rows || (gq & 3) >= at.cols) continue;
+          float* dst = part_sums(a, at, part, h + x, warp, gq & 3) + lane;
 #pragma unroll
-          for (int c = 0; c < 32; ++c) dst[c * kTile] = v[c];
+          for (int c = 0; c < 32; ++c) dst[c * 32] = v[c];
         } else if (r < nfull) {  // rows of the partial block (or past the end) belong to the other kernel
 #pragma unroll
           for (int c = 0; c < 32; ++c) v[c] = fmaf(a.scale, v[c], bias[c0 + c]);
@@ -275,24 +272,24 @@ constexpr int kSumThreads = kTile * (32 / kSumCols);
 template <int BLK>
 __global__ void __launch_bounds__(kSumThreads, 1024 / kSumThreads) antidiag_sum_kernel(const AntiArgs a) {
   __shared__ float metric[32][kTile];
-  const int n1 = a.n_tiles[1], i = (int)blockIdx.x;
-  const AntidiagTile tile = a.tiles[a.n_tiles[0] + i];
+  const AntidiagTile tile = a.tiles[a.n_tiles[0] + blockIdx.x];
   const int h = blockIdx.y, c0 = blockIdx.z * 32, m = threadIdx.x % kTile, first = threadIdx.x / kTile * kSumCols;
   const int seq = tile.seq, ti = tile.ti, tj = tile.tj;
   const int nb = a.rows.seq_nblk[seq], r0 = a.rows.seq_r0[seq];
   const int nfull = a.rows.kb_ntok[a.rows.seq_kb_first[seq] + nb - 1] == BLK ? nb : nb - 1;
   const int rl = ti * kTile + m;
   const bool row = r0 + rl < nfull;
-  const float* src = part_sums(a, i < n1 ? i : antidiag_parts(1) * n1 + i - n1, h) + (c0 + first) * kTile + m;
+  const float* src = part_sums(a, tile, 0, h, m / 32, blockIdx.z) + first * 32 + m % 32;
   const float* mv = a.mv + (int64_t)(h / a.g) * a.KB_tot + a.rows.seq_kb_off[seq];
-  const int64_t step = (int64_t)(i < n1 ? n1 : a.n_tiles[2]) * a.Hq * (kTile * kTile);
+  const int64_t step = (int64_t)a.Hq * (tile.rows * tile.cols) * 1024;
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if ((int)blockIdx.z >= tile.cols) return;
   auto add_up = [&](auto parts) {
     float v[kSumCols];
 #pragma unroll
     for (int p = 0; p < decltype(parts)::value; ++p) {
 #pragma unroll
-      for (int c = 0; c < kSumCols; ++c) v[c] = p == 0 ? src[c * kTile] : v[c] + src[p * step + c * kTile];
+      for (int c = 0; c < kSumCols; ++c) v[c] = p == 0 ? src[c * 32] : v[c] + src[p * step + c * 32];
     }
 #pragma unroll
     for (int c = 0; c < kSumCols; ++c) {
@@ -301,7 +298,7 @@ __global__ void __launch_bounds__(kSumThreads, 1024 / kSumThreads) antidiag_sum_
     }
   };
   if (row) {
-    if (i < n1) add_up(std::integral_constant<int, antidiag_parts(1)>{});
+    if ((int)blockIdx.x < a.n_tiles[1]) add_up(std::integral_constant<int, antidiag_parts(1)>{});
     else add_up(std::integral_constant<int, antidiag_parts(2)>{});
   }
   __syncthreads();
@@ -468,7 +465,7 @@ int antidiag_heads(const int32_t* n_tiles, int Hq, int g, int sms) {
   return g % 2 == 0 && 3 * done(2) < 2 * done(1) ? 2 : 1;
 }
 
-size_t antidiag_sums_bytes(int slots, int Hq) { return (size_t)slots * Hq * kTile * kTile * sizeof(float); }
+size_t antidiag_sums_bytes(int64_t sums_at, int Hq) { return (size_t)sums_at * Hq * 1024 * sizeof(float); }
 
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s) {

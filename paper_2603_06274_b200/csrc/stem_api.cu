@@ -309,15 +309,16 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
   // Anti-diagonal scoring has work only where a tile holds a full row and a full column.  What a tile costs and what it keeps
   // in the workspace follow from its own sequence, whatever is batched beside it.
   std::vector<AntidiagTile> anti_tiles;
-  int antidiag_slots = 0;
+  int32_t sums_at = 0;
   if (p.score_mode == 1) {
     for (int c = 0; c < kAntidiagClasses; ++c)
       for (size_t i = 0; i < gemm_tiles.size(); i += 3) {
         const int32_t b = gemm_tiles[i], ti = gemm_tiles[i + 1], tj = gemm_tiles[i + 2], n_full = (p.cu[b + 1] - p.cu[b]) / B;
         if (seq_class[b] != c || seq_r0[b] + ti * 128 >= n_full || tj * 128 >= n_full) continue;
-        anti_tiles.push_back({b, ti, tj});
+        auto squares = [](int32_t n) { return (std::min(n, 128) + 31) / 32; };
+        anti_tiles.push_back({b, ti, tj, squares(n_full - seq_r0[b] - ti * 128), squares(n_full - tj * 128), sums_at});
         ++p.n_antidiag_tiles[c];
-        antidiag_slots += c > 0 ? antidiag_parts(c) : 0;
+        if (c > 0) sums_at += antidiag_parts(c) * anti_tiles.back().rows * anti_tiles.back().cols;
       }
     gemm_tiles.clear();
   }
@@ -371,7 +372,7 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
     p.ws.qsplit = off; off = align_up(off + (vectors ? (size_t)3 * p.H_list * p.R_tot * kHeadDim * 2 : 0), 256);
     p.ws.ksplit = off; off = align_up(off + (own_k && vectors ? (size_t)3 * Hkv * p.KB_tot * kHeadDim * 2 : 0), 256);
     p.ws.metric = off; off = align_up(off + (size_t)p.H_list * (size_t)p.mt_tot * 4, 256);
-    p.ws.sums = off; off = align_up(off + antidiag_sums_bytes(antidiag_slots, Hq), 256);
+    p.ws.sums = off; off = align_up(off + antidiag_sums_bytes(sums_at, Hq), 256);
     p.ws.sel_idx = off; off = align_up(off + (size_t)p.H_list * p.R_tot * p.k_max * 4, 256);
     p.ws.sel_cnt = off; off = align_up(off + (size_t)p.H_list * p.R_tot * 4, 256);
     p.ws.total = off;

@@ -43,9 +43,10 @@ struct RowTables {
   const int32_t* kb_new;       // [n_kb_new] indices into the three arrays above of the blocks that the chunk adds
 };
 
-// A tile of the anti-diagonal contraction: sequence, row tile, column tile.
+// A tile of the anti-diagonal contraction: sequence, row tile, column tile.  Where it is summed in parts, the sums of its full rows
+// and columns are kept, in squares of 32: [part][H_q][cols][rows] squares from 1024 H_q sums_at floats on.
 struct AntidiagTile {
-  int32_t seq, ti, tj;
+  int32_t seq, ti, tj, rows, cols, sums_at;
 };
 // In how many parts the inner dimension is summed: the classes of antidiag_class.
 constexpr int kAntidiagClasses = 3;
@@ -58,7 +59,7 @@ struct WorkspaceLayout {
   size_t qsplit = 0;   // bf16 [3, H_list, R_tot, d]: Qbar as hi + mid + lo parts
   size_t ksplit = 0;   // bf16 [3, H_kv, KB_tot, d]: Kbar likewise
   size_t metric = 0;   // uint32 [H_list, mt_tot]: the metric of the fused path as bit planes of its selection keys
-  size_t sums = 0;     // fp32 [slots, H_q, 128, 128]: anti-diagonal scoring, the sums over parts of the inner dimension
+  size_t sums = 0;     // fp32: anti-diagonal scoring, the sums over parts of the inner dimension (AntidiagTile)
   size_t sel_idx = 0;  // int32 [H_list, R_tot, k_max]
   size_t sel_cnt = 0;  // int32 [H_list, R_tot]
   size_t total = 0;
@@ -146,7 +147,7 @@ cudaError_t launch_metric_gemm(const Plan& p, const void* qsplit, const void* ks
 int antidiag_max_sequences();
 int antidiag_class(int64_t n_blocks);
 int antidiag_heads(const int32_t* n_tiles, int Hq, int g, int sms);  // n_tiles: by class
-size_t antidiag_sums_bytes(int slots, int Hq);
+size_t antidiag_sums_bytes(int64_t sums_at, int Hq);
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s);
 

@@ -212,11 +212,17 @@ def test_a_batch_needs_no_more_memory_than_its_sequences_alone(block, seqlens, h
     assert total - lists <= sum(n - l for n, l in alone)
 
 
-def test_the_workspace_has_no_pooled_vectors():
-    # status words, MV, bit planes of the metric, lists; a sequence of more than 384 blocks keeps no sums over parts
-    hq, hkv, nb = 6, 2, 390
-    plan = StemPlan.from_workload(wl.small("ad_ws", seqlens=(128 * nb,), hq=hq, hkv=hkv, block=128, permille=50), score_mode=1)
-    sizes = (32, hkv * nb * 4, hq * nb * ((nb + 31) // 32 * 32) * 4, hq * nb * plan.info.k_max * 4, hq * nb * 4)
+@pytest.mark.parametrize("tokens,sums", [
+    (128 * 390, 0),                                                # more than 384 blocks: no sums over parts
+    (128 * 200 + 1, 3 * (128 * 128 + 96 * 128 + 96 * 96)),         # 200 full blocks: 72 rows and columns beyond the first 128
+    (1500, 8 * 32 * 32),                                           # 11 full blocks
+    (100, 0),                                                      # no full block
+])
+def test_the_workspace_has_no_pooled_vectors(tokens, sums):
+    # status words, MV, bit planes of the metric, the sums over parts of full rows and columns (rounded up to 32), lists
+    hq, hkv, nb = 6, 2, (tokens + 127) // 128
+    plan = StemPlan.from_workload(wl.small("ad_ws", seqlens=(tokens,), hq=hq, hkv=hkv, block=128, permille=50), score_mode=1)
+    sizes = (32, hkv * nb * 4, hq * nb * ((nb + 31) // 32 * 32) * 4, hq * sums * 4, hq * nb * plan.info.k_max * 4, hq * nb * 4)
     assert plan.info.workspace_bytes == sum((n + 255) // 256 * 256 for n in sizes)
     plan.close()
 
