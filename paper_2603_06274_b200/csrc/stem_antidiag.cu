@@ -15,7 +15,8 @@
 // each head, warps 0-3 write the tile as floats (the public M) or as bit planes of the selection keys (the fused path's
 // workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
 // heads share the key tile, 48 KB for two heads' step instead of 64, and short sequences, whose tiles are fewer than the SMs,
-// are computed in parts (antidiag_class), which a small kernel adds up in order.  Lists of a call at 32 / 8 heads, a head and a whole
+// are computed in parts (antidiag_class), which a small kernel adds up in order, or the CTA itself where a batch of them fills the SMs
+// (antidiag_form).  Lists of a call at 32 / 8 heads, a head and a whole
 // sum each / two heads, in parts: 16K tokens 89.8 / 61.2 us, 32K 119.5 / 101.0, 128K 877 / 780.  Only FULL
 // blocks go through the contraction (the maps end at the last full block, so nothing is read past a
 // sequence); a sequence's partial last block, whose anti-diagonal is truncated (the mean is over the
@@ -36,14 +37,16 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
+// Threads of the contraction: the epilogue's warps 0-3, copies, MMAs; where parts are added up in registers, a second head has an
+// epilogue of its own (warps 6-9).
+__host__ __device__ constexpr int antidiag_threads(int heads, bool add) { return add && heads == 2 ? 320 : 192; }
 constexpr int kTile = 128;
 constexpr int kRingTiles = 12;           // operand tiles in the ring: six stages of two, or four of three with two heads
 constexpr int kPartBytes = kTile * 128;  // one operand tile of a step: 128 rows x 64 columns bf16
 constexpr int kSmemBias = kRingTiles * kPartBytes;
-constexpr int kSmemBars = kSmemBias + kTile * 4;  // full[stages], empty[stages], acc_full
+constexpr int kSmemBars = kSmemBias + kTile * 4;  // full[stages], empty[stages], acc_full[2], acc_empty[2]
 constexpr int kStagesMax = kRingTiles / 2;
-constexpr int kSmemTmem = kSmemBars + (2 * kStagesMax + 1) * 8;
+constexpr int kSmemTmem = kSmemBars + (2 * kStagesMax + 4) * 8;
 constexpr int kSmemBytes = kSmemTmem + 16 + 1024;  // slack for manual 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 constexpr uint64_t kWaitLimitNs = 200ull * 1000 * 1000;
@@ -116,8 +119,10 @@ __device__ __forceinline__ void store_columns(const AntiArgs& a, int seq, int h,
   }
 }
 
-template <int BLK, int kHeads>
-__global__ void __launch_bounds__(kThreads, 1)
+// kAdd: a CTA computes all parts of its tile and adds them up itself, in the same order; the parts alternate between two accumulators
+// (a head), so that one is read while the next part is summed.
+template <int BLK, int kHeads, bool kAdd>
+__global__ void __launch_bounds__(antidiag_threads(kHeads, kAdd), 1)
 antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = ((uint32_t)__cvta_generic_to_shared(smem_raw) + 1023u) & ~1023u;
@@ -128,7 +133,9 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   constexpr int kStageBytes = (kHeads + 1) * kPartBytes;  // the key tile, then the heads' query tiles
   auto full = [&](int s) { return bars + 8 * s; };
   auto empty = [&](int s) { return bars + 8 * (kStages + s); };
-  const uint32_t acc_full = bars + 8 * 2 * kStages;
+  auto acc_full = [&](int n) { return bars + 8 * (2 * kStages + (n & 1)); };
+  auto acc_empty = [&](int n) { return bars + 8 * (2 * kStages + 2 + (n & 1)); };
+  constexpr int kTmemCols = kTile * kHeads * (kAdd ? 2 : 1);
   float* bias = (float*)(smem_gen + kSmemBias);
 
   // The CTAs in order: whole sums first; in a class all tiles and heads of the first part before those of the next, so that the
@@ -143,8 +150,9 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
       n_tiles = a.n_tiles[c];
       parts = antidiag_parts(c);
       const int per_part = n_tiles * (a.Hq / kHeads);
-      for (part = 0; part < parts && rest >= per_part; ++part) rest -= per_part;
-      if (part < parts) break;
+      const int shares = kAdd ? 1 : parts;
+      for (part = 0; part < shares && rest >= per_part; ++part) rest -= per_part;
+      if (part < shares) break;
     }
     y = rest / n_tiles;
     tile = tile0 + rest - y * n_tiles;
@@ -160,11 +168,11 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
-    mbar_init(acc_full, 1);
+    for (int n = 0; n < 2; ++n) { mbar_init(acc_full(n), 1); mbar_init(acc_empty(n), 4 * kHeads); }
     mbar_init_fence();
   }
   if (warp == 5) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_base + kSmemTmem), "n"(128 * kHeads)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_base + kSmemTmem), "n"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -173,7 +181,7 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   tc_fence_after();
   const uint32_t tmem = *(volatile uint32_t*)(smem_gen + kSmemTmem);
   constexpr int kIters = 2 * BLK;  // (token of the block, half of the head dimension)
-  const int first = part * kIters / parts, n_iters = (part + 1) * kIters / parts - first;
+  const int first = part * kIters / parts, n_iters = kAdd ? kIters : (part + 1) * kIters / parts - first;
 
   if (warp == 4) {
     // ============================== copies ==============================
@@ -199,12 +207,15 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
     // ============================== MMAs ==============================
     const bool leader = elect_one();
     bool ok = true;
+    int n = 0, start = 0, end = kAdd ? kIters / parts : n_iters;  // part in work (kAdd: of the tile's), its steps
 #pragma unroll 1
     for (int it = 0; it < n_iters && ok; ++it) {
       const int st = it % kStages;
-      ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status, tile, h));
+      if (kAdd && it == start && n >= 2) ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(n), ((n >> 1) - 1) & 1, a.status, tile, h));
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(full(st), (it / kStages) & 1, a.status, tile, h));
       if (!ok) break;
       tc_fence_after();
+      const uint32_t acc = tmem + (kAdd ? (n & 1) * kTile * kHeads : 0);
       if (leader) {
         const uint32_t b_addr = smem_base + st * kStageBytes;
 #pragma unroll
@@ -212,12 +223,17 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
           const uint32_t a_addr = b_addr + (x + 1) * kPartBytes;
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            mma_ss(tmem + x * kTile, smem_desc(a_addr + k * 32), smem_desc(b_addr + k * 32), kIdesc, (it | k) ? 1u : 0u);
+            mma_ss(acc + x * kTile, smem_desc(a_addr + k * 32), smem_desc(b_addr + k * 32), kIdesc, it > start || k > 0 ? 1u : 0u);
         }
         tc_commit(empty(st));
-        if (it == n_iters - 1) tc_commit(acc_full);
+        if (it == end - 1) tc_commit(acc_full(n));
       }
       __syncwarp();
+      if (kAdd && it == end - 1) {
+        ++n;
+        start = end;
+        end = (n + 1) * kIters / parts;
+      }
     }
   } else {
     // ============================== epilogue ==============================
@@ -230,19 +246,57 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
       const int c = threadIdx.x;
       bias[c] = (tj * kTile + c < nb) ? a.beta * a.mv[(int64_t)kvh * a.KB_tot + a.rows.seq_kb_off[seq] + tj * kTile + c] : 0.f;
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // these four warps
-    const int m = warp * 32 + lane;       // row of the tile == TMEM lane
+    asm volatile("bar.sync 1, %0;" ::"n"(antidiag_threads(kHeads, kAdd) - 64) : "memory");  // these warps
+    const int quarter = warp & 3;
+    const int m = quarter * 32 + lane;    // row of the tile == TMEM lane
     const int rl = ti * kTile + m;        // row inside the chunk
     const int r = r0 + rl;                // row inside the sequence
-    if (__all_sync(0xffffffffu, mbar_wait(acc_full, 0, a.status, tile, h))) {
-      tc_fence_after();
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+    // the heads of this warp: all, or (kAdd) the first for warps 0-3 and the second for warps 6-9
+    const int x0 = kAdd && warp > 4 ? 1 : 0, x1 = kAdd ? x0 + 1 : kHeads;
+    bool ok = true;
+    if (kAdd && parts > 1) {
+      float sum[kTile];
+      auto read = [&](int n, auto take) {  // take(columns of the n-th part's accumulator, where they begin)
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_full(n), (n >> 1) & 1, a.status, tile, h));
+        if (!ok) return;
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < kTile; c0 += 32) {
+          float v[32];
+          tmem_ld32_sync(taddr + ((n & 1) * kHeads + x0) * kTile + c0, v);
+          take(v, c0);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty(n));
+      };
+      read(0, [&](const float* v, int c0) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) sum[c0 + c] = v[c];
+      });
 #pragma unroll 1
-      for (int gq = 0; gq < 4 * kHeads; ++gq) {
+      for (int n = 1; n < parts && ok; ++n)
+        read(n, [&](const float* v, int c0) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) sum[c0 + c] += v[c];
+        });
+      // back to tensor memory, whose accumulators are all read by now: what follows has registers for 32 columns
+      if (ok) {
+#pragma unroll
+        for (int gq = 0; gq < 4; ++gq) tmem_st32_sync(taddr + x0 * kTile + gq * 32, sum + gq * 32);
+      }
+    } else {
+      ok = __all_sync(0xffffffffu, mbar_wait(acc_full(0), 0, a.status, tile, h));
+      tc_fence_after();
+    }
+    if (ok) {
+#pragma unroll 1
+      for (int gq = 4 * x0; gq < 4 * x1; ++gq) {
         float v[32];
         tmem_ld32_sync(taddr + gq * 32, v);
         const int x = gq >> 2, c0 = (gq & 3) * 32;
-        if (parts > 1) {
+        if (!kAdd && parts > 1) {
           if (warp >= at.rows || (gq & 3) >= at.cols) continue;
           float* dst = part_sums(a, at, part, h + x, warp, gq & 3) + lane;
 #pragma unroll
@@ -259,7 +313,7 @@ antidiag_metric_kernel(const __grid_constant__ MapSet maps, const AntiArgs a) {
   __syncthreads();
   if (warp == 5) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(128 * kHeads) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
   }
 }
 
@@ -442,30 +496,42 @@ int antidiag_max_sequences() { return kMaxSeqs; }
 // CTAs of 32 heads are a wave of the SMs or more; with fewer heads SMs stay idle there.
 int antidiag_class(int64_t n) { return n <= kTile ? 2 : n <= 3 * kTile ? 1 : 0; }
 
-// How many query heads a CTA computes (two or one of an even group; a head's sums are the same either way).  A step of two heads
-// moves 48 KB into the SM where one moves 32, so two are taken where the last CTA is then done in less than 2/3 of the shares.
-// Us of a call, two heads / one, by the waves of CTAs: 1 against 1: 4 / 2 heads, 400 blocks 124 / 82, 8 / 2, 640 132 / 104; 2 against
-// 3: 16 / 4, 768 290 / 282, 32 / 8, 512 307 / 289; 1 against 2: 8 / 2, 1024 183 / 205, 16 / 4, 512 149 / 169; 3 against 5: 32 / 8, 768
-// 502 / 514; 4 against 8: 32 / 8, 1024 780 / 856.
-int antidiag_heads(const int32_t* n_tiles, int Hq, int g, int sms) {
-  // when the last CTA is done, in 24ths of a tile's sum; CTAs start in order, each on the SM that is free first
-  auto done = [&](int heads) {
+size_t antidiag_sums_bytes(int64_t sums_at, int Hq) { return (size_t)sums_at * Hq * 1024 * sizeof(float); }
+
+// How the contraction is computed: a head or two (of an even group) to a CTA, the parts of a tile by a CTA each or all by one CTA that
+// adds them up.  A head's sums are the same bits in all four forms, so the form follows from what the plan holds.
+// A step of two heads moves 48 KB into the SM where one moves 32, so two are taken where the last CTA is then done in less than 2/3
+// of the steps.  Us of a call, two heads / one, by the waves of CTAs: 1 against 1: 4 / 2 heads, 400 blocks 124 / 82, 8 / 2, 640
+// 132 / 104; 2 against 3: 16 / 4, 768 290 / 282, 32 / 8, 512 307 / 289; 1 against 2: 8 / 2, 1024 183 / 205, 16 / 4, 512 149 / 169; 3
+// against 5: 32 / 8, 768 502 / 514; 4 against 8: 32 / 8, 1024 780 / 856.
+// Sums of parts go through memory, so a CTA takes all parts of its tile where the SMs are busy for 3/4 of the time even so.  Parts
+// apart / added up, by that share: 64 / 8 heads, 32K tokens (0.65) 222 / 243, 28 / 4, 32K (0.57) 93 / 101; 28 / 4, eight prompts of
+// 16K (0.76) 302 / 266, 32 / 8, likewise (0.86) 360 / 297, 64 / 8, likewise 640 / 573, 32 / 8, four of 48K (0.86) 665 / 640.
+AntidiagForm antidiag_form(const int32_t* n_tiles, int Hq, int g, int sms) {
+  int64_t work = 0;  // in 24ths of a tile's sum of a head
+  // when the last CTA is done, likewise; CTAs start in order, each on the SM that is free first
+  auto done = [&](int heads, bool add) {
     std::map<int64_t, int64_t> free_at{{0, sms}};  // SMs by the time they are free
-    for (int c = 0; c < kAntidiagClasses; ++c)
-      for (int64_t left = (int64_t)n_tiles[c] * antidiag_parts(c) * (Hq / heads); left > 0;) {
+    work = 0;
+    for (int c = 0; c < kAntidiagClasses; ++c) {
+      const int parts = add ? 1 : antidiag_parts(c);
+      for (int64_t left = (int64_t)n_tiles[c] * parts * (Hq / heads); left > 0;) {
         const auto first = *free_at.begin();
         const int64_t n = std::min(left, first.second);
         free_at.erase(free_at.begin());
         if (first.second > n) free_at[first.first] = first.second - n;
-        free_at[first.first + 24 / antidiag_parts(c)] += n;
+        free_at[first.first + 24 / parts] += n;
+        work += 24 / parts * n;
         left -= n;
       }
+    }
     return free_at.rbegin()->first;
   };
-  return g % 2 == 0 && 3 * done(2) < 2 * done(1) ? 2 : 1;
+  auto with = [&](bool add) { return AntidiagForm{g % 2 == 0 && 3 * done(2, add) < 2 * done(1, add) ? 2 : 1, add}; };
+  const AntidiagForm added = with(true);
+  const int64_t until = done(added.heads, true);
+  return n_tiles[1] + n_tiles[2] > 0 && 4 * work >= 3 * sms * until ? added : with(false);
 }
-
-size_t antidiag_sums_bytes(int64_t sums_at, int Hq) { return (size_t)sums_at * Hq * 1024 * sizeof(float); }
 
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s) {
@@ -505,20 +571,25 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   for (int c = 0; c < kAntidiagClasses; ++c) {
     a.n_tiles[c] = p.n_antidiag_tiles[c];
     n_tiles += a.n_tiles[c];
-    n_shares += a.n_tiles[c] * antidiag_parts(c);
+    n_shares += a.n_tiles[c] * (p.antidiag.add ? 1 : antidiag_parts(c));
   }
-  const int n_sum = n_tiles - a.n_tiles[0];
-  const bool two = p.antidiag_heads == 2;
+  const int n_sum = p.antidiag.add ? 0 : n_tiles - a.n_tiles[0];
+  const int heads = p.antidiag.heads;
+  const bool add = p.antidiag.add;
+  auto kernel = [&] {
+    auto of = [&](auto blk, auto h) {
+      return add ? antidiag_metric_kernel<decltype(blk)::value, decltype(h)::value, true> : antidiag_metric_kernel<decltype(blk)::value, decltype(h)::value, false>;
+    };
+    auto with = [&](auto blk) { return heads == 2 ? of(blk, std::integral_constant<int, 2>{}) : of(blk, std::integral_constant<int, 1>{}); };
+    return B == 128 ? with(std::integral_constant<int, 128>{}) : with(std::integral_constant<int, 64>{});
+  }();
 
-  static bool attr_set[64] = {};
-  const int dev_slot = p.device & 63;
-  if (!attr_set[dev_slot]) {
-    cudaError_t e = cudaFuncSetAttribute(antidiag_metric_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(antidiag_metric_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  static bool attr_set[64][8] = {};
+  bool& is_set = attr_set[p.device & 63][(B == 128 ? 4 : 0) + heads - 1 + (add ? 2 : 0)];
+  if (!is_set) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    attr_set[dev_slot] = true;
+    is_set = true;
   }
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -526,20 +597,18 @@ cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, 
   cudaError_t e = cudaSuccess;
   if (n_tiles > 0) {
     cudaLaunchConfig_t cfg = {};
-    const unsigned heads = (unsigned)(two ? a.Hq / 2 : a.Hq);
-    cfg.gridDim = dim3((unsigned)n_shares * heads);
+    const unsigned y = (unsigned)(a.Hq / heads);
+    cfg.gridDim = dim3((unsigned)n_shares * y);
     for (int c = 0; c < kAntidiagClasses; ++c)
       if (a.n_tiles[c] == n_tiles) {
         a.parts = antidiag_parts(c);
-        cfg.gridDim = dim3((unsigned)n_tiles, heads, (unsigned)a.parts);
+        cfg.gridDim = dim3((unsigned)n_tiles, y, add ? 1u : (unsigned)a.parts);
       }
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)antidiag_threads(heads, add));
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto kernel = B == 128 ? (two ? antidiag_metric_kernel<128, 2> : antidiag_metric_kernel<128, 1>)
-                           : (two ? antidiag_metric_kernel<64, 2> : antidiag_metric_kernel<64, 1>);
     e = cudaLaunchKernelEx(&cfg, kernel, maps, a);
     if (e != cudaSuccess) return e;
     ++*launched;

@@ -331,7 +331,10 @@ static int create_plan(const stem_config* cfg, const stem_options* opts, stem_pl
   }
 
   p.n_items = p.R_tot * Hq;
-  if (p.score_mode == 1) p.antidiag_heads = antidiag_heads(p.n_antidiag_tiles, Hq, g, p.sm_count);
+  if (p.score_mode == 1) {
+    p.antidiag = antidiag_form(p.n_antidiag_tiles, Hq, g, p.sm_count);
+    if (p.antidiag.add) sums_at = 0;
+  }
 
   Blob blob;
   const size_t o_row_seq = blob.add(row_seq), o_row_r = blob.add(row_r), o_row_tok0 = blob.add(row_tok0),

@@ -48,6 +48,11 @@ struct RowTables {
 struct AntidiagTile {
   int32_t seq, ti, tj, rows, cols, sums_at;
 };
+// Query heads to a CTA; whether a CTA adds up all parts of its tile.
+struct AntidiagForm {
+  int heads = 1;
+  bool add = false;
+};
 // In how many parts the inner dimension is summed: the classes of antidiag_class.
 constexpr int kAntidiagClasses = 3;
 __host__ __device__ constexpr int antidiag_parts(int c) { return c == 0 ? 1 : c == 1 ? 3 : 8; }
@@ -90,7 +95,7 @@ struct Plan {
   // Anti-diagonal scoring: the tiles with a full row and a full column, class by class.
   const AntidiagTile* d_antidiag_tiles = nullptr;
   int32_t n_antidiag_tiles[kAntidiagClasses] = {0, 0, 0};
-  int32_t antidiag_heads = 1;  // query heads a CTA
+  AntidiagForm antidiag;
   int32_t score_mode = 0;     // 0: product of block means (Eq. 7 on pooled blocks); 1: anti-diagonal scoring
   std::vector<int32_t> h_seq_r0, h_seq_qtok0;  // host copies: first chunk row, first packed Q token of every sequence
   int32_t H_list = 0;         // heads of the metric and of the lists: H_q, or H_kv with share_group
@@ -146,7 +151,7 @@ cudaError_t launch_metric_gemm(const Plan& p, const void* qsplit, const void* ks
 // *launched receives the number of kernels enqueued.
 int antidiag_max_sequences();
 int antidiag_class(int64_t n_blocks);
-int antidiag_heads(const int32_t* n_tiles, int Hq, int g, int sms);  // n_tiles: by class
+AntidiagForm antidiag_form(const int32_t* n_tiles, int Hq, int g, int sms);  // n_tiles: by class
 size_t antidiag_sums_bytes(int64_t sums_at, int Hq);
 cudaError_t launch_antidiag_metric(const Plan& p, const void* Q, const void* K, const float* mv, float* M, bool as_keys, float* sums,
                                    int32_t* status, int* launched, cudaStream_t s);

@@ -312,3 +312,34 @@ def test_lists_of_a_chunk_are_those_of_the_whole_sequence(block, n, q_start, hq,
         plan.close()
     assert row == whole.info.total_q_blocks
     whole.close()
+
+
+@pytest.mark.parametrize("block,seqlens,hq,hkv", [
+    (64, (64 * 100,) * 7 + (64 * 100 + 33,), 32, 8),      # eight parts, two heads to a CTA
+    (64, (64 * 250, 64 * 300 + 1, 64 * 200, 64 * 384), 28, 4),  # three parts, an odd group
+    (128, (128 * 100 + 100, 128 * 260, 128 * 390), 32, 8),  # all three kinds of sums
+])
+def test_parts_of_a_batch_that_fills_the_sms(block, seqlens, hq, hkv):
+    # A CTA adds up the parts of a tile where the batch fills the SMs (no room for sums then): the bits of each sequence alone.
+    n = sum(seqlens)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    q, k, v = (torch.randn((n, h, 128), generator=gen, device="cuda").to(torch.bfloat16) for h in (hq, hkv, hkv))
+
+    def scores(lens, q, k, v):
+        plan = StemPlan(lens, hq, hkv, block=block, budget_permille=50, score_mode=1)
+        M = torch.full((hq, plan.info.metric_elems), float("nan"), dtype=torch.float32, device="cuda")
+        binding.stem_score(plan, q, k, v, M)
+        idx, cnt = _lists_of(plan, q, k, v)
+        plan.close()
+        return M.nan_to_num(7e30), idx, cnt, plan.info
+
+    M, idx, cnt, info = scores(seqlens, q, k, v)
+    tok = off = row = 0
+    for length in seqlens:
+        part = slice(tok, tok + length)
+        M1, idx1, cnt1, info1 = scores((length,), q[part], k[part], v[part])
+        rows = slice(row, row + info1.total_q_blocks)
+        assert torch.equal(M1, M[:, off:off + info1.metric_elems])
+        assert np.array_equal(idx1, idx[:, rows, :info1.k_max]) and (idx[:, rows, info1.k_max:] == -1).all()
+        assert np.array_equal(cnt1, cnt[:, rows])
+        tok, off, row = part.stop, off + info1.metric_elems, rows.stop
