@@ -10,7 +10,7 @@
 // block, block) lets one TMA box fetch "64 columns of token t of 128 consecutive blocks" as a 128-row
 // K-major operand tile; the query map is walked with t = B-1-s, the key map with t = s.
 //
-// One CTA per (128 x 128 tile of one sequence's causal triangle, two query heads of a group or one (antidiag_heads),
+// One CTA per (128 x 128 tile of one sequence's causal triangle, two query heads of a group or one,
 // part of the inner dimension): warp 4 issues the copies through a ring of stages, warp 5 the MMAs into a TMEM accumulator for
 // each head, warps 0-3 write the tile as floats (the public M) or as bit planes of the selection keys (the fused path's
 // workspace form).  What bounds it is how fast operand tiles enter an SM (they come from the L2 at up to 64 bytes a cycle): two
