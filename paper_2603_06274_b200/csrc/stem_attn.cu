@@ -762,9 +762,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         continue;
       }
       const bool has_diag = (info >> 31) != 0u;
-      // Rows behind the sequence's last token hold what is packed behind it: they have no vote on the others' references.  (Rows
-      // without a token list are all -inf.)
-      const float threshold = kTok || row_valid ? kRescaleThreshold : INFINITY;
+      // Rows behind the sequence's last token hold what is packed behind it: they have no vote on the others' references, whatever
+      // their scores.  (Their O is not written; rows without a token list are all -inf.)  Blocks of 128: an infinite threshold; blocks
+      // of 64: an infinite reference, which needs no register in the loop.  Threshold / reference, us of a call: 64K + 40K tokens, 28 / 4
+      // heads 3177 / 3204; blocks of 64, dense: 6099 tokens, 64 / 8 heads 1193 / 1174, 16K, 32 / 8 4145 / 4055.
+      const bool no_vote = !kTok && !row_valid;
+      const float threshold = BLK == 128 && no_vote ? INFINITY : kRescaleThreshold;
       for (int e = 0; e < n; ++e, ++blk) {
         uint4 mask_w = make_uint4(0, 0, 0, 0);  // kTok: the block's mask words, here while S is still awaited
         if constexpr (kTok) {
@@ -807,7 +810,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (e == 0) {
           if (kDefer && d_has && !(ok = write_deferred())) break;
           l_run = 0.f;
-          m_run = fmaxf(mx_c, -FLT_MAX);  // finite: the row's list may name no token of the block, or all scores may be -inf
+          // finite where the row counts: its list may name no token of the block, or all scores may be -inf
+          m_run = BLK == 64 && no_vote ? INFINITY : fmaxf(mx_c, -FLT_MAX);
         } else {
           const bool grow = mx_c > m_run + threshold;
           rescale = __any_sync(0xffffffffu, grow);

@@ -629,7 +629,7 @@ def test_row_maxima_that_grow_from_block_to_block(block, seqlen, hq, hkv, dense)
 ])
 def test_a_sequence_does_not_see_what_is_packed_behind_it(block, seqlens, hq, hkv, dense):
     # The rows of a tile behind a sequence's last token hold the next sequence's queries.  Nothing of them may reach the rows
-    # before: the same bits, whether their scores are about 1 or about 2^60 (which outgrows every reference).
+    # before: the same bits, whether their scores are about 1, about 2^60 (which outgrows every reference) or not finite.
     w = wl.small("behind", seqlens=seqlens, hq=hq, hkv=hkv, block=block, permille=400, seed=sum(seqlens))
     data, plan, q, k, v = _setup(w)
     n = seqlens[0]
@@ -637,7 +637,7 @@ def test_a_sequence_does_not_see_what_is_packed_behind_it(block, seqlens, hq, hk
     binding.stem_score_select(plan, q, k, v, idx, cnt)
     lists = (None, None) if dense else (idx, cnt)
     got = []
-    for scale in (1.0, 2.0 ** 30):
+    for scale in (1.0, 2.0 ** 30, float("inf")):
         q[n:] *= scale
         k[n:] *= scale
         out = torch.full((w.total_tokens, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
@@ -646,5 +646,6 @@ def test_a_sequence_does_not_see_what_is_packed_behind_it(block, seqlens, hq, hk
         _ok(plan)
         got.append((out[:n].clone(), lse[:, :n].clone()))
     assert torch.isfinite(got[0][0].float()).all()
-    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    for o, l in got[1:]:
+        assert torch.equal(got[0][0], o) and torch.equal(got[0][1], l)
     plan.close()
